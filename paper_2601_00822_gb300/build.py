@@ -42,6 +42,7 @@ UNITS = [
     ("solver.cu", [], "solver.o"),
     ("noalloc.cu", [], "noalloc.o"),
     ("unet.cu", [], "unet.o"),
+    ("unet_conv.cu", [], "unet_conv.o"),
 ]
 
 

@@ -16,9 +16,7 @@
 // channels, K = voxels) staged through shared memory with ldmatrix.trans,
 // split over voxel chunks and reduced in a fixed order (deterministic).
 #include "bfcs.h"
-#include "kernels.h"
-
-#include <cuda_bf16.h>
+#include "unet_kernels.h"
 
 #include <algorithm>
 #include <cmath>
@@ -29,14 +27,6 @@
 
 namespace bfcs {
 namespace net {
-
-typedef __nv_bfloat16 bf16;
-
-constexpr float kSlope = 0.1f;
-
-struct Vol { int nx, ny, nz; };
-
-__device__ __forceinline__ int wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
 __device__ __forceinline__ unsigned ld32(const bf16* p) { return *reinterpret_cast<const unsigned*>(p); }
 
@@ -61,28 +51,6 @@ __device__ __forceinline__ void ldsm_x4_trans(unsigned* r, const void* smem_row)
 }
 
 // ------------------------------------------------------------------ convolution (forward / data gradient)
-enum InMode : int { IN_CONV = 0, IN_GATHER_UP = 1 };
-enum OutMode : int { OUT_BF16 = 0, OUT_SHUFFLE_UP = 1, OUT_F32 = 2 };
-
-struct ConvArgs {
-  const bf16* in;     // channels-last input: element (voxel, k) at in[voxel * ldi + offi + k]
-  int ldi, offi;
-  int cin;            // GEMM K per tap (multiple of 16)
-  const bf16* w;      // [tap][cout_p][cin], K fastest
-  const float* bias;  // bias[col % bias_mod], or null
-  int bias_mod;
-  int cout_p;         // GEMM columns (multiple of 8)
-  int cout;           // columns stored (OUT_F32)
-  int ksize;          // 1 or 3 (circular)
-  Vol v;              // grid of the GEMM rows (coarse grid for the gather / shuffle modes)
-  int batch;
-  int act;            // 1: leaky ReLU
-  int in_mode, out_mode;
-  void* out;          // channels-last output, element (voxel, col) at out[voxel * ldo + offo + col]
-  int ldo, offo;
-  int up_c;           // gather / shuffle: channels per sub-voxel (multiple of 16)
-};
-
 constexpr int kConvWarps = 4;
 constexpr int kConvNT = 8;   // n8 tiles per block (64 columns)
 
@@ -190,16 +158,7 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
   }
 }
 
-// Tiled 3^3 convolution (IN_CONV, OUT_BF16): a block computes a 16 x 8 x 2
-// voxel tile for 32 output columns.  The tile's circular halo (18 x 10 x 4
-// voxels, all cin channels) is staged once in shared memory with cp.async;
-// A fragments come from it by ldmatrix (rows = 16 consecutive x voxels, one
-// 16-byte chunk of 8 channels per row).  Chunk c of halo voxel v sits at
-// chunk c ^ ((v >> sh) & (chunks - 1)): 8 consecutive voxels then hit 8
-// distinct 16-byte bank groups (conflict-free ldmatrix) for cin = 16, 32, 64.
-// B fragments (weights, at most 110 KB per layer) are read from L1/L2.
-// Needs nx % 16 == 0, ny % 8 == 0, nz % 2 == 0, cin in {16, 32, 64}, ldi and
-// offi multiples of 8.
+// Voxel tile and circular halo of the tiled weight gradient (k_wgrad3t).
 constexpr int kTX = 16, kTY = 8, kTZ = 2;
 constexpr int kHX = kTX + 2, kHY = kTY + 2, kHZ = kTZ + 2, kHalo = kHX * kHY * kHZ;
 
@@ -209,345 +168,6 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::);
-}
-__device__ __forceinline__ void ldsm_x4(unsigned* r, unsigned saddr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(saddr));
-}
-
-size_t conv3t_smem(int cin) { return (size_t)kHalo * cin * sizeof(bf16); }
-
-__global__ void __launch_bounds__(128) k_conv3t(ConvArgs a) {
-  extern __shared__ __align__(128) unsigned char smh[];
-  const int chunks = a.cin >> 3;
-  const int sh = chunks == 8 ? 0 : chunks == 4 ? 1 : 2;
-  const int rowb = a.cin * 2;
-  const int ntx = a.v.nx / kTX, nty = a.v.ny / kTY;
-  int tb = blockIdx.x;
-  const int x0 = (tb % ntx) * kTX;
-  tb /= ntx;
-  const int y0 = (tb % nty) * kTY, z0 = (tb / nty) * kTZ;
-  const int b = blockIdx.z;
-  const long long nvox = (long long)a.v.nx * a.v.ny * a.v.nz;
-  const bf16* inb = a.in + (long long)b * nvox * a.ldi + a.offi;
-  for (int i = threadIdx.x; i < kHalo * chunks; i += blockDim.x) {
-    const int v = i / chunks, c = i - v * chunks;
-    const int hx = v % kHX, hy = (v / kHX) % kHY, hz = v / (kHX * kHY);
-    const int gx = wrap(x0 + hx - 1, a.v.nx), gy = wrap(y0 + hy - 1, a.v.ny), gz = wrap(z0 + hz - 1, a.v.nz);
-    const bf16* src = inb + (((long long)gz * a.v.ny + gy) * a.v.nx + gx) * a.ldi + c * 8;
-    cp_async16(smh + v * rowb + 16 * (c ^ ((v >> sh) & (chunks - 1))), src);
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, t = lane & 3;
-  const int col0 = blockIdx.y * 32;
-  const int ntiles = min(4, (a.cout_p - col0) / 8);
-  float acc[4][4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
-  int rowv[4];   // halo index of x = 0 of this warp's tile rows, plus the ldmatrix row of this lane
-  const int lrow = (lane & 7) + ((lane >> 3) & 1) * 8, lk = lane >> 4;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = warp * 4 + q;
-    rowv[q] = ((r / kTY + 1) * kHY + (r % kTY + 1)) * kHX + 1 + lrow;
-  }
-  const unsigned sbase = (unsigned)__cvta_generic_to_shared(smh);
-  for (int tap = 0; tap < 27; ++tap) {
-    const int doff = ((tap / 9 - 1) * kHY + ((tap / 3) % 3 - 1)) * kHX + (tap % 3 - 1);
-    const bf16* wt = a.w + (long long)tap * a.cout_p * a.cin + (long long)(col0 + g) * a.cin + 2 * t;
-    for (int kc = 0; kc < a.cin; kc += 16) {
-      const int c = (kc >> 3) + lk;
-      unsigned af[4][4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int v = rowv[q] + doff;
-        ldsm_x4(af[q], sbase + v * rowb + 16 * (c ^ ((v >> sh) & (chunks - 1))));
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j < ntiles) {
-          const bf16* wr = wt + (long long)j * 8 * a.cin + kc;
-          const unsigned bfr[2] = {ld32(wr), ld32(wr + 8)};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) mma16816(acc[q][j], af[q], bfr);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int r = warp * 4 + q;
-    const int y = y0 + r % kTY, z = z0 + r / kTY;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const long long vox = ((long long)z * a.v.ny + y) * a.v.nx + x0 + g + 8 * h;
-      bf16* orow = (bf16*)a.out + ((long long)b * nvox + vox) * a.ldo + a.offo;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j >= ntiles) continue;
-        const int col = col0 + j * 8 + 2 * t;
-        float v0 = acc[q][j][2 * h], v1 = acc[q][j][2 * h + 1];
-        if (a.bias != nullptr) {
-          v0 += a.bias[col % a.bias_mod];
-          v1 += a.bias[(col + 1) % a.bias_mod];
-        }
-        if (a.act) {
-          v0 = v0 > 0.f ? v0 : kSlope * v0;
-          v1 = v1 > 0.f ? v1 : kSlope * v1;
-        }
-        *reinterpret_cast<__nv_bfloat162*>(orow + col) = __floats2bfloat162_rn(v0, v1);
-      }
-    }
-  }
-}
-
-bool conv3t_ok(const ConvArgs& a) {
-  return a.ksize == 3 && a.in_mode == IN_CONV && a.out_mode == OUT_BF16 && a.v.nx % kTX == 0 &&
-         a.v.ny % kTY == 0 && a.v.nz % kTZ == 0 && (a.cin == 16 || a.cin == 32 || a.cin == 64) &&
-         a.ldi % 8 == 0 && a.offi % 8 == 0 && a.cout_p % 8 == 0;
-}
-
-// ------------------------------------------------------------------ tcgen05 convolution
-// 3^3 circular convolution on the 5th-generation tensor cores (tcgen05.mma,
-// kind::f16, BF16 operands, FP32 accumulator in tensor memory).  A persistent
-// block of 4 warps keeps the layer's weights in shared memory and walks
-// 128-voxel tiles (8 x-voxels x 16 y-rows x 1 z-slab).  Per tile the circular
-// halo (10 x 18 x 3 voxels, all cin channels) is staged with cp.async in the
-// canonical K-major no-swizzle layout: 8-channel chunk c of halo voxel v at
-// byte (c * NV + v) * 16.  Eight consecutive x-voxels then form one 8 x 16 B
-// core matrix, the next tile row (y + 1) sits HX voxels further (the stride
-// between 8-row groups, SBO) and the next channel chunk NV voxels further
-// (the stride along K, LBO) - so the A operand of every tap is the same
-// descriptor at a different start address.  Weights: chunk c of output
-// channel n of tap t at ((t * KC + c) * N + n) * 16 (SBO = 128 B, LBO = N * 16).
-// One thread issues 27 * cin / 16 MMAs of 128 x N x 16 into the accumulator,
-// tcgen05.commit arrives on an mbarrier, and the four warps read their 32
-// TMEM lanes (= tile voxels) back for bias, activation and the BF16 store.
-// Needs nx % 8 == 0, ny % 16 == 0, cin in {16, 32, 64}, cout_p in {32, 64},
-// IN_CONV / OUT_BF16, ldi, offi, ldo, offo multiples of 8.
-constexpr int kTcX = 8, kTcY = 16;
-constexpr int kTcHX = kTcX + 2, kTcHY = kTcY + 2, kTcHZ = 3, kTcNV = kTcHX * kTcHY * kTcHZ;
-constexpr unsigned kTcSpinLimit = 1u << 26;    // bounded wait on the MMA completion barrier
-
-// nbuf halo buffers (each rounded to 1 KB) + weights
-size_t conv3tc_smem(int cin, int n, int nbuf) {
-  return nbuf * (((size_t)kTcNV * (cin / 8) * 16 + 1023) / 1024 * 1024) + (size_t)27 * (cin / 8) * n * 16;
-}
-// two halo buffers only where two blocks still fit on an SM (measured: two
-// co-resident blocks beat one double-buffered block for the 32-channel layers)
-int conv3tc_nbuf(int cin, int n) { return conv3tc_smem(cin, n, 2) <= 111 * 1024 ? 2 : 1; }
-
-__device__ __forceinline__ uint64_t umma_sdesc(unsigned saddr, unsigned lbo, unsigned sbo) {
-  // start address, leading (K) and stride (M/N) byte offsets in 16-byte units,
-  // descriptor version 1 (bit 46), no swizzle, base offset 0
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
-}
-// instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
-// (bits 7-9 and 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-__device__ __forceinline__ unsigned umma_idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
-}
-
-// Pipelined: with two halo buffers (nbuf = 2) the halo of tile k+1 streams in
-// and the epilogue of tile k-1 runs while the tensor cores work on tile k (two
-// TMEM accumulators of N columns); with one buffer the next halo waits for
-// the current tile's MMAs.
-constexpr int kTcThreads = 256;   // 8 warps: warps w and w + 4 share TMEM lanes 32 (w % 4) .. + 31
-
-__global__ void __launch_bounds__(kTcThreads, 2) k_conv3_tc(ConvArgs a, int* err, int nbuf) {
-  extern __shared__ __align__(1024) unsigned char smt[];
-  __shared__ __align__(8) unsigned long long mbar[2];
-  __shared__ unsigned tmem_base_s;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int KC = a.cin >> 3, N = a.cout_p;
-  const unsigned h_stride = ((unsigned)kTcNV * KC * 16u + 1023u) & ~1023u;   // one halo buffer
-  unsigned char* sw = smt + nbuf * h_stride;                                 // weights after the halos
-  const unsigned sh_a = (unsigned)__cvta_generic_to_shared(smt);
-  const unsigned sw_a = (unsigned)__cvta_generic_to_shared(sw);
-  const unsigned mbar_a0 = (unsigned)__cvta_generic_to_shared(&mbar[0]);
-  const long long nvox = (long long)a.v.nx * a.v.ny * a.v.nz;
-  const int ntx = a.v.nx / kTcX, nty = a.v.ny / kTcY;
-  const int tiles_ps = ntx * nty * a.v.nz;
-  const int total = tiles_ps * a.batch;
-  const int G = gridDim.x;
-  // a network whose tensor-core wait once expired launches no more tensor-core
-  // work: the flag is sticky until the context is destroyed (see the exit below)
-  // (one thread reads it, so every thread of the block takes the same branch)
-  if (__syncthreads_or(tid == 0 && *(volatile int*)err != 0)) return;
-
-  if (warp == 0) {   // tensor memory: 2 accumulators of N FP32 columns x 128 lanes
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(&tmem_base_s);
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dst), "r"(2 * N));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
-  }
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mbar_a0));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mbar_a0 + 8));
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
-  }
-  for (int i = tid; i < 27 * N * KC; i += blockDim.x) {   // weights (core-matrix layout)
-    const int c = i % KC, n = (i / KC) % N, tap = i / (KC * N);
-    cp_async16(sw + ((tap * KC + c) * N + n) * 16, a.w + ((long long)tap * N + n) * a.cin + c * 8);
-  }
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-
-  struct TileXY { int b, x0, y0, z0; };
-  auto tile_of = [&](int t) {
-    TileXY r;
-    r.b = t / tiles_ps;
-    int tt = t - r.b * tiles_ps;
-    r.x0 = (tt % ntx) * kTcX;
-    tt /= ntx;
-    r.y0 = (tt % nty) * kTcY;
-    r.z0 = tt / nty;
-    return r;
-  };
-  auto issue_halo = [&](int t, int buf) {
-    const TileXY q = tile_of(t);
-    unsigned char* sh = smt + buf * h_stride;
-    const bf16* inb = a.in + (long long)q.b * nvox * a.ldi + a.offi;
-    for (int i = tid; i < kTcNV * KC; i += blockDim.x) {
-      const int v = i / KC, c = i - v * KC;
-      const int hx = v % kTcHX, hy = (v / kTcHX) % kTcHY, hz = v / (kTcHX * kTcHY);
-      const int gx = wrap(q.x0 + hx - 1, a.v.nx), gy = wrap(q.y0 + hy - 1, a.v.ny),
-                gz = wrap(q.z0 + hz - 1, a.v.nz);
-      cp_async16(sh + (c * kTcNV + v) * 16, inb + (((long long)gz * a.v.ny + gy) * a.v.nx + gx) * a.ldi + c * 8);
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  };
-  bool ok = true;
-  // bounded wait for the k-th commit on barrier k % 2 (its (k / 2)-th phase); one decision per block
-  auto wait_mma = [&](int k) {
-    const unsigned bar = mbar_a0 + 8u * (unsigned)(k & 1), parity = (unsigned)((k >> 1) & 1);
-    unsigned done = 0, spins = 0;
-    while (!done) {
-      asm volatile(
-          "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
-          : "=r"(done)
-          : "r"(bar), "r"(parity)
-          : "memory");
-      if (!done && ++spins > kTcSpinLimit) break;
-    }
-    if (__syncthreads_or(!done)) {
-      if (tid == 0) atomicExch(err, 1);
-      ok = false;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  };
-  auto epilogue = [&](const TileXY& q, int slot) {
-    const int quarter = warp & 3, half = warp >> 2;
-    const int r = quarter * 32 + lane;   // TMEM lane = tile voxel (x = r % 8, y = r / 8)
-    const long long vox = ((long long)q.z0 * a.v.ny + q.y0 + r / kTcX) * a.v.nx + q.x0 + r % kTcX;
-    bf16* orow = (bf16*)a.out + ((long long)q.b * nvox + vox) * a.ldo + a.offo;
-    for (int c0 = half * 16; c0 < N; c0 += 32) {   // this warp's 16-column slices
-      unsigned v[16];
-      const unsigned taddr = tmem_base_s + ((unsigned)(quarter * 32) << 16) + (unsigned)(slot * N + c0);
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(taddr));
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-      for (int q8 = 0; q8 < 16; q8 += 8) {
-        __align__(16) __nv_bfloat162 o[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int col = c0 + q8 + 2 * u;
-          float f0 = __uint_as_float(v[q8 + 2 * u]), f1 = __uint_as_float(v[q8 + 2 * u + 1]);
-          if (a.bias != nullptr) {
-            f0 += a.bias[col % a.bias_mod];
-            f1 += a.bias[(col + 1) % a.bias_mod];
-          }
-          if (a.act) {
-            f0 = f0 > 0.f ? f0 : kSlope * f0;
-            f1 = f1 > 0.f ? f1 : kSlope * f1;
-          }
-          o[u] = __floats2bfloat162_rn(f0, f1);
-        }
-        *reinterpret_cast<uint4*>(orow + c0 + q8) = *reinterpret_cast<const uint4*>(o);
-      }
-    }
-  };
-
-  const unsigned idesc = umma_idesc_bf16(128, N);
-  int t = blockIdx.x, k = 0;
-  TileXY prev{};
-  if (t < total) issue_halo(t, 0);
-  for (; t < total && ok; t += G, ++k) {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");   // weights and halo of tile k
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      const unsigned d_tmem = tmem_base_s + (unsigned)((k & 1) * N);
-      // descriptors of tap 0, chunk 0; later MMAs only move the start address
-      // (16-byte units in the low bits, which never carry past bit 13 here)
-      const uint64_t ad0 = umma_sdesc(sh_a + (unsigned)(k % nbuf) * h_stride, kTcNV * 16, kTcHX * 16);
-      const uint64_t bd0 = umma_sdesc(sw_a, N * 16, 128);
-      int first = 1;
-#pragma unroll 1
-      for (int tap = 0; tap < 27; ++tap) {
-        const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-        const unsigned aoff = (unsigned)((dz * kTcHY + dy) * kTcHX + dx);        // 16-byte units
-#pragma unroll 4
-        for (int kk = 0; kk < KC; kk += 2) {
-          const uint64_t ad = ad0 + aoff + (unsigned)(kk * kTcNV);
-          const uint64_t bd = bd0 + (unsigned)((tap * KC + kk) * N);
-          asm volatile(
-              "{\n.reg .pred p;\nsetp.eq.u32 p, %4, 0;\n"            // p: accumulate into D (not the first MMA)
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(first));
-          first = 0;
-        }
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                       mbar_a0 + 8u * (unsigned)(k & 1))
-                   : "memory");
-    }
-    const TileXY cur = tile_of(t);
-    if (k >= 1) {   // tile k-1: its MMAs are done, its accumulator is read while tile k's MMAs run
-      wait_mma(k - 1);
-      if (ok) epilogue(prev, (k - 1) & 1);
-    }
-    if (ok && t + G < total) {
-      if (nbuf == 1) wait_mma(k);   // the only halo buffer is still being read by tile k's MMAs
-      if (ok) issue_halo(t + G, (k + 1) % nbuf);
-    }
-    prev = cur;
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-  }
-  if (ok && k >= 1) {
-    wait_mma(k - 1);
-    if (ok) epilogue(prev, (k - 1) & 1);
-  }
-  // After an expired wait (ok == false) the MMAs of the last commit may still be
-  // in flight when the columns are released below: the contents of this CTA's
-  // TMEM columns are then undefined, and so would be a later CTA's accumulator
-  // placed in them.  The error flag is set before this point and is sticky, so
-  // no later tensor-core launch of this network runs and bfcs_net_status
-  // reports BFCS_ERR_TIMEOUT for every result from then on.
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base_s), "r"(2 * N));
-}
-
-bool conv3tc_ok(const ConvArgs& a) {
-  return a.ksize == 3 && a.in_mode == IN_CONV && a.out_mode == OUT_BF16 && a.v.nx % kTcX == 0 &&
-         a.v.ny % kTcY == 0 && (a.cin == 16 || a.cin == 32 || a.cin == 64) && (a.cout_p == 32 || a.cout_p == 64) &&
-         a.ldi % 8 == 0 && a.offi % 8 == 0 && a.ldo % 8 == 0 && a.offo % 8 == 0 &&
-         conv3tc_smem(a.cin, a.cout_p, 1) <= 225 * 1024;
 }
 
 // ------------------------------------------------------------------ weight gradient
@@ -1179,20 +799,9 @@ bool tcgen05_enabled() {
 }
 
 cudaError_t launch_conv(const ConvArgs& a, long long nvox, int* err, cudaStream_t st) {
-  if (tcgen05_enabled() && conv3tc_ok(a)) {
-    const long long tiles = (long long)(a.v.nx / kTcX) * (a.v.ny / kTcY) * a.v.nz * a.batch;
-    const int nbuf = conv3tc_nbuf(a.cin, a.cout_p);
-    const size_t smem = conv3tc_smem(a.cin, a.cout_p, nbuf);
-    const int per_sm = std::max(1, std::min(2, (int)((227 * 1024) / (smem + 2048))));
-    const int blocks = (int)std::min<long long>(tiles, (long long)sm_count() * per_sm);
-    k_conv3_tc<<<blocks, kTcThreads, smem, st>>>(a, err, nbuf);
-  } else if (conv3t_ok(a)) {
-    const int tiles = (a.v.nx / kTX) * (a.v.ny / kTY) * (a.v.nz / kTZ);
-    k_conv3t<<<dim3(tiles, ceil_div(a.cout_p, 32), a.batch), 128, conv3t_smem(a.cin), st>>>(a);
-  } else {
-    k_conv<<<dim3(ceil_div(nvox, kConvWarps * 32), ceil_div(a.cout_p, kConvNT * 8), a.batch), kConvWarps * 32, 0,
-             st>>>(a);
-  }
+  if (conv3_ok(a) && tcgen05_enabled()) return launch_conv3(a, sm_count(), err, st);
+  k_conv<<<dim3(ceil_div(nvox, kConvWarps * 32), ceil_div(a.cout_p, kConvNT * 8), a.batch), kConvWarps * 32, 0,
+           st>>>(a);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1500,9 +1109,7 @@ int bfcs_net_create(bfcs_net* out, int nx, int ny, int nz, int max_batch, int fl
     *r.first = N->base + pos;
     pos += (r.second + 255) / 256 * 256;
   }
-  if (cudaFuncSetAttribute(k_conv3t, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv3t_smem(64)) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(k_conv3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024) != cudaSuccess ||
+  if (conv3_init() != cudaSuccess ||
       cudaFuncSetAttribute(k_wgrad3t, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad3t_smem(64)) !=
           cudaSuccess) {
     cudaGetLastError();

@@ -170,3 +170,23 @@ def test_trained_warm_start_reduces_sweeps_and_matches_cold_solver():
     assert res["batched_warm"]["mean_sweeps"] < res["batched_cold"]["mean_sweeps"], res
     assert res["batched_warm"]["max_resid"] <= 1e-6 and res["batched_cold"]["max_resid"] <= 1e-6
     assert res["warm_vs_cold_eps_rel_l2_max"] < 1e-5, res
+
+
+@pytest.mark.parametrize("dims,batch", [((8, 8, 8), 1), ((40, 24, 16), 2), ((16, 8, 72), 3), ((24, 56, 8), 1),
+                                        ((64, 48, 64), 5)])
+def test_tensor_core_convolutions_equal_the_warp_level_ones_bit_for_bit(dims, batch, monkeypatch):
+    """Both forms sum each output's products in the same order (taps, then blocks of 16
+    channels, FP32 accumulators), so partial tiles, tiles that cross a column of planes,
+    blocks with one tile and blocks with many must reproduce the plain kernels exactly."""
+    flat = params(21).float().cuda()
+    x = inputs(22, batch, dims).float().cuda()
+    t = inputs(23, batch, dims, ch=6).float().cuda()
+    net = api.Net(dims, max_batch=batch, train=True)
+    out = []
+    for on in ("1", "0"):
+        monkeypatch.setenv("BFCS_NET_TCGEN05", on)
+        g, loss = net.grad(flat, x, t)
+        out.append((net.forward(flat, x).clone(), g.clone(), loss.clone()))
+    net.status()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
