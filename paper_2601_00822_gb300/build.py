@@ -43,6 +43,7 @@ UNITS = [
     ("noalloc.cu", [], "noalloc.o"),
     ("unet.cu", [], "unet.o"),
     ("unet_conv.cu", [], "unet_conv.o"),
+    ("unet_gemm.cu", [], "unet_gemm.o"),
 ]
 
 

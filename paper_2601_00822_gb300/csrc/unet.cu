@@ -10,11 +10,12 @@
 //   components.
 //
 // Activations are channels-last [b][z][y][x][c] BF16.  Convolutions are
-// implicit GEMMs on the tensor cores (mma.sync m16n8k16 BF16 -> FP32):
-// rows = voxels, columns = output channels, K = taps x input channels.  The
-// weight gradient is a second GEMM (rows = output channels, columns = input
-// channels, K = voxels) staged through shared memory with ldmatrix.trans,
-// split over voxel chunks and reduced in a fixed order (deterministic).
+// implicit GEMMs on the tensor cores: rows = voxels, columns = output channels,
+// K = taps x input channels (3^3 layers: tcgen05, unet_conv.cu; pointwise
+// layers: unet_gemm.cu).  The weight gradient is a second GEMM (rows = output
+// channels, columns = input channels, K = voxels) staged through shared memory
+// with ldmatrix.trans, split over voxel chunks and reduced in a fixed order
+// (deterministic).
 #include "bfcs.h"
 #include "unet_kernels.h"
 
@@ -51,6 +52,8 @@ __device__ __forceinline__ void ldsm_x4_trans(unsigned* r, const void* smem_row)
 }
 
 // ------------------------------------------------------------------ convolution (forward / data gradient)
+// 3^3 circular convolution on the warp-level tensor cores (BFCS_NET_TCGEN05=0),
+// operands straight from global memory
 constexpr int kConvWarps = 4;
 constexpr int kConvNT = 8;   // n8 tiles per block (64 columns)
 
@@ -78,38 +81,23 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
     cy[q] = (int)((r / a.v.nx) % a.v.ny);
     cz[q] = (int)(r / ((long long)a.v.nx * a.v.ny));
   }
-  const int taps = a.ksize == 3 ? 27 : 1;
-  const int FX = 2 * a.v.nx, FY = 2 * a.v.ny;
-  const long long in_batch = a.in_mode == IN_GATHER_UP ? nvox * 8 : nvox;
-  const bf16* inb = a.in + (long long)b * in_batch * a.ldi + a.offi;
-  for (int tap = 0; tap < taps; ++tap) {
-    const int dz = a.ksize == 3 ? tap / 9 - 1 : 0, dy = a.ksize == 3 ? (tap / 3) % 3 - 1 : 0,
-              dx = a.ksize == 3 ? tap % 3 - 1 : 0;
+  const bf16* inb = a.in + (long long)b * nvox * a.ldi + a.offi;
+  for (int tap = 0; tap < 27; ++tap) {
+    const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
     const bf16* rp[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      long long vox;
-      if (a.in_mode == IN_CONV)
-        vox = ((long long)wrap(cz[q] + dz, a.v.nz) * a.v.ny + wrap(cy[q] + dy, a.v.ny)) * a.v.nx +
-              wrap(cx[q] + dx, a.v.nx);
-      else
-        vox = ((long long)(2 * cz[q]) * FY + 2 * cy[q]) * FX + 2 * cx[q];
-      rp[q] = inb + vox * a.ldi;
-    }
+    for (int q = 0; q < 4; ++q)
+      rp[q] = inb + (((long long)wrap(cz[q] + dz, a.v.nz) * a.v.ny + wrap(cy[q] + dy, a.v.ny)) * a.v.nx +
+                     wrap(cx[q] + dx, a.v.nx)) * a.ldi;
     const bf16* wt = a.w + (long long)tap * a.cout_p * a.cin;
     for (int kc = 0; kc < a.cin; kc += 16) {
-      long long koff = kc;
-      if (a.in_mode == IN_GATHER_UP) {   // k = o * up_c + c -> fine voxel 2u + o, channel c
-        const int o = kc / a.up_c;
-        koff = sub_off(o, FX, FY) * a.ldi + (kc - o * a.up_c);
-      }
       unsigned af[2][4];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        af[i][0] = ld32(rp[2 * i] + koff + 2 * t);
-        af[i][1] = ld32(rp[2 * i + 1] + koff + 2 * t);
-        af[i][2] = ld32(rp[2 * i] + koff + 2 * t + 8);
-        af[i][3] = ld32(rp[2 * i + 1] + koff + 2 * t + 8);
+        af[i][0] = ld32(rp[2 * i] + kc + 2 * t);
+        af[i][1] = ld32(rp[2 * i + 1] + kc + 2 * t);
+        af[i][2] = ld32(rp[2 * i] + kc + 2 * t + 8);
+        af[i][3] = ld32(rp[2 * i + 1] + kc + 2 * t + 8);
       }
 #pragma unroll
       for (int j = 0; j < kConvNT; ++j) {
@@ -122,7 +110,7 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
       }
     }
   }
-  // epilogue: bias, activation, store
+  // epilogue: bias, activation or gate, store
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int i = q >> 1, h = q & 1;
@@ -141,19 +129,14 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
         v0 = v0 > 0.f ? v0 : kSlope * v0;
         v1 = v1 > 0.f ? v1 : kSlope * v1;
       }
-      if (a.out_mode == OUT_F32) {
-        float* o = (float*)a.out + ((long long)b * nvox + r) * a.ldo + a.offo;
-        if (col < a.cout) o[col] = v0;
-        if (col + 1 < a.cout) o[col + 1] = v1;
-      } else if (a.out_mode == OUT_BF16) {
-        bf16* o = (bf16*)a.out + ((long long)b * nvox + r) * a.ldo + a.offo + col;
-        *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(v0, v1);
-      } else {   // column o * up_c + c -> fine voxel 2u + o, channel c
-        const int o = col / a.up_c, c = col - o * a.up_c;
-        const long long fv = ((long long)(2 * cz[q]) * FY + 2 * cy[q]) * FX + 2 * cx[q] + sub_off(o, FX, FY);
-        bf16* out = (bf16*)a.out + ((long long)b * nvox * 8 + fv) * a.ldo + a.offo + c;
-        *reinterpret_cast<__nv_bfloat162*>(out) = __floats2bfloat162_rn(v0, v1);
+      __nv_bfloat162 o = __floats2bfloat162_rn(v0, v1);
+      if (a.gate != nullptr) {
+        const bf16* y = a.gate + ((long long)b * nvox + r) * a.ldg + a.offg + col;
+        if (!(__bfloat162float(y[0]) > 0.f)) o.x = __float2bfloat16(__bfloat162float(o.x) * kSlope);
+        if (!(__bfloat162float(y[1]) > 0.f)) o.y = __float2bfloat16(__bfloat162float(o.y) * kSlope);
       }
+      bf16* dst = (bf16*)a.out + ((long long)b * nvox + r) * a.ldo + a.offo + col;
+      *reinterpret_cast<__nv_bfloat162*>(dst) = o;
     }
   }
 }
@@ -415,15 +398,6 @@ bool wgrad3t_ok(const WgArgs& a) {
          a.ldx % 8 == 0 && a.offx % 8 == 0;
 }
 
-// out[i] = sum over c (in order) of part[c * per + i]
-__global__ void k_sum_chunks(const float* part, int nchunks, long long per, float* out) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < per; i += (long long)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int c = 0; c < nchunks; ++c) s += part[c * per + i];
-    out[i] = s;
-  }
-}
-
 // ------------------------------------------------------------------ elementwise
 // network input (B, 4, N) FP32 -> channels-last BF16 [B][N][16] (channels 4..15 zero)
 __global__ void k_features_in(const float* x, bf16* out, long long n, int batch) {
@@ -437,106 +411,137 @@ __global__ void k_features_in(const float* x, bf16* out, long long n, int batch)
     reinterpret_cast<uint4*>(out + i * 16)[1] = reinterpret_cast<const uint4*>(o)[1];
   }
 }
-// head output [B][N][6] FP32 -> (B, 6, N)
-__global__ void k_features_out(const float* y, float* out, long long n, int batch) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n * batch;
-       i += (long long)gridDim.x * blockDim.x) {
-    const long long b = i / n, v = i - b * n;
-#pragma unroll
-    for (int c = 0; c < 6; ++c) out[(b * 6 + c) * n + v] = y[i * 6 + c];
-  }
-}
-// 2^3 average pooling, fine -> coarse (channels-last views)
+// 2^3 average pooling, fine -> coarse (channels-last views), 8 channels (16 bytes) per thread
 __global__ void k_pool(const bf16* in, int ldi, int offi, bf16* out, int ldo, int offo, int C, Vol coarse,
                        int batch) {
   const long long nc = (long long)coarse.nx * coarse.ny * coarse.nz;
-  const int FX = 2 * coarse.nx, FY = 2 * coarse.ny;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc * batch * C;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    const long long r = i / C;
-    const long long b = r / nc, u = r - b * nc;
-    const int x = (int)(u % coarse.nx), y = (int)((u / coarse.nx) % coarse.ny),
-              z = (int)(u / ((long long)coarse.nx * coarse.ny));
-    const long long f0 = b * nc * 8 + ((long long)(2 * z) * FY + 2 * y) * FX + 2 * x;
-    float s = 0.f;
-#pragma unroll
-    for (int o = 0; o < 8; ++o) s += __bfloat162float(in[(f0 + sub_off(o, FX, FY)) * ldi + offi + c]);
-    out[r * ldo + offo + c] = __float2bfloat16(0.125f * s);
-  }
-}
-// pooling gradient added into the fine gradient: dfine[2u + o][c] += dcoarse[u][c] / 8
-__global__ void k_unpool_add(const bf16* dco, int ldc, int offc, bf16* dfine, int ldf, int offf, int C, Vol coarse,
-                             int batch) {
-  const long long nc = (long long)coarse.nx * coarse.ny * coarse.nz;
-  const int FX = 2 * coarse.nx, FY = 2 * coarse.ny;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc * batch * C * 8;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % C);
-    long long r = i / C;
-    const int o = (int)(r % 8);
-    r /= 8;
-    const long long b = r / nc, u = r - b * nc;
-    const int x = (int)(u % coarse.nx), y = (int)((u / coarse.nx) % coarse.ny),
-              z = (int)(u / ((long long)coarse.nx * coarse.ny));
-    const long long fv = b * nc * 8 + ((long long)(2 * z) * FY + 2 * y) * FX + 2 * x + sub_off(o, FX, FY);
-    bf16* d = dfine + fv * ldf + offf + c;
-    *d = __float2bfloat16(__bfloat162float(*d) + 0.125f * __bfloat162float(dco[r * ldc + offc + c]));
-  }
-}
-// dY *= act'(pre) in place; the sign of the saved post-activation output
-// equals the sign of the pre-activation.  8 channels (16 bytes) per thread.
-__global__ void k_act_bwd(bf16* dy, int ldd, int offd, const bf16* y, int ldy, int offy, int C, long long rows) {
-  const int cv = C / 8;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < rows * cv;
+  const int FX = 2 * coarse.nx, FY = 2 * coarse.ny, cv = C / 8;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc * batch * cv;
        i += (long long)gridDim.x * blockDim.x) {
     const long long r = i / cv;
     const int c = (int)(i - r * cv) * 8;
-    uint4* dp = reinterpret_cast<uint4*>(dy + r * ldd + offd + c);
-    uint4 dv = *dp;
+    const unsigned rr = (unsigned)r, yz = rr / coarse.nx, x = rr - yz * coarse.nx;   // rows < 2^31 / 8
+    const unsigned zb = yz / coarse.ny, y = yz - zb * coarse.ny;                      // zb = b nz + z
+    const long long f0 = ((long long)(2 * zb) * FY + 2 * y) * FX + 2 * x;
+    uint4 v[8];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) v[o] = *reinterpret_cast<const uint4*>(in + (f0 + sub_off(o, FX, FY)) * ldi + offi + c);
+    __align__(16) bf16 s8[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      float s = 0.f;
+#pragma unroll
+      for (int o = 0; o < 8; ++o) s += __bfloat162float(reinterpret_cast<const bf16*>(&v[o])[k]);
+      s8[k] = __float2bfloat16(0.125f * s);
+    }
+    *reinterpret_cast<uint4*>(out + r * ldo + offo + c) = *reinterpret_cast<const uint4*>(s8);
+  }
+}
+// pooling gradient added into the fine gradient, dfine[2u + o][c] += dcoarse[u][c] / 8,
+// then the activation's derivative there from the sign of the saved output y (gate8);
+// 8 channels (16 bytes) of one fine voxel per thread
+__global__ void k_unpool_gate(const bf16* dco, int ldc, int offc, bf16* dfine, int ldf, int offf, const bf16* y,
+                              int ldy, int offy, int C, Vol fine, int batch) {
+  const long long nf = (long long)fine.nx * fine.ny * fine.nz;
+  const int cv = C / 8;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nf * batch * cv;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long r = i / cv;
+    const int c = (int)(i - r * cv) * 8;
+    const unsigned rr = (unsigned)r, yz = rr / fine.nx, x = rr - yz * fine.nx;
+    const unsigned zb = yz / fine.ny, yy = yz - zb * fine.ny;
+    const long long u = ((long long)(zb / 2) * (fine.ny / 2) + yy / 2) * (fine.nx / 2) + x / 2;
+    uint4* dp = reinterpret_cast<uint4*>(dfine + r * ldf + offf + c);
+    const uint4 cg = *reinterpret_cast<const uint4*>(dco + u * ldc + offc + c);
     const uint4 yv = *reinterpret_cast<const uint4*>(y + r * ldy + offy + c);
-    bf16* d8 = reinterpret_cast<bf16*>(&dv);
-    const bf16* y8 = reinterpret_cast<const bf16*>(&yv);
+    uint4 d = *dp;
+    bf16* d8 = reinterpret_cast<bf16*>(&d);
+    const bf16* c8 = reinterpret_cast<const bf16*>(&cg);
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (!(__bfloat162float(y8[k]) > 0.f)) d8[k] = __float2bfloat16(__bfloat162float(d8[k]) * kSlope);
-    *dp = dv;
+      d8[k] = __float2bfloat16(__bfloat162float(d8[k]) + 0.125f * __bfloat162float(c8[k]));
+    gate8(reinterpret_cast<__nv_bfloat162*>(&d), yv);
+    *dp = d;
   }
 }
-// bias gradient partials: part[block][c] = sum over this block's rows of dY[r][c]
-constexpr int kBiasThreads = 256;
+// bias gradient partials: part[block][c] = sum over this block's rows of dY[r][c];
+// 8 channels (16 bytes) of a row per thread, thread sums added in thread order
+constexpr int kBiasThreads = 256, kBiasBlocks = 304;
 __global__ void __launch_bounds__(kBiasThreads) k_bias_grad(const bf16* dy, int ldd, int offd, int C, long long rows,
                                                             long long per, float* part) {
-  __shared__ float red[kBiasThreads];
-  const int nr = kBiasThreads / C;
-  const int c = threadIdx.x % C, j = threadIdx.x / C;
+  __shared__ float red[kBiasThreads * 8];
+  const int cv = C / 8, nr = kBiasThreads / cv;
+  const int c = threadIdx.x % cv, j = threadIdx.x / cv;
   const long long r0 = blockIdx.x * per, r1 = min(rows, r0 + per);
-  float s = 0.f;
-  if (j < nr)
-    for (long long r = r0 + j; r < r1; r += nr) s += __bfloat162float(dy[r * ldd + offd + c]);
-  red[threadIdx.x] = s;
+  float s[8] = {};
+  if (j < nr) {
+#pragma unroll 4
+    for (long long r = r0 + j; r < r1; r += nr) {
+      const uint4 v = *reinterpret_cast<const uint4*>(dy + r * ldd + offd + c * 8);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s[k] += __bfloat162float(reinterpret_cast<const bf16*>(&v)[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) red[k * kBiasThreads + threadIdx.x] = s[k];
   __syncthreads();
-  if (threadIdx.x < C) {
+  // 8 lanes per channel add the threads of its group in order, then one adds the lanes
+  const int ch = threadIdx.x / 8, l = threadIdx.x % 8;
+  for (int c0 = ch; c0 < C; c0 += kBiasThreads / 8) {
+    const float* col = red + (c0 % 8) * kBiasThreads + c0 / 8;
     float t = 0.f;
-    for (int q = 0; q < nr; ++q) t += red[q * C + threadIdx.x];
-    part[(long long)blockIdx.x * C + threadIdx.x] = t;
+    for (int q = l; q < nr; q += 8) t += col[q * cv];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o, 8);
+    if (l == 0) part[(long long)blockIdx.x * C + c0] = t;
   }
 }
-// relative squared L2 loss: per (block, sample) sums of (p - t)^2 and t^2 in
-// FP64; one voxel per thread (6 contiguous predictions, 6 coalesced targets)
+
+// p - t of two floats without rounding (TwoSum): hi + lo
+__device__ __forceinline__ ff exact_diff(float p, float t) {
+  const float s = __fsub_rn(p, t), v = __fsub_rn(s, p);
+  return ff_pair(s, __fsub_rn(__fsub_rn(p, __fsub_rn(s, v)), __fadd_rn(t, v)));
+}
+// the square of x and its rounding error stay inside the FP32 range (x finite)
+__device__ __forceinline__ bool ff_square_safe(float x) {
+  const float m = fabsf(x);
+  return (m > 1e-11f && m < 1e15f) || m == 0.f;
+}
+// relative squared L2 loss: per (block, sample) sums of (p - t)^2 and t^2; one voxel
+// per thread, planar fields (6 x n a sample).  The six squares of a voxel are formed
+// and added in float-float (about 48 bits, FP32 pipes), voxels in FP64: with every
+// term on the FP64 pipe the pass took 143 us for 8 samples of 64^3 instead of the
+// 15 us its 100 MB take.  Voxels with values outside the range of that form (tiny, huge,
+// not finite) are formed in FP64.
 constexpr int kLossBlocks = 64;
 __global__ void k_loss(const float* pred, const float* target, long long n, double* num, double* den) {
   __shared__ double rn[32], rd[32];
   const int b = blockIdx.y;
+  const float* pb = pred + (long long)b * 6 * n;
+  const float* tb = target + (long long)b * 6 * n;
   double sn = 0.0, sd = 0.0;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-    const float* pr = pred + ((long long)b * n + v) * 6;
+    ff vn = ff(0.0f), vd = ff(0.0f);
+    float p6[6], t6[6];
+    bool fast = true;
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-      const double p = pr[c];
-      const double t = target[((long long)b * 6 + c) * n + v];
-      sn += (p - t) * (p - t);
-      sd += t * t;
+      p6[c] = pb[c * n + v];
+      t6[c] = tb[c * n + v];
+      const ff d = exact_diff(p6[c], t6[c]);
+      vn = vn + d * d;
+      vd = vd + ff(t6[c]) * ff(t6[c]);
+      fast = fast && ff_square_safe(d.hi) && ff_square_safe(t6[c]);
+    }
+    if (fast) {
+      sn += f2d_bits(vn.hi) + f2d_bits(vn.lo);
+      sd += f2d_bits(vd.hi) + f2d_bits(vd.lo);
+    } else {
+      for (int c = 0; c < 6; ++c) {
+        const double t = t6[c], d = (double)p6[c] - t;
+        sn += d * d;
+        sd += t * t;
+      }
     }
   }
   for (int off = 16; off > 0; off >>= 1) {
@@ -552,34 +557,52 @@ __global__ void k_loss(const float* pred, const float* target, long long n, doub
     den[b * gridDim.x + blockIdx.x] = s1;
   }
 }
-// den_b[b], and loss = mean over b of num_b / den_b (written if loss != null)
-__global__ void k_loss_final(const double* num, const double* den, int nblk, int batch, double* den_b, double* loss) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double l = 0.0;
-  for (int b = 0; b < batch; ++b) {
+// den_b[b], and loss = mean over b of num_b / den_b (written if loss != null): one warp
+// per sample in turn, then thread 0 over the samples
+__global__ void k_loss_final(const double* num, const double* den, int nblk, int batch, double* den_b, double* rel_b,
+                             double* loss) {
+  const int lane = threadIdx.x & 31;
+  for (int b = threadIdx.x >> 5; b < batch; b += blockDim.x >> 5) {
     double s0 = 0, s1 = 0;
-    for (int k = 0; k < nblk; ++k) { s0 += num[b * nblk + k]; s1 += den[b * nblk + k]; }
-    den_b[b] = s1;
-    l += s0 / s1;
+    for (int k = lane; k < nblk; k += 32) { s0 += num[b * nblk + k]; s1 += den[b * nblk + k]; }
+    for (int off = 16; off > 0; off >>= 1) {
+      s0 += __shfl_down_sync(0xffffffffu, s0, off);
+      s1 += __shfl_down_sync(0xffffffffu, s1, off);
+    }
+    if (lane == 0) { den_b[b] = s1; rel_b[b] = s0 / s1; }
   }
-  if (loss != nullptr) *loss = l / batch;
+  __syncthreads();
+  if (threadIdx.x == 0 && loss != nullptr) {
+    double l = 0.0;
+    for (int b = 0; b < batch; ++b) l += rel_b[b];
+    *loss = l / batch;
+  }
 }
 // dL/dpred = 2 (p - t) / (den_b B), written as the head's output gradient
-// [B][N][16] BF16 (channels 6..15 zero); one voxel per thread
+// [B][N][16] BF16 (channels 6..15 zero); one voxel per thread; float-float products
+// (48 bits before the one rounding to FP32, where the FP64 form has 53; 155 us of FP64
+// pipe for 8 samples of 64^3), FP64 outside their range
 __global__ void k_loss_grad(const float* pred, const float* target, const double* den_b, long long n, int batch,
                             bf16* dy) {
-  for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < n * batch;
-       r += (long long)gridDim.x * blockDim.x) {
-    const long long b = r / n, v = r - b * n;
-    const double f = 2.0 / (den_b[b] * batch);
+  const int b = blockIdx.y;
+  const double fd = 2.0 / (den_b[b] * batch);
+  const ff f = ff(fd);
+  const bool fast = fd > 1e-18 && fd < 1e18;
+  const float* pb = pred + (long long)b * 6 * n;
+  const float* tb = target + (long long)b * 6 * n;
+  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
     __align__(16) bf16 o[16];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) o[c] = __float2bfloat16(0.f);
+    for (int c = 6; c < 16; ++c) o[c] = __float2bfloat16(0.f);
 #pragma unroll
-    for (int c = 0; c < 6; ++c)
-      o[c] = __float2bfloat16((float)(((double)pred[r * 6 + c] - (double)target[(b * 6 + c) * n + v]) * f));
-    reinterpret_cast<uint4*>(dy + r * 16)[0] = reinterpret_cast<const uint4*>(o)[0];
-    reinterpret_cast<uint4*>(dy + r * 16)[1] = reinterpret_cast<const uint4*>(o)[1];
+    for (int c = 0; c < 6; ++c) {
+      const float p = pb[c * n + v], t = tb[c * n + v];
+      const ff d = exact_diff(p, t);
+      o[c] = __float2bfloat16(fast && ff_square_safe(d.hi) ? (float)(d * f) : (float)(((double)p - (double)t) * fd));
+    }
+    uint4* d = reinterpret_cast<uint4*>(dy + ((long long)b * n + v) * 16);
+    d[0] = reinterpret_cast<const uint4*>(o)[0];
+    d[1] = reinterpret_cast<const uint4*>(o)[1];
   }
 }
 // Adam (Kingma and Ba 2014), bias-corrected, FP32 state
@@ -602,15 +625,24 @@ __global__ void k_adam(float* w, const float* g, float* m, float* v, long long n
 // [cin_p][8 cout].  The flat vector holds PyTorch's shapes: conv
 // W[co][ci][kz][ky][kx] (tap = 9 kz + 3 ky + kx), up W[ci][co][oz][oy][ox].
 struct LayerDef { int kind, cin, cout, cin_p, cout_p; long long woff, boff; };
+constexpr int kNumLayers = 18;
+struct PackArgs {
+  LayerDef def[kNumLayers];
+  bf16 *fw[kNumLayers], *bw[kNumLayers];
+};
 
-__global__ void k_pack(const float* flat, LayerDef L, bf16* fw, bf16* bw) {
+// every layer in one launch (blockIdx.y = layer)
+__global__ void k_pack(const float* flat, const __grid_constant__ PackArgs pa) {
+  const LayerDef& L = pa.def[blockIdx.y];
+  bf16* const fw = pa.fw[blockIdx.y];
+  bf16* const bw = pa.bw[blockIdx.y];
   const int taps = L.kind == 0 ? 27 : 1;
   const int ocols = L.kind == 2 ? 8 * L.cout : L.cout_p;
-  const long long nf = (long long)taps * ocols * L.cin_p;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nf; i += (long long)gridDim.x * blockDim.x) {
-    const int ci = (int)(i % L.cin_p);
-    const long long r = i / L.cin_p;
-    const int col = (int)(r % ocols), tap = (int)(r / ocols);
+  const int nf = taps * ocols * L.cin_p;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nf; i += gridDim.x * blockDim.x) {
+    const int ci = i % L.cin_p;
+    const int r = i / L.cin_p;
+    const int col = r % ocols, tap = r / ocols;
     float w = 0.f;
     if (ci < L.cin) {
       if (L.kind == 2) {
@@ -627,37 +659,66 @@ __global__ void k_pack(const float* flat, LayerDef L, bf16* fw, bf16* bw) {
   }
 }
 
-// summed weight gradient (layout of the forward weights) and bias gradient -> flat
-__global__ void k_unpack_grad(const float* gw, const float* gb, LayerDef L, float* gflat) {
+// A layer's gradients from their partials into the flat vector: weights [chunk][tap]
+// [cols][cin_p] (layout of the forward weights), biases [block][bcols].  Blocks of 32
+// outputs x 8 lanes: lane j adds partials j, j + 8, ... in order, the lanes are added
+// pairwise (a fixed order).  One thread per output over all partials left the pass to
+// the latency of up to 1024 dependent loads (18-120 us a layer).
+constexpr int kRedOut = 32, kRedLanes = 8;
+__global__ void __launch_bounds__(kRedOut * kRedLanes) k_reduce_grad(const float* wpart, int nchunks, const float* bpart,
+                                                                    int nblk, int bcols, LayerDef L, float* gflat) {
+  __shared__ float red[kRedLanes][kRedOut];
+  const int o = threadIdx.x % kRedOut, j = threadIdx.x / kRedOut;
   const int taps = L.kind == 0 ? 27 : 1;
   const int ocols = L.kind == 2 ? 8 * L.cout : L.cout_p;
-  const long long nw = (long long)taps * L.cout * L.cin * (L.kind == 2 ? 8 : 1);
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nw + L.cout;
-       i += (long long)gridDim.x * blockDim.x) {
-    if (i >= nw) { gflat[L.boff + (i - nw)] = gb[i - nw]; continue; }
-    if (L.kind == 2) {
-      const int o = (int)(i % 8);
-      const long long r = i / 8;
-      const int co = (int)(r % L.cout), ci = (int)(r / L.cout);
-      gflat[L.woff + i] = gw[(long long)(o * L.cout + co) * L.cin_p + ci];
-    } else {
-      const int tap = (int)(i % taps);
-      const long long r = i / taps;
-      const int ci = (int)(r % L.cin), co = (int)(r / L.cin);
-      gflat[L.woff + i] = gw[((long long)tap * ocols + co) * L.cin_p + ci];
-    }
+  const int per = taps * ocols * L.cin_p;
+  const int wblocks = (per + kRedOut - 1) / kRedOut;
+  const bool bias = (int)blockIdx.x >= wblocks;
+  const int i = (bias ? (int)blockIdx.x - wblocks : (int)blockIdx.x) * kRedOut + o;
+  const int count = bias ? bcols : per, parts = bias ? nblk : nchunks;
+  const float* p = bias ? bpart : wpart;
+  float s = 0.f;
+  if (i < count) {
+#pragma unroll 8
+    for (int c = j; c < parts; c += kRedLanes) s += p[(long long)c * count + i];
   }
+  red[j][o] = s;
+  __syncthreads();
+  if (j != 0 || i >= count) return;
+#pragma unroll
+  for (int h = 0; h < kRedLanes; h += 2) red[h][o] += red[h + 1][o];
+  const float t = (red[0][o] + red[2][o]) + (red[4][o] + red[6][o]);
+  if (bias) {
+    if (i < L.cout) gflat[L.boff + i] = t;
+    return;
+  }
+  const int ci = i % L.cin_p, r = i / L.cin_p, col = r % ocols, tap = r / ocols;
+  if (ci >= L.cin) return;
+  if (L.kind == 2) gflat[L.woff + ((long long)ci * L.cout + col % L.cout) * 8 + col / L.cout] = t;
+  else if (col < L.cout) gflat[L.woff + ((long long)col * L.cin + ci) * taps + tap] = t;
 }
 
 // ------------------------------------------------------------------ features / outputs
-// max |b| over 3 N values as the bits of a non-negative float (order-independent)
+// per sample: max |b| over 3 N values as the bits of a non-negative float
+// (order-independent); sample = blockIdx.y, one atomic per block
+template <typename R> struct SampleArgs {
+  const R* b[kSampleArgs];
+  const int8_t* phase[kSampleArgs];
+};
 template <typename R>
-__global__ void k_absmax(const R* b, long long n3, unsigned* out) {
+__global__ void k_absmax(const __grid_constant__ SampleArgs<R> sa, long long n3, unsigned* out) {
+  __shared__ float red[32];
+  const R* b = sa.b[blockIdx.y];
   float m = 0.f;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (long long)gridDim.x * blockDim.x)
     m = fmaxf(m, fabsf((float)b[i]));
   for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_down_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) m = fmaxf(m, red[w]);
+    atomicMax(out + blockIdx.y, __float_as_uint(m));
+  }
 }
 struct MuTab { float mu[BFCS_MAX_PHASES]; float mu_max; };
 // x (4, N): b / s and mu / mu_max - 1/2; target (6, N) = eps mu_max / s (if eps)
@@ -676,10 +737,14 @@ __global__ void k_prepare(const R* b, const int8_t* phase, MuTab mt, const unsig
     }
   }
 }
-// channels-last BF16 network input of one sample straight from b and phase
+// channels-last BF16 network inputs straight from b and phase (sample = blockIdx.y)
 template <typename R>
-__global__ void k_prepare_x0(const R* b, const int8_t* phase, MuTab mt, const unsigned* sbits, bf16* x0, long long n) {
-  const float s = __uint_as_float(*sbits);
+__global__ void k_prepare_x0(const __grid_constant__ SampleArgs<R> sa, MuTab mt, const unsigned* sbits, bf16* x0,
+                             long long n) {
+  const R* b = sa.b[blockIdx.y];
+  const int8_t* phase = sa.phase[blockIdx.y];
+  x0 += (long long)blockIdx.y * n * 16;
+  const float s = __uint_as_float(sbits[blockIdx.y]);
   const float inv = s > 0.f ? 1.f / s : 0.f;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
     __align__(16) bf16 o[16];
@@ -690,15 +755,6 @@ __global__ void k_prepare_x0(const R* b, const int8_t* phase, MuTab mt, const un
     o[3] = __float2bfloat16(mt.mu[phase[v]] / mt.mu_max - 0.5f);
     reinterpret_cast<uint4*>(x0 + v * 16)[0] = reinterpret_cast<const uint4*>(o)[0];
     reinterpret_cast<uint4*>(x0 + v * 16)[1] = reinterpret_cast<const uint4*>(o)[1];
-  }
-}
-// predicted strain (6, N) = y s / mu_max from the head output [N][6]
-template <typename R>
-__global__ void k_predict_out(const float* y, const unsigned* sbits, float mu_max, R* eps, long long n) {
-  const double f = (double)__uint_as_float(*sbits) / mu_max;
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) eps[c * n + v] = (R)(y[v * 6 + c] * f);
   }
 }
 
@@ -713,7 +769,6 @@ namespace {
 
 // (kind, cin, cout) in the order of the flat parameter vector
 struct LayerSpec { int kind, cin, cout; };
-constexpr int kNumLayers = 18;
 constexpr LayerSpec kSpec[kNumLayers] = {
     {0, 4, 32},  {0, 32, 32},                 // e0a e0b
     {0, 32, 32}, {0, 32, 32},                 // e1a e1b
@@ -750,12 +805,10 @@ struct bfcs_net_s {
   LayerDef def[kNumLayers];
   bf16* fw[kNumLayers];
   bf16* bw[kNumLayers];
-  float* gw[kNumLayers];     // summed weight gradients (forward layout)
-  float* gb[kNumLayers];
   char* base = nullptr;
   // activations
   bf16 *X0, *A0, *C0, *D0a, *D0b, *P0, *A1, *C1, *D1a, *D1b, *P1, *A2, *C2, *D2a, *D2b, *P2, *A3, *H3;
-  float* OUT;
+  float* OUT;                // head output (B, 6, n), training
   // gradients (training only)
   bf16 *dOUT = nullptr, *dA0, *dC0, *dD0a, *dD0b, *dP0, *dA1, *dC1, *dD1a, *dD1b, *dP1, *dA2, *dC2, *dD2a, *dD2b,
        *dP2, *dA3, *dH3;
@@ -764,6 +817,7 @@ struct bfcs_net_s {
   double* lnum;              // loss partials
   double* lden;
   double* den_b;
+  double* rel_b;
   unsigned* sbits;           // per-sample max |b|
   int* err;                  // set by a kernel whose bounded wait expired
 };
@@ -771,12 +825,10 @@ struct bfcs_net_s {
 namespace {
 
 cudaError_t pack_all(bfcs_net_s* N, const float* params) {
-  for (int l = 0; l < kNumLayers; ++l) {
-    const LayerDef& L = N->def[l];
-    const long long nf = (long long)(L.kind == 0 ? 27 : 1) * (L.kind == 2 ? 8 * L.cout : L.cout_p) * L.cin_p;
-    k_pack<<<grid_for(nf), 256, 0, N->st>>>(params, L, N->fw[l], N->bw[l]);
-  }
-  count_launches(kNumLayers);
+  PackArgs pa;
+  for (int l = 0; l < kNumLayers; ++l) { pa.def[l] = N->def[l]; pa.fw[l] = N->fw[l]; pa.bw[l] = N->bw[l]; }
+  k_pack<<<dim3(108, kNumLayers), 256, 0, N->st>>>(params, pa);
+  count_launches(1);
   return cudaGetLastError();
 }
 
@@ -799,7 +851,9 @@ bool tcgen05_enabled() {
 }
 
 cudaError_t launch_conv(const ConvArgs& a, long long nvox, int* err, cudaStream_t st) {
-  if (conv3_ok(a) && tcgen05_enabled()) return launch_conv3(a, sm_count(), err, st);
+  if (rows_ok(a)) return launch_rows(a, sm_count(), st);
+  if (!conv3_ok(a)) return cudaErrorInvalidValue;
+  if (tcgen05_enabled()) return launch_conv3(a, sm_count(), err, st);
   k_conv<<<dim3(ceil_div(nvox, kConvWarps * 32), ceil_div(a.cout_p, kConvNT * 8), a.batch), kConvWarps * 32, 0,
            st>>>(a);
   count_launches(1);
@@ -829,7 +883,7 @@ cudaError_t conv_fwd(bfcs_net_s* N, int l, const float* params, int B, View in, 
 }
 
 cudaError_t pool(bfcs_net_s* N, View in, View out, int C, int coarse_lv, int B) {
-  const long long tot = N->n[coarse_lv] * B * C;
+  const long long tot = N->n[coarse_lv] * B * C / 8;
   k_pool<<<grid_for(tot), 256, 0, N->st>>>(in.p, in.ld, in.off, out.p, out.ld, out.off, C, N->vol[coarse_lv], B);
   count_launches(1);
   return cudaGetLastError();
@@ -861,26 +915,46 @@ cudaError_t forward(bfcs_net_s* N, const float* params, int B) {
   NET_TRY(conv_fwd(N, U0, params, B, {N->D1b, 32, 0}, 1, OUT_SHUFFLE_UP, N->C0, 64, 0));
   NET_TRY(conv_fwd(N, D0A, params, B, {N->C0, 64, 0}, 0, F, N->D0a, 32, 0));
   NET_TRY(conv_fwd(N, D0B, params, B, {N->D0a, 32, 0}, 0, F, N->D0b, 32, 0));
-  NET_TRY(conv_fwd(N, HEAD, params, B, {N->D0b, 32, 0}, 0, OUT_F32, N->OUT, 6, 0));
   return cudaSuccess;
 }
 
-// Backward of layer l.  dout: gradient w.r.t. the layer output (post-activation;
-// turned into the pre-activation gradient in place); out: saved output; in:
-// saved input; din: where the input gradient goes (p == null: not needed).
-// lv: level of the GEMM rows (coarse level for an up layer).
-cudaError_t layer_bwd(bfcs_net_s* N, int l, int B, View dout, View out, View in, View din, int lv) {
+// the head over samples 0..B-1 of D0b: sample i to out[i] (6 x n), as the network's
+// output or (predict) as the strain prediction
+template <typename R>
+cudaError_t head(bfcs_net_s* N, const float* params, int B, R* const* out, bool predict, float mu_max) {
+  for (int i0 = 0; i0 < B; i0 += kSampleArgs) {
+    const int k = std::min(kSampleArgs, B - i0);
+    HeadArgs<R> a{};
+    a.in = N->D0b + (long long)i0 * N->n[0] * 32;
+    a.w = N->fw[HEAD];
+    a.bias = params + N->def[HEAD].boff;
+    a.n = N->n[0];
+    a.sbits = N->sbits + i0;
+    a.mu_max = mu_max;
+    for (int i = 0; i < k; ++i) a.out[i] = out[i0 + i];
+    const cudaError_t e = launch_head<R>(a, k, predict, sm_count(), N->st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+cudaError_t head_planar(bfcs_net_s* N, const float* params, int B, float* y) {
+  std::vector<float*> out(B);
+  for (int i = 0; i < B; ++i) out[i] = y + (long long)i * 6 * N->n[0];
+  return head<float>(N, params, B, out.data(), false, 1.f);
+}
+
+// Backward of layer l.  dout: gradient w.r.t. the layer's pre-activation (gated where
+// it was written); in: saved input; din: where the input gradient goes (p == null: not
+// needed); gate: the saved output whose activation's derivative din takes (p == null:
+// none: an up-convolution's or pooling's output, or a gradient still to be added to).
+// lv: level of the GEMM rows (coarse level for an up layer).  Gradients go to grad.
+cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View in, View din, View gate, int lv) {
   const LayerDef& L = N->def[l];
   const bool up = L.kind == 2;
   const int taps = L.kind == 0 ? 27 : 1;
   const long long rows = N->n[lv] * B;                  // GEMM K rows of the weight gradient
   const long long orows = up ? rows * 8 : rows;         // rows of the output gradient
   const int dch = up ? L.cout : L.cout_p;               // channels of the output gradient view
-  if (L.kind == 0) {
-    k_act_bwd<<<grid_for(orows * dch / 8), 256, 0, N->st>>>(dout.p, dout.ld, dout.off, out.p, out.ld, out.off, dch,
-                                                            orows);
-    count_launches(1);
-  }
   // weight gradient
   WgArgs w{};
   w.dy = dout.p; w.ldd = dout.ld; w.offd = dout.off;
@@ -898,7 +972,7 @@ cudaError_t layer_bwd(bfcs_net_s* N, int l, int B, View dout, View out, View in,
   nchunks = ceil_div(rows, w.chunk);
   const long long per = (long long)taps * w.cout_p * w.cin;
   const int bc = dch;
-  const int nblk = std::max(1, std::min(1024, ceil_div(orows, 512)));
+  const int nblk = std::max(1, std::min(kBiasBlocks, ceil_div(orows, 64)));
   if ((long long)nchunks * per + (long long)nblk * bc > N->part_cap) return cudaErrorInvalidValue;
   w.part = N->part;
   if (wgrad3t_ok(w)) {
@@ -911,13 +985,13 @@ cudaError_t layer_bwd(bfcs_net_s* N, int l, int B, View dout, View out, View in,
     const size_t smem = (size_t)kWgRows * (mcols + 8 + w.cin + 8) * sizeof(bf16);
     k_wgrad<<<dim3(nchunks, taps * mchunks), 128, smem, N->st>>>(w);
   }
-  k_sum_chunks<<<grid_for(per), 256, 0, N->st>>>(N->part, nchunks, per, N->gw[l]);
-  // bias gradient (over the rows of the output gradient)
+  // bias gradient (over the rows of the output gradient), then both sums
   const long long bper = (orows + nblk - 1) / nblk;
   float* bpart = N->part + (long long)nchunks * per;
   k_bias_grad<<<nblk, kBiasThreads, 0, N->st>>>(dout.p, dout.ld, dout.off, bc, orows, bper, bpart);
-  k_sum_chunks<<<grid_for(bc), 256, 0, N->st>>>(bpart, nblk, bc, N->gb[l]);
-  count_launches(4);
+  k_reduce_grad<<<ceil_div(per, kRedOut) + ceil_div(bc, kRedOut), kRedOut * kRedLanes, 0, N->st>>>(
+      N->part, nchunks, bpart, nblk, bc, L, grad);
+  count_launches(3);
   // input gradient: a convolution with the data-gradient weights
   if (din.p != nullptr) {
     ConvArgs a{};
@@ -934,62 +1008,55 @@ cudaError_t layer_bwd(bfcs_net_s* N, int l, int B, View dout, View out, View in,
     a.out_mode = OUT_BF16;
     a.out = din.p; a.ldo = din.ld; a.offo = din.off;
     a.up_c = L.cout;
+    a.gate = gate.p; a.ldg = gate.ld; a.offg = gate.off;
     const cudaError_t e = launch_conv(a, N->n[lv], N->err, N->st);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
 
-cudaError_t unpool_add(bfcs_net_s* N, View dco, View dfine, int C, int coarse_lv, int B) {
-  const long long tot = N->n[coarse_lv] * B * C * 8;
-  k_unpool_add<<<grid_for(tot), 256, 0, N->st>>>(dco.p, dco.ld, dco.off, dfine.p, dfine.ld, dfine.off, C,
-                                                 N->vol[coarse_lv], B);
+// pooling gradient into the skip half of a concatenation's gradient, and its gate
+cudaError_t unpool_gate(bfcs_net_s* N, View dco, View dfine, View y, int C, int fine_lv, int B) {
+  const long long tot = N->n[fine_lv] * B * C / 8;
+  k_unpool_gate<<<grid_for(tot), 256, 0, N->st>>>(dco.p, dco.ld, dco.off, dfine.p, dfine.ld, dfine.off, y.p, y.ld,
+                                                  y.off, C, N->vol[fine_lv], B);
   count_launches(1);
   return cudaGetLastError();
 }
 
-cudaError_t backward(bfcs_net_s* N, int B) {
+cudaError_t backward(bfcs_net_s* N, float* g, int B) {
   cudaError_t e;
   const View none{nullptr, 0, 0};
-  NET_TRY(layer_bwd(N, HEAD, B, {N->dOUT, 16, 0}, none, {N->D0b, 32, 0}, {N->dD0b, 32, 0}, 0));
-  NET_TRY(layer_bwd(N, D0B, B, {N->dD0b, 32, 0}, {N->D0b, 32, 0}, {N->D0a, 32, 0}, {N->dD0a, 32, 0}, 0));
-  NET_TRY(layer_bwd(N, D0A, B, {N->dD0a, 32, 0}, {N->D0a, 32, 0}, {N->C0, 64, 0}, {N->dC0, 64, 0}, 0));
-  NET_TRY(layer_bwd(N, U0, B, {N->dC0, 64, 0}, none, {N->D1b, 32, 0}, {N->dD1b, 32, 0}, 1));
-  NET_TRY(layer_bwd(N, D1B, B, {N->dD1b, 32, 0}, {N->D1b, 32, 0}, {N->D1a, 32, 0}, {N->dD1a, 32, 0}, 1));
-  NET_TRY(layer_bwd(N, D1A, B, {N->dD1a, 32, 0}, {N->D1a, 32, 0}, {N->C1, 64, 0}, {N->dC1, 64, 0}, 1));
-  NET_TRY(layer_bwd(N, U1, B, {N->dC1, 64, 0}, none, {N->D2b, 32, 0}, {N->dD2b, 32, 0}, 2));
-  NET_TRY(layer_bwd(N, D2B, B, {N->dD2b, 32, 0}, {N->D2b, 32, 0}, {N->D2a, 32, 0}, {N->dD2a, 32, 0}, 2));
-  NET_TRY(layer_bwd(N, D2A, B, {N->dD2a, 32, 0}, {N->D2a, 32, 0}, {N->C2, 64, 0}, {N->dC2, 64, 0}, 2));
-  NET_TRY(layer_bwd(N, U2, B, {N->dC2, 64, 0}, none, {N->H3, 48, 0}, {N->dH3, 48, 0}, 3));
-  NET_TRY(layer_bwd(N, E3B, B, {N->dH3, 48, 0}, {N->H3, 48, 0}, {N->A3, 48, 0}, {N->dA3, 48, 0}, 3));
-  NET_TRY(layer_bwd(N, E3A, B, {N->dA3, 48, 0}, {N->A3, 48, 0}, {N->P2, 32, 0}, {N->dP2, 32, 0}, 3));
-  NET_TRY(unpool_add(N, {N->dP2, 32, 0}, {N->dC2, 64, 32}, 32, 3, B));
-  NET_TRY(layer_bwd(N, E2B, B, {N->dC2, 64, 32}, {N->C2, 64, 32}, {N->A2, 32, 0}, {N->dA2, 32, 0}, 2));
-  NET_TRY(layer_bwd(N, E2A, B, {N->dA2, 32, 0}, {N->A2, 32, 0}, {N->P1, 32, 0}, {N->dP1, 32, 0}, 2));
-  NET_TRY(unpool_add(N, {N->dP1, 32, 0}, {N->dC1, 64, 32}, 32, 2, B));
-  NET_TRY(layer_bwd(N, E1B, B, {N->dC1, 64, 32}, {N->C1, 64, 32}, {N->A1, 32, 0}, {N->dA1, 32, 0}, 1));
-  NET_TRY(layer_bwd(N, E1A, B, {N->dA1, 32, 0}, {N->A1, 32, 0}, {N->P0, 32, 0}, {N->dP0, 32, 0}, 1));
-  NET_TRY(unpool_add(N, {N->dP0, 32, 0}, {N->dC0, 64, 32}, 32, 1, B));
-  NET_TRY(layer_bwd(N, E0B, B, {N->dC0, 64, 32}, {N->C0, 64, 32}, {N->A0, 32, 0}, {N->dA0, 32, 0}, 0));
-  NET_TRY(layer_bwd(N, E0A, B, {N->dA0, 32, 0}, {N->A0, 32, 0}, {N->X0, 16, 0}, none, 0));
+  NET_TRY(layer_bwd(N, g, HEAD, B, {N->dOUT, 16, 0}, {N->D0b, 32, 0}, {N->dD0b, 32, 0}, {N->D0b, 32, 0}, 0));
+  NET_TRY(layer_bwd(N, g, D0B, B, {N->dD0b, 32, 0}, {N->D0a, 32, 0}, {N->dD0a, 32, 0}, {N->D0a, 32, 0}, 0));
+  NET_TRY(layer_bwd(N, g, D0A, B, {N->dD0a, 32, 0}, {N->C0, 64, 0}, {N->dC0, 64, 0}, none, 0));
+  NET_TRY(layer_bwd(N, g, U0, B, {N->dC0, 64, 0}, {N->D1b, 32, 0}, {N->dD1b, 32, 0}, {N->D1b, 32, 0}, 1));
+  NET_TRY(layer_bwd(N, g, D1B, B, {N->dD1b, 32, 0}, {N->D1a, 32, 0}, {N->dD1a, 32, 0}, {N->D1a, 32, 0}, 1));
+  NET_TRY(layer_bwd(N, g, D1A, B, {N->dD1a, 32, 0}, {N->C1, 64, 0}, {N->dC1, 64, 0}, none, 1));
+  NET_TRY(layer_bwd(N, g, U1, B, {N->dC1, 64, 0}, {N->D2b, 32, 0}, {N->dD2b, 32, 0}, {N->D2b, 32, 0}, 2));
+  NET_TRY(layer_bwd(N, g, D2B, B, {N->dD2b, 32, 0}, {N->D2a, 32, 0}, {N->dD2a, 32, 0}, {N->D2a, 32, 0}, 2));
+  NET_TRY(layer_bwd(N, g, D2A, B, {N->dD2a, 32, 0}, {N->C2, 64, 0}, {N->dC2, 64, 0}, none, 2));
+  NET_TRY(layer_bwd(N, g, U2, B, {N->dC2, 64, 0}, {N->H3, 48, 0}, {N->dH3, 48, 0}, {N->H3, 48, 0}, 3));
+  NET_TRY(layer_bwd(N, g, E3B, B, {N->dH3, 48, 0}, {N->A3, 48, 0}, {N->dA3, 48, 0}, {N->A3, 48, 0}, 3));
+  NET_TRY(layer_bwd(N, g, E3A, B, {N->dA3, 48, 0}, {N->P2, 32, 0}, {N->dP2, 32, 0}, none, 3));
+  NET_TRY(unpool_gate(N, {N->dP2, 32, 0}, {N->dC2, 64, 32}, {N->C2, 64, 32}, 32, 2, B));
+  NET_TRY(layer_bwd(N, g, E2B, B, {N->dC2, 64, 32}, {N->A2, 32, 0}, {N->dA2, 32, 0}, {N->A2, 32, 0}, 2));
+  NET_TRY(layer_bwd(N, g, E2A, B, {N->dA2, 32, 0}, {N->P1, 32, 0}, {N->dP1, 32, 0}, none, 2));
+  NET_TRY(unpool_gate(N, {N->dP1, 32, 0}, {N->dC1, 64, 32}, {N->C1, 64, 32}, 32, 1, B));
+  NET_TRY(layer_bwd(N, g, E1B, B, {N->dC1, 64, 32}, {N->A1, 32, 0}, {N->dA1, 32, 0}, {N->A1, 32, 0}, 1));
+  NET_TRY(layer_bwd(N, g, E1A, B, {N->dA1, 32, 0}, {N->P0, 32, 0}, {N->dP0, 32, 0}, none, 1));
+  NET_TRY(unpool_gate(N, {N->dP0, 32, 0}, {N->dC0, 64, 32}, {N->C0, 64, 32}, 32, 0, B));
+  NET_TRY(layer_bwd(N, g, E0B, B, {N->dC0, 64, 32}, {N->A0, 32, 0}, {N->dA0, 32, 0}, {N->A0, 32, 0}, 0));
+  NET_TRY(layer_bwd(N, g, E0A, B, {N->dA0, 32, 0}, {N->X0, 16, 0}, none, none, 0));
   return cudaSuccess;
 }
 
 cudaError_t loss_and_grad(bfcs_net_s* N, int B, const float* target, double* loss_dev) {
   k_loss<<<dim3(kLossBlocks, B), 256, 0, N->st>>>(N->OUT, target, N->n[0], N->lnum, N->lden);
-  k_loss_final<<<1, 32, 0, N->st>>>(N->lnum, N->lden, kLossBlocks, B, N->den_b, loss_dev);
-  k_loss_grad<<<grid_for(N->n[0] * B), 256, 0, N->st>>>(N->OUT, target, N->den_b, N->n[0], B, N->dOUT);
+  k_loss_final<<<1, 256, 0, N->st>>>(N->lnum, N->lden, kLossBlocks, B, N->den_b, N->rel_b, loss_dev);
+  const int bx = std::max(1, std::min(ceil_div(N->n[0], 256), ceil_div(152 * 16, B)));
+  k_loss_grad<<<dim3(bx, B), 256, 0, N->st>>>(N->OUT, target, N->den_b, N->n[0], B, N->dOUT);
   count_launches(3);
-  return cudaGetLastError();
-}
-
-cudaError_t grads_to_flat(bfcs_net_s* N, float* grad) {
-  for (int l = 0; l < kNumLayers; ++l) {
-    const LayerDef& L = N->def[l];
-    const long long nw = (long long)(L.kind == 0 ? 27 : 1) * L.cout * L.cin * (L.kind == 2 ? 8 : 1) + L.cout;
-    k_unpack_grad<<<grid_for(nw), 256, 0, N->st>>>(N->gw[l], N->gb[l], L, grad);
-  }
-  count_launches(kNumLayers);
   return cudaGetLastError();
 }
 
@@ -1016,6 +1083,33 @@ bool valid_phases(int nphases, const bfcs_lame* phases) {
   for (int p = 0; p < nphases; ++p)
     if (!(phases[p].mu > 0.0) || !std::isfinite(phases[p].mu)) return false;
   return true;
+}
+
+// strain predictions of `batch` samples, maxb at a time
+template <typename R>
+int predict(bfcs_net_s* N, const float* params, int batch, const R* const* b, const int8_t* const* phase, int nphases,
+            const bfcs_lame* phases, R* const* eps_out) {
+  MuTab mt;
+  const float mu_max = mu_table(nphases, phases, &mt);
+  const long long n = N->n[0];
+  cudaError_t e = pack_all(N, params);
+  for (int i0 = 0; i0 < batch && e == cudaSuccess; i0 += N->maxb) {
+    const int B = std::min(N->maxb, batch - i0);
+    cudaMemsetAsync(N->sbits, 0, B * sizeof(unsigned), N->st);
+    for (int j0 = 0; j0 < B; j0 += kSampleArgs) {
+      const int k = std::min(kSampleArgs, B - j0);
+      SampleArgs<R> sa{};
+      for (int j = 0; j < k; ++j) { sa.b[j] = b[i0 + j0 + j]; sa.phase[j] = phase[i0 + j0 + j]; }
+      const int bx = std::max(1, std::min(ceil_div(n, 256), ceil_div(152 * 8, k)));
+      k_absmax<R><<<dim3(bx, k), 256, 0, N->st>>>(sa, 3 * n, N->sbits + j0);
+      k_prepare_x0<R><<<dim3(bx, k), 256, 0, N->st>>>(sa, mt, N->sbits + j0, N->X0 + (long long)j0 * n * 16, n);
+      count_launches(2);
+    }
+    e = forward(N, params, B);
+    if (e == cudaSuccess) e = head<R>(N, params, B, eps_out + i0, true, mu_max);
+  }
+  if (e == cudaSuccess) e = cudaGetLastError();
+  return status_of(e);
 }
 
 }  // namespace
@@ -1062,22 +1156,17 @@ int bfcs_net_create(bfcs_net* out, int nx, int ny, int nz, int max_batch, int fl
   act(&N->P0, 1, 32); act(&N->A1, 1, 32); act(&N->C1, 1, 64); act(&N->D1a, 1, 32); act(&N->D1b, 1, 32);
   act(&N->P1, 2, 32); act(&N->A2, 2, 32); act(&N->C2, 2, 64); act(&N->D2a, 2, 32); act(&N->D2b, 2, 32);
   act(&N->P2, 3, 32); act(&N->A3, 3, 48); act(&N->H3, 3, 48);
-  add(&N->OUT, (size_t)(B * n[0] * 6) * sizeof(float));
+  if (train) add(&N->OUT, (size_t)(B * n[0] * 6) * sizeof(float));
   for (int l = 0; l < kNumLayers; ++l) {
     const LayerDef& L = N->def[l];
     const size_t nw = (size_t)(L.kind == 0 ? 27 : 1) * (L.kind == 2 ? 8 * L.cout : L.cout_p) * L.cin_p;
     add(&N->fw[l], nw * sizeof(bf16));
     add(&N->bw[l], nw * sizeof(bf16));
-    N->gw[l] = nullptr;
-    N->gb[l] = nullptr;
-    if (train) {
-      add(&N->gw[l], nw * sizeof(float));
-      add(&N->gb[l], (size_t)L.cout * sizeof(float));
-    }
   }
   add(&N->lnum, (size_t)kLossBlocks * B * sizeof(double));
   add(&N->lden, (size_t)kLossBlocks * B * sizeof(double));
   add(&N->den_b, (size_t)B * sizeof(double));
+  add(&N->rel_b, (size_t)B * sizeof(double));
   add(&N->sbits, (size_t)B * sizeof(unsigned));
   add(&N->err, sizeof(int));
   if (train) {
@@ -1148,11 +1237,15 @@ int bfcs_net_prepare(bfcs_net N, int precision, const void* b, const int8_t* pha
   const long long n = N->n[0];
   cudaMemsetAsync(N->sbits, 0, sizeof(unsigned), N->st);
   if (precision == BFCS_FP64) {
-    k_absmax<double><<<grid_for(3 * n), 256, 0, N->st>>>((const double*)b, 3 * n, N->sbits);
+    SampleArgs<double> sa{};
+    sa.b[0] = (const double*)b;
+    k_absmax<double><<<std::min(304, grid_for(3 * n)), 256, 0, N->st>>>(sa, 3 * n, N->sbits);
     k_prepare<double><<<grid_for(n), 256, 0, N->st>>>((const double*)b, phase, mt, N->sbits, (const double*)eps, x_out,
                                                       target_out, n);
   } else {
-    k_absmax<float><<<grid_for(3 * n), 256, 0, N->st>>>((const float*)b, 3 * n, N->sbits);
+    SampleArgs<float> sa{};
+    sa.b[0] = (const float*)b;
+    k_absmax<float><<<std::min(304, grid_for(3 * n)), 256, 0, N->st>>>(sa, 3 * n, N->sbits);
     k_prepare<float><<<grid_for(n), 256, 0, N->st>>>((const float*)b, phase, mt, N->sbits, (const float*)eps, x_out,
                                                      target_out, n);
   }
@@ -1169,11 +1262,7 @@ int bfcs_net_forward(bfcs_net N, const float* params, int batch, const float* x,
     count_launches(1);
     e = forward(N, params, batch);
   }
-  if (e == cudaSuccess) {
-    k_features_out<<<grid_for(N->n[0] * batch), 256, 0, N->st>>>(N->OUT, y, N->n[0], batch);
-    count_launches(1);
-    e = cudaGetLastError();
-  }
+  if (e == cudaSuccess) e = head_planar(N, params, batch, y);
   return status_of(e);
 }
 
@@ -1188,9 +1277,9 @@ int bfcs_net_grad(bfcs_net N, const float* params, int batch, const float* x, co
     count_launches(1);
     e = forward(N, params, batch);
   }
+  if (e == cudaSuccess) e = head_planar(N, params, batch, N->OUT);
   if (e == cudaSuccess) e = loss_and_grad(N, batch, target, loss_dev);
-  if (e == cudaSuccess) e = backward(N, batch);
-  if (e == cudaSuccess) e = grads_to_flat(N, grad);
+  if (e == cudaSuccess) e = backward(N, grad, batch);
   return status_of(e);
 }
 
@@ -1219,39 +1308,10 @@ int bfcs_net_predict(bfcs_net N, const float* params, int precision, int batch, 
     return BFCS_ERR_INVALID_ARG;
   for (int i = 0; i < batch; ++i)
     if (b[i] == nullptr || phase[i] == nullptr || eps_out[i] == nullptr) return BFCS_ERR_INVALID_ARG;
-  MuTab mt;
-  const float mu_max = mu_table(nphases, phases, &mt);
-  const long long n = N->n[0];
-  cudaError_t e = pack_all(N, params);
-  for (int i0 = 0; i0 < batch && e == cudaSuccess; i0 += N->maxb) {
-    const int B = std::min(N->maxb, batch - i0);
-    cudaMemsetAsync(N->sbits, 0, B * sizeof(unsigned), N->st);
-    for (int i = 0; i < B; ++i) {
-      if (precision == BFCS_FP64) {
-        k_absmax<double><<<grid_for(3 * n), 256, 0, N->st>>>((const double*)b[i0 + i], 3 * n, N->sbits + i);
-        k_prepare_x0<double><<<grid_for(n), 256, 0, N->st>>>((const double*)b[i0 + i], phase[i0 + i], mt,
-                                                             N->sbits + i, N->X0 + i * n * 16, n);
-      } else {
-        k_absmax<float><<<grid_for(3 * n), 256, 0, N->st>>>((const float*)b[i0 + i], 3 * n, N->sbits + i);
-        k_prepare_x0<float><<<grid_for(n), 256, 0, N->st>>>((const float*)b[i0 + i], phase[i0 + i], mt,
-                                                            N->sbits + i, N->X0 + i * n * 16, n);
-      }
-    }
-    count_launches(2 * B);
-    e = forward(N, params, B);
-    for (int i = 0; i < B && e == cudaSuccess; ++i) {
-      if (precision == BFCS_FP64)
-        k_predict_out<double><<<grid_for(n), 256, 0, N->st>>>(N->OUT + i * n * 6, N->sbits + i, mu_max,
-                                                              (double*)eps_out[i0 + i], n);
-      else
-        k_predict_out<float><<<grid_for(n), 256, 0, N->st>>>(N->OUT + i * n * 6, N->sbits + i, mu_max,
-                                                             (float*)eps_out[i0 + i], n);
-      count_launches(1);
-      e = cudaGetLastError();
-    }
-  }
-  if (e == cudaSuccess) e = cudaGetLastError();
-  return status_of(e);
+  return precision == BFCS_FP64 ? predict<double>(N, params, batch, (const double* const*)b, phase, nphases, phases,
+                                                  (double* const*)eps_out)
+                                : predict<float>(N, params, batch, (const float* const*)b, phase, nphases, phases,
+                                                 (float* const*)eps_out);
 }
 
 }  // extern "C"

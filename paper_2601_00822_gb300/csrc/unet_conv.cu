@@ -16,7 +16,7 @@
 // (SBO 128 B, LBO 16 N B).
 //
 // Roles: warps 0-7 stage planes with cp.async and drain the accumulators (tcgen05.ld,
-// bias, leaky ReLU, BF16 store); one elected thread of warp 8 issues the 27 KC / 2
+// bias, leaky ReLU or the gate of a data gradient, BF16 store); one elected thread of warp 8 issues the 27 KC / 2
 // MMAs of a tile.  Two accumulators: the epilogue and the next plane's copies run
 // under the next tile's MMAs.  Barriers (mbarrier, two of each, used by alternate
 // tiles): full = operands staged, done = MMAs complete (tcgen05.commit), empty =
@@ -281,7 +281,9 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
         // epilogue of tile k
         const int x = ex + row % kCX, y = ey + row / kCX;
         const bool store = x < a.v.nx && y < a.v.ny;
-        bf16* orow = (bf16*)a.out + ((long long)eb * nvox + ((long long)z * a.v.ny + y) * a.v.nx + x) * a.ldo + a.offo;
+        const long long vox = (long long)eb * nvox + ((long long)z * a.v.ny + y) * a.v.nx + x;
+        bf16* orow = (bf16*)a.out + vox * a.ldo + a.offo;
+        const bf16* grow = a.gate != nullptr && store ? a.gate + vox * a.ldg + a.offg : nullptr;
 #pragma unroll
         for (int c0 = 0; c0 < N; c0 += 32) {           // this warp's 16-column slices
           const int cc = c0 + half * 16;
@@ -308,6 +310,7 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
               }
               o[u] = __floats2bfloat162_rn(f0, f1);
             }
+            if (grow != nullptr) gate8(o, *reinterpret_cast<const uint4*>(grow + cc + q8));
             if (store) *reinterpret_cast<uint4*>(orow + cc + q8) = *reinterpret_cast<const uint4*>(o);
           }
         }

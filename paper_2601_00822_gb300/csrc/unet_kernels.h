@@ -35,6 +35,32 @@ struct ConvArgs {
   void* out;          // channels-last output, element (voxel, col) at out[voxel * ldo + offo + col]
   int ldo, offo;
   int up_c;           // gather / shuffle: channels per sub-voxel (multiple of 16)
+  // data gradients: the activation's derivative at the layer below, from the sign of its
+  // saved output (voxel, col) at gate[voxel * ldg + offg + col]; null: none
+  const bf16* gate;
+  int ldg, offg;
+};
+
+// 8 values times act'(y) of the 8 saved outputs in y: the BF16 values are scaled and
+// rounded again, as a pass of its own over them would
+__device__ __forceinline__ void gate8(__nv_bfloat162* o, uint4 y) {
+  const bf16* y8 = reinterpret_cast<const bf16*>(&y);
+  bf16* o8 = reinterpret_cast<bf16*>(o);
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (!(__bfloat162float(y8[k]) > 0.f)) o8[k] = __float2bfloat16(__bfloat162float(o8[k]) * kSlope);
+}
+
+constexpr int kSampleArgs = 64;      // samples whose pointers travel in one launch's arguments
+
+template <typename R> struct HeadArgs {
+  const bf16* in;                    // [sample][n][32]
+  const bf16* w;                     // [16][32], rows 6.. zero
+  const float* bias;                 // 6
+  long long n;                       // voxels of a sample
+  const unsigned* sbits;             // prediction: per-sample max |b| (bits of a float)
+  float mu_max;
+  R* out[kSampleArgs];               // 6 x n each
 };
 
 // 3^3 circular convolution on the tensor cores (unet_conv.cu); conv3_ok: the layer
@@ -42,6 +68,14 @@ struct ConvArgs {
 bool conv3_ok(const ConvArgs& a);
 cudaError_t conv3_init();   // once per network context: shared-memory limits
 cudaError_t launch_conv3(const ConvArgs& a, int sms, int* err, cudaStream_t st);
+
+// pointwise GEMMs (unet_gemm.cu): up-convolutions, their data gradients, the head's
+// data gradient; rows_ok: the layer shapes they are compiled for
+bool rows_ok(const ConvArgs& a);
+cudaError_t launch_rows(const ConvArgs& a, int sms, cudaStream_t st);
+// the head for up to kSampleArgs samples
+template <typename R>
+cudaError_t launch_head(const HeadArgs<R>& a, int batch, bool predict, int sms, cudaStream_t st);
 
 }  // namespace net
 }  // namespace bfcs

@@ -190,3 +190,28 @@ def test_tensor_core_convolutions_equal_the_warp_level_ones_bit_for_bit(dims, ba
     net.status()
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-14, 1e-20, 1e18])
+def test_loss_and_its_gradient_over_the_range_of_the_fields(scale):
+    """The loss of the network's own output, written out in FP64, for targets and outputs
+    far below and above 1 (squares outside the FP32 range); the head's bias gradient is the
+    sum of the loss gradient over the voxels."""
+    dims = (24, 8, 16)
+    flat = params(31).float()
+    wslice, bslice = layer_slices()[-1][1:]
+    flat[wslice] *= scale
+    flat[bslice] *= scale
+    flat = flat.cuda()
+    x = inputs(32, 2, dims).float().cuda()
+    t = (scale * inputs(33, 2, dims, ch=6)).float().cuda()
+    t[:, 3] = 0.0
+    net = api.Net(dims, max_batch=2, train=True)
+    y = net.forward(flat, x).double()
+    g, loss = net.grad(flat, x, t)
+    d = y - t.double()
+    den = (t.double() ** 2).sum((1, 2, 3, 4))
+    want = ((d ** 2).sum((1, 2, 3, 4)) / den).mean()
+    assert abs(float(loss) - float(want)) <= 1e-12 * float(want)
+    db = (2.0 * d / (2 * den.view(-1, 1, 1, 1, 1))).sum((0, 2, 3, 4))
+    assert rel(g[bslice].double().cpu(), db.cpu()) <= 1e-2     # BF16 terms, 2^-9 each
