@@ -44,6 +44,7 @@ UNITS = [
     ("unet.cu", [], "unet.o"),
     ("unet_conv.cu", [], "unet_conv.o"),
     ("unet_gemm.cu", [], "unet_gemm.o"),
+    ("unet_wgrad.cu", [], "unet_wgrad.o"),
 ]
 
 

@@ -141,36 +141,12 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
   }
 }
 
-// Voxel tile and circular halo of the tiled weight gradient (k_wgrad3t).
-constexpr int kTX = 16, kTY = 8, kTZ = 2;
-constexpr int kHX = kTX + 2, kHY = kTY + 2, kHZ = kTZ + 2, kHalo = kHX * kHY * kHZ;
-
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::);
-}
-
 // ------------------------------------------------------------------ weight gradient
 // dW[tap][co][ci] = sum over (b, v) of dY[b][v][co] X[b][v + d_tap][ci]; for an
 // up-convolution (up_c > 0) dW[o up_c + co][ci] = sum over (b, u) of
 // dY[b][2u + o][co] X[b][u][ci] with dY read from the fine grid.
 // Block (chunk, tap x mchunk): voxels [chunk * rows_per, ...), 64 output
 // channels; partial[chunk][tap][cout_p][cin] in FP32.
-struct WgArgs {
-  const bf16* dy; int ldd, offd;   // output gradient (pre-activation)
-  const bf16* x; int ldx, offx;    // layer input
-  int cin, cout_p;                 // multiples of 16; cin <= 128; cout_p <= 64 or a multiple of 64
-  int ksize;
-  Vol v;                           // grid of the GEMM K index (coarse grid for the up mode)
-  int batch;
-  int up_c;
-  long long chunk;                 // voxels per block (multiple of 64)
-  float* part;
-};
-
 constexpr int kWgRows = 64;
 
 __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
@@ -191,13 +167,7 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mt = mcols / 16;
   const int FX = 2 * a.v.nx, FY = 2 * a.v.ny;
-  float acc[4][4][4];                               // [m16 tile][n8 tile of this warp][4]
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
+  float sum[4][4][4] = {};                          // [m16 tile][n8 tile of this warp][4]
   const int dvec = mcols / 8, xvec = a.cin / 8;
   for (long long r0 = start; r0 < stop; r0 += kWgRows) {
     __syncthreads();
@@ -229,6 +199,10 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
       *reinterpret_cast<uint4*>(dst) = val;
     }
     __syncthreads();
+    // the stage's 64 rows in accumulators of their own, added to the running sums with
+    // rounding: the tensor core truncates each accumulation, and over the thousand
+    // steps of a chunk that bias grows to 1e-5 of the sum
+    float acc[4][4][4] = {};
 #pragma unroll
     for (int ks = 0; ks < kWgRows; ks += 16) {
       const int mi = lane >> 3, rr = lane & 7;
@@ -255,6 +229,12 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
         }
       }
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sum[i][j][q] += acc[i][j][q];
   }
   const int g = lane >> 2, t = lane & 3;
   float* out = a.part + ((long long)blockIdx.x * taps + tap) * a.cout_p * a.cin;
@@ -267,7 +247,7 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
       for (int h = 0; h < 2; ++h) {
         const int n0 = (warp + 4 * p) * 16 + h * 8;
         if (n0 >= a.cin) continue;
-        const float* c = acc[i][2 * p + h];
+        const float* c = sum[i][2 * p + h];
         const int co = mc * mcols + i * 16 + g, ci = n0 + 2 * t;
         out[(long long)co * a.cin + ci] = c[0];
         out[(long long)co * a.cin + ci + 1] = c[1];
@@ -276,126 +256,6 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
       }
     }
   }
-}
-
-// Tiled weight gradient of a 3^3 convolution with 32 output channels:
-// block (i, s) walks voxel tiles i, i + gridDim.x, ... (16 x 8 x 2 voxels of
-// one sample); per tile it stages dY (256 x 32, row pitch 40 elements:
-// conflict-free ldmatrix.trans) and the circular halo of X for the input
-// channels [32 s, 32 s + 32) (swizzled as in k_conv3t), then warp w
-// accumulates the taps 3w .. 3w + 2 in registers: dW[tap] += dY^T X_shifted,
-// K = the 16 voxels of one tile row per step.  partial[i][tap][co][ci] FP32.
-// Needs cout_p == 32, the tiled grid, cin in {16, 32, 64}.
-constexpr int kWgtWarps = 9, kWgtDP = 40;
-
-size_t wgrad3t_smem(int cin) {
-  return (size_t)kTX * kTY * kTZ * kWgtDP * sizeof(bf16) + (size_t)kHalo * (cin < 32 ? cin : 32) * sizeof(bf16);
-}
-
-__global__ void __launch_bounds__(kWgtWarps * 32) k_wgrad3t(WgArgs a) {
-  extern __shared__ __align__(128) unsigned char smw[];
-  const int cs = min(a.cin, 32);
-  const int c0 = blockIdx.y * cs;
-  const int chunks = cs >> 3;
-  const int sh = chunks == 4 ? 1 : 2;
-  const int rowb = cs * 2;
-  bf16* sD = reinterpret_cast<bf16*>(smw);
-  unsigned char* sX = smw + kTX * kTY * kTZ * kWgtDP * sizeof(bf16);
-  const unsigned sXb = (unsigned)__cvta_generic_to_shared(sX);
-  const int ntx = a.v.nx / kTX, nty = a.v.ny / kTY, ntz = a.v.nz / kTZ;
-  const int per_sample = ntx * nty * ntz;
-  const long long nvox = (long long)a.v.nx * a.v.ny * a.v.nz;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int mi = lane >> 3, rr = lane & 7;
-  const int tap0 = warp * 3;
-  const int np = cs / 16;     // n16 pairs
-  float acc[3][2][4][4];
-#pragma unroll
-  for (int u = 0; u < 3; ++u)
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[u][i][j][q] = 0.f;
-  for (int tile = blockIdx.x; tile < per_sample * a.batch; tile += gridDim.x) {
-    const int b = tile / per_sample;
-    int tb = tile - b * per_sample;
-    const int x0 = (tb % ntx) * kTX;
-    tb /= ntx;
-    const int y0 = (tb % nty) * kTY, z0 = (tb / nty) * kTZ;
-    __syncthreads();   // the previous tile's shared-memory reads are done
-    for (int i = threadIdx.x; i < kTX * kTY * kTZ * 4; i += blockDim.x) {
-      const int v = i >> 2, c = i & 3;
-      const long long vox = ((long long)(z0 + v / (kTX * kTY)) * a.v.ny + y0 + (v / kTX) % kTY) * a.v.nx + x0 + v % kTX;
-      cp_async16(sD + v * kWgtDP + c * 8, a.dy + ((long long)b * nvox + vox) * a.ldd + a.offd + c * 8);
-    }
-    for (int i = threadIdx.x; i < kHalo * chunks; i += blockDim.x) {
-      const int v = i / chunks, c = i - v * chunks;
-      const int hx = v % kHX, hy = (v / kHX) % kHY, hz = v / (kHX * kHY);
-      const int gx = wrap(x0 + hx - 1, a.v.nx), gy = wrap(y0 + hy - 1, a.v.ny), gz = wrap(z0 + hz - 1, a.v.nz);
-      const bf16* src = a.x + ((long long)b * nvox + ((long long)gz * a.v.ny + gy) * a.v.nx + gx) * a.ldx + a.offx +
-                        c0 + c * 8;
-      cp_async16(sX + v * rowb + 16 * (c ^ ((v >> sh) & (chunks - 1))), src);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    if (tap0 >= 27) continue;
-    for (int r = 0; r < kTY * kTZ; ++r) {
-      const int yy = r % kTY, zz = r / kTY;
-      unsigned af[2][4];
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-        ldsm_x4_trans(af[i], sD + (r * kTX + (mi >> 1) * 8 + rr) * kWgtDP + i * 16 + (mi & 1) * 8);
-#pragma unroll
-      for (int u = 0; u < 3; ++u) {
-        const int tap = tap0 + u;
-        const int hv0 = ((zz + 1 + tap / 9 - 1) * kHY + (yy + 1 + (tap / 3) % 3 - 1)) * kHX + 1 + (tap % 3 - 1) +
-                        (mi & 1) * 8 + rr;
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          if (p < np) {
-            const int ch = 2 * p + (mi >> 1);
-            unsigned bq[4];
-            const unsigned addr = sXb + hv0 * rowb + 16 * (ch ^ ((hv0 >> sh) & (chunks - 1)));
-            asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                         : "=r"(bq[0]), "=r"(bq[1]), "=r"(bq[2]), "=r"(bq[3])
-                         : "r"(addr));
-            const unsigned b0[2] = {bq[0], bq[1]};
-            const unsigned b1[2] = {bq[2], bq[3]};
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              mma16816(acc[u][i][2 * p], af[i], b0);
-              mma16816(acc[u][i][2 * p + 1], af[i], b1);
-            }
-          }
-        }
-      }
-    }
-  }
-  if (tap0 >= 27) return;
-  const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-  for (int u = 0; u < 3; ++u) {
-    float* out = a.part + ((long long)blockIdx.x * 27 + tap0 + u) * 32 * a.cin + c0;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j >= 2 * np) continue;
-        const int co = i * 16 + g, ci = j * 8 + 2 * t;
-        out[(long long)co * a.cin + ci] = acc[u][i][j][0];
-        out[(long long)co * a.cin + ci + 1] = acc[u][i][j][1];
-        out[(long long)(co + 8) * a.cin + ci] = acc[u][i][j][2];
-        out[(long long)(co + 8) * a.cin + ci + 1] = acc[u][i][j][3];
-      }
-  }
-}
-
-bool wgrad3t_ok(const WgArgs& a) {
-  return a.ksize == 3 && a.up_c == 0 && a.cout_p == 32 && a.v.nx % kTX == 0 && a.v.ny % kTY == 0 &&
-         a.v.nz % kTZ == 0 && (a.cin == 16 || a.cin == 32 || a.cin == 64) && a.ldd % 8 == 0 && a.offd % 8 == 0 &&
-         a.ldx % 8 == 0 && a.offx % 8 == 0;
 }
 
 // ------------------------------------------------------------------ elementwise
@@ -972,26 +832,28 @@ cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View 
   nchunks = ceil_div(rows, w.chunk);
   const long long per = (long long)taps * w.cout_p * w.cin;
   const int bc = dch;
-  const int nblk = std::max(1, std::min(kBiasBlocks, ceil_div(orows, 64)));
+  const bool tc = wgrad3_ok(w) && tcgen05_enabled(), pw = wgrad1_ok(w);
+  if (tc) nchunks = wgrad3_chunks(w, sm_count());
+  else if (pw) nchunks = wgrad1_chunks(w, sm_count());
+  const int nblk = tc ? nchunks : pw ? (up ? 8 * nchunks : nchunks)
+                                     : std::max(1, std::min(kBiasBlocks, ceil_div(orows, 64)));
   if ((long long)nchunks * per + (long long)nblk * bc > N->part_cap) return cudaErrorInvalidValue;
   w.part = N->part;
-  if (wgrad3t_ok(w)) {
-    const long long tiles = (long long)(w.v.nx / kTX) * (w.v.ny / kTY) * (w.v.nz / kTZ) * B;
-    nchunks = (int)std::min<long long>(tiles, 152);
-    if ((long long)nchunks * per + (long long)nblk * bc > N->part_cap) return cudaErrorInvalidValue;
-    k_wgrad3t<<<dim3(nchunks, w.cin > 32 ? w.cin / 32 : 1), kWgtWarps * 32, wgrad3t_smem(w.cin), N->st>>>(w);
+  w.bpart = N->part + (long long)nchunks * per;
+  if (tc || pw) {   // with the bias gradient
+    const cudaError_t e = tc ? launch_wgrad3(w, nchunks, N->err, N->st) : launch_wgrad1(w, sm_count(), N->st);
+    if (e != cudaSuccess) return e;
   } else {
     const int mcols = std::min(64, w.cout_p);
     const size_t smem = (size_t)kWgRows * (mcols + 8 + w.cin + 8) * sizeof(bf16);
     k_wgrad<<<dim3(nchunks, taps * mchunks), 128, smem, N->st>>>(w);
+    const long long bper = (orows + nblk - 1) / nblk;
+    k_bias_grad<<<nblk, kBiasThreads, 0, N->st>>>(dout.p, dout.ld, dout.off, bc, orows, bper, w.bpart);
+    count_launches(2);
   }
-  // bias gradient (over the rows of the output gradient), then both sums
-  const long long bper = (orows + nblk - 1) / nblk;
-  float* bpart = N->part + (long long)nchunks * per;
-  k_bias_grad<<<nblk, kBiasThreads, 0, N->st>>>(dout.p, dout.ld, dout.off, bc, orows, bper, bpart);
   k_reduce_grad<<<ceil_div(per, kRedOut) + ceil_div(bc, kRedOut), kRedOut * kRedLanes, 0, N->st>>>(
-      N->part, nchunks, bpart, nblk, bc, L, grad);
-  count_launches(3);
+      N->part, nchunks, w.bpart, nblk, bc, L, grad);
+  count_launches(1);
   // input gradient: a convolution with the data-gradient weights
   if (din.p != nullptr) {
     ConvArgs a{};
@@ -1198,9 +1060,8 @@ int bfcs_net_create(bfcs_net* out, int nx, int ny, int nz, int max_batch, int fl
     *r.first = N->base + pos;
     pos += (r.second + 255) / 256 * 256;
   }
-  if (conv3_init() != cudaSuccess ||
-      cudaFuncSetAttribute(k_wgrad3t, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad3t_smem(64)) !=
-          cudaSuccess) {
+  if (conv3_init() != cudaSuccess || wgrad3_init() != cudaSuccess ||
+      wgrad1_init() != cudaSuccess) {
     cudaGetLastError();
     free_net(N);
     return BFCS_ERR_CUDA;

@@ -30,6 +30,7 @@
 // compile-time tap offsets on the uniform data path: a rolled tap loop on thread 0
 // measured 122 clocks per MMA, the unrolled loop under elect.sync 48.
 #include "unet_kernels.h"
+#include "unet_tc.cuh"
 
 #include <algorithm>
 
@@ -42,9 +43,8 @@ constexpr int kCX = 8, kCY = 16;                      // tile
 constexpr int kCHX = kCX + 2, kCHY = kCY + 2;         // halo plane
 constexpr int kCHalo = kCHX * kCHY;
 constexpr int kRing = 4;
-constexpr int kWorkers = 256;                         // warps 0-7
+constexpr int kWorkers = kTcWorkers;                  // warps 0-7
 constexpr int kConv3Threads = kWorkers + 32;
-constexpr unsigned kSpinLimit = 1u << 26;             // bound of every mbarrier wait
 
 template <int KC, int N> struct C3 {
   // plane pitch in voxels: chunk stride 16 PV such that the 16-byte writes of 8 / KC
@@ -59,64 +59,6 @@ template <int KC, int N> struct C3 {
   static constexpr int ACC = N <= 32 ? 32 : 64;       // TMEM columns of one accumulator (a power of two in all)
   static constexpr int NJ = (kCHalo * KC + kWorkers - 1) / kWorkers;   // plane copies per thread
 };
-
-__device__ __forceinline__ void cp16(unsigned dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int LEFT> __device__ __forceinline__ void cp_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(LEFT) : "memory");
-}
-__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-__device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-
-__device__ __forceinline__ bool elect_one() {
-  unsigned p;
-  asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
-  return p != 0;
-}
-__device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
-}
-// bounded wait for the phase of the given parity; gives up early once *fail is set
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int* fail) {
-  unsigned done = 0, spins = 0;
-  while (!done) {
-    asm volatile(
-        "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (!done && (++spins > kSpinLimit || *fail)) return false;
-  }
-  return true;
-}
-// barrier of the worker warps; true when the predicate held in all of them
-__device__ __forceinline__ bool workers_all(bool ok) {
-  unsigned r;
-  asm volatile(
-      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.and.pred q, 1, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"((unsigned)ok), "n"(kWorkers)
-      : "memory");
-  return r != 0;
-}
-
-__device__ __forceinline__ uint64_t sdesc(unsigned saddr, unsigned lbo, unsigned sbo) {
-  // start address, leading (K) and stride (M/N) byte offsets in 16-byte units,
-  // descriptor version 1 (bit 46), no swizzle, base offset 0
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
-}
-// instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
-// (bits 7-9 and 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-constexpr unsigned idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
-}
 
 }  // namespace
 
@@ -290,12 +232,7 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
           if (cc >= N) break;
           unsigned v[16];
           const unsigned taddr = tmem + ((unsigned)(quarter * 32) << 16) + (unsigned)((k & 1) * C::ACC + cc);
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-              : "r"(taddr));
-          asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+          tmem_ld16(v, taddr);
 #pragma unroll
           for (int q8 = 0; q8 < 16; q8 += 8) {
             __align__(16) __nv_bfloat162 o[4];

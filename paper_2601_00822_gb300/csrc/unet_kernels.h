@@ -69,6 +69,33 @@ bool conv3_ok(const ConvArgs& a);
 cudaError_t conv3_init();   // once per network context: shared-memory limits
 cudaError_t launch_conv3(const ConvArgs& a, int sms, int* err, cudaStream_t st);
 
+// weight gradients (see k_wgrad in unet.cu): partial[chunk][tap][cout_p][cin] in FP32
+struct WgArgs {
+  const bf16* dy; int ldd, offd;   // output gradient (pre-activation)
+  const bf16* x; int ldx, offx;    // layer input
+  int cin, cout_p;                 // multiples of 16; cin <= 128; cout_p <= 64 or a multiple of 64
+  int ksize;
+  Vol v;                           // grid of the GEMM K index (coarse grid for the up mode)
+  int batch;
+  int up_c;
+  long long chunk;                 // voxels per block (multiple of 64)
+  float* part;
+  float* bpart;                    // bias gradient partials of the fused forms: [chunk][32] (3^3), [chunk][8][32]
+                                   // (up), [chunk][16] (head)
+};
+// tcgen05 form of the 3^3 layers with 32 output channels (unet_wgrad.cu): wgrad3_chunks
+// partials, one per block
+bool wgrad3_ok(const WgArgs& a);
+cudaError_t wgrad3_init();
+int wgrad3_chunks(const WgArgs& a, int sms);
+cudaError_t launch_wgrad3(const WgArgs& a, int chunks, int* err, cudaStream_t st);
+
+// the up-convolutions and the head
+bool wgrad1_ok(const WgArgs& a);
+cudaError_t wgrad1_init();
+int wgrad1_chunks(const WgArgs& a, int sms);
+cudaError_t launch_wgrad1(const WgArgs& a, int sms, cudaStream_t st);
+
 // pointwise GEMMs (unet_gemm.cu): up-convolutions, their data gradients, the head's
 // data gradient; rows_ok: the layer shapes they are compiled for
 bool rows_ok(const ConvArgs& a);
