@@ -417,9 +417,9 @@ __global__ void k_loss(const float* pred, const float* target, long long n, doub
     den[b * gridDim.x + blockIdx.x] = s1;
   }
 }
-// den_b[b], and loss = mean over b of num_b / den_b (written if loss != null): one warp
-// per sample in turn, then thread 0 over the samples
-__global__ void k_loss_final(const double* num, const double* den, int nblk, int batch, double* den_b, double* rel_b,
+// The factor 2 / (den_b B) of the gradient, and loss = mean over b of num_b / den_b
+// (written if loss != null): one warp per sample in turn, then thread 0 over the samples
+__global__ void k_loss_final(const double* num, const double* den, int nblk, int batch, double* fac_b, double* rel_b,
                              double* loss) {
   const int lane = threadIdx.x & 31;
   for (int b = threadIdx.x >> 5; b < batch; b += blockDim.x >> 5) {
@@ -429,7 +429,7 @@ __global__ void k_loss_final(const double* num, const double* den, int nblk, int
       s0 += __shfl_down_sync(0xffffffffu, s0, off);
       s1 += __shfl_down_sync(0xffffffffu, s1, off);
     }
-    if (lane == 0) { den_b[b] = s1; rel_b[b] = s0 / s1; }
+    if (lane == 0) { fac_b[b] = 2.0 / (s1 * batch); rel_b[b] = s0 / s1; }
   }
   __syncthreads();
   if (threadIdx.x == 0 && loss != nullptr) {
@@ -442,12 +442,11 @@ __global__ void k_loss_final(const double* num, const double* den, int nblk, int
 // [B][N][16] BF16 (channels 6..15 zero); one voxel per thread; float-float products
 // (48 bits before the one rounding to FP32, where the FP64 form has 53; 155 us of FP64
 // pipe for 8 samples of 64^3), FP64 outside their range
-__global__ void k_loss_grad(const float* pred, const float* target, const double* den_b, long long n, int batch,
-                            bf16* dy) {
+__global__ void k_loss_grad(const float* pred, const float* target, const double* fac_b, long long n, bf16* dy) {
   const int b = blockIdx.y;
-  const double fd = 2.0 / (den_b[b] * batch);
-  const ff f = ff(fd);
-  const bool fast = fd > 1e-18 && fd < 1e18;
+  const double fd = fac_b[b];
+  const ff f = d2ff_bits(fd);       // (FP64 divisions and conversions by every thread took 65 us)
+  const bool fast = f.hi > 1e-18f && f.hi < 1e18f;
   const float* pb = pred + (long long)b * 6 * n;
   const float* tb = target + (long long)b * 6 * n;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
@@ -676,7 +675,7 @@ struct bfcs_net_s {
   long long part_cap = 0;
   double* lnum;              // loss partials
   double* lden;
-  double* den_b;
+  double* fac_b;
   double* rel_b;
   unsigned* sbits;           // per-sample max |b|
   int* err;                  // set by a kernel whose bounded wait expired
@@ -835,7 +834,7 @@ cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View 
   const bool tc = wgrad3_ok(w) && tcgen05_enabled(), pw = wgrad1_ok(w);
   if (tc) nchunks = wgrad3_chunks(w, sm_count());
   else if (pw) nchunks = wgrad1_chunks(w, sm_count());
-  const int nblk = tc ? nchunks : pw ? (up ? 8 * nchunks : nchunks)
+  const int nblk = tc ? nchunks : pw ? (up ? nchunks / 2 : nchunks)
                                      : std::max(1, std::min(kBiasBlocks, ceil_div(orows, 64)));
   if ((long long)nchunks * per + (long long)nblk * bc > N->part_cap) return cudaErrorInvalidValue;
   w.part = N->part;
@@ -915,9 +914,9 @@ cudaError_t backward(bfcs_net_s* N, float* g, int B) {
 
 cudaError_t loss_and_grad(bfcs_net_s* N, int B, const float* target, double* loss_dev) {
   k_loss<<<dim3(kLossBlocks, B), 256, 0, N->st>>>(N->OUT, target, N->n[0], N->lnum, N->lden);
-  k_loss_final<<<1, 256, 0, N->st>>>(N->lnum, N->lden, kLossBlocks, B, N->den_b, N->rel_b, loss_dev);
+  k_loss_final<<<1, 256, 0, N->st>>>(N->lnum, N->lden, kLossBlocks, B, N->fac_b, N->rel_b, loss_dev);
   const int bx = std::max(1, std::min(ceil_div(N->n[0], 256), ceil_div(152 * 16, B)));
-  k_loss_grad<<<dim3(bx, B), 256, 0, N->st>>>(N->OUT, target, N->den_b, N->n[0], B, N->dOUT);
+  k_loss_grad<<<dim3(bx, B), 256, 0, N->st>>>(N->OUT, target, N->fac_b, N->n[0], N->dOUT);
   count_launches(3);
   return cudaGetLastError();
 }
@@ -1027,7 +1026,7 @@ int bfcs_net_create(bfcs_net* out, int nx, int ny, int nz, int max_batch, int fl
   }
   add(&N->lnum, (size_t)kLossBlocks * B * sizeof(double));
   add(&N->lden, (size_t)kLossBlocks * B * sizeof(double));
-  add(&N->den_b, (size_t)B * sizeof(double));
+  add(&N->fac_b, (size_t)B * sizeof(double));
   add(&N->rel_b, (size_t)B * sizeof(double));
   add(&N->sbits, (size_t)B * sizeof(unsigned));
   add(&N->err, sizeof(int));

@@ -80,8 +80,7 @@ struct WgArgs {
   int up_c;
   long long chunk;                 // voxels per block (multiple of 64)
   float* part;
-  float* bpart;                    // bias gradient partials of the fused forms: [chunk][32] (3^3), [chunk][8][32]
-                                   // (up), [chunk][16] (head)
+  float* bpart;                    // bias gradient partials of the fused forms: [block][channels]
 };
 // tcgen05 form of the 3^3 layers with 32 output channels (unet_wgrad.cu): wgrad3_chunks
 // partials, one per block

@@ -20,8 +20,8 @@
 // the next tile starts from zero.
 //
 // A block marches along z over a run of tiles like k_conv3.  The four planes must lie
-// one after another, so planes are staged in segments of kSeg tiles (kSeg + 2 planes in
-// kSeg + 3 slots, the last one never written: it only feeds unused rows), and the slots
+// one after another, so planes are staged in segments of up to kSeg tiles (kSeg + 2 planes
+// in kSeg + 3 slots, the last one never written: it only feeds unused rows), and the slots
 // of finished tiles take the next segment's planes.  Voxels outside the grid (partial
 // tiles) have their dY zero-filled.  At the end the block writes its partial sums; they
 // are added in block order (k_reduce_grad).
@@ -175,92 +175,79 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
                   (yvalid >> j) & 1u);
       }
     };
-    // Tile j's loads: at the start of a segment three planes, else one, and its dY.
-    // Tile j + 2 is requested once tile j's MMAs are done.  A plane's slot was last read
-    // by tiles of the segment before: within a segment of at least three tiles those are
-    // done by then; planes of a new segment are requested only once the tile before it
-    // (the last reader of any of its slots) is done, that is one step later.
-    long long col = t0 / nz;
-    int z = (int)(t0 - col * nz), pos = 0;             // tile k
-    long long lcol = col;                              // column that the sources point to
-    set_column(col);
-    auto request = [&](long long jcol, int jz, int jpos, int jr) {
-      if (jcol != lcol) { set_column(jcol); lcol = jcol; }
-      if (jpos == 0) { load_x(jz - 1, 0); load_x(jz, 1); }
-      load_x(jz + 1, jpos + 2);
-      load_y(jz, jr);
-    };
-    struct Tile { long long col; int z, pos, r; };
+    // Tile j's loads: at the start of a segment three planes, else one, and its dY; one
+    // copy group each.  They are requested up to three tiles ahead (two copies in flight
+    // under two tiles' MMAs: one tile ahead left the pass to the copies' latency, 4600
+    // clocks a tile), but not before the last reader of their slots is done: dY slot j % 3
+    // was read by tile j - 3, plane slot p + 2 of segment position p (and 0 and 1 for p =
+    // 0) last by position min(p + 2, L - 1) of the segment before, of length L.
+    struct Tile { long long col; int z, pos, prev; };  // prev: length of the segment before (0: none)
     auto after = [&](Tile t) {
       Tile u;
       u.pos = next_pos(t.z, t.pos);
       u.z = t.z + 1 == nz ? 0 : t.z + 1;
       u.col = t.z + 1 == nz ? t.col + 1 : t.col;
-      u.r = t.r + 1 == kYRing ? 0 : t.r + 1;
+      u.prev = u.pos == 0 ? t.pos + 1 : t.prev;
       return u;
     };
-    Tile cur{col, z, pos, 0}, n1 = after(cur), n2 = after(n1);
-    request(cur.col, cur.z, cur.pos, cur.r);
-    cp_commit();
-    bool have1 = n > 1 && n1.pos != 0;                 // tile k + 1 already requested
-    if (have1) request(n1.col, n1.z, n1.pos, n1.r);
-    cp_commit();
-    cp_wait<1>();
-    fence_async();
-    bool ok = workers_all(true);
-    if (tid == 0) mbar_arrive(full);
-    unsigned phase[kYRing] = {};
+    auto last_reader = [&](Tile t, int j) { return t.prev == 0 ? -1 : j - t.pos - t.prev + min(t.pos + 2, t.prev - 1); };
+    long long lcol = t0 / nz;                          // column that the sources point to
+    Tile nt{lcol, (int)(t0 - lcol * nz), 0, 0};        // next tile to request, number `next`
+    int next = 0, nring = 0;
+    set_column(lcol);
+    auto request = [&]() {
+      if (nt.col != lcol) { set_column(nt.col); lcol = nt.col; }
+      if (nt.pos == 0) { load_x(nt.z - 1, 0); load_x(nt.z, 1); }
+      load_x(nt.z + 1, nt.pos + 2);
+      load_y(nt.z, nring);
+      cp_commit();
+      nt = after(nt);
+      ++next;
+      nring = nring + 1 == kYRing ? 0 : nring + 1;
+    };
+    // tile j (the oldest copy group still of interest) has landed for this thread
+    auto landed = [&](int j) {
+      if (next - 1 - j >= 2) cp_wait<2>();
+      else if (next - 1 - j == 1) cp_wait<1>();
+      else cp_wait<0>();
+      fence_async();
+    };
     // running sums: TMEM lane = 32 dz + ci, column = 96 dy + 32 dx + co; the two warps of a
     // quarter dz take alternate 16-column slices
     const int dz = warp & 3;
     float sum[9][16] = {};
     // bias gradient: this thread's chunk (tid % 4) of dY over voxels tid / 4 and tid / 4 + 64
-    // of every tile, from the unshifted copy
+    // of every tile, from the unshifted copy, once the tile has landed for all threads
     float bsum[8] = {};
+    auto bias = [&](int r) {
+      if (blockIdx.y != 0) return;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const unsigned off = kSlots * kXPlane + (unsigned)r * kYTile + (4u + (tid & 3)) * kYC + ((tid >> 2) + 64 * h) * 16u;
+        const uint4 v = *reinterpret_cast<const uint4*>(smem + off);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) bsum[q] += __bfloat162float(reinterpret_cast<const bf16*>(&v)[q]);
+      }
+    };
+    while (next < n && next < kYRing && last_reader(nt, next) < 0) request();
+    landed(0);
+    bool ok = workers_all(true);
+    if (tid == 0) mbar_arrive(full);
+    bias(0);
+    int ring = 0, phase = 0;                           // tile k's dY slot, the phase of its done barrier
     for (int k = 0; k < n; ++k) {
-      const bool more = k + 1 < n;
-      if (more && have1) {
-        cp_wait<0>();
-        fence_async();
+      const bool more = k + 1 < n, early = more && next > k + 1;
+      const int ring1 = ring + 1 == kYRing ? 0 : ring + 1;
+      if (early) {                                     // tile k + 1, requested before
+        landed(k + 1);
         ok = workers_all(ok);
         if (!ok) break;
         if (tid == 0) mbar_arrive(full + 8 * ((k + 1) & 1));
+        bias(ring1);
       }
-      unsigned ph = 0;
-#pragma unroll
-      for (int r = 0; r < kYRing; ++r)
-        if (r == cur.r) { ph = phase[r]; phase[r] ^= 1u; }
-      ok = mbar_wait(done + 8 * cur.r, ph, fail) && ok;
-      // (no barrier at the top of this step: the dY slot that tile k + 2 or k + 3 takes may
-      // still be read for the bias by a warp behind)
-      if (more && !have1) ok = workers_all(ok);
-      bool have2 = false;
-      if (ok) {
-        if (more && !have1) request(n1.col, n1.z, n1.pos, n1.r);
-        if (k + 2 < n && n2.pos != 0) { request(n2.col, n2.z, n2.pos, n2.r); have2 = true; }
-        cp_commit();
-      } else if (lane == 0) {
-        *fail = 1;
-        atomicExch(err, 1);
-      }
-      if (more && !have1) {
-        cp_wait<0>();
-        fence_async();
-        ok = workers_all(ok);
-        if (!ok) break;
-        if (tid == 0) mbar_arrive(full + 8 * ((k + 1) & 1));
-      }
-      // (tile k's dY slot is taken by tile k + 3, requested after the next workers_all)
-      if (ok && blockIdx.y == 0) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const unsigned off = kSlots * kXPlane + (unsigned)cur.r * kYTile + (4u + (tid & 3)) * kYC + ((tid >> 2) + 64 * h) * 16u;
-          const uint4 v = *reinterpret_cast<const uint4*>(smem + off);
-#pragma unroll
-          for (int q = 0; q < 8; ++q) bsum[q] += __bfloat162float(reinterpret_cast<const bf16*>(&v)[q]);
-        }
-      }
-      if (!more || (k + 1) % kFlush == 0) {
+      ok = mbar_wait(done + 8 * ring, (unsigned)phase, fail) && ok;
+      if (!ok && lane == 0) { *fail = 1; atomicExch(err, 1); }
+      if (!more || (k + 1) % kFlush == 0) {            // the next tile's MMAs wait for this
         if (ok && dz < 3) {
           tc_after();
 #pragma unroll
@@ -275,10 +262,20 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
         __syncwarp();
         if (lane == 0) mbar_arrive(drained);
       }
-      cur = n1;
-      n1 = n2;
-      n2 = after(n2);
-      have1 = have2;
+      // every thread has read the dY slots that are requested below (a step without the
+      // barrier above needs one here)
+      if (more && !early) ok = workers_all(ok);
+      if (ok)
+        while (next < n && next <= k + kYRing && last_reader(nt, next) <= k) request();
+      if (more && !early) {
+        landed(k + 1);
+        ok = workers_all(ok);
+        if (!ok) break;
+        if (tid == 0) mbar_arrive(full + 8 * ((k + 1) & 1));
+        bias(ring1);
+      }
+      ring = ring1;
+      if (ring == 0) phase ^= 1;
     }
     cp_wait<0>();
     ok = workers_all(ok);
@@ -443,13 +440,22 @@ __global__ void __launch_bounds__(256) k_wgrad1(WgArgs a, unsigned rows) {
         *reinterpret_cast<float2*>(out + co * cin + ci) = make_float2(sum[i][j][0], sum[i][j][1]);
         *reinterpret_cast<float2*>(out + (co + 8) * cin + ci) = make_float2(sum[i][j][2], sum[i][j][3]);
       }
+    // bias: the two sub-voxels of a warp, then the warps in order
+    __syncthreads();
+    float* red = reinterpret_cast<float*>(smem);      // [warp][32]
     if (t == 0) {
 #pragma unroll
-      for (int i = 0; i < C::MT; ++i) {
-        float* bo = a.bpart + (long long)s_id * 256 + o0 * 32 + i * 16 + g;   // [stream][o][32]
-        bo[0] = sum[i][2 * NP][0];
-        bo[8] = sum[i][2 * NP][2];
+      for (int i = 0; i < 2; ++i) {
+        red[warp * 32 + i * 16 + g] = sum[i][2 * NP][0] + sum[i + 2][2 * NP][0];
+        red[warp * 32 + i * 16 + g + 8] = sum[i][2 * NP][2] + sum[i + 2][2 * NP][2];
       }
+    }
+    __syncthreads();
+    if (tid < 32) {
+      float s = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) s += red[w * 32 + tid];
+      a.bpart[(long long)blockIdx.x * 32 + tid] = s;
     }
   } else {
     __syncthreads();
