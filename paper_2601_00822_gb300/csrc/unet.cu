@@ -367,6 +367,16 @@ __device__ __forceinline__ bool ff_square_safe(float x) {
   const float m = fabsf(x);
   return (m > 1e-11f && m < 1e15f) || m == 0.f;
 }
+// The FP64 forms of the loss terms, out of line: inlined they are computed for every
+// value and selected, and the FP64 pipe binds the pass again.
+__device__ __noinline__ void loss_terms_f64(const float* p, const float* t, double& sn, double& sd) {
+  for (int c = 0; c < 6; ++c) {
+    const double x = t[c], d = (double)p[c] - x;
+    sn += d * d;
+    sd += x * x;
+  }
+}
+__device__ __noinline__ float scaled_diff_f64(float p, float t, double f) { return (float)(((double)p - (double)t) * f); }
 // relative squared L2 loss: per (block, sample) sums of (p - t)^2 and t^2; one voxel
 // per thread, planar fields (6 x n a sample).  The six squares of a voxel are formed
 // and added in float-float (about 48 bits, FP32 pipes), voxels in FP64: with every
@@ -397,11 +407,10 @@ __global__ void k_loss(const float* pred, const float* target, long long n, doub
       sn += f2d_bits(vn.hi) + f2d_bits(vn.lo);
       sd += f2d_bits(vd.hi) + f2d_bits(vd.lo);
     } else {
-      for (int c = 0; c < 6; ++c) {
-        const double t = t6[c], d = (double)p6[c] - t;
-        sn += d * d;
-        sd += t * t;
-      }
+      double a0 = 0.0, a1 = 0.0;
+      loss_terms_f64(p6, t6, a0, a1);
+      sn += a0;
+      sd += a1;
     }
   }
   for (int off = 16; off > 0; off >>= 1) {
@@ -457,7 +466,7 @@ __global__ void k_loss_grad(const float* pred, const float* target, const double
     for (int c = 0; c < 6; ++c) {
       const float p = pb[c * n + v], t = tb[c * n + v];
       const ff d = exact_diff(p, t);
-      o[c] = __float2bfloat16(fast && ff_square_safe(d.hi) ? (float)(d * f) : (float)(((double)p - (double)t) * fd));
+      o[c] = __float2bfloat16(fast && ff_square_safe(d.hi) ? (float)(d * f) : scaled_diff_f64(p, t, fd));
     }
     uint4* d = reinterpret_cast<uint4*>(dy + ((long long)b * n + v) * 16);
     d[0] = reinterpret_cast<const uint4*>(o)[0];

@@ -150,6 +150,9 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows(ConvArgs a, unsigned ro
   }
 }
 
+// (out of line: inlined it is computed for every value and selected)
+__device__ __noinline__ float scaled_f64(float y, double f) { return (float)((double)y * f); }
+
 // The head: 32 channels to 6 strain components, written planar (sample b's component
 // c of voxel v at out[b][c n + v]) as FP32 (mode 0), or as the strain prediction
 // y s_b / mu_max in R (mode 1).
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_head(HeadArgs<R> a) {
     else if constexpr (sizeof(R) == 8) return (double)y * fd;
     else {
       const float m = fabsf(y);
-      return fast && ((m > 1e-12f && m < 1e15f) || m == 0.f) ? (float)(ff(y) * fs) : (float)((double)y * fd);
+      return fast && ((m > 1e-12f && m < 1e15f) || m == 0.f) ? (float)(ff(y) * fs) : scaled_f64(y, fd);
     }
   };
   const unsigned n = (unsigned)a.n;

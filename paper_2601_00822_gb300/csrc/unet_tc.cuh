@@ -67,6 +67,8 @@ __device__ __forceinline__ uint64_t sdesc(unsigned saddr, unsigned lbo, unsigned
 constexpr unsigned idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
 }
+// operand descriptor of the 64-byte swizzle (layout type 4 at bit 61)
+constexpr uint64_t kDescSwizzle64 = (uint64_t)4 << 61;
 // both operands MN-major (bits 15 and 16)
 constexpr unsigned kIdescMnMajorAB = (1u << 15) | (1u << 16);
 

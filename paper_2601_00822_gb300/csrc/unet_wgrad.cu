@@ -7,12 +7,15 @@
 //   B = three copies of the dY plane, copy dx shifted by dx - 1 along x (N = 96
 //       columns: dx, 32 output channels),
 //   K = the plane's 128 voxels in blocks of 16 (two rows of 8).
-// dy is a row offset of A's start address.  Both operands are MN-major without
-// swizzle, in the chunk-planar layout of the convolutions (8-channel chunk c of voxel v
-// at c * CS + 16 v): 8 channels x 8 voxels are one core matrix, the next 8 channels CS
-// further (SBO), the next 8 voxels 128 B further (LBO); four chunks to a plane or copy
-// make the stride uniform across planes and copies.  Three accumulators (dy) of 96
-// TMEM columns.
+// dy is a row offset of A's start address (whole rows of 8 voxels, so every start keeps
+// the swizzle's 512-byte alignment).  Both operands are MN-major in the 64-byte swizzle:
+// voxel v's 32 channels are 64 contiguous bytes at 64 v, 8-channel chunk c at 16-byte slot
+// c ^ ((v >> 1) & 3); eight voxels are one atom, the next eight 512 B further (SBO), the
+// next 32 channels one plane or copy further (LBO).  A voxel's four 16-byte copies land
+// side by side, which the copies need: in the chunk-planar layout of the convolutions
+// each fetched its 32-byte sector alone, twice the traffic from L2, and at 72 KB a tile
+// that bound the pass (209 us for the level-0 layer of 8 samples at 64^3).  Three
+// accumulators (dy) of 96 TMEM columns.
 //
 // The tensor core truncates when it accumulates, and a sum over a block's whole run
 // (860 steps for 8 samples of 64^3) came out 1.7e-5 off.  So every kFlush tiles the
@@ -43,15 +46,17 @@ constexpr int kGX = 8, kGY = 16, kGV = kGX * kGY;     // tile (one z plane)
 constexpr int kGHY = kGY + 2;
 constexpr int kSeg = 8;                               // tiles per staged segment
 constexpr int kSlots = kSeg + 3;
-constexpr unsigned kXC = 146 * 16;                    // chunk strides: 32 B past a multiple of 128 B, so the
-constexpr unsigned kYC = 130 * 16;                    // writes of two voxels x four chunks hit distinct banks
-constexpr unsigned kXPlane = 4 * kXC, kYTile = 12 * kYC;
+constexpr unsigned kXPlane = kGX * kGHY * 64;         // one staged plane: 8 x 18 voxels
+constexpr unsigned kYCopy = kGV * 64, kYTile = 3 * kYCopy;
 constexpr int kYRing = 3;
 constexpr int kFlush = 8;                             // tiles per accumulation in tensor memory
 constexpr unsigned kWgSmem = kSlots * kXPlane + kYRing * kYTile;
 constexpr unsigned kWgCols = 512;                     // TMEM allocation (3 x 96 columns used)
 constexpr int kXN = (kGX * kGHY * 4 + kTcWorkers - 1) / kTcWorkers;   // X copies per thread and plane
 constexpr int kYN = kGV * 12 / kTcWorkers;            // dY copies per thread and tile
+
+// byte offset of channel chunk c of voxel v (64-byte swizzle)
+__device__ __forceinline__ unsigned swz(int v, int c) { return (unsigned)v * 64u + (unsigned)((c ^ (v >> 1)) & 3) * 16u; }
 
 }  // namespace
 
@@ -103,15 +108,15 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
       }
       tc_after();
       if (elect_one()) {
-        const uint64_t ad0 = sdesc(xs + (unsigned)pos * kXPlane, 128, kXC);
-        const uint64_t bd0 = sdesc(ys + (unsigned)yr * kYTile, 128, kYC);
+        const uint64_t ad0 = sdesc(xs + (unsigned)pos * kXPlane, kXPlane, 512) | kDescSwizzle64;
+        const uint64_t bd0 = sdesc(ys + (unsigned)yr * kYTile, kYCopy, 512) | kDescSwizzle64;
         const unsigned acc = k % kFlush != 0 ? 1u : 0u;
 #pragma unroll
         for (int ks = 0; ks < kGY / 2; ++ks) {
 #pragma unroll
           for (int dy = 0; dy < 3; ++dy) {
-            const uint64_t ad = ad0 + (unsigned)((2 * ks + dy) * kGX);
-            const uint64_t bd = bd0 + (unsigned)(2 * ks * kGX);
+            const uint64_t ad = ad0 + (unsigned)((2 * ks + dy) * 32);   // 16-byte units
+            const uint64_t bd = bd0 + (unsigned)(2 * ks * 32);
             asm volatile(
                 "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tm + 96u * dy),
@@ -131,20 +136,23 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
     // ---- staging
     const long long nvox = (long long)a.v.nx * a.v.ny * nz, plane = (long long)a.v.nx * a.v.ny;
     const int c0 = blockIdx.y * 4;                     // first chunk of this half
-    const bf16 *xsrc[kXN], *ysrc[kYN];
-    unsigned yvalid = 0;
+    // this thread's copies in plane 0 of the loading column, as offsets in 16-byte units
+    // from the sample's first voxel
+    const bf16 *xbase = nullptr, *ybase = nullptr;
+    unsigned xsrc[kXN], ysrc[kYN], yvalid = 0;
+    const unsigned ldx8 = a.ldx / 8, ldd8 = a.ldd / 8;
     auto set_column = [&](long long col) {
       const int x0 = (int)(col % ntx) * kGX;
       col /= ntx;
       const int y0 = (int)(col % nty) * kGY, b = (int)(col / nty);
-      const bf16* xb = a.x + (long long)b * nvox * a.ldx + a.offx;
-      const bf16* yb = a.dy + (long long)b * nvox * a.ldd + a.offd;
+      xbase = a.x + (long long)b * nvox * a.ldx + a.offx;
+      ybase = a.dy + (long long)b * nvox * a.ldd + a.offd;
 #pragma unroll
       for (int j = 0; j < kXN; ++j) {
         const int i = tid + j * kTcWorkers, v = i / 4, c = i % 4;
         // (rows and voxels past the grid read wrapped values; their dY is zero)
         const int gx = (x0 + v % kGX) % a.v.nx, gy = (y0 + v / kGX - 1 + a.v.ny) % a.v.ny;
-        xsrc[j] = xb + ((long long)gy * a.v.nx + gx) * a.ldx + min((c0 + c) * 8, a.cin - 8);
+        xsrc[j] = (unsigned)(gy * a.v.nx + gx) * ldx8 + (unsigned)(c0 + c);
       }
       yvalid = 0;
 #pragma unroll
@@ -153,26 +161,30 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
         const int wx = x0 + v % kGX, wy = y0 + v / kGX;
         if (wx < a.v.nx && wy < a.v.ny) yvalid |= 1u << j;
         const int gx = (wx - (dx - 1) + a.v.nx) % a.v.nx, gy = wy % a.v.ny;
-        ysrc[j] = yb + ((long long)gy * a.v.nx + gx) * a.ldd + c * 8;
+        ysrc[j] = (unsigned)(gy * a.v.nx + gx) * ldd8 + (unsigned)c;
       }
     };
+    // where there is nothing to copy zeros are stored
+    auto copy = [&](unsigned dst, const bf16* src, bool valid) {
+      if (valid) cp16(dst, src);
+      else asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};\n" ::"r"(dst), "r"(0u) : "memory");
+    };
     auto load_x = [&](int z, int slot) {
-      const long long off = (long long)wrap(z, nz) * plane * a.ldx;
+      const bf16* base = xbase + (long long)wrap(z, nz) * plane * a.ldx;
 #pragma unroll
       for (int j = 0; j < kXN; ++j) {
         const int i = tid + j * kTcWorkers, v = i / 4, c = i % 4;
         if (v < kGX * kGHY)
-          cp16_fill(xs + (unsigned)slot * kXPlane + (unsigned)c * kXC + (unsigned)v * 16u, xsrc[j] + off,
-                    (c0 + c) * 8 < a.cin);
+          copy(xs + (unsigned)slot * kXPlane + swz(v, c), base + (long long)xsrc[j] * 8, (c0 + c) * 8 < a.cin);
       }
     };
     auto load_y = [&](int z, int r) {
-      const long long off = (long long)z * plane * a.ldd;
+      const bf16* base = ybase + (long long)z * plane * a.ldd;
 #pragma unroll
       for (int j = 0; j < kYN; ++j) {
         const int i = tid + j * kTcWorkers, c = i % 4, v = (i / 4) % kGV, dx = i / (4 * kGV);
-        cp16_fill(ys + (unsigned)r * kYTile + (unsigned)(dx * 4 + c) * kYC + (unsigned)v * 16u, ysrc[j] + off,
-                  (yvalid >> j) & 1u);
+        copy(ys + (unsigned)r * kYTile + (unsigned)dx * kYCopy + swz(v, c), base + (long long)ysrc[j] * 8,
+             (yvalid >> j) & 1u);
       }
     };
     // Tile j's loads: at the start of a segment three planes, else one, and its dY; one
@@ -223,7 +235,7 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
       if (blockIdx.y != 0) return;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const unsigned off = kSlots * kXPlane + (unsigned)r * kYTile + (4u + (tid & 3)) * kYC + ((tid >> 2) + 64 * h) * 16u;
+        const unsigned off = kSlots * kXPlane + (unsigned)r * kYTile + kYCopy + swz((tid >> 2) + 64 * h, tid & 3);
         const uint4 v = *reinterpret_cast<const uint4*>(smem + off);
 #pragma unroll
         for (int q = 0; q < 8; ++q) bsum[q] += __bfloat162float(reinterpret_cast<const bf16*>(&v)[q]);
