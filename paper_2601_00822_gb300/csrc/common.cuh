@@ -483,6 +483,7 @@ struct IterState {
   int next_check;    // sweep whose residual is evaluated next (sparse evaluation; else every sweep)
   int last_check;    // sweep of resid_last (valid once checks > 0)
   int checks;        // residual evaluations so far in this solve
+  int seen;          // 1 once a Green pass found `done` set: passes that run beside the residual step skip by this
   double stall_ref;  // residual at that checkpoint (0 = none yet)
   double resid_last;
   double bden;       // sqrt(sum |b_hat|^2) over modes with xi != 0

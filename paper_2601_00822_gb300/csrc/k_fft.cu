@@ -7,6 +7,7 @@
 // Compiled once per arithmetic type with BFCS_R = float, double or ff
 // (float-float arithmetic on FP64 fields, for the precision ladder).
 #include "kernels.h"
+#include "resid.cuh"
 
 #include <cuda.h>
 
@@ -275,16 +276,31 @@ template <typename R, int T> constexpr int col_min_blocks() {
 }
 
 template <typename R, int L, int DIR, int T, bool SW>
-__global__ void __launch_bounds__(CCfg<L, T, SW>::THREADS, col_min_blocks<R, T>()) k_colpass(CArgs<R> a) {
+__global__ void __launch_bounds__(CCfg<L, T, SW>::THREADS, col_min_blocks<R, T>())
+    k_colpass(const __grid_constant__ CArgs<R> a) {
   const int m = blockIdx.z;
-  if (a.st != nullptr && a.st[m].done) return;   // a member that has converged skips
+  int by = blockIdx.y;                           // (component, other axis)
+  if constexpr (DIR > 0) {
+    if (a.with_resid) {
+      if (by == 0) {
+        if (blockIdx.x == 0) resid_step(a.resid, m);
+        return;
+      }
+      --by;
+      if (a.st[m].seen) return;                  // a member that has converged skips
+    } else if (a.st != nullptr && a.st[m].done) {
+      return;
+    }
+  } else {
+    if (a.st != nullptr && a.st[m].done) return;
+  }
   constexpr int R1 = CCfg<L, T, SW>::F1, R2 = CCfg<L, T, SW>::F2;
   extern __shared__ unsigned char smem_raw[];
   C2<R>* s = reinterpret_cast<C2<R>*>(smem_raw);
   const int tid = threadIdx.x;
   const int mx = a.g.mx, p = a.g.p, ny = a.g.ny;
   const int other = a.axis == 1 ? a.g.nz : ny;
-  const int comp = blockIdx.y / other, o = blockIdx.y - comp * other;
+  const int comp = by / other, o = by - comp * other;
   const long long ls = a.axis == 1 ? (long long)p : (long long)ny * p;
   C2<R>* base = a.data + m * a.ms + comp * a.g.cs + (a.axis == 1 ? (long long)o * ny * p : (long long)o * p);
   const int c = tid % T, j = tid / T;
@@ -328,17 +344,31 @@ __global__ void __launch_bounds__(CCfg<L, T, SW>::THREADS, col_min_blocks<R, T>(
 
 template <int L, int DIR, int T>
 __global__ void __launch_bounds__(CCfg<L, T, false>::THREADS, T == 8 ? 6 : 3)
-    k_colpass_tma(CArgs<float> a, const __grid_constant__ CUtensorMap tm) {
+    k_colpass_tma(const __grid_constant__ CArgs<float> a, const __grid_constant__ CUtensorMap tm) {
   using R = float;
   const int m = blockIdx.z;
-  if (a.st != nullptr && a.st[m].done) return;   // a member that has converged skips
+  int by = blockIdx.y;                           // component * nz + z
+  if constexpr (DIR > 0) {
+    if (a.with_resid) {
+      if (by == 0) {
+        if (blockIdx.x == 0) resid_step(a.resid, m);
+        return;
+      }
+      --by;
+      if (a.st[m].seen) return;                  // a member that has converged skips
+    } else if (a.st != nullptr && a.st[m].done) {
+      return;
+    }
+  } else {
+    if (a.st != nullptr && a.st[m].done) return;
+  }
   constexpr int R1 = CCfg<L, T, false>::F1, R2 = CCfg<L, T, false>::F2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C2<R>* s = reinterpret_cast<C2<R>*>(smem_raw);   // [row][T], as the copy lands
   __shared__ __align__(8) unsigned long long bar;
   const int tid = threadIdx.x;
   const unsigned bar_a = (unsigned)__cvta_generic_to_shared(&bar);
-  const int plane = m * 6 * a.g.nz + blockIdx.y;   // (member, component, z) with blockIdx.y = comp * nz + z
+  const int plane = m * 6 * a.g.nz + by;   // (member, component, z)
   const int kx0 = blockIdx.x * T;
   if (tid == 0) {
     // fetch the tensor map while the barrier is set up: between y passes other
@@ -387,7 +417,7 @@ __global__ void __launch_bounds__(CCfg<L, T, false>::THREADS, T == 8 ? 6 : 3)
   const int kx = kx0 + c;
   const bool valid = kx < a.g.mx;
   const int ny = a.g.ny, p = a.g.p;
-  C2<R>* col = a.data + m * a.ms + (long long)blockIdx.y * ny * p + kx;
+  C2<R>* col = a.data + m * a.ms + (long long)by * ny * p + kx;
   // stage 1 from the landed tile, in place: thread (c, j) owns rows R2 n1 + j
   C2<R> x[R1];
   if (j < R2) {
@@ -459,7 +489,7 @@ cudaError_t launch_xpass_b(const XArgs<R>& a0, int batch, cudaStream_t st) {
 template <typename R, int L, int DIR, int T, bool SW>
 static cudaError_t colpass_LT(const CArgs<R>& a, int batch, cudaStream_t st) {
   const int other = a.axis == 1 ? a.g.nz : a.g.ny;
-  dim3 grid((a.g.mx + T - 1) / T, other * a.ncomp, batch);
+  dim3 grid((a.g.mx + T - 1) / T, other * a.ncomp + (DIR > 0 && a.with_resid ? 1 : 0), batch);
   const size_t smem = sizeof(C2<R>) * (size_t)L * T;
   cudaError_t e = cudaFuncSetAttribute(k_colpass<R, L, DIR, T, SW>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -471,7 +501,7 @@ static cudaError_t colpass_LT(const CArgs<R>& a, int batch, cudaStream_t st) {
 
 template <int L, int DIR, int T>
 static cudaError_t colpass_tma_LT(const CArgs<float>& a, int batch, cudaStream_t st) {
-  dim3 grid((a.g.mx + T - 1) / T, a.g.nz * 6, batch);
+  dim3 grid((a.g.mx + T - 1) / T, a.g.nz * 6 + (DIR > 0 && a.with_resid ? 1 : 0), batch);
   const size_t smem = sizeof(C2<float>) * (size_t)L * T;
   cudaError_t e = cudaFuncSetAttribute(k_colpass_tma<L, DIR, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);

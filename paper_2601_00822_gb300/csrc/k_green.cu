@@ -170,7 +170,10 @@ __device__ __forceinline__ R green_tile(const GArgs<R>& a, C2<R>* s, const C2<R>
 template <typename R, int L>
 __global__ void __launch_bounds__(GCfg<L>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgreen(GArgs<R> a) {
   const int mbr = blockIdx.z;
-  if (a.skip_done && a.st[mbr].done) return;     // a member that has converged skips
+  if (a.skip_done && a.st[mbr].done) {           // a member that has converged skips
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) a.st[mbr].seen = 1;
+    return;
+  }
   // this member's buffers and mean strain
   C2<R>* const spec = a.spec + mbr * a.spec_ms;
   const C2<R>* const bhat = a.bhat + mbr * a.b_ms;
@@ -376,6 +379,9 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
     __syncthreads();
   };
 
+  if (blockIdx.x == 0)                           // (as in k_zgreen)
+    for (int m = tid; m * tiles_pm < total; m += nthr)
+      if (a.st[m].done) a.st[m].seen = 1;
   int t = blockIdx.x;
   while (t < total && skip(t)) t += G;
   if (t < total) issue(t, 0);

@@ -2,10 +2,22 @@
 // body-force field, input validation, FP64 reductions of the residual and the
 // translated-averaging accumulation (Eqs. 3.5-3.6).
 #include "kernels.h"
+#include "resid.cuh"
 
 #include <atomic>
 
 namespace bfcs {
+
+__device__ __forceinline__ double block_sum(double v, double* red) {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)((blockDim.x + 31) / 32); ++w) t += red[w];
+  return t;   // valid in thread 0
+}
 
 static std::atomic<long long> g_launches{0};
 void count_launches(long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
@@ -20,17 +32,6 @@ bool supported_len(int n) {
 }
 
 constexpr int kRedThreads = 256;
-
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)((blockDim.x + 31) / 32); ++w) t += red[w];
-  return t;   // valid in thread 0
-}
 
 // ---------------------------------------------------------------- a1: phase map
 // A voxel with doubled centre 2i+1 (cell coordinates) is inside sphere
@@ -341,106 +342,10 @@ cudaError_t launch_bden(const C2<R>* bhat, const Geo& g, ResidSlot* part, IterSt
 }
 
 // ---------------------------------------------------------------- residual reduction (Eq. 5.11)
-// r = sqrt(sum partials) / D, D = ||b_hat|| + xi_min |sigma_hat(0)|_F with
-// sigma_hat(0) = N C0 E + tau_hat(0) and xi_min = 2 pi / max N_a.
-__global__ void k_resid_reduce(const ResidSlot* part, int nparts, IterState* sts, const Member* mem,
-                               double* hist, int hist_cap, double tol, double lam0, double mu0, double E0,
-                               double E1, double E2, double E3, double E4, double E5, double n, int maxdim,
-                               int mode, int warm_all, int stall_window, int check_max, int maxit,
-                               unsigned long long* io) {
-  __shared__ double red[32];
-  const int m = blockIdx.x;
-  IterState* st = sts + m;
-  if (mode == GM_SWEEP && st->done) return;
-  __shared__ int no_check;   // decided by one thread: thread 0 advances st->iters below
-  if (threadIdx.x == 0) {
-    const int sw = st->iters, nc = st->next_check;
-    no_check = mode == GM_SWEEP && check_max > 1 && sw != nc;
-    if (io != nullptr && mode == GM_SWEEP) {
-      // what the Green pass of this sweep moved besides its fixed traffic: d_prev read, d written
-      const bool rd = check_max <= 1 || sw == nc;
-      const bool wr = check_max <= 1 || rd || sw + 1 == nc || sw + 1 >= maxit;
-      atomicAdd(io, (unsigned long long)rd);
-      atomicAdd(io + 1, (unsigned long long)wr);
-    }
-  }
-  __syncthreads();
-  if (no_check) {
-    // no residual on this sweep (the Green pass wrote no partials)
-    if (threadIdx.x == 0) {
-      const int sweep = st->iters;
-      if (sweep < hist_cap && hist != nullptr) hist[(long long)m * hist_cap + sweep] = NAN;
-      st->iters = sweep + 1;
-    }
-    return;
-  }
-  part += m * nparts;
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[i].num;
-  const double t = block_sum(acc, red);
-  if (threadIdx.x != 0) return;
-  double E[6] = {E0, E1, E2, E3, E4, E5};
-  int warm = warm_all;
-  if (mem != nullptr) {
-    for (int c = 0; c < 6; ++c) E[c] = mem[m].E[c];
-    warm = mem[m].warm;
-    if (mem[m].tol >= 0.0) tol = mem[m].tol;
-  }
-  const double trE = E[0] + E[1] + E[2];
-  double s0[6];
-  for (int c = 0; c < 6; ++c)
-    s0[c] = mode == kReduceDefect ? st->tau0[c]
-                                  : n * (2.0 * mu0 * E[c] + (c < 3 ? lam0 * trE : 0.0)) + st->tau0[c];
-  const double s0n = sqrt(s0[0] * s0[0] + s0[1] * s0[1] + s0[2] * s0[2] +
-                          2.0 * (s0[3] * s0[3] + s0[4] * s0[4] + s0[5] * s0[5]));
-  const double den = st->bden + 6.283185307179586 / (double)maxdim * s0n;
-  double r = den > 0.0 ? sqrt(t) / den : sqrt(t);
-  if (mode == GM_FINAL || mode == kReduceDefect) { st->resid_final = r; return; }
-  const int sweep = st->iters;
-  const bool skip_check = warm && sweep == 0;
-  if (skip_check) r = INFINITY;
-  if (sweep < hist_cap && hist != nullptr) hist[(long long)m * hist_cap + sweep] = r;
-  // sweep of the next evaluation: with sparse evaluation, where the contraction
-  // rate between the last two evaluations predicts r <= tol (at most check_max
-  // sweeps ahead; every check_max sweeps when tol = 0), else the next sweep
-  int gap = 1;
-  if (check_max > 1 && !skip_check) {
-    if (!(tol > 0.0)) {
-      gap = check_max;
-    } else if (st->checks > 0 && sweep > st->last_check && r > tol && r < st->resid_last && r > 0.0) {
-      const double rate = pow(r / st->resid_last, 1.0 / (double)(sweep - st->last_check));
-      const double need = ceil(log(tol / r) / log(rate));
-      gap = (int)fmin(fmax(need, 1.0), (double)check_max);
-    }
-  }
-  st->next_check = sweep + gap;
-  if (!skip_check) {
-    st->last_check = sweep;
-    st->checks += 1;
-  }
-  st->resid_last = r;
-  st->iters = sweep + 1;
-  if (skip_check) return;
-  if (!(r == r && r < INFINITY)) { st->diverged = 1; st->done = 1; return; }
-  if (r <= tol) { st->done = 1; return; }
-  // stall: the residual did not drop by 10% over stall_window sweeps
-  if (stall_window > 0) {
-    if (st->stall_ref == 0.0) { st->stall_ref = r; st->stall_at = sweep; }
-    else if (sweep - st->stall_at >= stall_window) {
-      if (r > 0.9 * st->stall_ref) { st->stalled = 1; st->done = 1; }
-      else { st->stall_ref = r; st->stall_at = sweep; }
-    }
-  }
-}
+__global__ void k_resid_final(const __grid_constant__ ResidArgs a) { resid_step(a, blockIdx.x); }
 
-cudaError_t launch_resid_reduce(const ResidSlot* part, int nparts, IterState* st, const Member* mem,
-                                double* hist, int hist_cap, double tol, double lam0, double mu0,
-                                const double* E, long long n, int maxdim, int mode, int warm_all,
-                                int stall_window, int check_max, int maxit, unsigned long long* io, int batch,
-                                cudaStream_t s) {
-  k_resid_reduce<<<batch, 1024, 0, s>>>(part, nparts, st, mem, hist, hist_cap, tol, lam0, mu0, E[0], E[1],
-                                        E[2], E[3], E[4], E[5], (double)n, maxdim, mode, warm_all,
-                                        stall_window, check_max, maxit, io);
+cudaError_t launch_resid_final(const ResidArgs& a, int batch, cudaStream_t s) {
+  k_resid_final<<<batch, 1024, 0, s>>>(a);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -57,6 +57,27 @@ template <typename R> struct XArgs {
   XMember xm[kMaxBatch];
 };
 
+// ---- the residual step of a sweep (resid.cuh).  One block per member m: reduces
+// part[m * nparts ...], updates sts[m] and writes hist[m * hist_cap + sweep]; E, the warm
+// flag and a member's own tolerance come from mem[m].  The sweep index is the device
+// counter sts[m].iters.  check_max > 1: sparse evaluation, only sweeps s ==
+// sts[m].next_check carry a residual (others record NaN in hist); after each evaluation
+// the next one is placed at the sweep where the observed contraction rate predicts r <=
+// tol, at most check_max sweeps ahead (every check_max sweeps when tol = 0).  io
+// (nullable): two counters to which GM_SWEEP adds, per member, whether the sweep's Green
+// pass read d_prev and whether it wrote d (maxit: the call's sweep limit).
+struct ResidArgs {
+  const ResidSlot* part;
+  int nparts;
+  IterState* sts;
+  const Member* mem;
+  double* hist;
+  int hist_cap;
+  double tol, lam0, mu0, n;
+  int maxdim, mode, stall_window, check_max, maxit;
+  unsigned long long* io;
+};
+
 // ---- column passes along y (axis 1) or z (axis 2) on the half spectrum, in place.
 template <typename R> struct CArgs {
   C2<R>* data;
@@ -69,6 +90,11 @@ template <typename R> struct CArgs {
   int variant;            // FP32 only: column tile and factor order (kColVariants; 0 = default)
   const void* tmap;       // host array of the two tensor maps (8, 16 columns) of a y pass over 6-component spectra, or null
   const void* tmap_data;  // the buffer the maps address: the tensor-copy tiles run only when data is this buffer
+  // inverse passes: 1 adds one block row whose first block runs the sweep's residual step;
+  // members are then skipped by IterState.seen (set by the Green pass), since the step may
+  // set `done` while other blocks of the pass have not started
+  int with_resid;
+  ResidArgs resid;
 };
 
 // Column-pass variants an autotuner can pick from (FP32): tile width in kx
@@ -309,24 +335,8 @@ template <typename R>
 cudaError_t launch_bden(const C2<R>* bhat, const Geo& g, ResidSlot* part, IterState* st, cudaStream_t s,
                         int batch = 1, long long b_ms = 0);
 
-// residual reduction of the Green-pass partials; mode = GM_SWEEP, GM_FINAL or
-// kReduceDefect.  One block per member: member m reduces part[m * nparts ...],
-// updates st[m] and writes hist[m * hist_cap + sweep]; its E and warm flag
-// come from mem[m] when mem is given, else from E / warm_all.  In GM_SWEEP the
-// sweep index is the device counter st[m].iters.  check_max > 1: sparse
-// evaluation, only sweeps s == st[m].next_check carry a residual (others
-// record NaN in hist); after each evaluation the next one is placed at the
-// sweep where the observed contraction rate predicts r <= tol, at most
-// check_max sweeps ahead (every check_max sweeps when tol = 0).  io (nullable):
-// two counters that GM_SWEEP adds to, per member, whether the sweep's Green
-// pass read d_prev and whether it wrote d (maxit: the call's sweep limit).
-cudaError_t launch_resid_reduce(const ResidSlot* part, int nparts, IterState* st, const Member* mem,
-                                double* hist, int hist_cap, double tol, double c0_lam, double c0_mu,
-                                const double* E, long long n, int maxdim, int mode, int warm_all,
-                                int stall_window, int check_max, int maxit, unsigned long long* io, int batch,
-                                cudaStream_t s);
-// mode for launch_resid_reduce: tau0 already holds sigma_hat(0) (defect evaluation)
-constexpr int kReduceDefect = 7;
+// the residual of the final pass's partials (mode GM_FINAL) into st[m].resid_final
+cudaError_t launch_resid_final(const ResidArgs& a, int batch, cudaStream_t s);
 
 // elementwise helpers (k_misc.cu)
 cudaError_t launch_cast_d2f(float* dst, const double* src, long long count, cudaStream_t s);

@@ -548,6 +548,26 @@ struct SweepSet {
     return BFCS_OK;
   }
 
+  ResidArgs resid_args(int mode, int nparts) const {
+    ResidArgs r{};
+    r.part = P->part;
+    r.nparts = nparts;
+    r.sts = P->ist;
+    r.mem = P->mem_dev;
+    r.hist = P->hist;
+    r.hist_cap = P->hist_cap;
+    r.tol = tol;
+    r.lam0 = C0.lambda;
+    r.mu0 = C0.mu;
+    r.n = (double)P->g.n;
+    r.maxdim = maxdim;
+    r.mode = mode;
+    r.stall_window = P->stall_window;
+    r.check_max = P->resid_max;
+    r.maxit = ga.maxit;
+    return r;
+  }
+
   // one sweep for all members on stream q; identical launches every sweep
   // (graph-capturable); `sweep` labels profiled launches (-1: not profiled)
   int enqueue(cudaStream_t q, int sweep) {
@@ -571,12 +591,14 @@ struct SweepSet {
     ga.mode = GM_SWEEP;
     ga.skip_done = 1;
     CK(timed(3, [&] { return launch_zgreen_b<R>(ga, B, q); }));
-    CK(timed(2, [&] { return launch_colpass_b<R>(cy, +1, B, q); }));
-    // (the persistent form of the z pass does not run with sparse evaluation)
-    const int nparts = ga.sparse ? green_nparts<R>(P->g) : green_sweep_parts<R>(P->g);
-    unsigned long long* io = (P->prof_kind == 3 && sweep >= 0) ? P->io_dev : nullptr;
-    CK(launch_resid_reduce(P->part, nparts, P->ist, P->mem_dev, P->hist, P->hist_cap, tol, C0.lambda, C0.mu, E0,
-                           P->g.n, maxdim, GM_SWEEP, 0, P->stall_window, P->resid_max, ga.maxit, io, B, q));
+    // the inverse y pass, with the residual step beside it (the persistent form of the z
+    // pass does not run with sparse evaluation)
+    cy.with_resid = 1;
+    cy.resid = resid_args(GM_SWEEP, ga.sparse ? green_nparts<R>(P->g) : green_sweep_parts<R>(P->g));
+    cy.resid.io = (P->prof_kind == 3 && sweep >= 0) ? P->io_dev : nullptr;
+    const cudaError_t e = timed(2, [&] { return launch_colpass_b<R>(cy, +1, B, q); });
+    cy.with_resid = 0;
+    CK(e);
     return BFCS_OK;
   }
 
@@ -600,8 +622,7 @@ struct SweepSet {
     ga.mode = GM_FINAL;
     ga.skip_done = 0;
     CK(launch_zgreen_b<R>(ga, B, st));
-    CK(launch_resid_reduce(P->part, P->ngreen, P->ist, P->mem_dev, P->hist, P->hist_cap, tol, C0.lambda, C0.mu,
-                           E0, P->g.n, maxdim, GM_FINAL, 0, 0, P->resid_max, 0, nullptr, B, st));
+    CK(launch_resid_final(resid_args(GM_FINAL, P->ngreen), B, st));
     cy.ncomp = 3;
     CK(launch_colpass_b<R>(cy, +1, B, st));
     XArgs<R> xu{};
