@@ -336,8 +336,9 @@ __device__ __forceinline__ void fft_cols(C2<R>* s, int ncol, const C2<R>* __rest
 template <typename R, int L, int R1, int DIR>
 __device__ __forceinline__ void stage1f(C2<R>* x, int n2, const C2<R>* __restrict__ tw) {
   Dft<R, R1, DIR>::run(x);
-  if constexpr (R1 % 4 == 0 && R1 >= 8 && sizeof(R) <= 8 && !std::is_same<R, ff>::value) {
-    // W^(n2 k1) with k1 = 4 a + b as W^(4 n2 a) W^(n2 b): R1/4 - 1 + 3 table loads
+  if constexpr (R1 % 4 == 0 && R1 >= 8 && sizeof(R) == 4) {
+    // FP32 (FP64 is bound by its arithmetic pipe, not by the table's loads, and takes the
+    // entries as they are): W^(n2 k1) with k1 = 4 a + b as W^(4 n2 a) W^(n2 b): R1/4 - 1 + 3 table loads
     // and (R1/4 - 1) * 3 products instead of R1 - 1 loads (each product adds about
     // one rounding; float-float keeps the table, where a product costs more than a load)
     constexpr int A = R1 / 4, N2 = L / R1;
@@ -369,7 +370,7 @@ __device__ __forceinline__ void stage1f(C2<R>* x, int n2, const C2<R>* __restric
   } else {
 #pragma unroll
     for (int k1 = 1; k1 < R1; ++k1) {
-      C2<R> w = tw[(n2 * k1) % L];
+      C2<R> w = tw[n2 * k1];   // < L
       if (DIR > 0) w.y = -w.y;
       x[k1] = cmul(x[k1], w);
     }
@@ -382,7 +383,7 @@ __device__ __forceinline__ void stage1f(C2<R>* x, int n2, const C2<R>* __restric
 // then for each n2 this step on Y[k1][n2] (k1 = 0..R1-1) gives x[R2 n1 + n2].
 template <typename R, int L, int R1, int DIR>
 __device__ __forceinline__ void twiddle_then_dft(C2<R>* x, int n2, const C2<R>* __restrict__ tw) {
-  if constexpr (R1 % 4 == 0 && R1 >= 8 && sizeof(R) <= 8 && !std::is_same<R, ff>::value) {
+  if constexpr (R1 % 4 == 0 && R1 >= 8 && sizeof(R) == 4) {
     constexpr int A = R1 / 4, N2 = L / R1;
     const C2<R>* const f = tw + tw_offset<L, R1>() + n2;   // factored table, [entry][n2]
     C2<R> wb[4], wa[A];
@@ -400,7 +401,7 @@ __device__ __forceinline__ void twiddle_then_dft(C2<R>* x, int n2, const C2<R>* 
   } else {
 #pragma unroll
     for (int k1 = 1; k1 < R1; ++k1) {
-      C2<R> w = tw[(n2 * k1) % L];
+      C2<R> w = tw[n2 * k1];   // < L
       if (DIR > 0) w.y = -w.y;
       x[k1] = cmul(x[k1], w);
     }
@@ -421,6 +422,16 @@ __device__ __forceinline__ void stage2(C2<R>* y) {
   stage2f<R, LineInfo<L>::R2, DIR>(y);
 }
 
+// ------------------------------------------------------------------ chained launches
+// Kernels that are launched with programmatic stream serialisation (launch_chain): each
+// waits here, before its first access to global memory, for its predecessor to complete,
+// and then lets its successor's blocks be scheduled, so a launch's latency is spent while
+// the kernel before it runs.  Without effect on an ordinary launch.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
 // ------------------------------------------------------------------ async copies
 // 16-byte global -> shared copy that does not pass through registers
 // (cp.async, completion tracked per thread with commit/wait groups).
@@ -437,6 +448,7 @@ constexpr int kMaxPhases = 16;
 template <typename R> struct PhaseTab {
   R lam[kMaxPhases], mu[kMaxPhases];     // L(x)
   R lam1[kMaxPhases], mu1[kMaxPhases];   // L1(x) = L(x) - L0
+  R lamh[kMaxPhases], lam1h[kMaxPhases]; // lam / 2, lam1 / 2
 };
 
 // Half-spectrum geometry: [comp][z][y][kx], kx in [0, nx/2], row pitch p.

@@ -102,6 +102,7 @@ template <typename R>
 __global__ void __launch_bounds__(kCdThreads) k_cd_vec(CdArgs<R> a, int mode) {
   const int m = blockIdx.y;
   const bool all = mode == CdMode::FINAL || mode == CdMode::FINAL_U || mode == CdMode::RESID;
+  chain_wait();
   if (!all && a.cd[m].done) return;
   __shared__ double red[32];
   const Geo g = a.g;
@@ -266,6 +267,7 @@ static __global__ void k_cd_scalar(const double* part, int nparts, CdState* cd, 
   __shared__ double red[32];
   const int m = blockIdx.x;
   CdState& S = cd[m];
+  chain_wait();
   if (mode != CdMode::RESID && S.done) return;
   double a1 = 0.0, a2 = 0.0;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
@@ -354,6 +356,7 @@ __device__ __forceinline__ int cd_slot(int row, int c) { return c ^ (((row >> 1)
 template <typename R, int L, bool FWD>
 __global__ void __launch_bounds__(ZCfg<L>::BLOCK) k_zcd(CdArgs<R> a) {
   const int m = blockIdx.z;
+  chain_wait();
   if (a.cd[m].done) return;
   constexpr int T = kCdT, NCOL = kCdNcol;
   constexpr int R1 = LineInfo<L>::R1, R2 = LineInfo<L>::R2;
@@ -556,9 +559,8 @@ static cudaError_t zcd_L(const CdArgs<R>& a, bool fwd, int batch, cudaStream_t s
   auto k = fwd ? k_zcd<R, L, true> : k_zcd<R, L, false>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<grid, ZCfg<L>::BLOCK, smem, st>>>(a);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chain(true, k, grid, ZCfg<L>::BLOCK, smem, st, a);
 }
 
 template <typename R>
@@ -575,22 +577,20 @@ cudaError_t launch_zcd(const CdArgs<R>& a, bool fwd, int batch, IterState* ist, 
   if (e != cudaSuccess || !fwd) return e;
   // alpha from <p, q>: one partial pair per tile
   const int nparts = ((a.g.mx + kCdT - 1) / kCdT) * a.g.ny;
-  k_cd_scalar<<<batch, kCdThreads, 0, st>>>(a.part, nparts, a.cd, a.skip, ist, mem, a.lam0, a.mu0, (double)a.g.n,
-                                            maxdim, CdMode::PQ);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chain(true, k_cd_scalar, batch, kCdThreads, 0, st, (const double*)a.part, nparts, a.cd, a.skip, ist, mem,
+                      a.lam0, a.mu0, (double)a.g.n, maxdim, (int)CdMode::PQ);
 }
 
 template <typename R>
 cudaError_t launch_cd_vec(const CdArgs<R>& a, int mode, int batch, IterState* ist, const Member* mem, int maxdim,
                           cudaStream_t st) {
-  k_cd_vec<R><<<dim3(kCdParts, batch), kCdThreads, 0, st>>>(a, mode);
+  const cudaError_t e = launch_chain(true, k_cd_vec<R>, dim3(kCdParts, batch), kCdThreads, 0, st, a, mode);
   count_launches(1);
-  if (mode == CdMode::FINAL || mode == CdMode::FINAL_U) return cudaGetLastError();
-  k_cd_scalar<<<batch, kCdThreads, 0, st>>>(a.part, kCdParts, a.cd, a.skip, ist, mem, a.lam0, a.mu0,
-                                            (double)a.g.n, maxdim, mode);
+  if (e != cudaSuccess || mode == CdMode::FINAL || mode == CdMode::FINAL_U) return e;
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chain(true, k_cd_scalar, batch, kCdThreads, 0, st, (const double*)a.part, (int)kCdParts, a.cd, a.skip, ist,
+                      mem, a.lam0, a.mu0, (double)a.g.n, maxdim, mode);
 }
 
 template cudaError_t launch_cd_vec<BFCS_R>(const CdArgs<BFCS_R>&, int, int, IterState*, const Member*, int,

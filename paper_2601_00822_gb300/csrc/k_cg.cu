@@ -55,6 +55,7 @@ struct CgMode { enum : int { INIT = 0, PQ = 1, UPDATE = 2, DIR = 3 }; };
 template <typename R>
 __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
   const int m = blockIdx.y;
+  chain_wait();
   if (a.cg[m].done) return;
   __shared__ double red[32];
   const Geo g = a.g;
@@ -134,6 +135,7 @@ static __global__ void k_cg_scalar(const double* part, int nparts, CgState* cg, 
   __shared__ double red[32];
   const int m = blockIdx.x;
   CgState& S = cg[m];
+  chain_wait();
   if (S.done) return;
   double acc = 0.0;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[(long long)m * nparts + i];
@@ -163,12 +165,11 @@ static __global__ void k_cg_scalar(const double* part, int nparts, CgState* cg, 
 
 template <typename R>
 cudaError_t launch_cg_vec(const CgArgs<R>& a, int mode, int batch, cudaStream_t st) {
-  k_cg_vec<R><<<dim3(kCgParts, batch), kCgThreads, 0, st>>>(a, mode);
+  cudaError_t e = launch_chain(true, k_cg_vec<R>, dim3(kCgParts, batch), kCgThreads, 0, st, a, mode);
   count_launches(1);
-  if (mode == CgMode::DIR) return cudaGetLastError();
-  k_cg_scalar<<<batch, kCgThreads, 0, st>>>(a.part, kCgParts, a.cg, a.skip, mode);
+  if (e != cudaSuccess || mode == CgMode::DIR) return e;
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chain(true, k_cg_scalar, batch, kCgThreads, 0, st, (const double*)a.part, (int)kCgParts, a.cg, a.skip, mode);
 }
 
 template cudaError_t launch_cg_vec<BFCS_R>(const CgArgs<BFCS_R>&, int, int, cudaStream_t);

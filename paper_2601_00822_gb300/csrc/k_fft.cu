@@ -20,14 +20,19 @@ namespace bfcs {
 // x pass: LPB lines per block, each line as up to 3 complex pair-lines
 // (components 2q and 2q+1 as real and imaginary parts), one group of TPF
 // threads per pair-line.  Pair-line f keeps its L values in shared memory at
-// s[f * LP + pad(n)], pad(n) = n + n/16, which keeps every access below free
-// of bank conflicts.
+// s[f * LP + pad(n)], pad(n) = n + n/16.  LP spreads the pair-lines that share a half
+// warp (16 eight-byte accesses) over the banks: LP = R2 mod 16 with 16 threads a line
+// (step 1 packs R2 of them side by side), 8 or 4 mod 16 with 8 or 4 threads a line.
+// Step 1 (R2 tasks a line) is packed too: with its tasks on the first R2 of a line's TPF
+// threads, half the lanes of every warp issued nothing at L = 32 and 128, 60% at 24 and
+// 96.  The pass over 16 members of 64^3: 58 -> 53 us, one of 128^3: 42 -> 37 us (FP32).
 template <int L> struct XCfg {
   static constexpr int RMAX = LineInfo<L>::RMAX;
   static constexpr int TPF = RMAX <= 2 ? 2 : RMAX <= 4 ? 4 : RMAX <= 8 ? 8 : 16;   // threads per pair-line
   static constexpr int LPB = 64 / TPF;
   static constexpr int NCOL = 3 * LPB;
-  static constexpr int LP = L + L / 16 + 1;
+  static constexpr int LP0 = L + L / 16;
+  static constexpr int LP = TPF == 16 ? LP0 : TPF == 2 ? LP0 + 1 : LP0 + ((TPF - LP0) % 16 + 16) % 16;
   static constexpr int THREADS = NCOL * TPF;
 };
 
@@ -45,6 +50,7 @@ template <typename R> constexpr int xpass_min_blocks() {
 template <typename R, int L>
 __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpass(XArgs<R> a) {
   const int m = blockIdx.z;
+  chain_wait();
   if (a.st != nullptr && a.st[m].done) return;   // a member that has converged skips
   using C = XCfg<L>;
   using RT = typename RealOf<R>::T;   // storage type of the real fields
@@ -74,6 +80,11 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
   const bool fval = f < ncol && line < lines;
   const bool has_b = 2 * q + 1 < ncomp;
   C2<R>* sf = s + f * LP;
+  // the packed mapping of step 1: pair-line f1, task t1 < R2
+  const int f1 = tid / R2, t1 = tid % R2;
+  const int li1 = f1 / npair, q1 = f1 - li1 * npair;
+  const bool fval1 = f1 < ncol && line0 + li1 < lines;
+  C2<R>* sf1 = s + f1 * LP;
 
   // per-line translation bookkeeping of the polarization (made visible by the
   // barriers of step 1): the phase of voxel (n, y, z) is phase0(n - sx, y - sy, z - sz)
@@ -114,23 +125,24 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
 
   // ---- 1. inverse transform along x of the pair-line Z = A + i B (C2R), or load real data
   if (mode == XM_SWEEP || mode == XM_C2R || mode == XM_SWEEPSIG) {
-    if (fval && t < R2) {
-      const C2<R>* rowA = a.spec_in + m * a.spec_ms + (2 * q) * cs + line * p;
+    if (fval1) {
+      const C2<R>* rowA = a.spec_in + m * a.spec_ms + (2 * q1) * cs + (line0 + li1) * p;
       const C2<R>* rowB = rowA + cs;
+      const bool has_b1 = 2 * q1 + 1 < ncomp;
       C2<R> x[R1];
 #pragma unroll
       for (int n1 = 0; n1 < R1; ++n1) {
-        const int k = R2 * n1 + t;
+        const int k = R2 * n1 + t1;
         const int kk = k <= H ? k : L - k;
         C2<R> A = rowA[kk];
-        C2<R> B = has_b ? rowB[kk] : mk<R>(0, 0);
+        C2<R> B = has_b1 ? rowB[kk] : mk<R>(0, 0);
         if (kk == 0 || kk == H) { A.y = 0; B.y = 0; }     // DC and Nyquist keep their real parts
         if (k > H) { A.y = -A.y; B.y = -B.y; }            // Hermitian extension
         x[n1] = mk<R>(A.x - B.y, A.y + B.x);
       }
-      stage1<R, L, +1>(x, t, a.tw);
+      stage1<R, L, +1>(x, t1, a.tw);
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) sf[xpad(t * R1 + k1)] = x[k1];
+      for (int k1 = 0; k1 < R1; ++k1) sf1[xpad(t1 * R1 + k1)] = x[k1];
     }
     __syncthreads();
     // stage 2 reads and writes the same slots of its pair-line (t + R1 m, m < R2)
@@ -175,7 +187,9 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
   }
 
   // ---- 2. polarization tau = (L(x) - L0) eps, isotropic phases (Eq. 5.7);
-  //         sigma = L(x) eps instead in the stress modes
+  //         sigma = L(x) eps instead in the stress modes.  Half of it goes into the
+  //         forward transform: the split below then needs no factor 1/2 (exact, a power
+  //         of two)
   if (mode == XM_SWEEP || mode == XM_REALTAU || mode == XM_REALSIG || mode == XM_SWEEPSIG) {
     const bool full = mode == XM_REALSIG || mode == XM_SWEEPSIG;
     const int nx = a.g.nx;
@@ -205,11 +219,11 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
         o[0] = st_real<R>(lt + m2 * e0); o[rn] = st_real<R>(lt + m2 * e1); o[2 * rn] = st_real<R>(lt + m2 * e2);
         o[3 * rn] = st_real<R>(m2 * e3); o[4 * rn] = st_real<R>(m2 * e4); o[5 * rn] = st_real<R>(m2 * e5);
       }
-      const R lt = (full ? a.tab.lam[ph] : a.tab.lam1[ph]) * tr;
-      const R m2 = R(2) * (full ? a.tab.mu[ph] : a.tab.mu1[ph]);
-      c0[0] = mk<R>(lt + m2 * e0, lt + m2 * e1);
-      c0[LP] = mk<R>(lt + m2 * e2, m2 * e3);
-      c0[2 * LP] = mk<R>(m2 * e4, m2 * e5);
+      const R lt = (full ? a.tab.lamh[ph] : a.tab.lam1h[ph]) * tr;
+      const R mu = full ? a.tab.mu[ph] : a.tab.mu1[ph];
+      c0[0] = mk<R>(lt + mu * e0, lt + mu * e1);
+      c0[LP] = mk<R>(lt + mu * e2, mu * e3);
+      c0[2 * LP] = mk<R>(mu * e4, mu * e5);
     }
     __syncthreads();
   }
@@ -217,15 +231,15 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
   // ---- 3. forward transform along x and split the pair-line into two half spectra
   {
     C2<R> x[R1];
-    if (fval && t < R2) {
+    if (fval1) {
 #pragma unroll
-      for (int n1 = 0; n1 < R1; ++n1) x[n1] = sf[xpad(R2 * n1 + t)];
-      stage1<R, L, -1>(x, t, a.tw);
+      for (int n1 = 0; n1 < R1; ++n1) x[n1] = sf1[xpad(R2 * n1 + t1)];
+      stage1<R, L, -1>(x, t1, a.tw);
     }
     __syncthreads();
-    if (fval && t < R2) {
+    if (fval1) {
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) sf[xpad(t * R1 + k1)] = x[k1];
+      for (int k1 = 0; k1 < R1; ++k1) sf1[xpad(t1 * R1 + k1)] = x[k1];
     }
   }
   __syncthreads();
@@ -239,7 +253,9 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
   // k2' = R2 - 1 - k2 (k1 > 0) or (R2 - k2) % R2 (k1 = 0): one shuffle per k2.
   const int lane = threadIdx.x & 31;
   const int src = (lane & ~(TPF - 1)) | ((R1 - t) % R1);
-  const R half = R(0.5) * ((mode == XM_R2C && a.out_scale != R(0)) ? a.out_scale : R(1));
+  // real input data carries no factor yet
+  const bool scaled = mode == XM_R2C;
+  const R half = R(0.5) * (a.out_scale != R(0) ? a.out_scale : R(1));
   C2<R>* rowA = a.spec_out + m * a.spec_ms + (2 * q) * cs + line * p;
   C2<R>* rowB = rowA + cs;
   // only the outputs k <= H are stored: k = t + R1 k2 with t < R1 needs k2 <= H / R1
@@ -253,14 +269,20 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
     const int k = t + R1 * k2;
     if (fval && t < R1 && k <= H) {
       const C2<R> Z = y[k2];
-      rowA[k] = mk<R>(half * (Z.x + zm.x), half * (Z.y - zm.y));
-      if (has_b) rowB[k] = mk<R>(half * (Z.y + zm.y), -half * (Z.x - zm.x));
+      C2<R> A = mk<R>(Z.x + zm.x, Z.y - zm.y), B = mk<R>(Z.y + zm.y, zm.x - Z.x);
+      if (scaled) { A = scale(A, half); B = scale(B, half); }
+      rowA[k] = A;
+      if (has_b) rowB[k] = B;
     }
   }
 }
 
-// Column FFT along y or z: each block owns T consecutive kx columns of one
-// (other-axis, component) slab; loads are T-wide contiguous row segments.
+// Column FFT along y or z: each block owns T consecutive columns of one component, the
+// columns numbered kx first, then along the other axis, so few lanes are without work
+// (blocks per row of kx left a third of them idle at nx = 64, half at 32, and a pass in
+// FP64, bound by its arithmetic, paid for them); loads are T-wide row segments, in two
+// pieces where a row ends.  FP32 numbers the whole pitch (segments stay on 32-byte
+// sectors), the 16-byte types the stored modes.
 // L = F1 * F2 in the order given by SW (the default order of Fac<L>, or
 // swapped); T and SW are the autotuned choices of an FP32 plan.
 constexpr int kColT = 16;
@@ -275,11 +297,14 @@ template <typename R, int T> constexpr int col_min_blocks() {
   return sizeof(R) == 4 ? (T == 8 ? 6 : T == 16 ? 3 : 1) : 2;
 }
 
+template <typename R> __host__ __device__ __forceinline__ int col_width(const Geo& g) { return sizeof(R) == 4 ? g.p : g.mx; }
+
 template <typename R, int L, int DIR, int T, bool SW>
 __global__ void __launch_bounds__(CCfg<L, T, SW>::THREADS, col_min_blocks<R, T>())
     k_colpass(const __grid_constant__ CArgs<R> a) {
   const int m = blockIdx.z;
-  int by = blockIdx.y;                           // (component, other axis)
+  int by = blockIdx.y;                           // component
+  chain_wait();
   if constexpr (DIR > 0) {
     if (a.with_resid) {
       if (by == 0) {
@@ -300,13 +325,13 @@ __global__ void __launch_bounds__(CCfg<L, T, SW>::THREADS, col_min_blocks<R, T>(
   const int tid = threadIdx.x;
   const int mx = a.g.mx, p = a.g.p, ny = a.g.ny;
   const int other = a.axis == 1 ? a.g.nz : ny;
-  const int comp = by / other, o = by - comp * other;
   const long long ls = a.axis == 1 ? (long long)p : (long long)ny * p;
-  C2<R>* base = a.data + m * a.ms + comp * a.g.cs + (a.axis == 1 ? (long long)o * ny * p : (long long)o * p);
   const int c = tid % T, j = tid / T;
-  const int kx = blockIdx.x * T + c;
-  const bool valid = kx < mx;
-  C2<R>* col = base + kx;
+  const int flat = blockIdx.x * T + c;
+  const int width = col_width<R>(a.g);
+  const int o = flat / width, kx = flat - o * width;
+  const bool valid = o < other && kx < mx;
+  C2<R>* col = a.data + m * a.ms + by * a.g.cs + (long long)o * (a.axis == 1 ? (long long)ny * p : (long long)p) + kx;
   // stage 1 straight from global: thread (c, j) owns rows R2 n1 + j of column c
   if (j < R2) {
     C2<R> x[R1];
@@ -348,6 +373,7 @@ __global__ void __launch_bounds__(CCfg<L, T, false>::THREADS, T == 8 ? 6 : 3)
   using R = float;
   const int m = blockIdx.z;
   int by = blockIdx.y;                           // component * nz + z
+  chain_wait();
   if constexpr (DIR > 0) {
     if (a.with_resid) {
       if (by == 0) {
@@ -454,9 +480,8 @@ static cudaError_t xpass_L(const XArgs<R>& a, int batch, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_xpass<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_xpass<R, L><<<grid, C::THREADS, smem, st>>>(a);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chain(a.chain != 0, k_xpass<R, L>, grid, C::THREADS, smem, st, a);
 }
 
 template <typename R>
@@ -489,14 +514,13 @@ cudaError_t launch_xpass_b(const XArgs<R>& a0, int batch, cudaStream_t st) {
 template <typename R, int L, int DIR, int T, bool SW>
 static cudaError_t colpass_LT(const CArgs<R>& a, int batch, cudaStream_t st) {
   const int other = a.axis == 1 ? a.g.nz : a.g.ny;
-  dim3 grid((a.g.mx + T - 1) / T, other * a.ncomp + (DIR > 0 && a.with_resid ? 1 : 0), batch);
+  dim3 grid((col_width<R>(a.g) * other + T - 1) / T, a.ncomp + (DIR > 0 && a.with_resid ? 1 : 0), batch);
   const size_t smem = sizeof(C2<R>) * (size_t)L * T;
   cudaError_t e = cudaFuncSetAttribute(k_colpass<R, L, DIR, T, SW>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_colpass<R, L, DIR, T, SW><<<grid, CCfg<L, T, SW>::THREADS, smem, st>>>(a);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chain(a.chain != 0, k_colpass<R, L, DIR, T, SW>, grid, CCfg<L, T, SW>::THREADS, smem, st, a);
 }
 
 template <int L, int DIR, int T>
@@ -506,10 +530,9 @@ static cudaError_t colpass_tma_LT(const CArgs<float>& a, int batch, cudaStream_t
   cudaError_t e = cudaFuncSetAttribute(k_colpass_tma<L, DIR, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_colpass_tma<L, DIR, T><<<grid, CCfg<L, T, false>::THREADS, smem, st>>>(
-      a, reinterpret_cast<const CUtensorMap*>(a.tmap)[T == 8 ? 0 : 1]);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chain(a.chain != 0, k_colpass_tma<L, DIR, T>, grid, CCfg<L, T, false>::THREADS, smem, st, a,
+                      reinterpret_cast<const CUtensorMap*>(a.tmap)[T == 8 ? 0 : 1]);
 }
 
 template <typename R, int L, int DIR>

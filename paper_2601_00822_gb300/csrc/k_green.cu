@@ -26,8 +26,10 @@ namespace bfcs {
 
 constexpr int kGreenT = 4;   // kx columns per block; 6 components -> 24 line columns
 
-template <int L> struct GCfg {
-  static constexpr int NCOL = 6 * kGreenT;
+// T kx columns per block: 4 in FP32; FP64 plans, bound by the FP64 pipe of each SM, take 2
+// or 1 where that spreads a small grid's tiles more evenly over the SMs (green_cols)
+template <int L, int T = kGreenT> struct GCfg {
+  static constexpr int NCOL = 6 * T;
   static constexpr int THREADS = NCOL * LineInfo<L>::RMAX;
   // block size of the z pass: whole warps (the full-mask shuffles of the residual
   // reduction need them); threads past THREADS take no FFT task
@@ -41,7 +43,9 @@ template <int L> struct GCfg {
 // conflict-free, and the Green phase (8 rows x 4 columns of one component per
 // warp) covers all 16 eight-byte bank pairs twice instead of 8 of them 4 times.
 static_assert(kGreenT == 4 && (6 * kGreenT) % 8 == 0, "the swizzle flips one component bit");
-__device__ __forceinline__ int gslot(int row, int c) { return c ^ (((row >> 1) & 1) << 2); }
+template <int T> __device__ __forceinline__ int gslot(int row, int c) {
+  return T == kGreenT ? c ^ (((row >> 1) & 1) << 2) : c;
+}
 
 template <typename R>
 __device__ __forceinline__ void g0_apply(const C2<R> g[3], const R xi[3], R q, R inv_mu0, R c,
@@ -59,30 +63,27 @@ __device__ __forceinline__ void g0_apply(const C2<R> g[3], const R xi[3], R q, R
 // tile is replaced by eps_hat^{s+1} / N (GM_SWEEP / GM_INIT) or u_hat / N
 // (GM_FINAL); d = tau_hat . xi is written to dprev (sweep / init); returns this
 // thread's share of the residual numerator sum.
-template <typename R, int L>
+template <typename R, int L, int T>
 __device__ __forceinline__ R green_tile(const GArgs<R>& a, C2<R>* s, const C2<R>* pre, int col0, int ky, int mode,
                                         C2<R>* dprev, IterState* stm, const R* Em, bool rd = true,
                                         bool wr = true) {
   // GM_SWEEP: rd = this sweep forms the residual (d_prev staged), wr = it stores d
   const bool rd_d = mode == GM_FINAL || (mode == GM_SWEEP && rd);
   const bool wr_d = mode == GM_INIT || (mode == GM_SWEEP && wr);
-  constexpr int T = kGreenT;
-  constexpr int NCOL = GCfg<L>::NCOL;
+  constexpr int NCOL = GCfg<L, T>::NCOL;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int nx = a.g.nx, ny = a.g.ny, mx = a.g.mx, p = a.g.p;
   const long long cs = a.g.cs;
   const long long zs = (long long)ny * p;
   const long long rowbase = (long long)ky * p;
-  const R two_pi = R(6.283185307179586);
-  const R fx = two_pi / R(nx), fy = two_pi / R(ny), fz = two_pi / R(L);
-  const R mu0 = a.mu0, c0 = (a.lam0 + a.mu0) / (a.lam0 + R(2) * a.mu0);
+  const R fx = a.fx, fy = a.fy, fz = a.fz, c0 = a.c0, inv_mu0 = a.inv_mu0;   // (formed once, on the host)
   const R inv_n = a.inv_n;
   R acc = R(0);
   for (int idx = tid; idx < T * L; idx += nthr) {
     const int col = idx % T, n = idx / T;
     const int kx = col0 + col;
     C2<R>* const m = s + n * NCOL + col;
-    const int qs = (n >> 1) & 1;                    // component q sits at m[(q ^ qs) * T] (gslot)
+    const int qs = T == kGreenT ? (n >> 1) & 1 : 0; // component q sits at m[(q ^ qs) * T] (gslot)
     auto M = [&](int q) -> C2<R>& { return m[(q ^ qs) * T]; };
     const C2<R>* pm = pre + n * T + col;            // array r at pm[r * L * T]
     if (kx >= mx) {
@@ -143,7 +144,7 @@ __device__ __forceinline__ R green_tile(const GArgs<R>& a, C2<R>* s, const C2<R>
     w[1] = mk<R>(d[1].x + bh1.y, d[1].y - bh1.x);
     w[2] = mk<R>(d[2].x + bh2.y, d[2].y - bh2.x);
     C2<R> v[3];
-    g0_apply<R>(w, xi, qq, recip(mu0), c0, v);
+    g0_apply<R>(w, xi, qq, inv_mu0, c0, v);
     if (mode == GM_FINAL) {
       // u_hat = i v, scaled for the unnormalised inverse transforms
 #pragma unroll
@@ -167,9 +168,10 @@ __device__ __forceinline__ R green_tile(const GArgs<R>& a, C2<R>* s, const C2<R>
 // Each FFT stage is a loop over its (line column c, row group j) tasks; with the
 // block of GCfg<L>::BLOCK threads every thread takes at most one.  The b_hat and
 // d_prev tiles are staged in shared memory while the forward transform runs.
-template <typename R, int L>
-__global__ void __launch_bounds__(GCfg<L>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgreen(GArgs<R> a) {
+template <typename R, int L, int T>
+__global__ void __launch_bounds__(GCfg<L, T>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgreen(GArgs<R> a) {
   const int mbr = blockIdx.z;
+  chain_wait();
   if (a.skip_done && a.st[mbr].done) {           // a member that has converged skips
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) a.st[mbr].seen = 1;
     return;
@@ -181,8 +183,7 @@ __global__ void __launch_bounds__(GCfg<L>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgre
   ResidSlot* const part = a.part + mbr * a.part_ms;
   IterState* const stm = a.st + mbr;
   const R* const Em = a.use_me ? a.mE[mbr] : a.E;
-  constexpr int T = kGreenT;
-  constexpr int NCOL = GCfg<L>::NCOL;
+  constexpr int NCOL = GCfg<L, T>::NCOL;
   constexpr int R1 = LineInfo<L>::R1, R2 = LineInfo<L>::R2;
   constexpr int TASKS = NCOL * LineInfo<L>::RMAX;   // (column, row group) tasks of a stage
   extern __shared__ unsigned char smem_raw[];
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(GCfg<L>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgre
       for (int n1 = 0; n1 < R1; ++n1) x[n1] = cvalid ? gcol[(R2 * n1 + j) * zs] : mk<R>(0, 0);
       stage1<R, L, -1>(x, j, a.tw);
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) s[(j * R1 + k1) * NCOL + gslot(j * R1 + k1, c)] = x[k1];
+      for (int k1 = 0; k1 < R1; ++k1) s[(j * R1 + k1) * NCOL + gslot<T>(j * R1 + k1, c)] = x[k1];
     }
     __syncthreads();
     // stage 2 reads and writes the same slots (rows j + R1 m, m < R2, of column c):
@@ -246,10 +247,10 @@ __global__ void __launch_bounds__(GCfg<L>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgre
       if (j >= R1) continue;
       C2<R> y[R2];
 #pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) y[n2] = s[(n2 * R1 + j) * NCOL + gslot(n2 * R1 + j, c)];
+      for (int n2 = 0; n2 < R2; ++n2) y[n2] = s[(n2 * R1 + j) * NCOL + gslot<T>(n2 * R1 + j, c)];
       stage2<R, L, -1>(y);
 #pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2) s[(j + R1 * k2) * NCOL + gslot(j + R1 * k2, c)] = y[k2];
+      for (int k2 = 0; k2 < R2; ++k2) s[(j + R1 * k2) * NCOL + gslot<T>(j + R1 * k2, c)] = y[k2];
     }
     __syncthreads();
   }
@@ -258,7 +259,7 @@ __global__ void __launch_bounds__(GCfg<L>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgre
   __syncthreads();
 
   // ---- Green operators per mode
-  R acc = green_tile<R, L>(a, s, pre, col0, ky, mode, dprev, stm, Em, rd, wr);
+  R acc = green_tile<R, L, T>(a, s, pre, col0, ky, mode, dprev, stm, Em, rd, wr);
 
   // ---- residual partial of this block in FP64 (fixed order: deterministic)
   const bool resid = (mode == GM_SWEEP && rd) || mode == GM_FINAL;
@@ -283,10 +284,10 @@ __global__ void __launch_bounds__(GCfg<L>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgre
     if (j >= R1) continue;
     C2<R> y[R2];
 #pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) y[k2] = s[(j + R1 * k2) * NCOL + gslot(j + R1 * k2, c)];
+    for (int k2 = 0; k2 < R2; ++k2) y[k2] = s[(j + R1 * k2) * NCOL + gslot<T>(j + R1 * k2, c)];
     Dft<R, R2, +1>::run(y);
 #pragma unroll
-    for (int n2 = 0; n2 < R2; ++n2) s[(j + R1 * n2) * NCOL + gslot(j + R1 * n2, c)] = y[n2];
+    for (int n2 = 0; n2 < R2; ++n2) s[(j + R1 * n2) * NCOL + gslot<T>(j + R1 * n2, c)] = y[n2];
   }
   __syncthreads();
   for (int task = tid; task < TASKS; task += nthr) {
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(GCfg<L>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgre
     const bool keep = (mode != GM_FINAL || c / T < 3) && col0 + (c % T) < mx;
     C2<R> x[R1];
 #pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) x[k1] = s[(j * R1 + k1) * NCOL + gslot(j * R1 + k1, c)];
+    for (int k1 = 0; k1 < R1; ++k1) x[k1] = s[(j * R1 + k1) * NCOL + gslot<T>(j * R1 + k1, c)];
     twiddle_then_dft<R, L, R1, +1>(x, j, a.tw);
     if (keep) {
       C2<R>* gcol = column(c);
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
     for (int idx = tid; idx < 12 * L * 2; idx += nthr) {
       const int half = idx & 1, n = (idx >> 1) % L, arr = idx / (2 * L);
       if (arr < 6) {
-        cp_async16(S + n * NCOL + gslot(n, arr * T + 2 * half), spec + arr * cs + n * zs + 2 * half);
+        cp_async16(S + n * NCOL + gslot<T>(n, arr * T + 2 * half), spec + arr * cs + n * zs + 2 * half);
       } else {
         const int q = arr - 6;
         const C2<R>* src = (q < 3 ? bh + q * cs : dp + (q - 3) * cs) + n * zs + 2 * half;
@@ -379,6 +380,7 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
     __syncthreads();
   };
 
+  chain_wait();
   if (blockIdx.x == 0)                           // (as in k_zgreen)
     for (int m = tid; m * tiles_pm < total; m += nthr)
       if (a.st[m].done) a.st[m].seen = 1;
@@ -411,13 +413,13 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
       C2<R> x[R1];
       if (j < R2) {
 #pragma unroll
-        for (int n1 = 0; n1 < R1; ++n1) x[n1] = s[(R2 * n1 + j) * NCOL + gslot(R2 * n1 + j, c)];
+        for (int n1 = 0; n1 < R1; ++n1) x[n1] = s[(R2 * n1 + j) * NCOL + gslot<T>(R2 * n1 + j, c)];
         stage1<R, L, -1>(x, j, a.tw);
       }
       __syncthreads();
       if (j < R2) {
 #pragma unroll
-        for (int k1 = 0; k1 < R1; ++k1) s[(j * R1 + k1) * NCOL + gslot(j * R1 + k1, c)] = x[k1];
+        for (int k1 = 0; k1 < R1; ++k1) s[(j * R1 + k1) * NCOL + gslot<T>(j * R1 + k1, c)] = x[k1];
       }
     }
     __syncthreads();
@@ -425,17 +427,17 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
       C2<R> y[R2];
       if (j < R1) {
 #pragma unroll
-        for (int n2 = 0; n2 < R2; ++n2) y[n2] = s[(n2 * R1 + j) * NCOL + gslot(n2 * R1 + j, c)];
+        for (int n2 = 0; n2 < R2; ++n2) y[n2] = s[(n2 * R1 + j) * NCOL + gslot<T>(n2 * R1 + j, c)];
         stage2<R, L, -1>(y);
       }
       __syncthreads();
       if (j < R1) {
 #pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) s[(j + R1 * k2) * NCOL + gslot(j + R1 * k2, c)] = y[k2];
+        for (int k2 = 0; k2 < R2; ++k2) s[(j + R1 * k2) * NCOL + gslot<T>(j + R1 * k2, c)] = y[k2];
       }
     }
     __syncthreads();
-    acc += (double)green_tile<R, L>(a, s, pre, col0, ky, GM_SWEEP, dprev, stm, Em);
+    acc += (double)green_tile<R, L, T>(a, s, pre, col0, ky, GM_SWEEP, dprev, stm, Em);
     __syncthreads();
     // inverse z transform in the order of the one-tile-per-block form (the same
     // arithmetic, so the two forms give identical fields): in-place R2-point step,
@@ -443,16 +445,16 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
     if (j < R1) {
       C2<R> y[R2];
 #pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2) y[k2] = s[(j + R1 * k2) * NCOL + gslot(j + R1 * k2, c)];
+      for (int k2 = 0; k2 < R2; ++k2) y[k2] = s[(j + R1 * k2) * NCOL + gslot<T>(j + R1 * k2, c)];
       Dft<R, R2, +1>::run(y);
 #pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) s[(j + R1 * n2) * NCOL + gslot(j + R1 * n2, c)] = y[n2];
+      for (int n2 = 0; n2 < R2; ++n2) s[(j + R1 * n2) * NCOL + gslot<T>(j + R1 * n2, c)] = y[n2];
     }
     __syncthreads();
     if (j < R2) {
       C2<R> x[R1];
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) x[k1] = s[(j * R1 + k1) * NCOL + gslot(j * R1 + k1, c)];
+      for (int k1 = 0; k1 < R1; ++k1) x[k1] = s[(j * R1 + k1) * NCOL + gslot<T>(j * R1 + k1, c)];
       twiddle_then_dft<R, L, R1, +1>(x, j, a.tw);
       const int kx = col0 + ccol;
       if (kx < a.g.mx) {
@@ -792,21 +794,50 @@ cudaError_t launch_green_dense(C2<R>* spec, const C2<R>* bhat, C2<R>* dprev, con
   return cudaGetLastError();
 }
 
+// kx columns per block of the z pass for B members of grid g.  FP32: kGreenT (32-byte
+// sectors).  FP64: blocks that share an SM share its FP64 pipe, so the pass takes
+// (blocks on the busiest SM) x T; the widest T of least product.  32^3: 160 blocks of 4
+// columns put two on 8 of the 152 SMs, 288 of 2 columns the same work evenly.
 template <typename R>
-int green_nparts(const Geo& g) {
-  return ((g.mx + kGreenT - 1) / kGreenT) * g.ny;
+static int green_cols(const Geo& g, int B) {
+  if (sizeof(R) == 4) return kGreenT;
+  int best = kGreenT;
+  long long cost = -1;
+  for (int T = kGreenT; T >= 1; T /= 2) {
+    const long long blocks = (long long)((g.mx + T - 1) / T) * g.ny * B;
+    const long long c = (blocks + sm_count() - 1) / sm_count() * T;
+    if (cost < 0 || c < cost) { cost = c; best = T; }
+  }
+  return best;
+}
+
+template <typename R>
+int green_nparts(const Geo& g, int B) {
+  const int T = green_cols<R>(g, B);
+  return ((g.mx + T - 1) / T) * g.ny;
+}
+
+template <typename R, int L, int T>
+static cudaError_t zgreen_LT(const GArgs<R>& a, int batch, cudaStream_t st) {
+  dim3 grid((a.g.mx + T - 1) / T, a.g.ny, batch);
+  const size_t smem = sizeof(C2<R>) * (size_t)L * (GCfg<L, T>::NCOL + 6 * T);
+  cudaError_t e = cudaFuncSetAttribute(k_zgreen<R, L, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  count_launches(1);
+  return launch_chain(a.chain != 0, k_zgreen<R, L, T>, grid, GCfg<L, T>::BLOCK, smem, st, a);
 }
 
 template <typename R, int L>
 static cudaError_t zgreen_L(const GArgs<R>& a, int batch, cudaStream_t st) {
-  dim3 grid((a.g.mx + kGreenT - 1) / kGreenT, a.g.ny, batch);
-  const size_t smem = sizeof(C2<R>) * (size_t)L * (GCfg<L>::NCOL + 6 * kGreenT);
-  cudaError_t e = cudaFuncSetAttribute(k_zgreen<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  k_zgreen<R, L><<<grid, GCfg<L>::BLOCK, smem, st>>>(a);
-  count_launches(1);
-  return cudaGetLastError();
+  if constexpr (sizeof(R) == 8) {
+    switch (green_cols<R>(a.g, batch)) {
+      case 1: return zgreen_LT<R, L, 1>(a, batch, st);
+      case 2: return zgreen_LT<R, L, 2>(a, batch, st);
+      default: break;
+    }
+  }
+  return zgreen_LT<R, L, kGreenT>(a, batch, st);
 }
 
 template <int L>
@@ -816,19 +847,24 @@ static cudaError_t zgreen_p_L(const GArgs<float>& a, int batch, int blocks, cuda
   const size_t smem = GPCfg<L>::SMEM;
   cudaError_t e = cudaFuncSetAttribute(k_zgreen_p<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_zgreen_p<L><<<blocks, GCfg<L>::THREADS, smem, st>>>(a, tiles_x, tiles_pm, tiles_pm * batch);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_chain(a.chain != 0, k_zgreen_p<L>, blocks, GCfg<L>::THREADS, smem, st, a, tiles_x, tiles_pm, tiles_pm * batch);
 }
 
 template <typename R>
-int green_sweep_parts(const Geo& g) {
+int green_sweep_parts(const Geo& g, int B) {
   const int pb = green_persistent_blocks<R>(g);
-  return pb > 0 ? pb : green_nparts<R>(g);
+  return pb > 0 ? pb : green_nparts<R>(g, B);
 }
 
 template <typename R>
-cudaError_t launch_zgreen_b(const GArgs<R>& a, int batch, cudaStream_t st) {
+cudaError_t launch_zgreen_b(const GArgs<R>& a0, int batch, cudaStream_t st) {
+  GArgs<R> a = a0;
+  a.fx = R(6.283185307179586) / R(a.g.nx);
+  a.fy = R(6.283185307179586) / R(a.g.ny);
+  a.fz = R(6.283185307179586) / R(a.g.nz);
+  a.c0 = (a.lam0 + a.mu0) / (a.lam0 + R(2) * a.mu0);
+  a.inv_mu0 = R(1) / a.mu0;
   if constexpr (sizeof(R) == 4) {
     const int pb = green_persistent_blocks<R>(a.g);
     if (pb > 0 && a.mode == GM_SWEEP && a.skip_done && !a.sparse && GPCfg<256>::SMEM <= 227 * 1024) {
@@ -855,8 +891,8 @@ cudaError_t launch_zgreen(const GArgs<R>& a, cudaStream_t st) { return launch_zg
 #ifndef BFCS_FF   // the float-float build carries only the ladder's defect kernels
 template cudaError_t launch_zgreen<BFCS_R>(const GArgs<BFCS_R>&, cudaStream_t);
 template cudaError_t launch_zgreen_b<BFCS_R>(const GArgs<BFCS_R>&, int, cudaStream_t);
-template int green_nparts<BFCS_R>(const Geo&);
-template int green_sweep_parts<BFCS_R>(const Geo&);
+template int green_nparts<BFCS_R>(const Geo&, int);
+template int green_sweep_parts<BFCS_R>(const Geo&, int);
 template cudaError_t launch_green_dense<BFCS_R>(C2<BFCS_R>*, const C2<BFCS_R>*, C2<BFCS_R>*, const Geo&, double,
                                                 double, const double*, ResidSlot*, int, double*, cudaStream_t);
 #endif

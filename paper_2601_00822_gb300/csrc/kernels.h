@@ -6,6 +6,29 @@
 
 namespace bfcs {
 
+// Launch of a kernel that begins with chain_wait() (common.cuh), chained to its predecessor
+// when `chain` is set.  The Krylov loops chain their 8-10 launches per iteration (plain
+// stream launches with one-block kernels between the passes: a 128^3 solve by Algorithm 3
+// 38.9 -> 34.8 ms, a 64^3 FP64 solve by Algorithm 2 40.4 -> 37.7 ms); the sweeps do not:
+// their launches sit in CUDA graphs, whose gaps are small already, and blocks that wait on
+// an SM disturb the placement of the running pass (32^3 FP64 8.7 -> 11.0 ms, 64^3 3.54 ->
+// 3.66 ms, 256^3 121 -> 124 ms when chained).
+template <class... P, class... A>
+cudaError_t launch_chain(bool chain, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                         const A&... a) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = chain ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, a...);
+}
+
 // ---- x pass: along x (contiguous) with the real<->half-spectrum transform.
 enum XMode : int {
   XM_SWEEP = 0,    // spectrum -> C2R -> eps -> tau = L1 eps -> R2C -> spectrum (Eqs. 5.7, 5.8, 5.10)
@@ -54,6 +77,7 @@ template <typename R> struct XArgs {
   R out_scale;            // XM_R2C: factor applied to the stored half spectrum (0 means 1)
   int ncomp;
   int mode;
+  int chain;              // see launch_chain
   XMember xm[kMaxBatch];
 };
 
@@ -94,6 +118,7 @@ template <typename R> struct CArgs {
   // members are then skipped by IterState.seen (set by the Green pass), since the step may
   // set `done` while other blocks of the pass have not started
   int with_resid;
+  int chain;              // see launch_chain
   ResidArgs resid;
 };
 
@@ -202,6 +227,7 @@ enum GMode : int {
 };
 
 template <typename R> struct GArgs {
+  int chain;              // see launch_chain
   C2<R>* spec;            // 6 components, x- and y-transformed
   const C2<R>* bhat;      // 3 components, fully transformed body force
   C2<R>* dprev;           // 3 components: d = tau_hat . xi of the previous sweep
@@ -222,6 +248,7 @@ template <typename R> struct GArgs {
   // that sweep, the one before it and the last sweep (s + 1 == maxit)
   int sparse;
   int maxit;
+  R fx, fy, fz, c0, inv_mu0;       // 2 pi / n of the axes, G0's constants: filled by the launcher
   R mE[kMaxBatch][6];
 };
 
@@ -270,10 +297,10 @@ cudaError_t launch_defect_final(const ResidSlot* part, int nparts, IterState* st
                                 int maxdim, cudaStream_t s);
 template <typename R> cudaError_t launch_colpass(const CArgs<R>& a, int dir, cudaStream_t s);
 template <typename R> cudaError_t launch_zgreen(const GArgs<R>& a, cudaStream_t s);
-template <typename R> int green_nparts(const Geo& g);
+template <typename R> int green_nparts(const Geo& g, int B);
 // residual partial slots per member written by a GM_SWEEP launch of the z pass
 // (fewer than green_nparts when the persistent form runs)
-template <typename R> int green_sweep_parts(const Geo& g);
+template <typename R> int green_sweep_parts(const Geo& g, int B);
 template <typename R> cudaError_t launch_xpass_b(const XArgs<R>& a, int batch, cudaStream_t s);
 template <typename R> cudaError_t launch_colpass_b(const CArgs<R>& a, int dir, int batch, cudaStream_t s);
 template <typename R> cudaError_t launch_zgreen_b(const GArgs<R>& a, int batch, cudaStream_t s);

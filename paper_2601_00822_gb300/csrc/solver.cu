@@ -29,7 +29,6 @@ struct bfcs_plan_s {
   void* tw[3] = {nullptr, nullptr, nullptr};
   ResidSlot* part = nullptr;
   int npart = 0;              // slots allocated (>= every writer's block count)
-  int ngreen = 0;             // blocks of the fused z/Green pass = residual partials per sweep
   int stall_window = 100;     // sweeps without a 10% residual drop that end a solve
   IterState* ist = nullptr;        // max_batch members
   IterState* ist_host = nullptr;   // pinned, 3 slots x max_batch
@@ -328,6 +327,8 @@ PhaseTab<R> make_tab(int nph, const bfcs_lame* phases, bfcs_lame C0) {
     t.lam[p] = (R)q.lambda;
     t.mu[p] = (R)q.mu;
     t.lam1[p] = (R)(q.lambda - C0.lambda);
+    t.lamh[p] = (R)(0.5 * q.lambda);
+    t.lam1h[p] = (R)(0.5 * (q.lambda - C0.lambda));
     t.mu1[p] = (R)(q.mu - C0.mu);
   }
   return t;
@@ -497,7 +498,7 @@ struct SweepSet {
     ga.spec_ms = sms;
     ga.b_ms = 3 * g.cs;
     ga.d_ms = 3 * g.cs;
-    ga.part_ms = P->ngreen;
+    ga.part_ms = green_nparts<R>(P->g, B);
     cy.data = (C2<R>*)P->spec;
     cy.ms = sms;
     cy.g = g;
@@ -594,7 +595,7 @@ struct SweepSet {
     // the inverse y pass, with the residual step beside it (the persistent form of the z
     // pass does not run with sparse evaluation)
     cy.with_resid = 1;
-    cy.resid = resid_args(GM_SWEEP, ga.sparse ? green_nparts<R>(P->g) : green_sweep_parts<R>(P->g));
+    cy.resid = resid_args(GM_SWEEP, ga.sparse ? green_nparts<R>(P->g, B) : green_sweep_parts<R>(P->g, B));
     cy.resid.io = (P->prof_kind == 3 && sweep >= 0) ? P->io_dev : nullptr;
     const cudaError_t e = timed(2, [&] { return launch_colpass_b<R>(cy, +1, B, q); });
     cy.with_resid = 0;
@@ -622,7 +623,7 @@ struct SweepSet {
     ga.mode = GM_FINAL;
     ga.skip_done = 0;
     CK(launch_zgreen_b<R>(ga, B, st));
-    CK(launch_resid_final(resid_args(GM_FINAL, P->ngreen), B, st));
+    CK(launch_resid_final(resid_args(GM_FINAL, green_nparts<R>(P->g, B)), B, st));
     cy.ncomp = 3;
     CK(launch_colpass_b<R>(cy, +1, B, st));
     XArgs<R> xu{};
@@ -989,11 +990,14 @@ int run_cg(SweepSet<R>& ss, std::vector<double>& req, int maxit, std::vector<int
   xa.spec_in = ca.p;
   xa.spec_out = ca.q;
   xa.st = P->cg_skip;
+  xa.chain = 1;
   CArgs<R> cy = ss.cy;
   cy.data = ca.q;   // not the mapped spectrum: the same tile with direct loads (tmap_data != data)
   cy.st = P->cg_skip;
   cy.ncomp = 6;
+  cy.chain = 1;
   GArgs<R> ga = ss.ga;
+  ga.chain = 1;
   ga.spec = ca.q;
   ga.st = P->cg_skip;
   ga.mode = GM_APPLY;
@@ -1119,6 +1123,7 @@ int run_cd(SweepSet<R>& ss, int maxit, bfcs_info* infos) {
   xs.st = P->cg_skip;
   cy.st = P->cg_skip;
   cz.st = P->cg_skip;
+  xs.chain = cy.chain = 1;
   int it = 0, chunk = 8;
   std::vector<double> obs_r(B, -1.0);
   std::vector<int> obs_it(B, -1);
@@ -1959,8 +1964,8 @@ int bfcs_plan_create(bfcs_plan* out, int nx, int ny, int nz, int max_batch, int 
             cudaStreamCreateWithFlags(&P->loop_st, cudaStreamNonBlocking) == cudaSuccess;
   if (!ok) { free_plan(P); return BFCS_ERR_CUDA; }
   const size_t cs = (size_t)P->g.cs;
-  P->ngreen = P->fp64 ? green_nparts<double>(P->g) : green_nparts<float>(P->g);
-  P->npart = std::max(P->ngreen, 512);
+  // residual partials: one per block of the z/Green pass (FP64: down to one column a block)
+  P->npart = std::max(P->fp64 ? P->g.mx * P->g.ny : green_nparts<float>(P->g, 1), 512);
   const size_t MB = (size_t)max_batch;
   ok = cudaMalloc(&P->spec, MB * 6 * cs * P->csz) == cudaSuccess &&
        cudaMalloc(&P->bhat, MB * 3 * cs * P->csz) == cudaSuccess &&

@@ -754,3 +754,27 @@ def test_loads_with_vanishing_components(comps, precision):
         ev = ~np.isnan(hist)
         h_ref = np.array(ref["hist"])
         assert np.all(np.abs(hist[ev] - h_ref[ev]) <= 1e-4 * h_ref[ev] + (1e-12 if precision == "fp64" else 1e-6))
+
+
+@pytest.mark.parametrize("dims,cell", [((32, 32, 32), (16, 16, 16)), ((48, 24, 16), (24, 12, 16)), ((16, 12, 6), (8, 12, 6)),
+                                       ((24, 64, 32), (24, 16, 16))])
+def test_fp64_column_widths_of_the_z_pass_agree(dims, cell):
+    """FP64 plans choose the z pass's columns per block (4, 2 or 1) by how the batch's
+    blocks fall on the SMs, so batches of 1 to 9 run different widths: the same fields bit
+    for bit, and residuals that differ by the order of their FP64 partial sums (<= 1e-13
+    for up to 10^4 terms of one sign)."""
+    nx, ny, nz = dims
+    p = small_problem(dims, cell, [[cell[0], cell[1], cell[2], cell[2] ** 2 // 4, 1]], (nx / 2, ny / 2, nz / 2),
+                      min(dims) / 3.0, E=(0.002, 0.0, -0.001, 0.0, 0.0, 0.003))
+    ph, b = gpu_inputs(p, "fp64")
+    ref = None
+    for B in (1, 2, 4, 9):
+        with api.Plan(dims, "fp64", max_batch=B) as plan:
+            mem, infos = plan.solve_batched([dict(phase=ph, b=b, E=p.mean_strain) for _ in range(B)], p.phases, p.c0,
+                                            tol=0.0, maxit=6)
+        for m, i in zip(mem, infos):
+            got = (m["eps_out"], m["sig_out"], m["u_out"], i.resid)
+            if ref is None:
+                ref = got
+            assert all(torch.equal(a, c) for a, c in zip(got[:3], ref[:3])), B
+            assert abs(got[3] - ref[3]) <= 1e-13 * ref[3], B
