@@ -168,8 +168,14 @@ __device__ __forceinline__ R green_tile(const GArgs<R>& a, C2<R>* s, const C2<R>
 // Each FFT stage is a loop over its (line column c, row group j) tasks; with the
 // block of GCfg<L>::BLOCK threads every thread takes at most one.  The b_hat and
 // d_prev tiles are staged in shared memory while the forward transform runs.
+// Blocks per SM the register budget is sized for.  FP32 to 64 lines: 6 (56 registers
+// instead of 71, no spills); 96 and 128: 3; longer lines: 2, by their shared memory.
+template <typename R, int L> constexpr int green_min_blocks() {
+  return sizeof(R) != 4 ? 1 : L <= 64 ? 6 : L <= 128 ? 3 : 2;
+}
+
 template <typename R, int L, int T>
-__global__ void __launch_bounds__(GCfg<L, T>::BLOCK, sizeof(R) == 4 ? 2 : 1) k_zgreen(GArgs<R> a) {
+__global__ void __launch_bounds__(GCfg<L, T>::BLOCK, green_min_blocks<R, L>()) k_zgreen(GArgs<R> a) {
   const int mbr = blockIdx.z;
   chain_wait();
   if (a.skip_done && a.st[mbr].done) {           // a member that has converged skips
