@@ -269,16 +269,46 @@ static __global__ void k_cd_scalar(const double* part, int nparts, CdState* cd, 
   CdState& S = cd[m];
   chain_wait();
   if (mode != CdMode::RESID && S.done) return;
+  // One chain of latencies (FP64 add 64 clocks, square root and division 600 each): both
+  // sums go through the same shuffles, and the normaliser of an update's residual is
+  // formed by another warp beside them.
+  __shared__ double red2[32], iden_s;
+  IterState& st = ist[m];
+  const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5;
+  const double xmin = 6.283185307179586 / (double)maxdim;
   double a1 = 0.0, a2 = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
+#pragma unroll 4
+  for (int i = tid; i < nparts; i += blockDim.x) {
     a1 += part[((long long)m * nparts + i) * 2];
     a2 += part[((long long)m * nparts + i) * 2 + 1];
   }
-  const double t1 = cd_reduce(a1, red);
-  const double t2 = cd_reduce(a2, red);
-  if (threadIdx.x != 0) return;
-  IterState& st = ist[m];
-  const double xmin = 6.283185307179586 / (double)maxdim;
+  if (mode == CdMode::UPDATE && tid >= (int)blockDim.x - 32) {
+    // s0u += alpha s0p, and 1 / (bden + xi_min |s0b + s0u|_F): lane k < 6 a component
+    double q = 0.0;
+    if (lane < 6) {
+      const double u = S.s0u[lane] + S.alpha * S.s0p[lane], v = S.s0b[lane] + u;
+      S.s0u[lane] = u;
+      q = (lane < 3 ? 1.0 : 2.0) * v * v;
+    }
+    for (int off = 4; off > 0; off >>= 1) q += __shfl_down_sync(0xffffffffu, q, off);
+    if (lane == 0) {
+      const double den = st.bden + xmin * sqrt(q);
+      iden_s = den > 0.0 ? 1.0 / den : 1.0;
+    }
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    a1 += __shfl_down_sync(0xffffffffu, a1, off);
+    a2 += __shfl_down_sync(0xffffffffu, a2, off);
+  }
+  if (lane == 0) { red[tid >> 5] = a1; red2[tid >> 5] = a2; }
+  __syncthreads();
+  if (tid >= 32) return;
+  double t1 = tid < nw ? red[tid] : 0.0, t2 = tid < nw ? red2[tid] : 0.0;
+  for (int off = 16; off > 0; off >>= 1) {
+    t1 += __shfl_down_sync(0xffffffffu, t1, off);
+    t2 += __shfl_down_sync(0xffffffffu, t2, off);
+  }
+  if (tid != 0) return;
   auto resid = [&](const double (&s0)[6], double rr) {
     const double den = st.bden + xmin * cd_s0norm(s0);
     return den > 0.0 ? sqrt(rr) / den : sqrt(rr);
@@ -311,11 +341,8 @@ static __global__ void k_cd_scalar(const double* part, int nparts, CdState* cd, 
   } else if (mode == CdMode::UPDATE) {
     S.beta = S.rz > 0.0 ? t1 / S.rz : 0.0;
     S.rz = t1;
-    for (int k = 0; k < 6; ++k) S.s0u[k] += S.alpha * S.s0p[k];
     S.iters += 1;
-    double s0[6];
-    for (int k = 0; k < 6; ++k) s0[k] = S.s0b[k] + S.s0u[k];
-    S.resid = resid(s0, t2);
+    S.resid = sqrt(t2) * iden_s;
     st.resid_last = S.resid;
     if (!(S.resid == S.resid)) { S.status = 3; fin = true; }
     else if (S.resid <= S.tol) { S.status = 1; fin = true; }

@@ -138,8 +138,14 @@ static __global__ void k_cg_scalar(const double* part, int nparts, CgState* cg, 
   chain_wait();
   if (S.done) return;
   double acc = 0.0;
+#pragma unroll 4
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[(long long)m * nparts + i];
-  const double t = block_reduce(acc, red);
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  double t = threadIdx.x < blockDim.x / 32 ? red[threadIdx.x] : 0.0;
+  for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
   if (threadIdx.x != 0) return;
   bool fin = false;
   if (mode == CgMode::INIT) {

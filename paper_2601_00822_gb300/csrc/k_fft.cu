@@ -308,7 +308,11 @@ __global__ void __launch_bounds__(CCfg<L, T, SW>::THREADS, col_min_blocks<R, T>(
   if constexpr (DIR > 0) {
     if (a.with_resid) {
       if (by == 0) {
-        if (blockIdx.x == 0) resid_step(a.resid, m);
+        if (m == 0)
+          for (int k = blockIdx.x; k < (int)gridDim.z; k += gridDim.x) {
+            resid_step(a.resid, k);
+            __syncthreads();
+          }
         return;
       }
       --by;
@@ -377,7 +381,11 @@ __global__ void __launch_bounds__(CCfg<L, T, false>::THREADS, T == 8 ? 6 : 3)
   if constexpr (DIR > 0) {
     if (a.with_resid) {
       if (by == 0) {
-        if (blockIdx.x == 0) resid_step(a.resid, m);
+        if (m == 0)
+          for (int k = blockIdx.x; k < (int)gridDim.z; k += gridDim.x) {
+            resid_step(a.resid, k);
+            __syncthreads();
+          }
         return;
       }
       --by;

@@ -226,10 +226,15 @@ cudaError_t launch_polarize(R* tau, const R* eps, const int8_t* phase, const Pha
 // ---------------------------------------------------------------- validation
 constexpr int kValBlocks = 512;
 
+// partials of member blockIdx.y: [8][gridDim.x]: per component sum b_c, sum |b_c|, then
+// the phase ids' minimum and maximum
 template <typename R>
-__global__ void k_validate(const int8_t* phase, const R* b, long long n, int* iout, double* part) {
+__global__ void k_validate(const __grid_constant__ ValArgs<R> va, long long n, double* part) {
   __shared__ double red[32];
   __shared__ int smin, smax;
+  const int8_t* phase = va.phase[blockIdx.y];
+  const R* b = va.b[blockIdx.y];
+  part += (long long)blockIdx.y * 8 * gridDim.x;
   if (threadIdx.x == 0) { smin = 127; smax = -128; }
   __syncthreads();
   int lmin = 127, lmax = -128;
@@ -253,31 +258,43 @@ __global__ void k_validate(const int8_t* phase, const R* b, long long n, int* io
     if (threadIdx.x == 0) part[(2 * c + 1) * gridDim.x + blockIdx.x] = ta;
   }
   __syncthreads();
-  if (threadIdx.x == 0) { atomicMin(&iout[0], smin); atomicMax(&iout[1], smax); }
-}
-
-__global__ void k_validate_final(const double* part, int nparts, double* dout) {
-  __shared__ double red[32];
-  for (int j = 0; j < 6; ++j) {
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[j * nparts + i];
-    const double t = block_sum(acc, red);
-    if (threadIdx.x == 0) dout[(j & 1) * 3 + j / 2] = t;
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    part[6 * gridDim.x + blockIdx.x] = (double)smin;
+    part[7 * gridDim.x + blockIdx.x] = (double)smax;
   }
 }
 
-__global__ void k_init_minmax(int* iout) { iout[0] = 127; iout[1] = -128; }
+// one warp per quantity of member blockIdx.x
+__global__ void k_validate_final(const double* part, int nparts, int* iout, double* dout) {
+  const int m = blockIdx.x, j = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* p = part + ((long long)m * 8 + j) * nparts;
+  if (j < 6) {
+    double acc = 0.0;
+    for (int i = lane; i < nparts; i += 32) acc += p[i];
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+    if (lane == 0) dout[6 * m + (j & 1) * 3 + j / 2] = acc;
+  } else {
+    int v = j == 6 ? 127 : -128;
+    for (int i = lane; i < nparts; i += 32) v = j == 6 ? min(v, (int)p[i]) : max(v, (int)p[i]);
+    for (int off = 16; off > 0; off >>= 1) {
+      const int w = __shfl_down_sync(0xffffffffu, v, off);
+      v = j == 6 ? min(v, w) : max(v, w);
+    }
+    if (lane == 0) iout[2 * m + j - 6] = v;
+  }
+}
 
-int validate_scratch(long long) { return 6 * kValBlocks; }
+int validate_scratch() { return 8 * kValBlocks; }
 
+// All members in two launches (three a member, each a few blocks' latency, took 3% of a
+// batch of 64^3 solves); at least four voxels a thread.
 template <typename R>
-cudaError_t launch_validate(const int8_t* phase, const R* b, long long n, int* iout, double* dout,
-                            double* scratch, cudaStream_t s) {
-  k_init_minmax<<<1, 1, 0, s>>>(iout);
-  k_validate<R><<<kValBlocks, kRedThreads, 0, s>>>(phase, b, n, iout, scratch);
-  k_validate_final<<<1, kRedThreads, 0, s>>>(scratch, kValBlocks, dout);
-  count_launches(3);
+cudaError_t launch_validate(const ValArgs<R>& va, int batch, long long n, int* iout, double* dout, double* scratch,
+                            cudaStream_t s) {
+  const int blocks = (int)std::max<long long>(1, std::min<long long>(kValBlocks, n / (4 * kRedThreads)));
+  k_validate<R><<<dim3(blocks, batch), kRedThreads, 0, s>>>(va, n, scratch);
+  k_validate_final<<<batch, 256, 0, s>>>(scratch, blocks, iout, dout);
+  count_launches(2);
   return cudaGetLastError();
 }
 
@@ -569,28 +586,23 @@ __global__ void k_cast_d2f(float* dst, const double* src, long long count) {
        i += (long long)gridDim.x * blockDim.x)
     dst[i] = (float)src[i];
 }
-__global__ void k_cast_f2d(double* dst, const float* src, long long count) {
+template <bool ADD>
+__global__ void k_f2d(const __grid_constant__ F2dArgs a, long long count) {
+  double* dst = a.dst[blockIdx.y];
+  const float* src = a.src[blockIdx.y];
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
        i += (long long)gridDim.x * blockDim.x)
-    dst[i] = (double)src[i];
-}
-__global__ void k_add_f2d(double* dst, const float* src, long long count) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x)
-    dst[i] += (double)src[i];
+    dst[i] = ADD ? dst[i] + (double)src[i] : (double)src[i];
 }
 cudaError_t launch_cast_d2f(float* dst, const double* src, long long count, cudaStream_t s) {
   k_cast_d2f<<<8 * 152, 256, 0, s>>>(dst, src, count);
   count_launches(1);
   return cudaGetLastError();
 }
-cudaError_t launch_cast_f2d(double* dst, const float* src, long long count, cudaStream_t s) {
-  k_cast_f2d<<<8 * 152, 256, 0, s>>>(dst, src, count);
-  count_launches(1);
-  return cudaGetLastError();
-}
-cudaError_t launch_add_f2d(double* dst, const float* src, long long count, cudaStream_t s) {
-  k_add_f2d<<<8 * 152, 256, 0, s>>>(dst, src, count);
+cudaError_t launch_f2d(const F2dArgs& a, int batch, long long count, bool add, cudaStream_t s) {
+  const int blocks = (int)std::max<long long>(1, std::min<long long>(8 * 152, (count + 1023) / 1024));
+  if (add) k_f2d<true><<<dim3(blocks, batch), 256, 0, s>>>(a, count);
+  else k_f2d<false><<<dim3(blocks, batch), 256, 0, s>>>(a, count);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -622,8 +634,14 @@ cudaError_t launch_cast_spec_ff(C2<float>* dst, const C2<ff>* src, const Geo& g,
   return cudaGetLastError();
 }
 
-__global__ void k_stress(double* sig, const double* eps, const int8_t* phase, PhaseTab<double> tab, int sx,
-                         int sy, int sz, int nx, int ny, int nz) {
+__global__ void k_stress(const __grid_constant__ StressArgs a, const __grid_constant__ PhaseTab<double> tab, int nx,
+                         int ny, int nz) {
+  const int m = blockIdx.y;
+  double* const sig = a.sig[m];
+  if (sig == nullptr) return;                    // a member without this output
+  const double* const eps = a.eps[m];
+  const int8_t* const phase = a.phase[m];
+  const int sx = a.sx[m], sy = a.sy[m], sz = a.sz[m];
   const long long n = (long long)nx * ny * nz;
   const bool small = n <= 0xFFFFFFFFLL;
   // shifts reduced to [0, n) once: the per-voxel translation is then one compare
@@ -644,9 +662,11 @@ __global__ void k_stress(double* sig, const double* eps, const int8_t* phase, Ph
     for (int c = 3; c < 6; ++c) sig[c * n + v] = m2 * eps[c * n + v];
   }
 }
-cudaError_t launch_stress(double* sig, const double* eps, const int8_t* phase, const PhaseTab<double>& tab,
-                          int sx, int sy, int sz, int nx, int ny, int nz, cudaStream_t s) {
-  k_stress<<<8 * 152, 256, 0, s>>>(sig, eps, phase, tab, sx, sy, sz, nx, ny, nz);
+cudaError_t launch_stress(const StressArgs& a, int batch, const PhaseTab<double>& tab, int nx, int ny, int nz,
+                          cudaStream_t s) {
+  const long long n = (long long)nx * ny * nz;
+  const int blocks = (int)std::max<long long>(1, std::min<long long>(8 * 152, (n + 255) / 256));
+  k_stress<<<dim3(blocks, batch), 256, 0, s>>>(a, tab, nx, ny, nz);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -658,8 +678,7 @@ cudaError_t launch_stress(double* sig, const double* eps, const int8_t* phase, c
                                           cudaStream_t);                                          \
   template cudaError_t launch_body_force_blocks<R>(R*, int, int, int, double, double, double,      \
                                                    double, int, double*, cudaStream_t);           \
-  template cudaError_t launch_validate<R>(const int8_t*, const R*, long long, int*, double*,       \
-                                          double*, cudaStream_t);                                 \
+  template cudaError_t launch_validate<R>(const ValArgs<R>&, int, long long, int*, double*, double*, cudaStream_t);                                 \
   template cudaError_t launch_bden<R>(const C2<R>*, const Geo&, ResidSlot*, IterState*,            \
                                       cudaStream_t, int, long long);                              \
   template cudaError_t launch_accumulate<R>(double*, int*, const R*, const R*, const R*,           \

@@ -98,7 +98,8 @@ struct ResidArgs {
   double* hist;
   int hist_cap;
   double tol, lam0, mu0, n;
-  int maxdim, mode, stall_window, check_max, maxit;
+  double ximin;           // 2 pi / max N_a
+  int mode, stall_window, check_max, maxit;
   unsigned long long* io;
 };
 
@@ -114,8 +115,8 @@ template <typename R> struct CArgs {
   int variant;            // FP32 only: column tile and factor order (kColVariants; 0 = default)
   const void* tmap;       // host array of the two tensor maps (8, 16 columns) of a y pass over 6-component spectra, or null
   const void* tmap_data;  // the buffer the maps address: the tensor-copy tiles run only when data is this buffer
-  // inverse passes: 1 adds one block row whose first block runs the sweep's residual step;
-  // members are then skipped by IterState.seen (set by the Green pass), since the step may
+  // inverse passes: 1 adds one block row whose blocks of the first member run the sweep's
+  // residual steps (scheduled first; a member each); members are then skipped by IterState.seen (set by the Green pass), since the step may
   // set `done` while other blocks of the pass have not started
   int with_resid;
   int chain;              // see launch_chain
@@ -349,12 +350,17 @@ cudaError_t launch_body_force_blocks(R* b, int nx, int ny, int nz, double cx, do
                                      double a, int blocks, double* scratch /* >= blocks + 1 doubles */,
                                      cudaStream_t s);
 
-// validation: phase id range and body-force sums; out[0..1] = min/max phase,
-// dout[0..2] = sum b_c, dout[3..5] = sum |b_c|
+// Phase-id range and load sums of `batch` members (phase maps and loads in va), member m:
+// iout[2 m] = min, iout[2 m + 1] = max; dout[6 m + c] = sum b_c, dout[6 m + 3 + c] =
+// sum |b_c|; scratch: validate_scratch() doubles a member
+template <typename R> struct ValArgs {
+  const int8_t* phase[kMaxBatch];
+  const R* b[kMaxBatch];
+};
 template <typename R>
-cudaError_t launch_validate(const int8_t* phase, const R* b, long long n, int* iout, double* dout,
-                            double* scratch, cudaStream_t s);
-int validate_scratch(long long n);
+cudaError_t launch_validate(const ValArgs<R>& va, int batch, long long n, int* iout, double* dout, double* scratch,
+                            cudaStream_t s);
+int validate_scratch();
 
 // sum over modes with xi != 0 of w |b_hat|^2 -> st->bden = sqrt(sum); batched:
 // member m uses bhat + m * b_ms, part + m * 512 and st + m
@@ -367,14 +373,24 @@ cudaError_t launch_resid_final(const ResidArgs& a, int batch, cudaStream_t s);
 
 // elementwise helpers (k_misc.cu)
 cudaError_t launch_cast_d2f(float* dst, const double* src, long long count, cudaStream_t s);
-cudaError_t launch_cast_f2d(double* dst, const float* src, long long count, cudaStream_t s);
-cudaError_t launch_add_f2d(double* dst, const float* src, long long count, cudaStream_t s);
+// dst[m] = src[m] (add: +=) over count values, FP32 into FP64, for `batch` pairs
+struct F2dArgs {
+  double* dst[kMaxBatch];
+  const float* src[kMaxBatch];
+};
+cudaError_t launch_f2d(const F2dArgs& a, int batch, long long count, bool add, cudaStream_t s);
 // complex128 -> complex64 copy of ncomp spectral components (same geometry)
 cudaError_t launch_cast_spec(C2<float>* dst, const C2<double>* src, const Geo& g, int ncomp, cudaStream_t s);
 cudaError_t launch_cast_spec_ff(C2<float>* dst, const C2<ff>* src, const Geo& g, int ncomp, cudaStream_t s);
 // sigma = L(x) eps pointwise (FP64), phase translated by (sx, sy, sz)
-cudaError_t launch_stress(double* sig, const double* eps, const int8_t* phase, const PhaseTab<double>& tab,
-                          int sx, int sy, int sz, int nx, int ny, int nz, cudaStream_t s);
+struct StressArgs {
+  double* sig[kMaxBatch];
+  const double* eps[kMaxBatch];
+  const int8_t* phase[kMaxBatch];
+  int sx[kMaxBatch], sy[kMaxBatch], sz[kMaxBatch];
+};
+cudaError_t launch_stress(const StressArgs& a, int batch, const PhaseTab<double>& tab, int nx, int ny, int nz,
+                          cudaStream_t s);
 
 template <typename R>
 cudaError_t launch_accumulate(double* acc, int* hits, const R* eps, const R* sig, const R* u,

@@ -13,62 +13,69 @@ namespace bfcs {
 // Member m's step; all threads of a block (at least one warp; threads past the last whole
 // warp add nothing).  Sums the Green pass's partials in a fixed order for the block size.  r = sqrt(sum) / D, D = ||b_hat|| +
 // xi_min |sigma_hat(0)|_F with sigma_hat(0) = N C0 E + tau_hat(0) and xi_min = 2 pi / max N_a.
+//
+// The step is one chain of latencies (an FP64 add takes 64 clocks, a square root or a
+// division 600), and a small grid's y pass is no longer than it: the partials are
+// requested before anything else is looked at, the normaliser and its reciprocal are
+// formed by another warp beside the sum, and the warps' sums are added by shuffles.
 static __device__ __noinline__ void resid_step(const ResidArgs& a, int m) {
   __shared__ double red[32];
-  __shared__ double den_s;
-  __shared__ int no_check;   // decided by one thread: thread 0 advances st->iters below
+  __shared__ double den_s, iden_s;
   IterState* st = a.sts + m;
-  if (a.mode == GM_SWEEP && st->seen) return;   // (written by the Green pass: the block's threads agree)
-  if (threadIdx.x == 0) {
-    const int sw = st->iters, nc = st->next_check;
-    no_check = a.mode == GM_SWEEP && a.check_max > 1 && sw != nc;
-    if (a.io != nullptr && a.mode == GM_SWEEP) {
-      // what the Green pass of this sweep moved besides its fixed traffic: d_prev read, d written
-      const bool rd = a.check_max <= 1 || sw == nc;
-      const bool wr = a.check_max <= 1 || rd || sw + 1 == nc || sw + 1 >= a.maxit;
-      atomicAdd(a.io, (unsigned long long)rd);
-      atomicAdd(a.io + 1, (unsigned long long)wr);
-    }
+  const ResidSlot* part = a.part + (long long)m * a.nparts;
+  const int tid = threadIdx.x, nthr = blockDim.x & ~31, nw = nthr >> 5;
+  const bool sweep_mode = a.mode == GM_SWEEP;
+  const int seen = sweep_mode ? st->seen : 0;   // (written by the Green pass: the block's threads agree)
+  const int sweep = st->iters, nc = st->next_check;
+  double acc = 0.0;
+  if (tid < nthr) {
+#pragma unroll 4
+    for (int i = tid; i < a.nparts; i += nthr) acc += part[i].num;
   }
-  __syncthreads();
+  if (seen) return;
+  if (tid == 0 && sweep_mode && a.io != nullptr) {
+    // what the Green pass of this sweep moved besides its fixed traffic: d_prev read, d written
+    const bool rd = a.check_max <= 1 || sweep == nc;
+    const bool wr = a.check_max <= 1 || rd || sweep + 1 == nc || sweep + 1 >= a.maxit;
+    atomicAdd(a.io, (unsigned long long)rd);
+    atomicAdd(a.io + 1, (unsigned long long)wr);
+  }
+  const bool no_check = sweep_mode && a.check_max > 1 && sweep != nc;
   if (no_check) {
     // no residual on this sweep (the Green pass wrote no partials)
-    if (threadIdx.x == 0) {
-      const int sweep = st->iters;
+    __syncthreads();         // every thread has read the counters
+    if (tid == 0) {
       if (sweep < a.hist_cap && a.hist != nullptr) a.hist[(long long)m * a.hist_cap + sweep] = NAN;
       st->iters = sweep + 1;
     }
     return;
   }
-  const int nthr = blockDim.x & ~31, nw = nthr >> 5;
-  if (threadIdx.x == (nw > 1 ? 32 : 0)) {   // the normaliser, beside the sum
+  if (tid == (nw > 1 ? nthr - 32 : 0)) {   // the normaliser, beside the sum
     const double* E = a.mem[m].E;
     const double trE = E[0] + E[1] + E[2];
     double s0[6];
     for (int c = 0; c < 6; ++c)
       s0[c] = a.n * (2.0 * a.mu0 * E[c] + (c < 3 ? a.lam0 * trE : 0.0)) + st->tau0[c];
-    const double s0n = sqrt(s0[0] * s0[0] + s0[1] * s0[1] + s0[2] * s0[2] +
-                            2.0 * (s0[3] * s0[3] + s0[4] * s0[4] + s0[5] * s0[5]));
-    den_s = st->bden + 6.283185307179586 / (double)a.maxdim * s0n;
+    const double s0n = sqrt((s0[0] * s0[0] + s0[1] * s0[1]) + s0[2] * s0[2] +
+                            2.0 * ((s0[3] * s0[3] + s0[4] * s0[4]) + s0[5] * s0[5]));
+    const double den = st->bden + a.ximin * s0n;
+    den_s = den;
+    iden_s = 1.0 / den;
   }
-  const ResidSlot* part = a.part + (long long)m * a.nparts;
-  if ((int)threadIdx.x < nthr) {
-    double acc = 0.0;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < a.nparts; i += nthr) acc += part[i].num;
+  if (tid < nthr) {
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    if ((tid & 31) == 0) red[tid >> 5] = acc;
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  double t = 0.0;
-  for (int w = 0; w < nw; ++w) t += red[w];
-  const double den = den_s;
+  if (tid >= 32) return;
+  double t = tid < nw ? red[tid] : 0.0;
+  for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+  if (tid != 0) return;
   const int warm = a.mem[m].warm;
   const double tol = a.mem[m].tol >= 0.0 ? a.mem[m].tol : a.tol;
-  double r = den > 0.0 ? sqrt(t) / den : sqrt(t);
-  if (a.mode == GM_FINAL) { st->resid_final = r; return; }
-  const int sweep = st->iters;
+  double r = sqrt(t);
+  if (den_s > 0.0) r *= iden_s;
+  if (!sweep_mode) { st->resid_final = r; return; }
   const bool skip_check = warm && sweep == 0;
   if (skip_check) r = INFINITY;
   if (sweep < a.hist_cap && a.hist != nullptr) a.hist[(long long)m * a.hist_cap + sweep] = r;

@@ -349,9 +349,12 @@ int check_material(int nph, const bfcs_lame* phases, bfcs_lame C0) {
 // whose phase maps and loads are given in the host arrays.
 template <typename R>
 int validate_members(bfcs_plan P, int B, const int8_t* const* phase, const void* const* b, int nph) {
-  for (int m = 0; m < B; ++m)
-    CK(launch_validate<R>(phase[m], (const R*)b[m], P->g.n, P->ival + 2 * m, P->dval + 6 * m, P->dscratch,
-                          P->st));
+  ValArgs<R> va{};
+  for (int m = 0; m < B; ++m) {
+    va.phase[m] = phase[m];
+    va.b[m] = (const R*)b[m];
+  }
+  CK(launch_validate<R>(va, B, P->g.n, P->ival, P->dval, P->dscratch, P->st));
   CK(read_small(P->ival_host, P->ival, 2 * B * sizeof(int), P->st));
   CK(read_small(P->dval_host, P->dval, 6 * B * sizeof(double), P->st));
   const int w = sync_stream(P);
@@ -561,7 +564,7 @@ struct SweepSet {
     r.lam0 = C0.lambda;
     r.mu0 = C0.mu;
     r.n = (double)P->g.n;
-    r.maxdim = maxdim;
+    r.ximin = 6.283185307179586 / (double)maxdim;
     r.mode = mode;
     r.stall_window = P->stall_window;
     r.check_max = P->resid_max;
@@ -1627,11 +1630,14 @@ int solve_mixed_batch(bfcs_plan P, int B, const Member* in, int nph, const bfcs_
   const int s1 = run_batch<float>(P, B, tab32, C0, in[0].E, std::max(tol, P->switch_tol), maxit, inf.data(),
                                   any_warm, true);
   if (s1 < 0) return s1;
+  F2dArgs fa{};
   for (int m = 0; m < B; ++m) {
     sweeps[m] += inf[m].iters;
     r_last[m] = inf[m].resid;
-    CK(launch_cast_f2d(u64[m], u32(m), 3 * n, st));
+    fa.dst[m] = u64[m];
+    fa.src[m] = u32(m);
   }
+  CK(launch_f2d(fa, B, 3 * n, false, st));
 
   for (int round = 0;; ++round) {
     std::vector<int> act;
@@ -1683,18 +1689,29 @@ int solve_mixed_batch(bfcs_plan P, int B, const Member* in, int nph, const bfcs_
     if (e != BFCS_OK) return e;
     const int s2 = run_batch<float>(P, k, tab32, C0, zeroE, 0.5, std::max(left, 1), inf.data(), false, true);
     if (s2 < 0) return s2;
+    F2dArgs fe{};
     for (int j = 0; j < k; ++j) {
       const int m = next[j];
       sweeps[m] += inf[j].iters;
       stalled[m] = inf[j].stalled;
-      CK(launch_add_f2d(u64[m], u32(j), 3 * n, st));
-      if (inc_eps) CK(launch_add_f2d((double*)in[m].eps_out, eps32(j), 6 * n, st));
+      fa.dst[j] = u64[m];
+      fa.src[j] = u32(j);
+      fe.dst[j] = (double*)in[m].eps_out;
+      fe.src[j] = eps32(j);
     }
+    CK(launch_f2d(fa, k, 3 * n, true, st));
+    if (inc_eps) CK(launch_f2d(fe, k, 6 * n, true, st));
   }
-  for (int m = 0; m < B; ++m)
-    if (in[m].sig_out != nullptr)
-      CK(launch_stress((double*)in[m].sig_out, (const double*)in[m].eps_out, in[m].phase, tab64, in[m].sx,
-                       in[m].sy, in[m].sz, g.nx, g.ny, g.nz, st));
+  StressArgs sa{};
+  bool any_sig = false;
+  for (int m = 0; m < B; ++m) {
+    sa.sig[m] = (double*)in[m].sig_out;
+    sa.eps[m] = (const double*)in[m].eps_out;
+    sa.phase[m] = in[m].phase;
+    sa.sx[m] = in[m].sx; sa.sy[m] = in[m].sy; sa.sz[m] = in[m].sz;
+    any_sig = any_sig || in[m].sig_out != nullptr;
+  }
+  if (any_sig) CK(launch_stress(sa, B, tab64, g.nx, g.ny, g.nz, st));
   const int w = sync_stream(P);
   if (w != BFCS_OK) return w;
   P->last_iters = 0;     // history of the FP32 phases is not kept across rounds
@@ -1978,8 +1995,8 @@ int bfcs_plan_create(bfcs_plan* out, int nx, int ny, int nz, int max_batch, int 
        cudaMallocHost(&P->mem_host, MB * sizeof(Member)) == cudaSuccess &&
        cudaMalloc(&P->ival, MB * 2 * sizeof(int)) == cudaSuccess &&
        cudaMalloc(&P->dval, MB * 6 * sizeof(double)) == cudaSuccess &&
-       cudaMalloc(&P->dscratch, std::max(validate_scratch(P->g.n), body_force_scratch(P->g.n)) *
-                                    sizeof(double)) == cudaSuccess &&
+       cudaMalloc(&P->dscratch, std::max<size_t>(MB * validate_scratch(), body_force_scratch(P->g.n)) *
+                                     sizeof(double)) == cudaSuccess &&
        cudaMallocHost(&P->ist_host, 3 * MB * sizeof(IterState)) == cudaSuccess &&
        cudaMallocHost(&P->ival_host, MB * 2 * sizeof(int)) == cudaSuccess &&
        cudaMallocHost(&P->dval_host, MB * 6 * sizeof(double)) == cudaSuccess;
