@@ -1,5 +1,5 @@
 // Shared device building blocks of the BFCS solver: complex arithmetic,
-// register-resident small DFTs and the shared-memory four-step line FFT.
+// register-resident small DFTs and the steps of the four-step line FFT.
 //
 // Transform convention (Eqs. 4.3-4.5 of the paper): forward uses
 // omega^{-kn} = exp(-2 pi i kn/N), inverse exp(+2 pi i kn/N); the 1/|N| of the
@@ -130,6 +130,35 @@ template <typename R, int DIR> __device__ __forceinline__ C2<R> mul_di(C2<R> a) 
   return DIR > 0 ? mk<R>(-a.y, a.x) : mk<R>(a.y, -a.x);
 }
 
+// Complex sum and difference of the register butterflies.  FP32 with P (packed): both
+// parts in one instruction, with the same roundings; the passes along lines are short of
+// issue slots.  Cold, per launch: y pass of 256^3 117 -> 103 us, x pass 166 -> 160 us, of
+// 16 members of 64^3 52.9 -> 51.9 us, z pass 75.9 -> 74.8 us; the z pass of 256 lines took
+// 308 us instead of 298 and stays with single instructions (kPackZ).
+template <typename R, bool P> __device__ __forceinline__ C2<R> badd(C2<R> a, C2<R> b) {
+  if constexpr (P && std::is_same<R, float>::value) {
+    C2<R> r;
+    asm("{\n.reg .b64 p, q;\nmov.b64 p, {%2, %3};\nmov.b64 q, {%4, %5};\nadd.rn.f32x2 p, p, q;\nmov.b64 {%0, %1}, p;\n}\n"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+  } else {
+    return a + b;
+  }
+}
+template <typename R, bool P> __device__ __forceinline__ C2<R> bsub(C2<R> a, C2<R> b) {
+  if constexpr (P && std::is_same<R, float>::value) {
+    C2<R> r;
+    asm("{\n.reg .b64 p, q;\nmov.b64 p, {%2, %3};\nmov.b64 q, {%4, %5};\nsub.rn.f32x2 p, p, q;\nmov.b64 {%0, %1}, p;\n}\n"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+  } else {
+    return a - b;
+  }
+}
+constexpr bool kPackZ(int L) { return L <= 128; }
+
 // |z|^2 accumulated in FP64 (float-float: from the leading parts, which carry
 // the 24 bits a norm needs)
 template <typename R> __device__ __forceinline__ double norm2(C2<R> z) {
@@ -163,18 +192,18 @@ __host__ __device__ constexpr double sin48(int j) { return cos48(j - 12); }
 
 // ------------------------------------------------------------------ register DFTs
 // X[k] = sum_n x[n] exp(DIR 2 pi i n k / RADIX), in place, natural order.
-template <typename R, int RADIX, int DIR> struct Dft;
+template <typename R, int RADIX, int DIR, bool P = true> struct Dft;
 
-template <typename R, int DIR> struct Dft<R, 1, DIR> {
+template <typename R, int DIR, bool P> struct Dft<R, 1, DIR, P> {
   static __device__ __forceinline__ void run(C2<R>*) {}
 };
-template <typename R, int DIR> struct Dft<R, 2, DIR> {
+template <typename R, int DIR, bool P> struct Dft<R, 2, DIR, P> {
   static __device__ __forceinline__ void run(C2<R>* x) {
     C2<R> a = x[0], b = x[1];
-    x[0] = a + b; x[1] = a - b;
+    x[0] = badd<R, P>(a, b); x[1] = bsub<R, P>(a, b);
   }
 };
-template <typename R, int DIR> struct Dft<R, 3, DIR> {
+template <typename R, int DIR, bool P> struct Dft<R, 3, DIR, P> {
   static __device__ __forceinline__ void run(C2<R>* x) {
     const R h = R(0.8660254037844386);   // sin(2 pi / 3)
     C2<R> t1 = x[1] + x[2];
@@ -183,11 +212,11 @@ template <typename R, int DIR> struct Dft<R, 3, DIR> {
     x[0] = x[0] + t1; x[1] = t2 + t3; x[2] = t2 - t3;
   }
 };
-template <typename R, int DIR> struct Dft<R, 4, DIR> {
+template <typename R, int DIR, bool P> struct Dft<R, 4, DIR, P> {
   static __device__ __forceinline__ void run(C2<R>* x) {
-    C2<R> a = x[0] + x[2], b = x[0] - x[2], c = x[1] + x[3];
-    C2<R> d = mul_di<R, DIR>(x[1] - x[3]);
-    x[0] = a + c; x[2] = a - c; x[1] = b + d; x[3] = b - d;
+    C2<R> a = badd<R, P>(x[0], x[2]), b = bsub<R, P>(x[0], x[2]), c = badd<R, P>(x[1], x[3]);
+    C2<R> d = mul_di<R, DIR>(bsub<R, P>(x[1], x[3]));
+    x[0] = badd<R, P>(a, c); x[2] = bsub<R, P>(a, c); x[1] = badd<R, P>(b, d); x[3] = bsub<R, P>(b, d);
   }
 };
 
@@ -199,7 +228,7 @@ template <> struct Split<8> { static constexpr int A = 4, B = 2; };
 template <> struct Split<12> { static constexpr int A = 4, B = 3; };
 template <> struct Split<16> { static constexpr int A = 4, B = 4; };
 
-template <typename R, int RADIX, int DIR> struct Dft {
+template <typename R, int RADIX, int DIR, bool P> struct Dft {
   static __device__ __forceinline__ void run(C2<R>* x) {
     constexpr int A = Split<RADIX>::A, B = Split<RADIX>::B;
     C2<R> u[B][A];
@@ -207,7 +236,7 @@ template <typename R, int RADIX, int DIR> struct Dft {
     for (int n2 = 0; n2 < B; ++n2) {
 #pragma unroll
       for (int n1 = 0; n1 < A; ++n1) u[n2][n1] = x[B * n1 + n2];
-      Dft<R, A, DIR>::run(u[n2]);
+      Dft<R, A, DIR, P>::run(u[n2]);
 #pragma unroll
       for (int k1 = 1; k1 < A; ++k1) {
         if (n2 * k1 == 0) continue;
@@ -229,7 +258,7 @@ template <typename R, int RADIX, int DIR> struct Dft {
       C2<R> v[B];
 #pragma unroll
       for (int n2 = 0; n2 < B; ++n2) v[n2] = u[n2][k1];
-      Dft<R, B, DIR>::run(v);
+      Dft<R, B, DIR, P>::run(v);
 #pragma unroll
       for (int k2 = 0; k2 < B; ++k2) x[k1 + A * k2] = v[k2];
     }
@@ -275,67 +304,15 @@ template <int L, int R1> constexpr int tw_offset() {
   return L + (R1 == Fac<L>::R1 ? 0 : tw_block(L, Fac<L>::R1));
 }
 
-// Shared-memory four-step FFT over NCOL independent lines of length L stored
-// column-wise: element n of line f at s[n * NCOL + f].  Needs at least
-// NCOL * RMAX threads (one task per thread per stage so it can run in place);
-// extra threads idle.  tw[j] = exp(-2 pi i j / L) (forward sign).
-// Stage 1 (thread (f, n2)): DFT_R1 over n1 of x[R2 n1 + n2], twiddle W_L^{n2 k1}.
-// Stage 2 (thread (f, k1)): DFT_R2 over n2, output X[k1 + R1 k2].
-// Begins and ends with __syncthreads().
-template <typename R, int L, int DIR>
-__device__ __forceinline__ void fft_cols(C2<R>* s, int ncol, const C2<R>* __restrict__ tw) {
-  constexpr int R1 = LineInfo<L>::R1, R2 = LineInfo<L>::R2;
-  const int tid = threadIdx.x;
-  __syncthreads();
-  {
-    const int f = tid % ncol, n2 = tid / ncol;
-    const bool act = n2 < R2;
-    C2<R> x[R1];
-    if (act) {
-#pragma unroll
-      for (int n1 = 0; n1 < R1; ++n1) x[n1] = s[(R2 * n1 + n2) * ncol + f];
-      Dft<R, R1, DIR>::run(x);
-#pragma unroll
-      for (int k1 = 1; k1 < R1; ++k1) {
-        C2<R> w = tw[(n2 * k1) % L];
-        if (DIR > 0) w.y = -w.y;
-        x[k1] = cmul(x[k1], w);
-      }
-    }
-    __syncthreads();
-    if (act) {
-#pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) s[(n2 * R1 + k1) * ncol + f] = x[k1];
-    }
-  }
-  __syncthreads();
-  {
-    const int f = tid % ncol, k1 = tid / ncol;
-    const bool act = k1 < R1;
-    C2<R> y[R2];
-    if (act) {
-#pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) y[n2] = s[(n2 * R1 + k1) * ncol + f];
-      Dft<R, R2, DIR>::run(y);
-    }
-    __syncthreads();
-    if (act) {
-#pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2) s[(k1 + R1 * k2) * ncol + f] = y[k2];
-    }
-  }
-  __syncthreads();
-}
-
-// Register-staged pieces of the same four-step FFT.  A thread holding the R1
+// Four-step FFT of a line, L = R1 R2, in register-staged pieces.  A thread holding the R1
 // inputs x[R2 n1 + n2] (n1 = 0..R1-1) of one line runs stage1(); after the
 // exchange through shared memory a thread holding the R2 values Y[n2][k1]
 // (n2 = 0..R2-1) runs stage2() and owns the outputs X[k1 + R1 k2].
 // stage1f / stage2f take the factor R1 explicitly (L = R1 * (L / R1), either
 // order of the two radices); stage1 / stage2 use the default order of Fac<L>.
-template <typename R, int L, int R1, int DIR>
+template <typename R, int L, int R1, int DIR, bool P = true>
 __device__ __forceinline__ void stage1f(C2<R>* x, int n2, const C2<R>* __restrict__ tw) {
-  Dft<R, R1, DIR>::run(x);
+  Dft<R, R1, DIR, P>::run(x);
   if constexpr (R1 % 4 == 0 && R1 >= 8 && sizeof(R) == 4) {
     // FP32 (FP64 is bound by its arithmetic pipe, not by the table's loads, and takes the
     // entries as they are): W^(n2 k1) with k1 = 4 a + b as W^(4 n2 a) W^(n2 b): R1/4 - 1 + 3 table loads
@@ -381,7 +358,7 @@ __device__ __forceinline__ void stage1f(C2<R>* x, int n2, const C2<R>* __restric
 // four-step rule: with k = k1 + R1 k2 and n = R2 n1 + n2, a first in-place step
 // Y[k1][n2] = DFT_R2 over k2 of X[k1 + R1 k2] (rows k1 + R1 m read and written),
 // then for each n2 this step on Y[k1][n2] (k1 = 0..R1-1) gives x[R2 n1 + n2].
-template <typename R, int L, int R1, int DIR>
+template <typename R, int L, int R1, int DIR, bool P = true>
 __device__ __forceinline__ void twiddle_then_dft(C2<R>* x, int n2, const C2<R>* __restrict__ tw) {
   if constexpr (R1 % 4 == 0 && R1 >= 8 && sizeof(R) == 4) {
     constexpr int A = R1 / 4, N2 = L / R1;
@@ -406,20 +383,20 @@ __device__ __forceinline__ void twiddle_then_dft(C2<R>* x, int n2, const C2<R>* 
       x[k1] = cmul(x[k1], w);
     }
   }
-  Dft<R, R1, DIR>::run(x);
+  Dft<R, R1, DIR, P>::run(x);
 }
 
-template <typename R, int R2, int DIR>
+template <typename R, int R2, int DIR, bool P = true>
 __device__ __forceinline__ void stage2f(C2<R>* y) {
-  Dft<R, R2, DIR>::run(y);
+  Dft<R, R2, DIR, P>::run(y);
 }
-template <typename R, int L, int DIR>
+template <typename R, int L, int DIR, bool P = true>
 __device__ __forceinline__ void stage1(C2<R>* x, int n2, const C2<R>* __restrict__ tw) {
-  stage1f<R, L, LineInfo<L>::R1, DIR>(x, n2, tw);
+  stage1f<R, L, LineInfo<L>::R1, DIR, P>(x, n2, tw);
 }
-template <typename R, int L, int DIR>
+template <typename R, int L, int DIR, bool P = true>
 __device__ __forceinline__ void stage2(C2<R>* y) {
-  stage2f<R, LineInfo<L>::R2, DIR>(y);
+  stage2f<R, LineInfo<L>::R2, DIR, P>(y);
 }
 
 // ------------------------------------------------------------------ chained launches

@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(ZCfg<L>::BLOCK) k_zcd(CdArgs<R> a) {
       C2<R> x[R1];
 #pragma unroll
       for (int n1 = 0; n1 < R1; ++n1) x[n1] = cvalid ? gcol[(R2 * n1 + j) * zs] : mk<R>(0, 0);
-      stage1<R, L, -1>(x, j, a.tw);
+      stage1<R, L, -1, kPackZ(L)>(x, j, a.tw);
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) sm[(j * R1 + k1) * NCOL + cd_slot(j * R1 + k1, c)] = x[k1];
     }
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(ZCfg<L>::BLOCK) k_zcd(CdArgs<R> a) {
       C2<R> y[R2];
 #pragma unroll
       for (int n2 = 0; n2 < R2; ++n2) y[n2] = sm[(n2 * R1 + j) * NCOL + cd_slot(n2 * R1 + j, c)];
-      stage2<R, L, -1>(y);
+      stage2<R, L, -1, kPackZ(L)>(y);
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) sm[(j + R1 * k2) * NCOL + cd_slot(j + R1 * k2, c)] = y[k2];
     }
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(ZCfg<L>::BLOCK) k_zcd(CdArgs<R> a) {
     C2<R> y[R2];
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) y[k2] = sm[(j + R1 * k2) * NCOL + cd_slot(j + R1 * k2, c)];
-    Dft<R, R2, +1>::run(y);
+    Dft<R, R2, +1, kPackZ(L)>::run(y);
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) sm[(j + R1 * n2) * NCOL + cd_slot(j + R1 * n2, c)] = y[n2];
   }
@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(ZCfg<L>::BLOCK) k_zcd(CdArgs<R> a) {
     C2<R> x[R1];
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) x[k1] = sm[(j * R1 + k1) * NCOL + cd_slot(j * R1 + k1, c)];
-    twiddle_then_dft<R, L, R1, +1>(x, j, a.tw);
+    twiddle_then_dft<R, L, R1, +1, kPackZ(L)>(x, j, a.tw);
     if (col0 + (c % T) < g.mx) {
       C2<R>* gcol = column(c);
 #pragma unroll

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(GCfg<L, T>::BLOCK, green_min_blocks<R, L>()) k
       C2<R> x[R1];
 #pragma unroll
       for (int n1 = 0; n1 < R1; ++n1) x[n1] = cvalid ? gcol[(R2 * n1 + j) * zs] : mk<R>(0, 0);
-      stage1<R, L, -1>(x, j, a.tw);
+      stage1<R, L, -1, kPackZ(L)>(x, j, a.tw);
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) s[(j * R1 + k1) * NCOL + gslot<T>(j * R1 + k1, c)] = x[k1];
     }
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(GCfg<L, T>::BLOCK, green_min_blocks<R, L>()) k
       C2<R> y[R2];
 #pragma unroll
       for (int n2 = 0; n2 < R2; ++n2) y[n2] = s[(n2 * R1 + j) * NCOL + gslot<T>(n2 * R1 + j, c)];
-      stage2<R, L, -1>(y);
+      stage2<R, L, -1, kPackZ(L)>(y);
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) s[(j + R1 * k2) * NCOL + gslot<T>(j + R1 * k2, c)] = y[k2];
     }
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(GCfg<L, T>::BLOCK, green_min_blocks<R, L>()) k
     C2<R> y[R2];
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) y[k2] = s[(j + R1 * k2) * NCOL + gslot<T>(j + R1 * k2, c)];
-    Dft<R, R2, +1>::run(y);
+    Dft<R, R2, +1, kPackZ(L)>::run(y);
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) s[(j + R1 * n2) * NCOL + gslot<T>(j + R1 * n2, c)] = y[n2];
   }
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(GCfg<L, T>::BLOCK, green_min_blocks<R, L>()) k
     C2<R> x[R1];
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) x[k1] = s[(j * R1 + k1) * NCOL + gslot<T>(j * R1 + k1, c)];
-    twiddle_then_dft<R, L, R1, +1>(x, j, a.tw);
+    twiddle_then_dft<R, L, R1, +1, kPackZ(L)>(x, j, a.tw);
     if (keep) {
       C2<R>* gcol = column(c);
 #pragma unroll
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
       if (j < R2) {
 #pragma unroll
         for (int n1 = 0; n1 < R1; ++n1) x[n1] = s[(R2 * n1 + j) * NCOL + gslot<T>(R2 * n1 + j, c)];
-        stage1<R, L, -1>(x, j, a.tw);
+        stage1<R, L, -1, kPackZ(L)>(x, j, a.tw);
       }
       __syncthreads();
       if (j < R2) {
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
       if (j < R1) {
 #pragma unroll
         for (int n2 = 0; n2 < R2; ++n2) y[n2] = s[(n2 * R1 + j) * NCOL + gslot<T>(n2 * R1 + j, c)];
-        stage2<R, L, -1>(y);
+        stage2<R, L, -1, kPackZ(L)>(y);
       }
       __syncthreads();
       if (j < R1) {
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
       C2<R> y[R2];
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) y[k2] = s[(j + R1 * k2) * NCOL + gslot<T>(j + R1 * k2, c)];
-      Dft<R, R2, +1>::run(y);
+      Dft<R, R2, +1, kPackZ(L)>::run(y);
 #pragma unroll
       for (int n2 = 0; n2 < R2; ++n2) s[(j + R1 * n2) * NCOL + gslot<T>(j + R1 * n2, c)] = y[n2];
     }
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
       C2<R> x[R1];
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) x[k1] = s[(j * R1 + k1) * NCOL + gslot<T>(j * R1 + k1, c)];
-      twiddle_then_dft<R, L, R1, +1>(x, j, a.tw);
+      twiddle_then_dft<R, L, R1, +1, kPackZ(L)>(x, j, a.tw);
       const int kx = col0 + ccol;
       if (kx < a.g.mx) {
         C2<R>* gcol = a.spec + m * a.spec_ms + ccomp * cs + (long long)ky * p + kx;

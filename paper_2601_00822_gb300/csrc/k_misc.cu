@@ -404,41 +404,63 @@ bool col_variant_valid(int v, int n) {
 
 // ---------------------------------------------------------------- a10: translated averaging
 // acc layout (30 x N, FP64): <u> 3, <u>^(1) 3, <eps> 6, <eps>^(1) 6, <sigma> 6, <sigma>^(1) 6.
+// Members are added in order, each voxel by one thread: the sums stay in registers over
+// the members of a launch (a launch per member read and wrote all 30 sums each time).
 template <typename R>
-__global__ void k_accumulate(double* acc, int* hits, const R* eps, const R* sig, const R* u,
-                             const int8_t* phase, int sx, int sy, int sz, int nx, int ny, int nz) {
+__global__ void k_accumulate(double* acc, int* hits, const __grid_constant__ AccArgs<R> a, int batch, int nx, int ny,
+                             int nz) {
   const long long n = (long long)nx * ny * nz;
   const bool small = n <= 0xFFFFFFFFLL;
-  // shifts reduced to [0, n) once: the per-voxel translation is then one compare
-  const int sxr = ((sx % nx) + nx) % nx, syr = ((sy % ny) + ny) % ny, szr = ((sz % nz) + nz) % nz;
+  // blockIdx.y: 0 the displacement (3 + 3 sums and the hits), 1 and 2 the strain, 3 and 4
+  // the stress, three components each (6 + 6 sums of registers)
+  const int part = blockIdx.y;
+  const int field0 = part == 0 ? 12 : part <= 2 ? (part - 1) * 3 : 6 + (part - 3) * 3;   // in eps | sig | u
+  const int out0 = part == 0 ? 0 : part <= 2 ? 6 + (part - 1) * 3 : 18 + (part - 3) * 3;
+  const int in_off = part == 0 ? 3 : 6;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n;
        v += (long long)gridDim.x * blockDim.x) {
     int x, y, z;
     lin_xyz(v, nx, ny, small, x, y, z);
-    int xs = x - sxr; if (xs < 0) xs += nx;
-    int ys = y - syr; if (ys < 0) ys += ny;
-    int zs = z - szr; if (zs < 0) zs += nz;
-    const bool in = phase[((long long)zs * ny + ys) * nx + xs] != 0;
+    double s[3], si[3];
+    int h = part == 0 ? hits[v] : 0;
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const double val = (double)u[c * n + v];
-      acc[c * n + v] += val;
-      if (in) acc[(3 + c) * n + v] += val;
+      s[c] = acc[(out0 + c) * n + v];
+      si[c] = acc[(out0 + in_off + c) * n + v];
     }
-    for (int c = 0; c < 6; ++c) {
-      const double e = (double)eps[c * n + v], sg = (double)sig[c * n + v];
-      acc[(6 + c) * n + v] += e;
-      acc[(18 + c) * n + v] += sg;
-      if (in) { acc[(12 + c) * n + v] += e; acc[(24 + c) * n + v] += sg; }
+    for (int m = 0; m < batch; ++m) {
+      int xs = x - a.sx[m]; if (xs < 0) xs += nx;
+      int ys = y - a.sy[m]; if (ys < 0) ys += ny;
+      int zs = z - a.sz[m]; if (zs < 0) zs += nz;
+      const bool in = a.phase[m][((long long)zs * ny + ys) * nx + xs] != 0;
+      const R* f = a.fields[m] + (long long)field0 * n + v;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const double val = (double)f[c * n];
+        s[c] += val;
+        if (in) si[c] += val;
+      }
+      if (in) ++h;
     }
-    if (in) hits[v] += 1;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      acc[(out0 + c) * n + v] = s[c];
+      acc[(out0 + in_off + c) * n + v] = si[c];
+    }
+    if (part == 0) hits[v] = h;
   }
 }
 
 template <typename R>
-cudaError_t launch_accumulate(double* acc, int* hits, const R* eps, const R* sig, const R* u,
-                              const int8_t* phase, int sx, int sy, int sz, int nx, int ny, int nz,
+cudaError_t launch_accumulate(double* acc, int* hits, AccArgs<R> a, int batch, int nx, int ny, int nz,
                               cudaStream_t s) {
-  k_accumulate<R><<<4 * 152, 256, 0, s>>>(acc, hits, eps, sig, u, phase, sx, sy, sz, nx, ny, nz);
+  // shifts reduced to [0, n) once: the per-voxel translation is then one compare
+  for (int m = 0; m < batch; ++m) {
+    a.sx[m] = ((a.sx[m] % nx) + nx) % nx;
+    a.sy[m] = ((a.sy[m] % ny) + ny) % ny;
+    a.sz[m] = ((a.sz[m] % nz) + nz) % nz;
+  }
+  k_accumulate<R><<<dim3(2 * 152, 5), 256, 0, s>>>(acc, hits, a, batch, nx, ny, nz);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -681,9 +703,7 @@ cudaError_t launch_stress(const StressArgs& a, int batch, const PhaseTab<double>
   template cudaError_t launch_validate<R>(const ValArgs<R>&, int, long long, int*, double*, double*, cudaStream_t);                                 \
   template cudaError_t launch_bden<R>(const C2<R>*, const Geo&, ResidSlot*, IterState*,            \
                                       cudaStream_t, int, long long);                              \
-  template cudaError_t launch_accumulate<R>(double*, int*, const R*, const R*, const R*,           \
-                                            const int8_t*, int, int, int, int, int, int,          \
-                                            cudaStream_t);                                        \
+  template cudaError_t launch_accumulate<R>(double*, int*, AccArgs<R>, int, int, int, int, cudaStream_t);                                        \
   template cudaError_t launch_moduli<R>(const ModArgs<R>&, int, double*, double*, cudaStream_t);   \
   template cudaError_t launch_radial_max<R>(const R*, int, int, int, int, const int*, int,           \
                                             unsigned long long*, unsigned long long*, cudaStream_t);

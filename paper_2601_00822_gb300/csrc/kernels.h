@@ -392,9 +392,15 @@ struct StressArgs {
 cudaError_t launch_stress(const StressArgs& a, int batch, const PhaseTab<double>& tab, int nx, int ny, int nz,
                           cudaStream_t s);
 
+// adds the fields of `batch` members (each eps 6 | sig 6 | u 3 of n values at fields[m],
+// phase map phase[m] translated by (sx, sy, sz)) to the 30 sums and the hit counts
+template <typename R> struct AccArgs {
+  const R* fields[kMaxBatch];
+  const int8_t* phase[kMaxBatch];
+  int sx[kMaxBatch], sy[kMaxBatch], sz[kMaxBatch];
+};
 template <typename R>
-cudaError_t launch_accumulate(double* acc, int* hits, const R* eps, const R* sig, const R* u,
-                              const int8_t* phase, int sx, int sy, int sz, int nx, int ny, int nz,
+cudaError_t launch_accumulate(double* acc, int* hits, AccArgs<R> a, int batch, int nx, int ny, int nz,
                               cudaStream_t s);
 cudaError_t launch_scale(double* acc, long long count, double f, cudaStream_t s);
 

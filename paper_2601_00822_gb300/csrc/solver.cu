@@ -1811,11 +1811,13 @@ int average_impl(bfcs_plan P, int count, const AvgMembers& am, int nph, const bf
     const int s = run_batch<R>(P, B, tab, C0, E, tol, maxit, infos != nullptr ? infos + start : nullptr, false);
     if (s < 0) return s;
     if (severity(s) > severity(worst)) worst = s;
+    AccArgs<R> aa{};
     for (int m = 0; m < B; ++m) {
-      const R* eps = (const R*)P->tmp + (size_t)m * 15 * n;
-      CK(launch_accumulate<R>(avg, h, eps, eps + 6 * n, eps + 12 * n, mem[m].phase, mem[m].sx, mem[m].sy,
-                              mem[m].sz, P->g.nx, P->g.ny, P->g.nz, P->st));
+      aa.fields[m] = (const R*)P->tmp + (size_t)m * 15 * n;
+      aa.phase[m] = mem[m].phase;
+      aa.sx[m] = mem[m].sx; aa.sy[m] = mem[m].sy; aa.sz[m] = mem[m].sz;
     }
+    CK(launch_accumulate<R>(avg, h, aa, B, P->g.nx, P->g.ny, P->g.nz, P->st));
   }
   CK(launch_scale(avg, 30 * n, 1.0 / count, P->st));
   const int w = sync_stream(P);
@@ -1851,11 +1853,13 @@ int average_mixed(bfcs_plan P, int count, const AvgMembers& am, int nph, const b
                                     infos != nullptr ? infos + start : nullptr);
     if (s < 0) return s;
     if (severity(s) > severity(worst)) worst = s;
+    AccArgs<double> aa{};
     for (int m = 0; m < B; ++m) {
-      const double* eps = (const double*)mem[m].eps_out;
-      CK(launch_accumulate<double>(avg, h, eps, eps + 6 * n, eps + 12 * n, mem[m].phase, mem[m].sx, mem[m].sy,
-                                   mem[m].sz, P->g.nx, P->g.ny, P->g.nz, P->st));
+      aa.fields[m] = (const double*)P->tmp + (size_t)m * 15 * n;
+      aa.phase[m] = mem[m].phase;
+      aa.sx[m] = mem[m].sx; aa.sy[m] = mem[m].sy; aa.sz[m] = mem[m].sz;
     }
+    CK(launch_accumulate<double>(avg, h, aa, B, P->g.nx, P->g.ny, P->g.nz, P->st));
   }
   CK(launch_scale(avg, 30 * n, 1.0 / count, P->st));
   const int w = sync_stream(P);
