@@ -478,6 +478,8 @@ struct IterState {
   double bden;       // sqrt(sum |b_hat|^2) over modes with xi != 0
   double resid_final;
   double tau0[6];    // k = 0 mode of tau (unnormalised), current sweep
+  double tol;        // the member's tolerance, set at its start
+  int maxit;         // the loop's sweep limit, set when it starts (the last sweep stores d)
 };
 
 }  // namespace bfcs

@@ -88,17 +88,19 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
 
   // per-line translation bookkeeping of the polarization (made visible by the
   // barriers of step 1): the phase of voxel (n, y, z) is phase0(n - sx, y - sy, z - sz)
+  const int8_t* phase_map = a.mem != nullptr ? a.mem[m].phase : a.xm[m].phase;
   if (tid < LPB && (mode == XM_SWEEP || mode == XM_REALTAU || mode == XM_REALSIG || mode == XM_SWEEPSIG)) {
-    const XMember& M = a.xm[m];
     const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
+    const int msx = a.mem != nullptr ? a.mem[m].sx : a.xm[m].sx, msy = a.mem != nullptr ? a.mem[m].sy : a.xm[m].sy,
+              msz = a.mem != nullptr ? a.mem[m].sz : a.xm[m].sz;
     const long long ln = line0 + tid;
     if (ln < lines) {
-      int y = (int)(ln % ny) - ((M.sy % ny) + ny) % ny, z = (int)(ln / ny) - ((M.sz % nz) + nz) % nz;
+      int y = (int)(ln % ny) - ((msy % ny) + ny) % ny, z = (int)(ln / ny) - ((msz % nz) + nz) % nz;
       if (y < 0) y += ny;
       if (z < 0) z += nz;
       prow_s[tid] = (z * ny + y) * nx;
     }
-    if (tid == 0) sx_s = ((M.sx % nx) + nx) % nx;
+    if (tid == 0) sx_s = ((msx % nx) + nx) % nx;
   }
   // the block's phase-map rows (untranslated in x) stream into shared memory during
   // the inverse transform, so the polarization does not wait on one load per voxel
@@ -106,19 +108,19 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
   __shared__ __align__(16) int8_t ph_s[kPhaseStaged ? LPB : 1][kPhaseStaged ? L : 16];
   const bool polar = mode == XM_SWEEP || mode == XM_REALTAU || mode == XM_REALSIG || mode == XM_SWEEPSIG;
   // 16-byte copies need a 16-byte aligned map (a caller may pass an offset view: then direct loads)
-  const bool staged = kPhaseStaged && polar && ((reinterpret_cast<uintptr_t>(a.xm[m].phase) & 15u) == 0);
+  const bool staged = kPhaseStaged && polar && ((reinterpret_cast<uintptr_t>(phase_map) & 15u) == 0);
   if (staged) {
-    const XMember& M = a.xm[m];
+    const int msy = a.mem != nullptr ? a.mem[m].sy : a.xm[m].sy, msz = a.mem != nullptr ? a.mem[m].sz : a.xm[m].sz;
     const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
     constexpr int CH = kPhaseStaged ? L / 16 : 1;  // 16-byte pieces per row
     for (int q = tid; q < LPB * CH; q += blockDim.x) {
       const int i = q / CH, ch = q - i * CH;
       const long long ln = line0 + i;
       if (ln >= lines) continue;
-      int y = (int)(ln % ny) - ((M.sy % ny) + ny) % ny, z = (int)(ln / ny) - ((M.sz % nz) + nz) % nz;
+      int y = (int)(ln % ny) - ((msy % ny) + ny) % ny, z = (int)(ln / ny) - ((msz % nz) + nz) % nz;
       if (y < 0) y += ny;
       if (z < 0) z += nz;
-      cp_async16(&ph_s[i][ch * 16], M.phase + (long long)(z * ny + y) * nx + ch * 16);
+      cp_async16(&ph_s[i][ch * 16], phase_map + (long long)(z * ny + y) * nx + ch * 16);
     }
     cp_async_commit();
   }
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(XCfg<L>::THREADS, xpass_min_blocks<R>()) k_xpa
       const XMember& M = a.xm[m];
       int xs = n - sx;
       if (xs < 0) xs += nx;
-      const int ph = staged ? (int)ph_s[kPhaseStaged ? i : 0][kPhaseStaged ? xs : 0] : (int)M.phase[prow_s[i] + xs];
+      const int ph = staged ? (int)ph_s[kPhaseStaged ? i : 0][kPhaseStaged ? xs : 0] : (int)(a.mem != nullptr ? a.mem[m].phase : M.phase)[prow_s[i] + xs];
       const R tr = e0 + e1 + e2;
       const long long vox = ln * L + n;
       if (M.eps_out != nullptr) {

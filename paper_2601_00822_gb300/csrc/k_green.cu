@@ -65,7 +65,7 @@ __device__ __forceinline__ void g0_apply(const C2<R> g[3], const R xi[3], R q, R
 // thread's share of the residual numerator sum.
 template <typename R, int L, int T>
 __device__ __forceinline__ R green_tile(const GArgs<R>& a, C2<R>* s, const C2<R>* pre, int col0, int ky, int mode,
-                                        C2<R>* dprev, IterState* stm, const R* Em, bool rd = true,
+                                        C2<R>* dprev, IterState* stm, const Member* mem, bool rd = true,
                                         bool wr = true) {
   // GM_SWEEP: rd = this sweep forms the residual (d_prev staged), wr = it stores d
   const bool rd_d = mode == GM_FINAL || (mode == GM_SWEEP && rd);
@@ -110,7 +110,7 @@ __device__ __forceinline__ R green_tile(const GArgs<R>& a, C2<R>* s, const C2<R>
       }
 #pragma unroll
       for (int q = 0; q < 6; ++q)
-        M(q) = (mode != GM_FINAL && mode != GM_APPLY && k0) ? mk<R>(Em[q], R(0)) : mk<R>(0, 0);
+        M(q) = (mode != GM_FINAL && mode != GM_APPLY && k0) ? mk<R>((R)mem->E[q], R(0)) : mk<R>(0, 0);
       continue;
     }
     const bool load = mode != GM_APPLY;
@@ -188,7 +188,6 @@ __global__ void __launch_bounds__(GCfg<L, T>::BLOCK, green_min_blocks<R, L>()) k
   C2<R>* const dprev = a.dprev + mbr * a.d_ms;
   ResidSlot* const part = a.part + mbr * a.part_ms;
   IterState* const stm = a.st + mbr;
-  const R* const Em = a.use_me ? a.mE[mbr] : a.E;
   constexpr int NCOL = GCfg<L, T>::NCOL;
   constexpr int R1 = LineInfo<L>::R1, R2 = LineInfo<L>::R2;
   constexpr int TASKS = NCOL * LineInfo<L>::RMAX;   // (column, row group) tasks of a stage
@@ -212,7 +211,7 @@ __global__ void __launch_bounds__(GCfg<L, T>::BLOCK, green_min_blocks<R, L>()) k
   if (mode == GM_SWEEP && a.sparse) {
     const int sw = stm->iters, nc = stm->next_check;
     rd = sw == nc;
-    wr = rd || sw + 1 == nc || sw + 1 >= a.maxit;
+    wr = rd || sw + 1 == nc || sw + 1 >= stm->maxit;
   }
   // element z of line column c at column(c)[z * zs]
   auto column = [&](int c) { const int q = c / T; return spec + q * cs + rowbase + col0 + (c - q * T); };
@@ -265,7 +264,7 @@ __global__ void __launch_bounds__(GCfg<L, T>::BLOCK, green_min_blocks<R, L>()) k
   __syncthreads();
 
   // ---- Green operators per mode
-  R acc = green_tile<R, L, T>(a, s, pre, col0, ky, mode, dprev, stm, Em, rd, wr);
+  R acc = green_tile<R, L, T>(a, s, pre, col0, ky, mode, dprev, stm, a.mem + mbr, rd, wr);
 
   // ---- residual partial of this block in FP64 (fixed order: deterministic)
   const bool resid = (mode == GM_SWEEP && rd) || mode == GM_FINAL;
@@ -413,7 +412,6 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
     const C2<R>* pre = s + TILE;
     C2<R>* const dprev = a.dprev + m * a.d_ms;
     IterState* const stm = a.st + m;
-    const R* const Em = a.use_me ? a.mE[m] : a.E;
     // forward z transform, in place in the tile
     {
       C2<R> x[R1];
@@ -443,7 +441,7 @@ __global__ void __launch_bounds__(GCfg<L>::THREADS, 1)
       }
     }
     __syncthreads();
-    acc += (double)green_tile<R, L, T>(a, s, pre, col0, ky, GM_SWEEP, dprev, stm, Em);
+    acc += (double)green_tile<R, L, T>(a, s, pre, col0, ky, GM_SWEEP, dprev, stm, a.mem + m);
     __syncthreads();
     // inverse z transform in the order of the one-tile-per-block form (the same
     // arithmetic, so the two forms give identical fields): in-place R2-point step,

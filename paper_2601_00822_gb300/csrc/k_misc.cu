@@ -5,6 +5,7 @@
 #include "resid.cuh"
 
 #include <atomic>
+#include <cstddef>
 
 namespace bfcs {
 
@@ -359,6 +360,30 @@ cudaError_t launch_bden(const C2<R>* bhat, const Geo& g, ResidSlot* part, IterSt
 }
 
 // ---------------------------------------------------------------- residual reduction (Eq. 5.11)
+__global__ void k_init_states(IterState* st, const Member* mem, double tol) {
+  IterState* s = st + blockIdx.x;
+  int* w = reinterpret_cast<int*>(s);
+  for (int i = threadIdx.x; i < (int)(offsetof(IterState, resid_last) / sizeof(int)); i += blockDim.x) w[i] = 0;
+  if (threadIdx.x == 0) {
+    const double t = mem[blockIdx.x].tol;
+    s->tol = t >= 0.0 ? t : tol;
+    s->maxit = 0;
+  }
+}
+cudaError_t launch_init_states(IterState* st, const Member* mem, int batch, double tol, cudaStream_t s) {
+  k_init_states<<<batch, 32, 0, s>>>(st, mem, tol);
+  count_launches(1);
+  return cudaGetLastError();
+}
+__global__ void k_set_maxit(IterState* st, int batch, int maxit) {
+  for (int m = threadIdx.x; m < batch; m += blockDim.x) st[m].maxit = maxit;
+}
+cudaError_t launch_set_maxit(IterState* st, int batch, int maxit, cudaStream_t s) {
+  k_set_maxit<<<1, 64, 0, s>>>(st, batch, maxit);
+  count_launches(1);
+  return cudaGetLastError();
+}
+
 __global__ void k_resid_final(const __grid_constant__ ResidArgs a) { resid_step(a, blockIdx.x); }
 
 cudaError_t launch_resid_final(const ResidArgs& a, int batch, cudaStream_t s) {

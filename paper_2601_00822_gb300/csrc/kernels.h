@@ -78,18 +78,20 @@ template <typename R> struct XArgs {
   int ncomp;
   int mode;
   int chain;              // see launch_chain
+  const Member* mem;      // nullable: phase map and shift of member m from mem[m] instead of xm[m] (the sweeps, whose
+                          // captured graphs then hold no input's address)
   XMember xm[kMaxBatch];
 };
 
 // ---- the residual step of a sweep (resid.cuh).  One block per member m: reduces
-// part[m * nparts ...], updates sts[m] and writes hist[m * hist_cap + sweep]; E, the warm
-// flag and a member's own tolerance come from mem[m].  The sweep index is the device
+// part[m * nparts ...], updates sts[m] and writes hist[m * hist_cap + sweep]; E and the
+// warm flag come from mem[m], the tolerance and the loop's sweep limit from sts[m].  The sweep index is the device
 // counter sts[m].iters.  check_max > 1: sparse evaluation, only sweeps s ==
 // sts[m].next_check carry a residual (others record NaN in hist); after each evaluation
 // the next one is placed at the sweep where the observed contraction rate predicts r <=
 // tol, at most check_max sweeps ahead (every check_max sweeps when tol = 0).  io
 // (nullable): two counters to which GM_SWEEP adds, per member, whether the sweep's Green
-// pass read d_prev and whether it wrote d (maxit: the call's sweep limit).
+// pass read d_prev and whether it wrote d.
 struct ResidArgs {
   const ResidSlot* part;
   int nparts;
@@ -97,9 +99,9 @@ struct ResidArgs {
   const Member* mem;
   double* hist;
   int hist_cap;
-  double tol, lam0, mu0, n;
+  double lam0, mu0, n;
   double ximin;           // 2 pi / max N_a
-  int mode, stall_window, check_max, maxit;
+  int mode, stall_window, check_max;
   unsigned long long* io;
 };
 
@@ -234,7 +236,6 @@ template <typename R> struct GArgs {
   C2<R>* dprev;           // 3 components: d = tau_hat . xi of the previous sweep
   Geo g;
   R lam0, mu0;
-  R E[6];
   R inv_n;                // 1 / |N| of Eq. 4.4
   const C2<R>* tw;        // exp(-2 pi i j / nz)
   ResidSlot* part;        // one slot per block (per member: part_ms slots)
@@ -242,15 +243,13 @@ template <typename R> struct GArgs {
   long long spec_ms, b_ms, d_ms;   // member strides (complex elements)
   int part_ms;
   int skip_done;          // 1: members with st[m].done skip the launch
-  int use_me;             // 1: member m takes its mean strain from mE[m]
+  const Member* mem;      // per member: the mean strain
   int mode;
   // GM_SWEEP with sparse residual evaluation: sweep s = st[m].iters reads d_prev
   // and forms the residual only when s == st[m].next_check, and writes d only on
-  // that sweep, the one before it and the last sweep (s + 1 == maxit)
+  // that sweep, the one before it and the last sweep (s + 1 == st[m].maxit)
   int sparse;
-  int maxit;
   R fx, fy, fz, c0, inv_mu0;       // 2 pi / n of the axes, G0's constants: filled by the launcher
-  R mE[kMaxBatch][6];
 };
 
 // ---- defect of an approximate strain on the fully transformed stress spectrum:
@@ -367,6 +366,11 @@ int validate_scratch();
 template <typename R>
 cudaError_t launch_bden(const C2<R>* bhat, const Geo& g, ResidSlot* part, IterState* st, cudaStream_t s,
                         int batch = 1, long long b_ms = 0);
+
+// start of a solve: st[m] = 0 up to resid_last, its tolerance (mem[m].tol, or tol where that
+// is negative); limit of a sweep loop
+cudaError_t launch_init_states(IterState* st, const Member* mem, int batch, double tol, cudaStream_t s);
+cudaError_t launch_set_maxit(IterState* st, int batch, int maxit, cudaStream_t s);
 
 // the residual of the final pass's partials (mode GM_FINAL) into st[m].resid_final
 cudaError_t launch_resid_final(const ResidArgs& a, int batch, cudaStream_t s);

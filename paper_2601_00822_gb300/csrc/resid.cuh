@@ -36,7 +36,7 @@ static __device__ __noinline__ void resid_step(const ResidArgs& a, int m) {
   if (tid == 0 && sweep_mode && a.io != nullptr) {
     // what the Green pass of this sweep moved besides its fixed traffic: d_prev read, d written
     const bool rd = a.check_max <= 1 || sweep == nc;
-    const bool wr = a.check_max <= 1 || rd || sweep + 1 == nc || sweep + 1 >= a.maxit;
+    const bool wr = a.check_max <= 1 || rd || sweep + 1 == nc || sweep + 1 >= st->maxit;
     atomicAdd(a.io, (unsigned long long)rd);
     atomicAdd(a.io + 1, (unsigned long long)wr);
   }
@@ -72,7 +72,7 @@ static __device__ __noinline__ void resid_step(const ResidArgs& a, int m) {
   for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
   if (tid != 0) return;
   const int warm = a.mem[m].warm;
-  const double tol = a.mem[m].tol >= 0.0 ? a.mem[m].tol : a.tol;
+  const double tol = st->tol;
   double r = sqrt(t);
   if (den_s > 0.0) r *= iden_s;
   if (!sweep_mode) { st->resid_final = r; return; }

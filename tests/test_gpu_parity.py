@@ -778,3 +778,35 @@ def test_fp64_column_widths_of_the_z_pass_agree(dims, cell):
                 ref = got
             assert all(torch.equal(a, c) for a, c in zip(got[:3], ref[:3])), B
             assert abs(got[3] - ref[3]) <= 1e-13 * ref[3], B
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64", "mixed"])
+def test_a_plan_serves_other_inputs_after_a_solve(precision):
+    """A plan keeps its sweep graph between solves.  Solves that change the phase map (other
+    addresses and contents), the load, the mean strain, the shift, the tolerance, the sweep
+    limit, the batch size or the material equal those of fresh plans bit for bit."""
+    dims = (32, 24, 16)
+    base = small_problem(dims, (16, 12, 16), [[16, 12, 16, 80, 1]], (16.0, 12.0, 8.0), 5.0)
+    other = small_problem(dims, (16, 12, 8), [[16, 12, 8, 30, 1], [4, 4, 4, 12, 1]], (8.0, 6.0, 4.0), 4.0,
+                          E=(0.01, -0.004, 0.002, 0.001, -0.003, 0.005))
+    phb, bb = gpu_inputs(base, precision)
+    pho, bo = gpu_inputs(other, precision)
+    stiff = [(1.0, 0.5), (4.0, 2.0)]
+    tol = 1e-4 if precision == "fp32" else 1e-8
+    calls = [(1, phb, bb, (0.0,) * 6, (0, 0, 0), base.phases, tol, 4000), (1, pho, bo, other.mean_strain, (3, 5, 7), base.phases, tol, 4000),
+             (3, pho, bb, other.mean_strain, (0, 0, 1), base.phases, 10 * tol, 4000), (3, phb, bo, (0.0,) * 6, (1, 2, 3), stiff, tol, 4000),
+             (1, phb, bb, (0.0,) * 6, (0, 0, 0), base.phases, tol, 13), (1, phb, bb, (0.0,) * 6, (0, 0, 0), base.phases, tol, 4000)]
+
+    def run(plan, c):
+        B, ph, b, E, shift, phases, t, maxit = c
+        mem = [dict(phase=ph, b=b, E=tuple((m + 1) * e for e in E), shift=shift) for m in range(B)]
+        mem, infos = plan.solve_batched(mem, phases, W.reference_medium(phases), tol=t, maxit=maxit)
+        return [(m["eps_out"], m["sig_out"], m["u_out"], i.iters) for m, i in zip(mem, infos)]
+
+    with api.Plan(dims, precision, max_batch=3) as kept:
+        for c in calls:
+            got = run(kept, c)
+            with api.Plan(dims, precision, max_batch=3) as fresh:
+                want = run(fresh, c)
+            for g, w in zip(got, want):
+                assert g[3] == w[3] and all(torch.equal(x, y) for x, y in zip(g[:3], w[:3])), c[0]
