@@ -404,6 +404,11 @@ __device__ __forceinline__ void stage2(C2<R>* y) {
 // waits here, before its first access to global memory, for its predecessor to complete,
 // and then lets its successor's blocks be scheduled, so a launch's latency is spent while
 // the kernel before it runs.  Without effect on an ordinary launch.
+// A chained kernel's blocks are scheduled once every block of its predecessor has passed
+// this wait, so whatever was written before the predecessor is complete by then: a kernel
+// may read it ahead of its own wait (the network's layers do so with their parameters,
+// which are packed at least two launches earlier).  Tensor memory is allocated after the
+// wait only: a waiting block that held some could keep its predecessor from starting.
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");

@@ -12,7 +12,9 @@ namespace bfcs {
 // 38.9 -> 34.8 ms, a 64^3 FP64 solve by Algorithm 2 40.4 -> 37.7 ms); the sweeps do not:
 // their launches sit in CUDA graphs, whose gaps are small already, and blocks that wait on
 // an SM disturb the placement of the running pass (32^3 FP64 8.7 -> 11.0 ms, 64^3 3.54 ->
-// 3.66 ms, 256^3 121 -> 124 ms when chained).
+// 3.66 ms, 256^3 121 -> 124 ms when chained).  The network chains all of its launches (26 a
+// forward pass of some microseconds each at 32^3): one 32^3 sample 242 -> 195 us, and 160
+// us with the layers' parameters loaded before the wait.
 template <class... P, class... A>
 cudaError_t launch_chain(bool chain, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                          const A&... a) {

@@ -58,6 +58,7 @@ constexpr int kConvWarps = 4;
 constexpr int kConvNT = 8;   // n8 tiles per block (64 columns)
 
 __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
+  chain_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const long long nvox = (long long)a.v.nx * a.v.ny * a.v.nz;
@@ -150,6 +151,7 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
 constexpr int kWgRows = 64;
 
 __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int mcols = min(64, a.cout_p);
   const int mchunks = a.cout_p / mcols;
@@ -261,6 +263,7 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
 // ------------------------------------------------------------------ elementwise
 // network input (B, 4, N) FP32 -> channels-last BF16 [B][N][16] (channels 4..15 zero)
 __global__ void k_features_in(const float* x, bf16* out, long long n, int batch) {
+  chain_wait();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n * batch;
        i += (long long)gridDim.x * blockDim.x) {
     const long long b = i / n, v = i - b * n;
@@ -274,6 +277,7 @@ __global__ void k_features_in(const float* x, bf16* out, long long n, int batch)
 // 2^3 average pooling, fine -> coarse (channels-last views), 8 channels (16 bytes) per thread
 __global__ void k_pool(const bf16* in, int ldi, int offi, bf16* out, int ldo, int offo, int C, Vol coarse,
                        int batch) {
+  chain_wait();
   const long long nc = (long long)coarse.nx * coarse.ny * coarse.nz;
   const int FX = 2 * coarse.nx, FY = 2 * coarse.ny, cv = C / 8;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc * batch * cv;
@@ -302,6 +306,7 @@ __global__ void k_pool(const bf16* in, int ldi, int offi, bf16* out, int ldo, in
 // 8 channels (16 bytes) of one fine voxel per thread
 __global__ void k_unpool_gate(const bf16* dco, int ldc, int offc, bf16* dfine, int ldf, int offf, const bf16* y,
                               int ldy, int offy, int C, Vol fine, int batch) {
+  chain_wait();
   const long long nf = (long long)fine.nx * fine.ny * fine.nz;
   const int cv = C / 8;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nf * batch * cv;
@@ -329,6 +334,7 @@ __global__ void k_unpool_gate(const bf16* dco, int ldc, int offc, bf16* dfine, i
 constexpr int kBiasThreads = 256, kBiasBlocks = 304;
 __global__ void __launch_bounds__(kBiasThreads) k_bias_grad(const bf16* dy, int ldd, int offd, int C, long long rows,
                                                             long long per, float* part) {
+  chain_wait();
   __shared__ float red[kBiasThreads * 8];
   const int cv = C / 8, nr = kBiasThreads / cv;
   const int c = threadIdx.x % cv, j = threadIdx.x / cv;
@@ -385,6 +391,7 @@ __device__ __noinline__ float scaled_diff_f64(float p, float t, double f) { retu
 // not finite) are formed in FP64.
 constexpr int kLossBlocks = 64;
 __global__ void k_loss(const float* pred, const float* target, long long n, double* num, double* den) {
+  chain_wait();
   __shared__ double rn[32], rd[32];
   const int b = blockIdx.y;
   const float* pb = pred + (long long)b * 6 * n;
@@ -430,6 +437,7 @@ __global__ void k_loss(const float* pred, const float* target, long long n, doub
 // (written if loss != null): one warp per sample in turn, then thread 0 over the samples
 __global__ void k_loss_final(const double* num, const double* den, int nblk, int batch, double* fac_b, double* rel_b,
                              double* loss) {
+  chain_wait();
   const int lane = threadIdx.x & 31;
   for (int b = threadIdx.x >> 5; b < batch; b += blockDim.x >> 5) {
     double s0 = 0, s1 = 0;
@@ -452,6 +460,7 @@ __global__ void k_loss_final(const double* num, const double* den, int nblk, int
 // (48 bits before the one rounding to FP32, where the FP64 form has 53; 155 us of FP64
 // pipe for 8 samples of 64^3), FP64 outside their range
 __global__ void k_loss_grad(const float* pred, const float* target, const double* fac_b, long long n, bf16* dy) {
+  chain_wait();
   const int b = blockIdx.y;
   const double fd = fac_b[b];
   const ff f = d2ff_bits(fd);       // (FP64 divisions and conversions by every thread took 65 us)
@@ -476,6 +485,7 @@ __global__ void k_loss_grad(const float* pred, const float* target, const double
 // Adam (Kingma and Ba 2014), bias-corrected, FP32 state
 __global__ void k_adam(float* w, const float* g, float* m, float* v, long long n, float lr, float b1, float b2,
                        float eps, float c1, float c2) {
+  chain_wait();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -501,6 +511,7 @@ struct PackArgs {
 
 // every layer in one launch (blockIdx.y = layer)
 __global__ void k_pack(const float* flat, const __grid_constant__ PackArgs pa) {
+  chain_wait();
   const LayerDef& L = pa.def[blockIdx.y];
   bf16* const fw = pa.fw[blockIdx.y];
   bf16* const bw = pa.bw[blockIdx.y];
@@ -535,6 +546,7 @@ __global__ void k_pack(const float* flat, const __grid_constant__ PackArgs pa) {
 constexpr int kRedOut = 32, kRedLanes = 8;
 __global__ void __launch_bounds__(kRedOut * kRedLanes) k_reduce_grad(const float* wpart, int nchunks, const float* bpart,
                                                                     int nblk, int bcols, LayerDef L, float* gflat) {
+  chain_wait();
   __shared__ float red[kRedLanes][kRedOut];
   const int o = threadIdx.x % kRedOut, j = threadIdx.x / kRedOut;
   const int taps = L.kind == 0 ? 27 : 1;
@@ -575,6 +587,7 @@ template <typename R> struct SampleArgs {
 };
 template <typename R>
 __global__ void k_absmax(const __grid_constant__ SampleArgs<R> sa, long long n3, unsigned* out) {
+  chain_wait();
   __shared__ float red[32];
   const R* b = sa.b[blockIdx.y];
   float m = 0.f;
@@ -593,6 +606,7 @@ struct MuTab { float mu[BFCS_MAX_PHASES]; float mu_max; };
 template <typename R>
 __global__ void k_prepare(const R* b, const int8_t* phase, MuTab mt, const unsigned* sbits, const R* eps, float* x,
                           float* target, long long n) {
+  chain_wait();
   const float s = __uint_as_float(*sbits);
   const float inv = s > 0.f ? 1.f / s : 0.f;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
@@ -609,6 +623,7 @@ __global__ void k_prepare(const R* b, const int8_t* phase, MuTab mt, const unsig
 template <typename R>
 __global__ void k_prepare_x0(const __grid_constant__ SampleArgs<R> sa, MuTab mt, const unsigned* sbits, bf16* x0,
                              long long n) {
+  chain_wait();
   const R* b = sa.b[blockIdx.y];
   const int8_t* phase = sa.phase[blockIdx.y];
   x0 += (long long)blockIdx.y * n * 16;
@@ -630,6 +645,7 @@ __global__ void k_prepare_x0(const __grid_constant__ SampleArgs<R> sa, MuTab mt,
 }  // namespace bfcs
 
 // ====================================================================== host side
+using bfcs::launch_chain;
 using namespace bfcs::net;
 using bfcs::count_launches;
 
@@ -695,7 +711,7 @@ namespace {
 cudaError_t pack_all(bfcs_net_s* N, const float* params) {
   PackArgs pa;
   for (int l = 0; l < kNumLayers; ++l) { pa.def[l] = N->def[l]; pa.fw[l] = N->fw[l]; pa.bw[l] = N->bw[l]; }
-  k_pack<<<dim3(108, kNumLayers), 256, 0, N->st>>>(params, pa);
+  launch_chain(true, k_pack, dim3(108, kNumLayers), 256, 0, N->st, params, pa);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -722,8 +738,8 @@ cudaError_t launch_conv(const ConvArgs& a, long long nvox, int* err, cudaStream_
   if (rows_ok(a)) return launch_rows(a, sm_count(), st);
   if (!conv3_ok(a)) return cudaErrorInvalidValue;
   if (tcgen05_enabled()) return launch_conv3(a, sm_count(), err, st);
-  k_conv<<<dim3(ceil_div(nvox, kConvWarps * 32), ceil_div(a.cout_p, kConvNT * 8), a.batch), kConvWarps * 32, 0,
-           st>>>(a);
+  launch_chain(true, k_conv, dim3(ceil_div(nvox, kConvWarps * 32), ceil_div(a.cout_p, kConvNT * 8), a.batch),
+               kConvWarps * 32, 0, st, a);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -752,7 +768,8 @@ cudaError_t conv_fwd(bfcs_net_s* N, int l, const float* params, int B, View in, 
 
 cudaError_t pool(bfcs_net_s* N, View in, View out, int C, int coarse_lv, int B) {
   const long long tot = N->n[coarse_lv] * B * C / 8;
-  k_pool<<<grid_for(tot), 256, 0, N->st>>>(in.p, in.ld, in.off, out.p, out.ld, out.off, C, N->vol[coarse_lv], B);
+  launch_chain(true, k_pool, grid_for(tot), 256, 0, N->st, in.p, in.ld, in.off, out.p, out.ld, out.off, C,
+               N->vol[coarse_lv], B);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -854,13 +871,14 @@ cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View 
   } else {
     const int mcols = std::min(64, w.cout_p);
     const size_t smem = (size_t)kWgRows * (mcols + 8 + w.cin + 8) * sizeof(bf16);
-    k_wgrad<<<dim3(nchunks, taps * mchunks), 128, smem, N->st>>>(w);
+    launch_chain(true, k_wgrad, dim3(nchunks, taps * mchunks), 128, smem, N->st, w);
     const long long bper = (orows + nblk - 1) / nblk;
-    k_bias_grad<<<nblk, kBiasThreads, 0, N->st>>>(dout.p, dout.ld, dout.off, bc, orows, bper, w.bpart);
+    launch_chain(true, k_bias_grad, nblk, kBiasThreads, 0, N->st, dout.p, dout.ld, dout.off, bc, orows, bper,
+                 w.bpart);
     count_launches(2);
   }
-  k_reduce_grad<<<ceil_div(per, kRedOut) + ceil_div(bc, kRedOut), kRedOut * kRedLanes, 0, N->st>>>(
-      N->part, nchunks, w.bpart, nblk, bc, L, grad);
+  launch_chain(true, k_reduce_grad, ceil_div(per, kRedOut) + ceil_div(bc, kRedOut), kRedOut * kRedLanes, 0, N->st,
+               N->part, nchunks, w.bpart, nblk, bc, L, grad);
   count_launches(1);
   // input gradient: a convolution with the data-gradient weights
   if (din.p != nullptr) {
@@ -888,8 +906,8 @@ cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View 
 // pooling gradient into the skip half of a concatenation's gradient, and its gate
 cudaError_t unpool_gate(bfcs_net_s* N, View dco, View dfine, View y, int C, int fine_lv, int B) {
   const long long tot = N->n[fine_lv] * B * C / 8;
-  k_unpool_gate<<<grid_for(tot), 256, 0, N->st>>>(dco.p, dco.ld, dco.off, dfine.p, dfine.ld, dfine.off, y.p, y.ld,
-                                                  y.off, C, N->vol[fine_lv], B);
+  launch_chain(true, k_unpool_gate, grid_for(tot), 256, 0, N->st, dco.p, dco.ld, dco.off, dfine.p, dfine.ld,
+               dfine.off, y.p, y.ld, y.off, C, N->vol[fine_lv], B);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -922,10 +940,10 @@ cudaError_t backward(bfcs_net_s* N, float* g, int B) {
 }
 
 cudaError_t loss_and_grad(bfcs_net_s* N, int B, const float* target, double* loss_dev) {
-  k_loss<<<dim3(kLossBlocks, B), 256, 0, N->st>>>(N->OUT, target, N->n[0], N->lnum, N->lden);
-  k_loss_final<<<1, 256, 0, N->st>>>(N->lnum, N->lden, kLossBlocks, B, N->fac_b, N->rel_b, loss_dev);
+  launch_chain(true, k_loss, dim3(kLossBlocks, B), 256, 0, N->st, N->OUT, target, N->n[0], N->lnum, N->lden);
+  launch_chain(true, k_loss_final, 1, 256, 0, N->st, N->lnum, N->lden, kLossBlocks, B, N->fac_b, N->rel_b, loss_dev);
   const int bx = std::max(1, std::min(ceil_div(N->n[0], 256), ceil_div(152 * 16, B)));
-  k_loss_grad<<<dim3(bx, B), 256, 0, N->st>>>(N->OUT, target, N->fac_b, N->n[0], N->dOUT);
+  launch_chain(true, k_loss_grad, dim3(bx, B), 256, 0, N->st, N->OUT, target, N->fac_b, N->n[0], N->dOUT);
   count_launches(3);
   return cudaGetLastError();
 }
@@ -971,8 +989,9 @@ int predict(bfcs_net_s* N, const float* params, int batch, const R* const* b, co
       SampleArgs<R> sa{};
       for (int j = 0; j < k; ++j) { sa.b[j] = b[i0 + j0 + j]; sa.phase[j] = phase[i0 + j0 + j]; }
       const int bx = std::max(1, std::min(ceil_div(n, 256), ceil_div(152 * 8, k)));
-      k_absmax<R><<<dim3(bx, k), 256, 0, N->st>>>(sa, 3 * n, N->sbits + j0);
-      k_prepare_x0<R><<<dim3(bx, k), 256, 0, N->st>>>(sa, mt, N->sbits + j0, N->X0 + (long long)j0 * n * 16, n);
+      launch_chain(true, k_absmax<R>, dim3(bx, k), 256, 0, N->st, sa, 3 * n, N->sbits + j0);
+      launch_chain(true, k_prepare_x0<R>, dim3(bx, k), 256, 0, N->st, sa, mt, N->sbits + j0,
+                   N->X0 + (long long)j0 * n * 16, n);
       count_launches(2);
     }
     e = forward(N, params, B);
@@ -1108,15 +1127,15 @@ int bfcs_net_prepare(bfcs_net N, int precision, const void* b, const int8_t* pha
   if (precision == BFCS_FP64) {
     SampleArgs<double> sa{};
     sa.b[0] = (const double*)b;
-    k_absmax<double><<<std::min(304, grid_for(3 * n)), 256, 0, N->st>>>(sa, 3 * n, N->sbits);
-    k_prepare<double><<<grid_for(n), 256, 0, N->st>>>((const double*)b, phase, mt, N->sbits, (const double*)eps, x_out,
-                                                      target_out, n);
+    launch_chain(true, k_absmax<double>, std::min(304, grid_for(3 * n)), 256, 0, N->st, sa, 3 * n, N->sbits);
+    launch_chain(true, k_prepare<double>, grid_for(n), 256, 0, N->st, (const double*)b, phase, mt, N->sbits,
+                 (const double*)eps, x_out, target_out, n);
   } else {
     SampleArgs<float> sa{};
     sa.b[0] = (const float*)b;
-    k_absmax<float><<<std::min(304, grid_for(3 * n)), 256, 0, N->st>>>(sa, 3 * n, N->sbits);
-    k_prepare<float><<<grid_for(n), 256, 0, N->st>>>((const float*)b, phase, mt, N->sbits, (const float*)eps, x_out,
-                                                     target_out, n);
+    launch_chain(true, k_absmax<float>, std::min(304, grid_for(3 * n)), 256, 0, N->st, sa, 3 * n, N->sbits);
+    launch_chain(true, k_prepare<float>, grid_for(n), 256, 0, N->st, (const float*)b, phase, mt, N->sbits,
+                 (const float*)eps, x_out, target_out, n);
   }
   count_launches(2);
   return status_of(cudaGetLastError());
@@ -1127,7 +1146,7 @@ int bfcs_net_forward(bfcs_net N, const float* params, int batch, const float* x,
     return BFCS_ERR_INVALID_ARG;
   cudaError_t e = pack_all(N, params);
   if (e == cudaSuccess) {
-    k_features_in<<<grid_for(N->n[0] * batch), 256, 0, N->st>>>(x, N->X0, N->n[0], batch);
+    launch_chain(true, k_features_in, grid_for(N->n[0] * batch), 256, 0, N->st, x, N->X0, N->n[0], batch);
     count_launches(1);
     e = forward(N, params, batch);
   }
@@ -1142,7 +1161,7 @@ int bfcs_net_grad(bfcs_net N, const float* params, int batch, const float* x, co
     return BFCS_ERR_INVALID_ARG;
   cudaError_t e = pack_all(N, params);
   if (e == cudaSuccess) {
-    k_features_in<<<grid_for(N->n[0] * batch), 256, 0, N->st>>>(x, N->X0, N->n[0], batch);
+    launch_chain(true, k_features_in, grid_for(N->n[0] * batch), 256, 0, N->st, x, N->X0, N->n[0], batch);
     count_launches(1);
     e = forward(N, params, batch);
   }
@@ -1158,7 +1177,7 @@ int bfcs_net_adam(bfcs_net N, float* params, const float* grad, float* m, float*
     return BFCS_ERR_INVALID_ARG;
   const float c1 = (float)(1.0 - std::pow(0.9, (double)t)), c2 = (float)(1.0 - std::pow(0.999, (double)t));
   const long long n = param_count();
-  k_adam<<<grid_for(n), 256, 0, N->st>>>(params, grad, m, v, n, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
+  launch_chain(true, k_adam, grid_for(n), 256, 0, N->st, params, grad, m, v, n, lr, 0.9f, 0.999f, 1e-8f, c1, c2);
   count_launches(1);
   return status_of(cudaGetLastError());
 }

@@ -60,6 +60,45 @@ template <int KC, int N> struct C3 {
   static constexpr int NJ = (kCHalo * KC + kWorkers - 1) / kWorkers;   // plane copies per thread
 };
 
+// column col of tiles (x fastest, then y, then the sample)
+__device__ __forceinline__ void conv3_column(const ConvArgs& a, long long col, int& b, int& x0, int& y0) {
+  const int ntx = (a.v.nx + kCX - 1) / kCX, nty = (a.v.ny + kCY - 1) / kCY;
+  x0 = (int)(col % ntx) * kCX;
+  col /= ntx;
+  y0 = (int)(col % nty) * kCY;
+  b = (int)(col / nty);
+}
+
+// worker tid's copies in plane 0 of column col
+template <int KC, int NJ>
+__device__ __forceinline__ void conv3_sources(const ConvArgs& a, long long col, int tid, const bf16* (&src)[NJ]) {
+  int b, x0, y0;
+  conv3_column(a, col, b, x0, y0);
+  const bf16* inb = a.in + (long long)b * ((long long)a.v.nx * a.v.ny * a.v.nz) * a.ldi + a.offi;
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    const int i = tid + j * kWorkers;
+    const int v = i / KC, c = i % KC;
+    // (a partial tile's rows past the grid read wrapped voxels; they are not stored)
+    const int gx = (x0 + v % kCHX - 1 + a.v.nx) % a.v.nx, gy = (y0 + v / kCHX - 1 + a.v.ny) % a.v.ny;
+    src[j] = inb + ((long long)gy * a.v.nx + gx) * a.ldi + c * 8;
+  }
+}
+
+// requests plane z into ring slot id
+template <int KC, int N>
+__device__ __forceinline__ void conv3_load_plane(const ConvArgs& a, unsigned ring, int z, unsigned id, int tid,
+                                                 const bf16* const (&src)[C3<KC, N>::NJ]) {
+  using C = C3<KC, N>;
+  const long long off = (long long)wrap(z, a.v.nz) * ((long long)a.v.nx * a.v.ny * a.ldi);
+  const unsigned base = ring + (id & (kRing - 1)) * C::PLANE;
+#pragma unroll
+  for (int j = 0; j < C::NJ; ++j) {
+    const int i = tid + j * kWorkers;
+    if (i < kCHalo * KC) cp16(base + (unsigned)((i % KC) * C::PV + i / KC) * 16u, src[j] + off);
+  }
+}
+
 }  // namespace
 
 template <int KC, int N>
@@ -79,10 +118,29 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
   const long long total = (long long)ntx * nty * nz * a.batch;
   const long long t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
   const int n = (int)(t1 - t0);
+  // The parameters, ahead of the wait for the predecessor (they were written before it,
+  // see chain_wait): one 32^3 sample 189 -> 160 us, sixteen of 64^3 1982 -> 1916 us.  The
+  // first tile's planes right after the wait, before the flag and the allocation, took
+  // 153 us at 32^3 but 2253 us for the batch: their addresses spill.
+  if (warp != 8 && n > 0) {
+    for (int i = tid; i < 27 * N * KC; i += kWorkers) {   // weights (core-matrix layout)
+      const int c = i % KC, m = (i / KC) % N, tap = i / (KC * N);
+      cp16(wsm + (unsigned)((tap * KC + c) * N + m) * 16u, a.w + ((long long)tap * N + m) * a.cin + c * 8);
+    }
+    if (tid < N) bias_s[tid] = a.bias != nullptr ? __ldcg(a.bias + tid % a.bias_mod) : 0.f;
+    cp_commit();
+  }
+  chain_wait();
+  // the warp's role once more, as a value of its own: with the test above repeated the
+  // compiler joins the parts of a role and spills
+  const bool issuer = __shfl_sync(0xffffffffu, warp, 0) == 8;
   // a network whose tensor-core wait once expired launches no more tensor-core work:
   // the flag is sticky until the context is destroyed (one thread reads it, so that
   // every thread of the block takes the same branch)
-  if (__syncthreads_or(tid == 0 && *(volatile int*)err != 0) || n <= 0) return;
+  if (__syncthreads_or(tid == 0 && *(volatile int*)err != 0) || n <= 0) {
+    cp_wait<0>();
+    return;
+  }
 
   if (warp == 8) {
     const unsigned dst = (unsigned)__cvta_generic_to_shared(&tmem_s);
@@ -98,12 +156,11 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
   }
-  if (tid < N) bias_s[tid] = a.bias != nullptr ? a.bias[tid % a.bias_mod] : 0.f;
   tc_before();
   __syncthreads();
   tc_after();
 
-  if (warp == 8) {
+  if (issuer) {
     // ---- MMA issue
     const unsigned tmem = __shfl_sync(0xffffffffu, tmem_s, 0);
     unsigned q = 0;                                    // ring index of the tile's lowest plane
@@ -147,58 +204,26 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
   } else {
     // ---- plane staging and epilogue
     const long long nvox = (long long)a.v.nx * a.v.ny * nz;
-    const long long zstride = (long long)a.v.nx * a.v.ny * a.ldi;
     const bf16* src[C::NJ];                            // this thread's copies in plane 0 of the loading column
-    auto column = [&](long long col, int& b, int& x0, int& y0) {
-      x0 = (int)(col % ntx) * kCX;
-      col /= ntx;
-      y0 = (int)(col % nty) * kCY;
-      b = (int)(col / nty);
-    };
-    auto set_column = [&](long long col) {
-      int b, x0, y0;
-      column(col, b, x0, y0);
-      const bf16* inb = a.in + (long long)b * nvox * a.ldi + a.offi;
-#pragma unroll
-      for (int j = 0; j < C::NJ; ++j) {
-        const int i = tid + j * kWorkers;
-        const int v = i / KC, c = i % KC;
-        // (a partial tile's rows past the grid read wrapped voxels; they are not stored)
-        const int gx = (x0 + v % kCHX - 1 + a.v.nx) % a.v.nx, gy = (y0 + v / kCHX - 1 + a.v.ny) % a.v.ny;
-        src[j] = inb + ((long long)gy * a.v.nx + gx) * a.ldi + c * 8;
-      }
-    };
-    auto load_plane = [&](int z, unsigned id) {
-      const long long off = (long long)wrap(z, nz) * zstride;
-      const unsigned base = ring + (id & (kRing - 1)) * C::PLANE;
-#pragma unroll
-      for (int j = 0; j < C::NJ; ++j) {
-        const int i = tid + j * kWorkers;
-        if (i < kCHalo * KC) cp16(base + (unsigned)((i % KC) * C::PV + i / KC) * 16u, src[j] + off);
-      }
-    };
     const int quarter = warp & 3, half = warp >> 2;
     const int row = quarter * 32 + lane;               // TMEM lane = tile voxel (x = row % 8, y = row / 8)
     const unsigned tmem = tmem_s;
 
-    for (int i = tid; i < 27 * N * KC; i += kWorkers) {   // weights (core-matrix layout)
-      const int c = i % KC, m = (i / KC) % N, tap = i / (KC * N);
-      cp16(wsm + (unsigned)((tap * KC + c) * N + m) * 16u, a.w + ((long long)tap * N + m) * a.cin + c * 8);
-    }
     long long col = t0 / nz;
     int z = (int)(t0 - col * nz);
-    set_column(col);
+    asm volatile("" : "+l"(col));
+    conv3_sources<KC>(a, col, tid, src);
     unsigned id = 0;                                   // ring index of tile k's lowest plane
-    for (int d = 0; d < 3; ++d) load_plane(z - 1 + d, d);
+    for (int d = 0; d < 3; ++d) conv3_load_plane<KC, N>(a, ring, z - 1 + d, d, tid, src);
     cp_commit();
-    if (n > 1 && z + 1 < nz) load_plane(z + 2, 3);
+    if (n > 1 && z + 1 < nz) conv3_load_plane<KC, N>(a, ring, z + 2, 3, tid, src);
     cp_commit();
     cp_wait<1>();
     fence_async();
     bool ok = workers_all(true);
     if (tid == 0) mbar_arrive(full);
     int eb, ex, ey;
-    column(col, eb, ex, ey);
+    conv3_column(a, col, eb, ex, ey);
     for (int k = 0; k < n; ++k) {
       const bool more = k + 1 < n, newcol = more && z + 1 == nz;
       if (more && !newcol) {                           // tile k + 1's plane, requested one tile ago
@@ -214,11 +239,11 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
       if (ok) {
         // tile k's lowest plane is free: request what tiles k + 1 and k + 2 still need
         if (newcol) {
-          set_column(col + 1);
-          for (int d = 0; d < 3; ++d) load_plane(d - 1, idn + d);
+          conv3_sources<KC>(a, col + 1, tid, src);
+          for (int d = 0; d < 3; ++d) conv3_load_plane<KC, N>(a, ring, d - 1, idn + d, tid, src);
         }
         const int zn = newcol ? 0 : z + 1;
-        if (k + 2 < n && zn + 1 < nz) load_plane(zn + 2, idn + 3);
+        if (k + 2 < n && zn + 1 < nz) conv3_load_plane<KC, N>(a, ring, zn + 2, idn + 3, tid, src);
         cp_commit();
         // epilogue of tile k
         const int x = ex + row % kCX, y = ey + row / kCX;
@@ -265,7 +290,7 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
         if (tid == 0) mbar_arrive(full + 8 * ((k + 1) & 1));
         ++col;
         z = 0;
-        column(col, eb, ex, ey);
+        conv3_column(a, col, eb, ex, ey);
       } else {
         ++z;
       }
@@ -316,7 +341,7 @@ cudaError_t launch_conv3(const ConvArgs& a, int sms, int* err, cudaStream_t st) 
 #define BFCS_X(KC, N)                                                                                          \
   if (a.cin == 8 * KC && a.cout_p == N) {                                                                      \
     const int blocks = (int)std::min<long long>(tiles, (long long)sms * C3<KC, N>::BLOCKS);                    \
-    k_conv3<KC, N><<<blocks, kConv3Threads, C3<KC, N>::SMEM, st>>>(a, err);                                    \
+    launch_chain(true, k_conv3<KC, N>, blocks, kConv3Threads, C3<KC, N>::SMEM, st, a, err);                    \
     count_launches(1);                                                                                         \
     return cudaGetLastError();                                                                                 \
   }

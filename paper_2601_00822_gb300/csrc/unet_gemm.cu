@@ -49,10 +49,11 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows(ConvArgs a, unsigned ro
     const int l = i & 31, j = (i >> 5) & 3, grp = (i >> 7) % NG, s = i / (128 * NG);
     const int col = grp * 32 + 8 * ((l >> 2) >> 1) + 2 * j + ((l >> 2) & 1);
     uint2 w = make_uint2(0u, 0u);
-    if (col < a.cout_p) w = *reinterpret_cast<const uint2*>(a.w + (long long)col * K + 16 * s + 4 * (l & 3));
+    if (col < a.cout_p) w = __ldcg(reinterpret_cast<const uint2*>(a.w + (long long)col * K + 16 * s + 4 * (l & 3)));
     wfrag[i] = w;
   }
-  if (tid < NG * 32) bias_s[tid] = a.bias != nullptr && tid < a.cout_p ? a.bias[tid % a.bias_mod] : 0.f;
+  if (tid < NG * 32) bias_s[tid] = a.bias != nullptr && tid < a.cout_p ? __ldcg(a.bias + tid % a.bias_mod) : 0.f;
+  chain_wait();
   __syncthreads();
   const unsigned nx = a.v.nx, ny = a.v.ny;
   const long long FX = 2 * nx, FY = 2 * ny;
@@ -162,8 +163,9 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_head(HeadArgs<R> a) {
   const int g = lane >> 2, t = lane & 3;
   uint2 w[2];
 #pragma unroll
-  for (int s = 0; s < 2; ++s) w[s] = *reinterpret_cast<const uint2*>(a.w + g * 32 + 16 * s + 4 * t);   // column g
-  const float b0 = 2 * t < 6 ? a.bias[2 * t] : 0.f, b1 = 2 * t + 1 < 6 ? a.bias[2 * t + 1] : 0.f;
+  for (int s = 0; s < 2; ++s) w[s] = __ldcg(reinterpret_cast<const uint2*>(a.w + g * 32 + 16 * s + 4 * t));   // column g
+  const float b0 = 2 * t < 6 ? __ldcg(a.bias + 2 * t) : 0.f, b1 = 2 * t + 1 < 6 ? __ldcg(a.bias + 2 * t + 1) : 0.f;
+  chain_wait();
   const int b = blockIdx.y;
   const bf16* in = a.in + (long long)b * a.n * 32;
   R* out = a.out[b];
@@ -227,7 +229,7 @@ namespace {
 template <int KS, int NG, bool GATHER, bool SHUFFLE>
 cudaError_t rows_launch(const ConvArgs& a, unsigned rows, int sms, cudaStream_t st) {
   const unsigned blocks = std::min<unsigned>((rows + kRowWarps * kRowsPerWarp - 1) / (kRowWarps * kRowsPerWarp), 4u * sms);
-  k_rows<KS, NG, GATHER, SHUFFLE><<<blocks, kRowWarps * 32, KS * NG * 128 * sizeof(uint2), st>>>(a, rows);
+  launch_chain(true, k_rows<KS, NG, GATHER, SHUFFLE>, blocks, kRowWarps * 32, KS * NG * 128 * sizeof(uint2), st, a, rows);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -261,9 +263,9 @@ cudaError_t launch_head(const HeadArgs<R>& a, int batch, bool predict, int sms, 
   const long long per = kRowWarps * kRowsPerWarp;
   const unsigned bx = (unsigned)std::max<long long>(1, std::min((a.n + per - 1) / per, (long long)(8 * sms / batch + 1)));
   if (predict) {
-    k_head<R, true><<<dim3(bx, batch), kRowWarps * 32, 0, st>>>(a);
+    launch_chain(true, k_head<R, true>, dim3(bx, batch), kRowWarps * 32, 0, st, a);
   } else {
-    if constexpr (sizeof(R) == 4) k_head<R, false><<<dim3(bx, batch), kRowWarps * 32, 0, st>>>(a);
+    if constexpr (sizeof(R) == 4) launch_chain(true, k_head<R, false>, dim3(bx, batch), kRowWarps * 32, 0, st, a);
     else return cudaErrorInvalidValue;
   }
   count_launches(1);

@@ -62,6 +62,7 @@ __device__ __forceinline__ unsigned swz(int v, int c) { return (unsigned)v * 64u
 
 // cin channels of the 32-channel half blockIdx.y (cin = 16: chunks 2 and 3 are zero)
 __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* err) {
+  chain_wait();
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) unsigned long long bars[3 + kYRing];   // full 0/1, done 0..2, drained
   __shared__ unsigned tmem_s;
@@ -358,6 +359,7 @@ template <int NP, bool UP> struct W1 {
 
 template <int NP, bool UP>
 __global__ void __launch_bounds__(256) k_wgrad1(WgArgs a, unsigned rows) {
+  chain_wait();
   using C = W1<NP, UP>;
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -521,9 +523,9 @@ int wgrad1_chunks(const WgArgs& a, int sms) { return wgrad1_blocks(a, sms) * (a.
 cudaError_t launch_wgrad1(const WgArgs& a, int sms, cudaStream_t st) {
   const unsigned rows = (unsigned)((long long)a.v.nx * a.v.ny * a.v.nz * a.batch);
   const int blocks = wgrad1_blocks(a, sms);
-  if (a.up_c == 0) k_wgrad1<2, false><<<blocks, 256, W1<2, false>::SMEM, st>>>(a, rows);
-  else if (a.cin == 32) k_wgrad1<2, true><<<blocks, 256, W1<2, true>::SMEM, st>>>(a, rows);
-  else k_wgrad1<3, true><<<blocks, 256, W1<3, true>::SMEM, st>>>(a, rows);
+  if (a.up_c == 0) launch_chain(true, k_wgrad1<2, false>, blocks, 256, W1<2, false>::SMEM, st, a, rows);
+  else if (a.cin == 32) launch_chain(true, k_wgrad1<2, true>, blocks, 256, W1<2, true>::SMEM, st, a, rows);
+  else launch_chain(true, k_wgrad1<3, true>, blocks, 256, W1<3, true>::SMEM, st, a, rows);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -543,7 +545,7 @@ int wgrad3_chunks(const WgArgs& a, int sms) {
 }
 
 cudaError_t launch_wgrad3(const WgArgs& a, int chunks, int* err, cudaStream_t st) {
-  k_wgrad3<<<dim3(chunks, a.cin > 32 ? a.cin / 32 : 1), kTcWorkers + 32, kWgSmem, st>>>(a, err);
+  launch_chain(true, k_wgrad3, dim3(chunks, a.cin > 32 ? a.cin / 32 : 1), kTcWorkers + 32, kWgSmem, st, a, err);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -220,3 +220,43 @@ def test_loss_and_its_gradient_over_the_range_of_the_fields(scale):
     assert abs(float(loss) - float(want)) <= 1e-12 * float(want)
     db = (2.0 * d / (2 * den.view(-1, 1, 1, 1, 1))).sum((0, 2, 3, 4))
     assert rel(g[bslice].double().cpu(), db.cpu()) <= 1e-2     # BF16 terms, 2^-9 each
+
+
+@pytest.mark.parametrize("dims,batch", [((8, 8, 8), 1), ((32, 16, 24), 3)])
+def test_captured_passes_equal_the_direct_ones(dims, batch):
+    """Forward pass, strain prediction and gradient recorded in a CUDA graph and replayed
+    with other parameters and inputs: the chained launches keep their order, and the
+    layers' early parameter loads see the values of the replay."""
+    r = np.random.default_rng(41)
+    flat = params(42).float().cuda()
+    x = inputs(43, batch, dims).float().cuda()
+    t = inputs(44, batch, dims, ch=6).float().cuda()
+    b = [torch.tensor(r.standard_normal((3,) + dims[::-1]), dtype=torch.float32, device="cuda") for _ in range(batch)]
+    ph = [torch.tensor(r.integers(0, 2, dims[::-1]), dtype=torch.int8, device="cuda") for _ in range(batch)]
+    phases = [(1.0, 0.5), (0.3, 2.0)]
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        net = api.Net(dims, max_batch=batch, train=True, stream=side)
+
+        def passes():
+            y = net.forward(flat, x)
+            p = net.predict(flat, b, ph, phases)
+            g, loss = net.grad(flat, x, t)
+            return [y, *p, g, loss]
+
+        passes()
+        side.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            got = passes()
+        for k in range(3):
+            flat.copy_(params(45 + k).float())
+            x.copy_(inputs(48 + k, batch, dims).float())
+            b[0].copy_(torch.tensor(r.standard_normal(b[0].shape), dtype=torch.float32))
+            graph.replay()
+            replayed = [v.clone() for v in got]
+            want = passes()
+            assert all(torch.equal(u, v) for u, v in zip(replayed, want))
+        net.status()
+        side.synchronize()
