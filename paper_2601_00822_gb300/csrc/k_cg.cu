@@ -12,28 +12,39 @@
 // computed on the device, so an iteration needs no host synchronisation.
 #include "kernels.h"
 
+#include <algorithm>
+
 #ifndef BFCS_R
 #define BFCS_R float
 #endif
 
 namespace bfcs {
 
-constexpr int kCgThreads = 256;
+// Vector kernels: blocks of 128 threads, one mode a thread, up to the eight blocks an SM
+// holds (kCgParts).  In FP64 they are bound by the FP64 pipe (about 45 operations a mode
+// and two lanes an SM: 9.4 us at 64^3 when every SM has the same share), so the work has
+// to be even: 512 blocks of 256 gave some SMs four blocks and others three, and 16 blocks
+// a second round.
+constexpr int kCgThreads = 128;
+constexpr int kCgScalarThreads = 256;
 
-// Re(a : C0 : conj b) for the 6 tensorial components (xx yy zz yz xz xy), in the
+__device__ __forceinline__ float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_r(double a, double b, double c) { return fma(a, b, c); }
+
+// Re(a : C0 : conj b) for the 6 tensorial components (xx yy zz yz xz xy), mu2 = 2 mu0, in the
 // vectors' precision (FP32 vectors: FP32 per mode; the caller sums 16 modes in R
 // and then adds in FP64: GB300's FP64 pipe would otherwise bound the vector kernels)
 template <typename R>
-__device__ __forceinline__ R c0dot(const C2<R> (&a)[6], const C2<R> (&b)[6], R lam0, R mu0) {
+__device__ __forceinline__ R c0dot(const C2<R> (&a)[6], const C2<R> (&b)[6], R lam0, R mu2) {
   const R ta_r = a[0].x + a[1].x + a[2].x, ta_i = a[0].y + a[1].y + a[2].y;
   const R tb_r = b[0].x + b[1].x + b[2].x, tb_i = b[0].y + b[1].y + b[2].y;
-  R s = R(0);
+  R s = R(0), o = R(0);
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    const R w = c < 3 ? R(1) : R(2);
-    s += w * (a[c].x * b[c].x + a[c].y * b[c].y);
+  for (int c = 0; c < 3; ++c) {
+    s = fma_r(a[c].x, b[c].x, fma_r(a[c].y, b[c].y, s));
+    o = fma_r(a[c + 3].x, b[c + 3].x, fma_r(a[c + 3].y, b[c + 3].y, o));
   }
-  return lam0 * (ta_r * tb_r + ta_i * tb_i) + R(2) * mu0 * s;
+  return fma_r(lam0, fma_r(ta_r, tb_r, ta_i * tb_i), mu2 * fma_r(R(2), o, s));
 }
 
 __device__ __forceinline__ double block_reduce(double v, double* red) {
@@ -65,15 +76,15 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
   C2<R>* p = a.p + off;
   C2<R>* q = a.q + off;
   const C2<R>* s = a.s != nullptr ? a.s + off : nullptr;
-  __shared__ R cst[4];          // alpha, beta, lam0, mu0, converted once per block
+  __shared__ R cst[4];          // alpha, beta, lam0, 2 mu0, converted once per block
   if (threadIdx.x == 0) {
     cst[0] = (R)a.cg[m].alpha;
     cst[1] = (R)a.cg[m].beta;
     cst[2] = (R)a.lam0;
-    cst[3] = (R)a.mu0;
+    cst[3] = (R)(2 * a.mu0);
   }
   __syncthreads();
-  const R alpha = cst[0], beta = cst[1], lam0 = cst[2], mu0 = cst[3];
+  const R alpha = cst[0], beta = cst[1], lam0 = cst[2], mu2 = cst[3];
   const long long modes = (long long)g.nz * g.ny * g.mx;
   // partial sums: 16 grid-stride modes in R (their products are R), then one FP64 add
   double acc = 0.0;
@@ -96,7 +107,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
           p[k * g.cs + gi] = x;
           u[k] = x;
         }
-        part += w * c0dot<R>(u, u, lam0, mu0);
+        part += w * c0dot<R>(u, u, lam0, mu2);
       } else if (mode == CgMode::PQ) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
@@ -104,7 +115,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
           v[k] = u[k] - q[k * g.cs + gi];
           q[k * g.cs + gi] = v[k];
         }
-        part += w * c0dot<R>(u, v, lam0, mu0);
+        part += w * c0dot<R>(u, v, lam0, mu2);
       } else if (mode == CgMode::UPDATE) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
@@ -112,7 +123,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
           u[k] = r[k * g.cs + gi] - scale(q[k * g.cs + gi], alpha);
           r[k * g.cs + gi] = u[k];
         }
-        part += w * c0dot<R>(u, u, lam0, mu0);
+        part += w * c0dot<R>(u, u, lam0, mu2);
       } else {
 #pragma unroll
         for (int k = 0; k < 6; ++k) p[k * g.cs + gi] = r[k * g.cs + gi] + scale(p[k * g.cs + gi], beta);
@@ -171,11 +182,13 @@ static __global__ void k_cg_scalar(const double* part, int nparts, CgState* cg, 
 
 template <typename R>
 cudaError_t launch_cg_vec(const CgArgs<R>& a, int mode, int batch, cudaStream_t st) {
-  cudaError_t e = launch_chain(true, k_cg_vec<R>, dim3(kCgParts, batch), kCgThreads, 0, st, a, mode);
+  const int modes = a.g.nz * a.g.ny * a.g.mx, nparts = std::min(kCgParts, (modes + kCgThreads - 1) / kCgThreads);
+  cudaError_t e = launch_chain(true, k_cg_vec<R>, dim3(nparts, batch), kCgThreads, 0, st, a, mode);
   count_launches(1);
   if (e != cudaSuccess || mode == CgMode::DIR) return e;
   count_launches(1);
-  return launch_chain(true, k_cg_scalar, batch, kCgThreads, 0, st, (const double*)a.part, (int)kCgParts, a.cg, a.skip, mode);
+  return launch_chain(true, k_cg_scalar, batch, kCgScalarThreads, 0, st, (const double*)a.part, nparts, a.cg, a.skip,
+                      mode);
 }
 
 template cudaError_t launch_cg_vec<BFCS_R>(const CgArgs<BFCS_R>&, int, int, cudaStream_t);

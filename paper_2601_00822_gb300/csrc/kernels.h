@@ -150,7 +150,7 @@ struct CgState {
   int best_it;           // iteration of `best`; no new best for kCgStagnation iterations ends the member
 };
 constexpr int kCgStagnation = 50;
-constexpr int kCgParts = 512;       // partial sums per member
+constexpr int kCgParts = 152 * 8;   // most partial sums per member: one block each, eight blocks an SM
 template <typename R> struct CgArgs {
   C2<R>* c;              // iterate (state layout, members at ms)
   C2<R>* r;              // residual

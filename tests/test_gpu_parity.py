@@ -609,6 +609,23 @@ def test_cg_inside_the_mixed_ladder_and_batched_equals_individual():
             assert r <= 2e-9, (sh, r)
 
 
+@pytest.mark.parametrize("dims,spheres,centre,a", [
+    ((8, 8, 4), [[8, 8, 4, 12, 1]], (4.0, 4.0, 2.0), 1.8),                  # 160 modes: a full and a partial block
+    ((16, 12, 6), [[8, 12, 6, 16, 1]], (8.0, 6.0, 3.0), 2.5),               # 648 modes
+    ((96, 64, 64), [[96, 64, 64, 2000, 1]], (48.0, 32.0, 32.0), 9.0)])      # more modes than threads: two rounds
+def test_cg_vectors_over_the_range_of_their_grids(dims, spheres, centre, a):
+    """Vector kernels of the conjugate gradients with few, partial and several modes a
+    thread: the solution meets the residual tolerance by the oracle's own residual (twice
+    the tolerance, for the rounding of either)."""
+    p = small_problem(dims, dims, spheres, centre, a)
+    ph_o, b_o = oracle_inputs(p)
+    ph, b = gpu_inputs(p, "fp64")
+    with api.Plan(p.dims, "fp64", cg=True) as plan:
+        eps, sig, u, info = plan.solve(ph, p.phases, p.c0, b, tol=1e-10, maxit=4000)
+    assert info.status == _lib.OK and info.resid <= 1e-10
+    assert O.residual(ph_o, p.phases, eps.cpu().numpy(), O.fft3(b_o), O.wavevectors(p.dims)) <= 2e-10
+
+
 # ---------------------------------------------------------------- full size (256^3, the benchmarked launch)
 def test_full_size_solve_meets_tolerance_independently_checked():
     p = W.config_c2(contrast=10.0, seed=1)
