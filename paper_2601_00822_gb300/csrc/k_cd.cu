@@ -587,7 +587,7 @@ static cudaError_t zcd_L(const CdArgs<R>& a, bool fwd, int batch, cudaStream_t s
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   count_launches(1);
-  return launch_chain(true, k, grid, ZCfg<L>::BLOCK, smem, st, a);
+  return launch_chain(chain_passes<R>(), k, grid, ZCfg<L>::BLOCK, smem, st, a);
 }
 
 template <typename R>

@@ -9,12 +9,22 @@ namespace bfcs {
 // Launch of a kernel that begins with chain_wait() (common.cuh), chained to its predecessor
 // when `chain` is set.  The Krylov loops chain their 8-10 launches per iteration (plain
 // stream launches with one-block kernels between the passes: a 128^3 solve by Algorithm 3
-// 38.9 -> 34.8 ms, a 64^3 FP64 solve by Algorithm 2 40.4 -> 37.7 ms); the sweeps do not:
+// 38.9 -> 34.8 ms, a 64^3 FP64 solve by Algorithm 2 36.0 -> 33.6 ms with the vectors and
+// scalars chained instead of everything); the sweeps do not:
 // their launches sit in CUDA graphs, whose gaps are small already, and blocks that wait on
 // an SM disturb the placement of the running pass (32^3 FP64 8.7 -> 11.0 ms, 64^3 3.54 ->
 // 3.66 ms, 256^3 121 -> 124 ms when chained).  The network chains all of its launches (26 a
 // forward pass of some microseconds each at 32^3): one 32^3 sample 242 -> 195 us, and 160
 // us with the layers' parameters loaded before the wait.
+//
+// Of an FP64 Krylov loop only the vector kernels and scalars are chained (chain_passes).
+// Blocks of a waiting pass take the slots that the running kernel leaves free, which are
+// on few SMs when it does not fill the chip, and the FP64 pipe of those SMs then bounds
+// the pass: Algorithm 2 at 64 x 64 x 32 takes 13.3 ms with the passes chained and 9.8 ms
+// without, Algorithm 3 there 17.4 and 12.9, 64^3 19.9 and 19.4; only 32 x 48 x 96 and
+// 24 x 32 x 128 lose, by 0-6 % (Algorithm 3).  The FP32 passes gain at every size measured
+// (24^3 to 128^3, 5-25 %).
+template <typename R> constexpr bool chain_passes() { return !std::is_same<R, double>::value; }
 template <class... P, class... A>
 cudaError_t launch_chain(bool chain, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                          const A&... a) {

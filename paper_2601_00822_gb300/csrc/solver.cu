@@ -1037,14 +1037,14 @@ int run_cg(SweepSet<R>& ss, std::vector<double>& req, int maxit, std::vector<int
   xa.spec_in = ca.p;
   xa.spec_out = ca.q;
   xa.st = P->cg_skip;
-  xa.chain = 1;
+  xa.chain = chain_passes<R>();
   CArgs<R> cy = ss.cy;
   cy.data = ca.q;   // not the mapped spectrum: the same tile with direct loads (tmap_data != data)
   cy.st = P->cg_skip;
   cy.ncomp = 6;
-  cy.chain = 1;
+  cy.chain = chain_passes<R>();
   GArgs<R> ga = ss.ga;
-  ga.chain = 1;
+  ga.chain = chain_passes<R>();
   ga.spec = ca.q;
   ga.st = P->cg_skip;
   ga.mode = GM_APPLY;
@@ -1170,7 +1170,7 @@ int run_cd(SweepSet<R>& ss, int maxit, bfcs_info* infos) {
   xs.st = P->cg_skip;
   cy.st = P->cg_skip;
   cz.st = P->cg_skip;
-  xs.chain = cy.chain = 1;
+  xs.chain = cy.chain = chain_passes<R>();
   int it = 0, chunk = 8;
   std::vector<double> obs_r(B, -1.0);
   std::vector<int> obs_it(B, -1);
