@@ -20,31 +20,38 @@
 
 namespace bfcs {
 
-// Vector kernels: blocks of 128 threads, one mode a thread, up to the eight blocks an SM
-// holds (kCgParts).  In FP64 they are bound by the FP64 pipe (about 45 operations a mode
+// Vector kernels.  In FP64 they are bound by the FP64 pipe (about 45 operations a mode
 // and two lanes an SM: 9.4 us at 64^3 when every SM has the same share), so the work has
-// to be even: 512 blocks of 256 (20 us a launch) gave some SMs four blocks and others three,
-// and 16 blocks a second round.  A 64^3 FP64 solve 37.8 -> 36.0 ms.
-constexpr int kCgThreads = 128;
+// to be even: blocks of 128 threads, one mode a thread, up to the eight blocks an SM holds.
+// 512 blocks of 256 (20 us a launch) gave some SMs four blocks and others three, and 16
+// blocks a second round.  A 64^3 FP64 solve 37.8 -> 36.0 ms.  FP32 vectors, bound by
+// memory, keep 512 blocks of 256.
+template <typename R> constexpr int cg_threads() { return sizeof(R) == 8 ? 128 : 256; }
 constexpr int kCgScalarThreads = 256;
 
-__device__ __forceinline__ float fma_r(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fma_r(double a, double b, double c) { return fma(a, b, c); }
-
-// Re(a : C0 : conj b) for the 6 tensorial components (xx yy zz yz xz xy), mu2 = 2 mu0, in the
+// Re(a : C0 : conj b) for the 6 tensorial components (xx yy zz yz xz xy), in the
 // vectors' precision (FP32 vectors: FP32 per mode; the caller sums 16 modes in R
 // and then adds in FP64: GB300's FP64 pipe would otherwise bound the vector kernels)
 template <typename R>
-__device__ __forceinline__ R c0dot(const C2<R> (&a)[6], const C2<R> (&b)[6], R lam0, R mu2) {
+__device__ __forceinline__ R c0dot(const C2<R> (&a)[6], const C2<R> (&b)[6], R lam0, R mu0) {
   const R ta_r = a[0].x + a[1].x + a[2].x, ta_i = a[0].y + a[1].y + a[2].y;
   const R tb_r = b[0].x + b[1].x + b[2].x, tb_i = b[0].y + b[1].y + b[2].y;
-  R s = R(0), o = R(0);
+  if constexpr (sizeof(R) == 8) {
+    double d = 0.0, o = 0.0;              // diagonal and shear terms apart: five operations less
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    s = fma_r(a[c].x, b[c].x, fma_r(a[c].y, b[c].y, s));
-    o = fma_r(a[c + 3].x, b[c + 3].x, fma_r(a[c + 3].y, b[c + 3].y, o));
+    for (int c = 0; c < 3; ++c) {
+      d = fma(a[c].x, b[c].x, fma(a[c].y, b[c].y, d));
+      o = fma(a[c + 3].x, b[c + 3].x, fma(a[c + 3].y, b[c + 3].y, o));
+    }
+    return fma(lam0, fma(ta_r, tb_r, ta_i * tb_i), 2.0 * mu0 * fma(2.0, o, d));
   }
-  return fma_r(lam0, fma_r(ta_r, tb_r, ta_i * tb_i), mu2 * fma_r(R(2), o, s));
+  R s = R(0);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const R w = c < 3 ? R(1) : R(2);
+    s += w * (a[c].x * b[c].x + a[c].y * b[c].y);
+  }
+  return lam0 * (ta_r * tb_r + ta_i * tb_i) + R(2) * mu0 * s;
 }
 
 __device__ __forceinline__ double block_reduce(double v, double* red) {
@@ -64,7 +71,7 @@ struct CgMode { enum : int { INIT = 0, PQ = 1, UPDATE = 2, DIR = 3 }; };
 // UPDATE: c += alpha p, r -= alpha q, partial <r, r>
 // DIR:    p = r + beta p
 template <typename R>
-__global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
+__global__ void __launch_bounds__(cg_threads<R>()) k_cg_vec(CgArgs<R> a, int mode) {
   const int m = blockIdx.y;
   chain_wait();
   if (a.cg[m].done) return;
@@ -76,15 +83,15 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
   C2<R>* p = a.p + off;
   C2<R>* q = a.q + off;
   const C2<R>* s = a.s != nullptr ? a.s + off : nullptr;
-  __shared__ R cst[4];          // alpha, beta, lam0, 2 mu0, converted once per block
+  __shared__ R cst[4];          // alpha, beta, lam0, mu0, converted once per block
   if (threadIdx.x == 0) {
     cst[0] = (R)a.cg[m].alpha;
     cst[1] = (R)a.cg[m].beta;
     cst[2] = (R)a.lam0;
-    cst[3] = (R)(2 * a.mu0);
+    cst[3] = (R)a.mu0;
   }
   __syncthreads();
-  const R alpha = cst[0], beta = cst[1], lam0 = cst[2], mu2 = cst[3];
+  const R alpha = cst[0], beta = cst[1], lam0 = cst[2], mu0 = cst[3];
   const long long modes = (long long)g.nz * g.ny * g.mx;
   // partial sums: 16 grid-stride modes in R (their products are R), then one FP64 add
   double acc = 0.0;
@@ -107,7 +114,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
           p[k * g.cs + gi] = x;
           u[k] = x;
         }
-        part += w * c0dot<R>(u, u, lam0, mu2);
+        part += w * c0dot<R>(u, u, lam0, mu0);
       } else if (mode == CgMode::PQ) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
@@ -115,7 +122,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
           v[k] = u[k] - q[k * g.cs + gi];
           q[k * g.cs + gi] = v[k];
         }
-        part += w * c0dot<R>(u, v, lam0, mu2);
+        part += w * c0dot<R>(u, v, lam0, mu0);
       } else if (mode == CgMode::UPDATE) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
@@ -123,7 +130,7 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_vec(CgArgs<R> a, int mode) {
           u[k] = r[k * g.cs + gi] - scale(q[k * g.cs + gi], alpha);
           r[k * g.cs + gi] = u[k];
         }
-        part += w * c0dot<R>(u, u, lam0, mu2);
+        part += w * c0dot<R>(u, u, lam0, mu0);
       } else {
 #pragma unroll
         for (int k = 0; k < 6; ++k) p[k * g.cs + gi] = r[k * g.cs + gi] + scale(p[k * g.cs + gi], beta);
@@ -182,8 +189,10 @@ static __global__ void k_cg_scalar(const double* part, int nparts, CgState* cg, 
 
 template <typename R>
 cudaError_t launch_cg_vec(const CgArgs<R>& a, int mode, int batch, cudaStream_t st) {
-  const int modes = a.g.nz * a.g.ny * a.g.mx, nparts = std::min(kCgParts, (modes + kCgThreads - 1) / kCgThreads);
-  cudaError_t e = launch_chain(true, k_cg_vec<R>, dim3(nparts, batch), kCgThreads, 0, st, a, mode);
+  constexpr int threads = cg_threads<R>();
+  const int modes = a.g.nz * a.g.ny * a.g.mx;
+  const int nparts = sizeof(R) == 8 ? std::min(kCgParts, (modes + threads - 1) / threads) : 512;
+  cudaError_t e = launch_chain(true, k_cg_vec<R>, dim3(nparts, batch), threads, 0, st, a, mode);
   count_launches(1);
   if (e != cudaSuccess || mode == CgMode::DIR) return e;
   count_launches(1);
