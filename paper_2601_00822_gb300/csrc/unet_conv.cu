@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kConv3Threads, C3<KC, N>::BLOCKS) k_conv3(Conv
     for (int k = 0; k < n; ++k) {
       bool ok = mbar_wait(full + 8 * (k & 1), (unsigned)((k >> 1) & 1), fail);
       if (ok && k >= 2) ok = mbar_wait(empty + 8 * (k & 1), (unsigned)(((k >> 1) - 1) & 1), fail);
-      if (__any_sync(0xffffffffu, !ok)) {
+      if (!ok) {
         if (lane == 0) { *fail = 1; atomicExch(err, 1); }
         break;
       }

@@ -32,18 +32,21 @@ __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
 __device__ __forceinline__ void mbar_arrive(unsigned bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
-// bounded wait for the phase of the given parity; gives up early once *fail is set
+// Bounded wait of a whole warp for the phase of the given parity; gives up early once *fail
+// is set.  The result is the same in all lanes (an expired limit in one of them counts for
+// all): the tensor-memory loads that follow a wait are warp-wide instructions.
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, volatile int* fail) {
   unsigned done = 0, spins = 0;
+  bool ok = true;
   while (!done) {
     asm volatile(
         "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
         : "=r"(done)
         : "r"(bar), "r"(parity)
         : "memory");
-    if (!done && (++spins > kTcSpinLimit || *fail)) return false;
+    if (!done && (++spins > kTcSpinLimit || *fail)) { ok = false; break; }
   }
-  return true;
+  return __all_sync(0xffffffffu, ok);
 }
 // barrier of the worker warps; true when the predicate held in all of them
 __device__ __forceinline__ bool workers_all(bool ok) {

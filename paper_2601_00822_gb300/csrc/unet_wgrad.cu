@@ -36,6 +36,7 @@
 // nine warps of mma.sync and sums over the blocks as a launch of their own.
 #include "unet_kernels.h"
 #include "unet_tc.cuh"
+#include "unet_wgrad_flow.h"
 
 #include <algorithm>
 
@@ -46,12 +47,9 @@ namespace {
 
 constexpr int kGX = 8, kGY = 16, kGV = kGX * kGY;     // tile (one z plane)
 constexpr int kGHY = kGY + 2;
-constexpr int kSeg = 8;                               // tiles per staged segment
 constexpr int kSlots = kSeg + 3;
 constexpr unsigned kXPlane = kGX * kGHY * 64;         // one staged plane: 8 x 18 voxels
 constexpr unsigned kYCopy = kGV * 64, kYTile = 3 * kYCopy;
-constexpr int kYRing = 3;
-constexpr int kFlush = 8;                             // tiles per accumulation in tensor memory
 constexpr unsigned kWgSmem = kSlots * kXPlane + kYRing * kYTile;
 constexpr unsigned kWgCols = 512;                     // TMEM allocation (3 x 96 columns used)
 constexpr int kXN = (kGX * kGHY * 4 + kTcWorkers - 1) / kTcWorkers;   // X copies per thread and plane
@@ -95,9 +93,6 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
   tc_after();
   const unsigned tmem = tmem_s;
 
-  // position of tile k in its segment: segments end after kSeg tiles or with the column
-  auto next_pos = [&](int z, int pos) { return z + 1 == nz || pos + 1 == kSeg ? 0 : pos + 1; };
-
   if (warp == 8) {
     // ---- MMA issue
     const unsigned tm = __shfl_sync(0xffffffffu, tmem, 0);
@@ -105,7 +100,7 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
     for (int k = 0; k < n; ++k) {
       bool ok = mbar_wait(full + 8 * (k & 1), (unsigned)((k >> 1) & 1), fail);
       if (ok && k > 0 && k % kFlush == 0) ok = mbar_wait(drained, (unsigned)((k / kFlush - 1) & 1), fail);
-      if (__any_sync(0xffffffffu, !ok)) {
+      if (!ok) {
         if (lane == 0) { *fail = 1; atomicExch(err, 1); }
         break;
       }
@@ -131,7 +126,7 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
                      : "memory");
       }
       __syncwarp();
-      pos = next_pos(z, pos);
+      pos = wg_next_pos(z, nz, pos);
       z = z + 1 == nz ? 0 : z + 1;
       yr = yr + 1 == kYRing ? 0 : yr + 1;
     }
@@ -190,40 +185,17 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
              (yvalid >> j) & 1u);
       }
     };
-    // Tile j's loads: at the start of a segment three planes, else one, and its dY; one
-    // copy group each.  They are requested up to three tiles ahead (two copies in flight
-    // under two tiles' MMAs: one tile ahead left the pass to the copies' latency, 4600
-    // clocks a tile), but not before the last reader of their slots is done: dY slot j % 3
-    // was read by tile j - 3, plane slot p + 2 of segment position p (and 0 and 1 for p =
-    // 0) last by position min(p + 2, L - 1) of the segment before, of length L.
-    struct Tile { long long col; int z, pos, prev; };  // prev: length of the segment before (0: none)
-    auto after = [&](Tile t) {
-      Tile u;
-      u.pos = next_pos(t.z, t.pos);
-      u.z = t.z + 1 == nz ? 0 : t.z + 1;
-      u.col = t.z + 1 == nz ? t.col + 1 : t.col;
-      u.prev = u.pos == 0 ? t.pos + 1 : t.prev;
-      return u;
-    };
-    auto last_reader = [&](Tile t, int j) { return t.prev == 0 ? -1 : j - t.pos - t.prev + min(t.pos + 2, t.prev - 1); };
-    long long lcol = t0 / nz;                          // column that the sources point to
-    Tile nt{lcol, (int)(t0 - lcol * nz), 0, 0};        // next tile to request, number `next`
-    int next = 0, nring = 0;
-    set_column(lcol);
-    auto request = [&]() {
-      if (nt.col != lcol) { set_column(nt.col); lcol = nt.col; }
-      if (nt.pos == 0) { load_x(nt.z - 1, 0); load_x(nt.z, 1); }
-      load_x(nt.z + 1, nt.pos + 2);
-      load_y(nt.z, nring);
+    set_column(t0 / nz);
+    auto request = [&](const WgTile& t, int slot) {
+      if (t.z == 0) set_column(t.col);                 // a new column
+      if (t.pos == 0) { load_x(t.z - 1, 0); load_x(t.z, 1); }
+      load_x(t.z + 1, t.pos + 2);
+      load_y(t.z, slot);
       cp_commit();
-      nt = after(nt);
-      ++next;
-      nring = nring + 1 == kYRing ? 0 : nring + 1;
     };
-    // tile j (the oldest copy group still of interest) has landed for this thread
-    auto landed = [&](int j) {
-      if (next - 1 - j >= 2) cp_wait<2>();
-      else if (next - 1 - j == 1) cp_wait<1>();
+    auto landed = [&](int younger) {
+      if (younger >= 2) cp_wait<2>();
+      else if (younger == 1) cp_wait<1>();
       else cp_wait<0>();
       fence_async();
     };
@@ -244,56 +216,30 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
         for (int q = 0; q < 8; ++q) bsum[q] += __bfloat162float(reinterpret_cast<const bf16*>(&v)[q]);
       }
     };
-    while (next < n && next < kYRing && last_reader(nt, next) < 0) request();
-    landed(0);
-    bool ok = workers_all(true);
-    if (tid == 0) mbar_arrive(full);
-    bias(0);
-    int ring = 0, phase = 0;                           // tile k's dY slot, the phase of its done barrier
-    for (int k = 0; k < n; ++k) {
-      const bool more = k + 1 < n, early = more && next > k + 1;
-      const int ring1 = ring + 1 == kYRing ? 0 : ring + 1;
-      if (early) {                                     // tile k + 1, requested before
-        landed(k + 1);
-        ok = workers_all(ok);
-        if (!ok) break;
-        if (tid == 0) mbar_arrive(full + 8 * ((k + 1) & 1));
-        bias(ring1);
-      }
-      ok = mbar_wait(done + 8 * ring, (unsigned)phase, fail) && ok;
+    auto publish = [&](int k) {
+      if (tid == 0) mbar_arrive(full + 8 * (k & 1));
+    };
+    auto wait_done = [&](int slot, int phase) {
+      const bool ok = mbar_wait(done + 8 * slot, (unsigned)phase, fail);
       if (!ok && lane == 0) { *fail = 1; atomicExch(err, 1); }
-      if (!more || (k + 1) % kFlush == 0) {            // the next tile's MMAs wait for this
-        if (ok && dz < 3) {
-          tc_after();
+      return ok;
+    };
+    auto drain = [&](bool ok) {
+      if (ok && dz < 3) {
+        tc_after();
 #pragma unroll
-          for (int i = 0; i < 9; ++i) {
-            unsigned v[16];
-            tmem_ld16(v, tmem + ((unsigned)(dz * 32) << 16) + 16u * (unsigned)(2 * i + (warp >> 2)));
+        for (int i = 0; i < 9; ++i) {
+          unsigned v[16];
+          tmem_ld16(v, tmem + ((unsigned)(dz * 32) << 16) + 16u * (unsigned)(2 * i + (warp >> 2)));
 #pragma unroll
-            for (int j = 0; j < 16; ++j) sum[i][j] += __uint_as_float(v[j]);
-          }
-          tc_before();
+          for (int j = 0; j < 16; ++j) sum[i][j] += __uint_as_float(v[j]);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(drained);
+        tc_before();
       }
-      // every thread has read the dY slots that are requested below (a step without the
-      // barrier above needs one here)
-      if (more && !early) ok = workers_all(ok);
-      if (ok)
-        while (next < n && next <= k + kYRing && last_reader(nt, next) <= k) request();
-      if (more && !early) {
-        landed(k + 1);
-        ok = workers_all(ok);
-        if (!ok) break;
-        if (tid == 0) mbar_arrive(full + 8 * ((k + 1) & 1));
-        bias(ring1);
-      }
-      ring = ring1;
-      if (ring == 0) phase ^= 1;
-    }
-    cp_wait<0>();
-    ok = workers_all(ok);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(drained);
+    };
+    const bool ok = wgrad3_workers(n, nz, t0, request, landed, workers_all, publish, bias, wait_done, drain);
     if (ok && blockIdx.y == 0) {                       // threads of a channel added in thread order
       float* red = reinterpret_cast<float*>(smem);     // [tid / 4][32] (every MMA and copy is done)
 #pragma unroll
