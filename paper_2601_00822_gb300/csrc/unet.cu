@@ -368,7 +368,7 @@ __device__ __forceinline__ ff exact_diff(float p, float t) {
   const float s = __fsub_rn(p, t), v = __fsub_rn(s, p);
   return ff_pair(s, __fsub_rn(__fsub_rn(p, __fsub_rn(s, v)), __fadd_rn(t, v)));
 }
-// the square of x and its rounding error stay inside the FP32 range (x finite)
+// the square of x and its rounding errors stay inside the FP32 range (x finite)
 __device__ __forceinline__ bool ff_square_safe(float x) {
   const float m = fabsf(x);
   return (m > 1e-11f && m < 1e15f) || m == 0.f;
@@ -383,12 +383,38 @@ __device__ __noinline__ void loss_terms_f64(const float* p, const float* t, doub
   }
 }
 __device__ __noinline__ float scaled_diff_f64(float p, float t, double f) { return (float)(((double)p - (double)t) * f); }
+// Sum of squares as three floats, each at most an ulp of the one before it: TwoSum carries
+// the rounding errors of the leading sum into the second and of that into the third, whose
+// own rounding is 2^-24 of 2^-47 of the sum.  A voxel's squares (products without rounding
+// from fused multiply-adds) come out to about 2^-68, so that their one rounding to FP64 is
+// all that differs from an exact sum; 6 FP64 operations for 12 squares.
+struct SqSum {
+  float a = 0.f, b = 0.f, c = 0.f;
+  static __device__ __forceinline__ float two_sum(float& s, float x) {
+    const float t = __fadd_rn(s, x), v = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(x, v));
+    s = t;
+    return e;
+  }
+  __device__ __forceinline__ void low(float x) { c = __fadd_rn(c, two_sum(b, x)); }
+  __device__ __forceinline__ void add(float x) {                       // x^2
+    const float q = __fmul_rn(x, x);
+    low(two_sum(a, q));
+    low(__fmaf_rn(x, x, -q));
+  }
+  __device__ __forceinline__ void add(ff x) {                          // (hi + lo)^2
+    add(x.hi);
+    const float h2 = __fadd_rn(x.hi, x.hi), q = __fmul_rn(h2, x.lo);
+    low(q);
+    c = __fadd_rn(c, __fmaf_rn(x.lo, x.lo, __fmaf_rn(h2, x.lo, -q)));
+  }
+  __device__ __forceinline__ double sum() const { return f2d_bits(a) + (f2d_bits(b) + f2d_bits(c)); }
+};
 // relative squared L2 loss: per (block, sample) sums of (p - t)^2 and t^2; one voxel
-// per thread, planar fields (6 x n a sample).  The six squares of a voxel are formed
-// and added in float-float (about 48 bits, FP32 pipes), voxels in FP64: with every
-// term on the FP64 pipe the pass took 143 us for 8 samples of 64^3 instead of the
-// 15 us its 100 MB take.  Voxels with values outside the range of that form (tiny, huge,
-// not finite) are formed in FP64.
+// per thread, planar fields (6 x n a sample).  The squares of a voxel are added in FP32
+// pieces without loss (SqSum), voxels in FP64: with every term on the FP64 pipe the pass
+// took 143 us for 8 samples of 64^3 instead of the 15 us its 100 MB take.  Voxels with
+// values outside the range of that form (tiny, huge, not finite) are formed in FP64.
 constexpr int kLossBlocks = 64;
 __global__ void k_loss(const float* pred, const float* target, long long n, double* num, double* den) {
   chain_wait();
@@ -398,7 +424,7 @@ __global__ void k_loss(const float* pred, const float* target, long long n, doub
   const float* tb = target + (long long)b * 6 * n;
   double sn = 0.0, sd = 0.0;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-    ff vn = ff(0.0f), vd = ff(0.0f);
+    SqSum vn, vd;
     float p6[6], t6[6];
     bool fast = true;
 #pragma unroll
@@ -406,13 +432,13 @@ __global__ void k_loss(const float* pred, const float* target, long long n, doub
       p6[c] = pb[c * n + v];
       t6[c] = tb[c * n + v];
       const ff d = exact_diff(p6[c], t6[c]);
-      vn = vn + d * d;
-      vd = vd + ff(t6[c]) * ff(t6[c]);
+      vn.add(d);
+      vd.add(t6[c]);
       fast = fast && ff_square_safe(d.hi) && ff_square_safe(t6[c]);
     }
     if (fast) {
-      sn += f2d_bits(vn.hi) + f2d_bits(vn.lo);
-      sd += f2d_bits(vd.hi) + f2d_bits(vd.lo);
+      sn += vn.sum();
+      sd += vd.sum();
     } else {
       double a0 = 0.0, a1 = 0.0;
       loss_terms_f64(p6, t6, a0, a1);

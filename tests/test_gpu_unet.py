@@ -8,6 +8,8 @@ Bars (relative L2): output <= 2e-2, loss <= 1e-2, each layer's weight and
 bias gradient <= 5e-2.  A wrong tap, transposed weight, missing bias or a
 skip connection in the wrong place gives errors of order 1.
 """
+from fractions import Fraction
+
 import numpy as np
 import pytest
 import torch
@@ -260,3 +262,30 @@ def test_captured_passes_equal_the_direct_ones(dims, batch):
             assert all(torch.equal(u, v) for u, v in zip(replayed, want))
         net.status()
         side.synchronize()
+
+
+def constant_output(bias):
+    """Parameters whose output is `bias` at every voxel (FP32, exactly): zero head weights."""
+    flat = params(51).float()
+    ws, bs = list(layer_slices())[-1][1:]
+    flat[ws] = 0.0
+    flat[bs] = torch.tensor(bias, dtype=torch.float32)
+    return flat.cuda()
+
+
+@pytest.mark.parametrize("n,roundings", [(8, 13), (64, 43)])
+def test_the_loss_is_summed_to_fp64(n, roundings):
+    """Constant output and target: every voxel has the same terms, so that what is lost on
+    one of them is lost on all, and the sums over voxels are multiples of one number.  Each
+    of the two sums rounds a voxel (2), k v for k up to the voxels of a thread (15 at 64^3)
+    and for 3, 5, 6, 7 warps; then the quotient: 2 (2 + 4) + 1 or 2 (2 + 15 + 4) + 1 roundings
+    of 2^-53.  The values are such that sums of 48 bits miss by 1.6e-14."""
+    p = [float.fromhex(v) for v in ("-0x1.5bd8e8p+0", "0x1.094478p+1", "0x1.78f4p+0", "-0x1.581092p-2",
+                                    "-0x1.85381ap-1", "0x1.1108bcp+0")]
+    q = [float.fromhex(v) for v in ("0x1.18d16ep-2", "-0x1.afdb24p-2", "0x1.c6bcb6p-10", "0x1.081ab6p-10",
+                                    "0x1.8f6894p-8", "-0x1.79607p-11")]
+    net = api.Net((n, n, n), max_batch=1, train=True)
+    t = torch.tensor(q, dtype=torch.float32, device="cuda").view(1, 6, 1, 1, 1).expand(1, 6, n, n, n).contiguous()
+    _, loss = net.grad(constant_output(p), inputs(52, 1, (n, n, n)).float().cuda(), t)
+    want = sum((Fraction(a) - Fraction(b)) ** 2 for a, b in zip(p, q)) / sum(Fraction(b) ** 2 for b in q)
+    assert abs(Fraction(float(loss)) - want) <= roundings * Fraction(1, 2 ** 53) * want
