@@ -482,9 +482,9 @@ __global__ void k_loss_final(const double* num, const double* den, int nblk, int
   }
 }
 // dL/dpred = 2 (p - t) / (den_b B), written as the head's output gradient
-// [B][N][16] BF16 (channels 6..15 zero); one voxel per thread; float-float products
-// (48 bits before the one rounding to FP32, where the FP64 form has 53; 155 us of FP64
-// pipe for 8 samples of 64^3), FP64 outside their range
+// [B][N][16] BF16 (channels 6..15 zero); one voxel per thread.  The product is rounded to
+// FP32 once; it comes from float-float arithmetic where that rounds as FP64 does (155 us of
+// FP64 pipe for 8 samples of 64^3 otherwise) and from FP64 where not, or outside its range
 __global__ void k_loss_grad(const float* pred, const float* target, const double* fac_b, long long n, bf16* dy) {
   chain_wait();
   const int b = blockIdx.y;
@@ -500,8 +500,8 @@ __global__ void k_loss_grad(const float* pred, const float* target, const double
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       const float p = pb[c * n + v], t = tb[c * n + v];
-      const ff d = exact_diff(p, t);
-      o[c] = __float2bfloat16(fast && ff_square_safe(d.hi) ? (float)(d * f) : scaled_diff_f64(p, t, fd));
+      const ff d = exact_diff(p, t), r = d * f;
+      o[c] = __float2bfloat16(fast && ff_square_safe(d.hi) && ff_rounds_as_fp64(r) ? r.hi : scaled_diff_f64(p, t, fd));
     }
     uint4* d = reinterpret_cast<uint4*>(dy + ((long long)b * n + v) * 16);
     d[0] = reinterpret_cast<const uint4*>(o)[0];

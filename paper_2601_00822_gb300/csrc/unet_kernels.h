@@ -51,6 +51,16 @@ __device__ __forceinline__ void gate8(__nv_bfloat162* o, uint4 y) {
     if (!(__bfloat162float(y8[k]) > 0.f)) o8[k] = __float2bfloat16(__bfloat162float(o8[k]) * kSlope);
 }
 
+// Whether r, a product of float-float arithmetic, rounds to FP32 (r.hi) as the product in
+// FP64 does: true unless the value lies within 2^-43 of a boundary between two floats.
+// The two products differ by less than 2^-44 (a factor cut to 47 bits, two roundings of
+// 2^-47 and the product of the low parts; the FP64 form rounds at 2^-53), so the few
+// values that fail (2^-18 of them) are formed in FP64 and every result is that of FP64.
+__device__ __forceinline__ bool ff_rounds_as_fp64(ff r) {
+  const float w = fabsf(r.hi) * 1.1368683772161603e-13f;   // 2^-43
+  return __fadd_rn(r.hi, __fadd_rn(r.lo, w)) == r.hi && __fadd_rn(r.hi, __fsub_rn(r.lo, w)) == r.hi;
+}
+
 constexpr int kSampleArgs = 64;      // samples whose pointers travel in one launch's arguments
 
 template <typename R> struct HeadArgs {

@@ -289,3 +289,19 @@ def test_the_loss_is_summed_to_fp64(n, roundings):
     _, loss = net.grad(constant_output(p), inputs(52, 1, (n, n, n)).float().cuda(), t)
     want = sum((Fraction(a) - Fraction(b)) ** 2 for a, b in zip(p, q)) / sum(Fraction(b) ** 2 for b in q)
     assert abs(Fraction(float(loss)) - want) <= roundings * Fraction(1, 2 ** 53) * want
+
+
+def test_the_loss_gradient_rounds_as_fp64_does():
+    """The loss gradient (p - t) 2 / den is rounded to FP32 and then to BF16.  Here the
+    product lies between a tie of two BF16 values and the next float, 2^-46 from where FP32
+    decides between them: 48 bits give the other neighbour.  512 voxels with the same value:
+    den and the head's bias gradient, 512 times the value, are exact."""
+    p, q = float.fromhex("0x1.429116p+7"), float.fromhex("0x1.23aaap-1")
+    net = api.Net((8, 8, 8), max_batch=1, train=True)
+    t = torch.zeros((1, 6, 8, 8, 8), device="cuda")
+    t[:, 5] = q
+    g, _ = net.grad(constant_output([p, 0.0, 0.0, 0.0, 0.0, q]), inputs(53, 1, (8, 8, 8)).float().cuda(), t)
+    want = torch.tensor(p * (2.0 / (512.0 * q * q)), dtype=torch.float64).float().to(torch.bfloat16).double()
+    bias = g[list(layer_slices())[-1][2]].double().cpu()
+    assert float(bias[0]) == 512.0 * float(want), (float(bias[0]) / 512.0, float(want))
+    assert torch.equal(bias[1:], torch.zeros(5, dtype=torch.float64))
