@@ -177,16 +177,17 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_head(HeadArgs<R> a) {
     fs = ff(fd);
     fast = fd > 1e-18 && fd < 1e18;
   }
-  // y s / mu_max.  FP32 fields: rounded once from about 48 bits (float-float); FP64
-  // multiplies and conversions of every value would bind the pass to the FP64 pipe (16
-  // us a 64^3 sample), so they serve only values whose product's parts could leave the
-  // FP32 range.
+  // y s / mu_max.  FP32 fields: from float-float arithmetic where it rounds as FP64 does;
+  // FP64 multiplies and conversions of every value would bind the pass to the FP64 pipe (16
+  // us a 64^3 sample), so they serve only the other values (one in 2^18) and those whose
+  // product's parts could leave the FP32 range.
   auto value = [&](float y) -> R {
     if constexpr (!PREDICT) return y;
     else if constexpr (sizeof(R) == 8) return (double)y * fd;
     else {
       const float m = fabsf(y);
-      return fast && ((m > 1e-12f && m < 1e15f) || m == 0.f) ? (float)(ff(y) * fs) : scaled_f64(y, fd);
+      const ff r = ff(y) * fs;
+      return fast && m > 1e-12f && m < 1e15f && ff_rounds_as_fp64(r) ? r.hi : scaled_f64(y, fd);
     }
   };
   const unsigned n = (unsigned)a.n;

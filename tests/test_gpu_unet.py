@@ -305,3 +305,18 @@ def test_the_loss_gradient_rounds_as_fp64_does():
     bias = g[list(layer_slices())[-1][2]].double().cpu()
     assert float(bias[0]) == 512.0 * float(want), (float(bias[0]) / 512.0, float(want))
     assert torch.equal(bias[1:], torch.zeros(5, dtype=torch.float64))
+
+
+@pytest.mark.parametrize("s,y", [("0x1.d16d7p-1", "0x1.98p+0"), ("0x1.8p+0", "-0x1.fffffep+3"), ("0x1.4p-30", "0x1.23456p-60"),
+                                 ("0x1.4p+20", "0x1.23456p-60")])
+def test_the_fp32_prediction_rounds_as_fp64_does(s, y):
+    """Predicted strain y s / mu_max, one FP64 product rounded to FP32.  The first
+    product lies 2^-47 from where FP32 decides between two values."""
+    s, y = float.fromhex(s), float.fromhex(y)
+    net = api.Net((8, 8, 8), max_batch=1)
+    b = torch.zeros((3, 8, 8, 8), device="cuda")
+    b[1, 2, 3, 4], b[1, 5, 3, 4] = s, -s
+    ph = torch.zeros((8, 8, 8), dtype=torch.int8, device="cuda")
+    got = net.predict(constant_output([y, -y, 0.5, y, y, y]), [b], [ph], [(1.0, 3.0)])[0].cpu()
+    want = torch.tensor([v * (s / 3.0) for v in (y, -y, 0.5, y, y, y)], dtype=torch.float64).float()
+    assert torch.equal(got.view(torch.int32), want.view(6, 1, 1, 1).expand(6, 8, 8, 8).contiguous().view(torch.int32))
