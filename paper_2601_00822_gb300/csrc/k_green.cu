@@ -14,6 +14,7 @@
 // The displacement consistent with eps^{s+1} is u_hat = i v (Eq. 2.9-2.10).
 // Modes with xi = 0: eps_hat = N E at k = 0 (prescribed mean strain), else 0.
 #include "kernels.h"
+#include "green_cols.h"
 
 #include <algorithm>
 #include <cstdlib>
@@ -800,20 +801,10 @@ cudaError_t launch_green_dense(C2<R>* spec, const C2<R>* bhat, C2<R>* dprev, con
 }
 
 // kx columns per block of the z pass for B members of grid g.  FP32: kGreenT (32-byte
-// sectors).  FP64: blocks that share an SM share its FP64 pipe, so the pass takes
-// (blocks on the busiest SM) x T; the widest T of least product.  32^3: 160 blocks of 4
-// columns put two on 8 of the 152 SMs, 288 of 2 columns the same work evenly.
+// sectors); FP64: see green_cols.h.
 template <typename R>
 static int green_cols(const Geo& g, int B) {
-  if (sizeof(R) == 4) return kGreenT;
-  int best = kGreenT;
-  long long cost = -1;
-  for (int T = kGreenT; T >= 1; T /= 2) {
-    const long long blocks = (long long)((g.mx + T - 1) / T) * g.ny * B;
-    const long long c = (blocks + sm_count() - 1) / sm_count() * T;
-    if (cost < 0 || c < cost) { cost = c; best = T; }
-  }
-  return best;
+  return sizeof(R) == 4 ? kGreenT : green_cols_fp64(g.mx, g.ny, B, sm_count());
 }
 
 template <typename R>
