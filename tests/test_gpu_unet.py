@@ -320,3 +320,141 @@ def test_the_fp32_prediction_rounds_as_fp64_does(s, y):
     got = net.predict(constant_output([y, -y, 0.5, y, y, y]), [b], [ph], [(1.0, 3.0)])[0].cpu()
     want = torch.tensor([v * (s / 3.0) for v in (y, -y, 0.5, y, y, y)], dtype=torch.float64).float()
     assert torch.equal(got.view(torch.int32), want.view(6, 1, 1, 1).expand(6, 8, 8, 8).contiguous().view(torch.int32))
+
+
+def layer_spans():
+    return {name: (ws, bs) for name, ws, bs in layer_slices()}
+
+
+def set_identity(flat, name, cin, cout=32, first=0):
+    """Layer `name` passes its input channels first .. first + cout - 1 through unchanged: the
+    centre tap of a 3^3 layer, every sub-voxel of an up-convolution, the six rows of the head."""
+    ws, bs = layer_spans()[name]
+    w = torch.zeros_like(flat[ws])
+    if name.startswith("u"):
+        w.view(cin, cout, 8)[first:first + cout][torch.arange(cout), torch.arange(cout)] = 1.0
+    elif name == "head":
+        w.view(6, 32)[torch.arange(min(6, 32 - first)), first + torch.arange(min(6, 32 - first))] = 1.0
+    else:
+        w.view(cout, cin, 27)[torch.arange(cout), first + torch.arange(cout), 13] = 1.0
+    flat[ws] = w
+    flat[bs] = 0.0
+
+
+def pass_through_from(flat, level):
+    """Everything after the up-convolution of `level` hands its output on: the decoder's
+    convolutions and the finer up-convolutions are identities (for positive values)."""
+    for k in range(level, -1, -1):
+        set_identity(flat, f"d{k}a", 64)
+        set_identity(flat, f"d{k}b", 32)
+        if k > 0:
+            set_identity(flat, f"u{k - 1}", 32)
+
+
+def read_channels(net, flat, x, level):
+    """The 32 channels that reach the head, at the resolution of `level` (replicated above it)."""
+    out = []
+    for first in range(0, 32, 6):
+        f = flat.clone()
+        set_identity(f, "head", 32, first=first)
+        y = net.forward(f.cuda(), x).double().cpu()
+        out.append(y[:, :min(6, 32 - first)])
+    s = 2 ** level
+    y = torch.cat(out, 1)
+    return y[:, :, ::s, ::s, ::s]
+
+
+@pytest.mark.parametrize("dims,batch", [((8, 8, 8), 1), ((24, 16, 8), 3), ((40, 8, 24), 2)])
+@pytest.mark.parametrize("level", [2, 1, 0])
+def test_pointwise_layers_against_fp64_sums(dims, batch, level):
+    """The up-convolutions and the head against FP64 sums of the BF16 operands that they get
+    (rows in numbers that are no multiples of a warp's 32 or a block's 256 at levels 2 and 1).
+    With identities after the up-convolution of `level` the output shows what it writes, and
+    with an identity in its place what it reads.  Values stay positive, so that no activation
+    or its derivative changes them.  Forward: rounded to BF16 from an FP32 sum of up to 48
+    products within 1e-5.  Weight and bias gradients: FP32 sums of BF16 products, 1e-5.  The gradient it hands down, rounded to
+    BF16 (a few values the other way), through the bias gradient of the layer below: 1e-3."""
+    cin = 48 if level == 2 else 32
+    below = {2: "e3b", 1: "d2b", 0: "d1b"}[level]
+    g = torch.Generator().manual_seed(60 + level)
+    flat = params(61).float()
+    ws, bs = layer_spans()[f"u{level}"]
+    pass_through_from(flat, level)
+    flat[layer_spans()[below][1]] += 8.0
+    w = (torch.rand(cin, 32, 8, generator=g) * 0.1 - 0.05).float()
+    bias = 40.0 + torch.rand(32, generator=g)
+    x = inputs(62, batch, dims).float().cuda()
+    t = (40.0 + 4.0 * inputs(63, batch, dims, ch=6)).float()
+    net = api.Net(dims, max_batch=batch, train=True)
+    # what the layer reads, 32 channels at a time
+    got_in = []
+    for first in range(0, cin, 16 if cin == 48 else 32):
+        if first + 32 > cin:
+            break
+        f = flat.clone()
+        set_identity(f, f"u{level}", cin, first=first)
+        got_in.append(read_channels(net, f, x, level + 1))
+    u = got_in[0] if cin == 32 else torch.cat([got_in[0], got_in[1][:, 16:]], 1)
+    assert (u > 0).all()
+    # what it writes
+    flat[ws] = w.reshape(-1)
+    flat[bs] = bias
+    wb = bf16(w)
+    nz, ny, nx = u.shape[2:]
+
+    def spread(v):                                   # (b, 32, 8, z, y, x) -> fine grid
+        return v.view(batch, 32, 2, 2, 2, nz, ny, nx).permute(0, 1, 5, 2, 6, 3, 7, 4).reshape(batch, 32, 2 * nz, 2 * ny, 2 * nx)
+
+    want = spread(torch.einsum("bizyx,ico->bcozyx", u, wb) + bias.double().view(1, 32, 1, 1, 1, 1))
+    got = read_channels(net, flat, x, level)
+    assert ((bf16(want * (1 - 1e-5)) <= got) & (got <= bf16(want * (1 + 1e-5)))).all()
+    # the head with weights of its own, on what reaches it
+    fine = got
+    for _ in range(level):
+        fine = fine.repeat_interleave(2, 2).repeat_interleave(2, 3).repeat_interleave(2, 4)
+    f = flat.clone()
+    hw = (torch.rand(6, 32, generator=g) - 0.5).float()
+    f[layer_spans()["head"][0]] = hw.reshape(-1)
+    y = net.forward(f.cuda(), x).double().cpu()
+    want = torch.einsum("bczyx,hc->bhzyx", fine, bf16(hw)) + f[layer_spans()["head"][1]].double().view(1, 6, 1, 1, 1)
+    assert ((y - want).abs() <= 1e-5 * torch.einsum("bczyx,hc->bhzyx", fine, bf16(hw).abs())).all()
+    # gradients with the head on six of the channels
+    set_identity(f, "head", 32, first=13)
+    y = net.forward(f.cuda(), x).double().cpu()
+    grad, _ = net.grad(f.cuda(), x, t.cuda())
+    grad = grad.double().cpu()
+    d = y - t.double()
+    den = (t.double() ** 2).sum((1, 2, 3, 4)).view(-1, 1, 1, 1, 1)
+    dout = bf16((d * (2.0 / (den * batch))).float())
+    assert rel(grad[layer_spans()["head"][1]], dout.sum((0, 2, 3, 4))) <= 1e-5
+    assert rel(grad[layer_spans()["head"][0]], torch.einsum("bhzyx,bczyx->hc", dout, fine)) <= 1e-5
+    dy = torch.zeros_like(fine)
+    dy[:, 13:19] = dout
+    for _ in range(level):                           # the identity up-convolutions add their eight sub-voxels
+        b_, c_, z_, y_, x_ = dy.shape
+        dy = bf16(dy.view(b_, c_, z_ // 2, 2, y_ // 2, 2, x_ // 2, 2).sum((3, 5, 7)).float())
+    dyo = dy.view(batch, 32, nz, 2, ny, 2, nx, 2).permute(0, 1, 3, 5, 7, 2, 4, 6).reshape(batch, 32, 8, nz, ny, nx)
+    assert rel(grad[bs], dy.sum((0, 2, 3, 4))) <= 1e-5
+    assert rel(grad[ws], torch.einsum("bcozyx,bizyx->ico", dyo, u)) <= 1e-5
+    du = bf16(torch.einsum("bcozyx,ico->bizyx", dyo, wb).float())
+    assert rel(grad[layer_spans()[below][1]], du.sum((0, 2, 3, 4))) <= 1e-3
+    net.status()
+
+
+def test_batches_beyond_one_launch_of_pointers():
+    """More samples than travel in one launch's arguments (64), and predictions of more
+    samples than the context holds: equal to smaller batches bit for bit."""
+    dims, n = (8, 8, 8), 70
+    r = np.random.default_rng(71)
+    flat = params(72).float().cuda()
+    x = inputs(73, n, dims).float().cuda()
+    b = [torch.tensor(r.standard_normal((3, 8, 8, 8)), dtype=torch.float32, device="cuda") for _ in range(n)]
+    ph = [torch.tensor(r.integers(0, 2, (8, 8, 8)), dtype=torch.int8, device="cuda") for _ in range(n)]
+    phases = [(1.0, 0.5), (0.3, 2.0)]
+    big, small = api.Net(dims, max_batch=n), api.Net(dims, max_batch=9)
+    want = torch.cat([small.forward(flat, x[i:i + 9]) for i in range(0, n, 9)])
+    assert torch.equal(big.forward(flat, x), want)
+    alone = [small.predict(flat, [bi], [pi], phases)[0].clone() for bi, pi in zip(b, ph)]
+    for net in (big, small):
+        assert all(torch.equal(p, a) for p, a in zip(net.predict(flat, b, ph, phases), alone))
+        net.status()
