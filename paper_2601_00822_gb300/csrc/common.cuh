@@ -123,7 +123,6 @@ template <typename R> __device__ __forceinline__ C2<R> operator-(C2<R> a, C2<R> 
 template <typename R> __device__ __forceinline__ C2<R> cmul(C2<R> a, C2<R> b) {
   return mk<R>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-template <typename R> __device__ __forceinline__ C2<R> conjg(C2<R> a) { return mk<R>(a.x, -a.y); }
 template <typename R> __device__ __forceinline__ C2<R> scale(C2<R> a, R s) { return mk<R>(a.x * s, a.y * s); }
 // multiply by dir * i, dir = +-1
 template <typename R, int DIR> __device__ __forceinline__ C2<R> mul_di(C2<R> a) {
@@ -295,7 +294,8 @@ template <int L> struct LineInfo {
 // (one 128-byte line per warp load, where the strided W^((4 n2 a) mod L) spans up
 // to 12).  The values equal the entries W^((n2 b) mod L), W^((4 n2 a) mod L).
 // One block per eligible radix of the line (Fac<L>::R1, then Fac<L>::R2 if it
-// differs) in float and double tables.  Float-float tables, where a product costs
+// differs) in float and double tables; the double kernels, bound by their arithmetic
+// pipe, take the entries W^j as they are.  Float-float tables, where a product costs
 // more than a load, hold instead the block [k1 - 1][n2] = W^((n2 k1) mod L),
 // k1 = 1..R1-1, n2 < L/R1, for R1 = Fac<L>::R1.
 constexpr bool tw_factored(int r1) { return r1 % 4 == 0 && r1 >= 8; }

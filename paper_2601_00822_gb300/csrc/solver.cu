@@ -163,8 +163,9 @@ static void line_radices(int n, int& r1, int& r2) {
   }
 }
 
-// Twiddles W^j = exp(-2 pi i j / n), j < n, then (FP32 and FP64 tables) the
-// factored stage-1 blocks that tw_offset / stage1f read: for each eligible
+// Twiddles W^j = exp(-2 pi i j / n), j < n, then (FP32 and FP64 tables; the FP64
+// kernels read the entries W^j alone) the factored stage-1 blocks that tw_offset /
+// stage1f read: for each eligible
 // first radix r (Fac<n>::R1, then Fac<n>::R2 if it differs), entries
 // [b - 1][n2] = W^((n2 b) mod n), b = 1..3, and [a + 2][n2] = W^((4 n2 a) mod n),
 // a = 1..r/4-1, for n2 < n / r; float-float tables instead [k1 - 1][n2] =
@@ -475,14 +476,13 @@ struct SweepSet {
   int B = 0;
   double tol = 0.0;
   bfcs_lame C0{};
-  const double* E0 = nullptr;
   int maxdim = 0;
   GArgs<R> ga{};
   CArgs<R> cy{};
   XArgs<R> xa{};
 
-  void prepare(bfcs_plan plan, int batch, const PhaseTab<R>& tab, bfcs_lame c0, const double* e0, double t) {
-    P = plan; B = batch; tol = t; C0 = c0; E0 = e0;
+  void prepare(bfcs_plan plan, int batch, const PhaseTab<R>& tab, bfcs_lame c0, double t) {
+    P = plan; B = batch; tol = t; C0 = c0;
     const Geo g = P->g;
     maxdim = std::max(g.nx, std::max(g.ny, g.nz));
     const long long sms = 6 * g.cs;
@@ -1242,10 +1242,10 @@ int run_cd(SweepSet<R>& ss, int maxit, bfcs_info* infos) {
 // start, whose residual is not evaluated); rounds repeat while they at least
 // halve the residual, then plain sweeps finish the job.
 template <typename R>
-int run_batch(bfcs_plan P, int B, const PhaseTab<R>& tab, bfcs_lame C0, const double* E0, double tol,
-              int maxit, bfcs_info* infos, bool any_warm, bool u_only = false) {
+int run_batch(bfcs_plan P, int B, const PhaseTab<R>& tab, bfcs_lame C0, double tol, int maxit,
+              bfcs_info* infos, bool any_warm, bool u_only = false) {
   SweepSet<R> ss;
-  ss.prepare(P, B, tab, C0, E0, tol);
+  ss.prepare(P, B, tab, C0, tol);
   ss.u_only = u_only;
   if (P->use_cd && any_warm) return BFCS_ERR_INVALID_ARG;   // Algorithm 3 starts from u1 = 0
   int e = ss.init(any_warm);
@@ -1340,7 +1340,7 @@ int solve_core(bfcs_plan P, const int8_t* phase, const PhaseTab<R>& tab, bfcs_la
   const Member m = make_member(phase, shift, E, nullptr, eps_init, out);
   int e = upload_members(P, 1, &m);
   if (e != BFCS_OK) return e;
-  return run_batch<R>(P, 1, tab, C0, E, tol, maxit, info, eps_init != nullptr);
+  return run_batch<R>(P, 1, tab, C0, tol, maxit, info, eps_init != nullptr);
 }
 
 template <typename R>
@@ -1360,7 +1360,7 @@ int solve_impl(bfcs_plan P, const int8_t* phase, int nph, const bfcs_lame* phase
   if (e != BFCS_OK) return e;
   e = transform_members<R>(P, 1);
   if (e != BFCS_OK) return e;
-  return run_batch<R>(P, 1, make_tab<R>(nph, phases, C0), C0, E, tol, maxit, info, eps_init != nullptr);
+  return run_batch<R>(P, 1, make_tab<R>(nph, phases, C0), C0, tol, maxit, info, eps_init != nullptr);
 }
 
 // bfcs_solve_batched on FP32/FP64 plans: groups of up to max_batch members
@@ -1399,7 +1399,7 @@ int solve_batch_impl(bfcs_plan P, int batch, const bfcs_problem* pr, int nph, co
     if (e != BFCS_OK) return e;
     e = transform_members<R>(P, B);
     if (e != BFCS_OK) return e;
-    const int s = run_batch<R>(P, B, tab, C0, pr[start].E, tol, maxit, infos != nullptr ? infos + start : nullptr,
+    const int s = run_batch<R>(P, B, tab, C0, tol, maxit, infos != nullptr ? infos + start : nullptr,
                                warm);
     if (s < 0) return s;
     if (severity(s) > severity(worst)) worst = s;
@@ -1443,7 +1443,7 @@ int solve_group_impl(int n, const bfcs_group_item* items, int nph, const bfcs_la
     if (e != BFCS_OK) return e;
     e = transform_members<R>(P, B);
     if (e != BFCS_OK) return e;
-    sets[i].prepare(P, B, tab, C0, pr[0].E, tol);
+    sets[i].prepare(P, B, tab, C0, tol);
     e = sets[i].init(warm);
     if (e != BFCS_OK) return e;
     ptrs.push_back(&sets[i]);
@@ -1671,7 +1671,7 @@ int solve_mixed_batch(bfcs_plan P, int B, const Member* in, int nph, const bfcs_
   e = upload_members(P, B, mem.data());
   if (e != BFCS_OK) return e;
   // (the ladder's FP32 solves need the displacement and strain only: no final pass)
-  const int s1 = run_batch<float>(P, B, tab32, C0, in[0].E, std::max(tol, P->switch_tol), maxit, inf.data(),
+  const int s1 = run_batch<float>(P, B, tab32, C0, std::max(tol, P->switch_tol), maxit, inf.data(),
                                   any_warm, true);
   if (s1 < 0) return s1;
   F2dArgs fa{};
@@ -1731,7 +1731,7 @@ int solve_mixed_batch(bfcs_plan P, int B, const Member* in, int nph, const bfcs_
     CK(launch_bden<float>(bhat32, g, P->part, P->ist, st, k, 3 * cs));
     e = upload_members(P, k, mem.data());
     if (e != BFCS_OK) return e;
-    const int s2 = run_batch<float>(P, k, tab32, C0, zeroE, 0.5, std::max(left, 1), inf.data(), false, true);
+    const int s2 = run_batch<float>(P, k, tab32, C0, 0.5, std::max(left, 1), inf.data(), false, true);
     if (s2 < 0) return s2;
     F2dArgs fe{};
     for (int j = 0; j < k; ++j) {
@@ -1852,7 +1852,7 @@ int average_impl(bfcs_plan P, int count, const AvgMembers& am, int nph, const bf
     if (e != BFCS_OK) return e;
     e = transform_members<R>(P, B);            // b is fixed (Eq. 3.4)
     if (e != BFCS_OK) return e;
-    const int s = run_batch<R>(P, B, tab, C0, E, tol, maxit, infos != nullptr ? infos + start : nullptr, false);
+    const int s = run_batch<R>(P, B, tab, C0, tol, maxit, infos != nullptr ? infos + start : nullptr, false);
     if (s < 0) return s;
     if (severity(s) > severity(worst)) worst = s;
     AccArgs<R> aa{};

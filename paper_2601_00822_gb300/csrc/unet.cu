@@ -12,10 +12,11 @@
 // Activations are channels-last [b][z][y][x][c] BF16.  Convolutions are
 // implicit GEMMs on the tensor cores: rows = voxels, columns = output channels,
 // K = taps x input channels (3^3 layers: tcgen05, unet_conv.cu; pointwise
-// layers: unet_gemm.cu).  The weight gradient is a second GEMM (rows = output
-// channels, columns = input channels, K = voxels) staged through shared memory
-// with ldmatrix.trans, split over voxel chunks and reduced in a fixed order
-// (deterministic).
+// layers: unet_gemm.cu).  A weight gradient is a second GEMM (rows = output channels,
+// columns = input channels, K = voxels): tcgen05 for the 3^3 layers with 32 output
+// channels, mma.sync for the pointwise ones (unet_wgrad.cu) and for the two 48-channel
+// layers (k_wgrad below).  Each block sums a run of voxels, and the blocks' partial sums are
+// added in a fixed order (deterministic).
 #include "bfcs.h"
 #include "unet_kernels.h"
 
@@ -34,21 +35,6 @@ __device__ __forceinline__ unsigned ld32(const bf16* p) { return *reinterpret_ca
 // fine voxel offset of sub-voxel o = 4 oz + 2 oy + ox on a grid of pitch (FX, FY)
 __device__ __forceinline__ long long sub_off(int o, int FX, int FY) {
   return ((long long)(o >> 2) * FY + ((o >> 1) & 1)) * FX + (o & 1);
-}
-
-__device__ __forceinline__ void mma16816(float* c, const unsigned* a, const unsigned* b) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-__device__ __forceinline__ void ldsm_x4_trans(unsigned* r, const void* smem_row) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(smem_row);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(a));
 }
 
 // ------------------------------------------------------------------ convolution (forward / data gradient)
@@ -104,9 +90,9 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
       for (int j = 0; j < kConvNT; ++j) {
         if (j < ntiles) {
           const bf16* wr = wt + (long long)(col0 + j * 8 + g) * a.cin + kc + 2 * t;
-          const unsigned bfr[2] = {ld32(wr), ld32(wr + 8)};
-          mma16816(acc[0][j], af[0], bfr);
-          mma16816(acc[1][j], af[1], bfr);
+          const unsigned b0 = ld32(wr), b1 = ld32(wr + 8);
+          mma16816(acc[0][j], af[0], b0, b1);
+          mma16816(acc[1][j], af[1], b0, b1);
         }
       }
     }
@@ -143,34 +129,29 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(ConvArgs a) {
 }
 
 // ------------------------------------------------------------------ weight gradient
-// dW[tap][co][ci] = sum over (b, v) of dY[b][v][co] X[b][v + d_tap][ci]; for an
-// up-convolution (up_c > 0) dW[o up_c + co][ci] = sum over (b, u) of
-// dY[b][2u + o][co] X[b][u][ci] with dY read from the fine grid.
-// Block (chunk, tap x mchunk): voxels [chunk * rows_per, ...), 64 output
-// channels; partial[chunk][tap][cout_p][cin] in FP32.
+// dW[tap][co][ci] = sum over (b, v) of dY[b][v][co] X[b][v + d_tap][ci] of a 3^3 layer on the
+// warp-level tensor cores: the 48-channel layers (0.2% of a gradient's products), and every
+// 3^3 layer with BFCS_NET_TCGEN05=0.  Block (chunk, tap): voxels [chunk * rows_per, ...);
+// partial[chunk][tap][cout_p][cin] in FP32.
 constexpr int kWgRows = 64;
 
 __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
   chain_wait();
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int mcols = min(64, a.cout_p);
-  const int mchunks = a.cout_p / mcols;
-  const int tap = blockIdx.y / mchunks, mc = blockIdx.y - tap * mchunks;
-  const int taps = gridDim.y / mchunks;
-  const int CP = mcols + 8, XP = a.cin + 8;         // row pitches: 16-byte multiples, conflict-free ldmatrix
+  const int tap = blockIdx.y;
+  const int CP = a.cout_p + 8, XP = a.cin + 8;      // row pitches: 16-byte multiples, conflict-free ldmatrix
   bf16* sD = reinterpret_cast<bf16*>(smraw);        // [64][CP]
   bf16* sX = sD + kWgRows * CP;                     // [64][XP]
-  const int dz = a.ksize == 3 ? tap / 9 - 1 : 0, dy = a.ksize == 3 ? (tap / 3) % 3 - 1 : 0,
-            dx = a.ksize == 3 ? tap % 3 - 1 : 0;
+  const unsigned sDa = (unsigned)__cvta_generic_to_shared(sD), sXa = (unsigned)__cvta_generic_to_shared(sX);
+  const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
   const long long nvox = (long long)a.v.nx * a.v.ny * a.v.nz;
   const long long total = nvox * a.batch;
   const long long start = (long long)blockIdx.x * a.chunk;
   const long long stop = min(start + a.chunk, total);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int mt = mcols / 16;
-  const int FX = 2 * a.v.nx, FY = 2 * a.v.ny;
+  const int mt = a.cout_p / 16;
   float sum[4][4][4] = {};                          // [m16 tile][n8 tile of this warp][4]
-  const int dvec = mcols / 8, xvec = a.cin / 8;
+  const int dvec = a.cout_p / 8, xvec = a.cin / 8;
   for (long long r0 = start; r0 < stop; r0 += kWgRows) {
     __syncthreads();
     for (int idx = threadIdx.x; idx < kWgRows * (dvec + xvec); idx += blockDim.x) {
@@ -178,20 +159,13 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
       const long long gr = r0 + row;
       uint4 val = make_uint4(0u, 0u, 0u, 0u);
       if (gr < stop) {
-        const long long b = gr / nvox;
-        const long long vv = gr - b * nvox;
-        const int x = (int)(vv % a.v.nx), y = (int)((vv / a.v.nx) % a.v.ny),
-                  z = (int)(vv / ((long long)a.v.nx * a.v.ny));
         if (cv < dvec) {
-          const int col = mc * mcols + cv * 8;
-          if (a.up_c > 0) {
-            const int o = col / a.up_c, c = col - o * a.up_c;
-            const long long fv = ((long long)(2 * z) * FY + 2 * y) * FX + 2 * x + sub_off(o, FX, FY);
-            val = *reinterpret_cast<const uint4*>(a.dy + (b * nvox * 8 + fv) * a.ldd + a.offd + c);
-          } else {
-            val = *reinterpret_cast<const uint4*>(a.dy + gr * a.ldd + a.offd + col);
-          }
+          val = *reinterpret_cast<const uint4*>(a.dy + gr * a.ldd + a.offd + cv * 8);
         } else {
+          const long long b = gr / nvox;
+          const long long vv = gr - b * nvox;
+          const int x = (int)(vv % a.v.nx), y = (int)((vv / a.v.nx) % a.v.ny),
+                    z = (int)(vv / ((long long)a.v.nx * a.v.ny));
           const long long nb = ((long long)wrap(z + dz, a.v.nz) * a.v.ny + wrap(y + dy, a.v.ny)) * a.v.nx +
                                wrap(x + dx, a.v.nx);
           val = *reinterpret_cast<const uint4*>(a.x + (b * nvox + nb) * a.ldx + a.offx + (cv - dvec) * 8);
@@ -212,21 +186,19 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         const int n0 = (warp + 4 * p) * 16;
-        if (n0 < a.cin) ldsm_x4_trans(bq[p], sX + (ks + (mi & 1) * 8 + rr) * XP + n0 + (mi >> 1) * 8);
+        if (n0 < a.cin) ldsm_x4_trans(bq[p], sXa + 2u * ((ks + (mi & 1) * 8 + rr) * XP + n0 + (mi >> 1) * 8));
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         if (i >= mt) continue;
         unsigned af[4];
-        ldsm_x4_trans(af, sD + (ks + (mi >> 1) * 8 + rr) * CP + i * 16 + (mi & 1) * 8);
+        ldsm_x4_trans(af, sDa + 2u * ((ks + (mi >> 1) * 8 + rr) * CP + i * 16 + (mi & 1) * 8));
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
           const int n0 = (warp + 4 * p) * 16;
           if (n0 < a.cin) {
-            const unsigned b0[2] = {bq[p][0], bq[p][1]};
-            const unsigned b1[2] = {bq[p][2], bq[p][3]};
-            mma16816(acc[i][2 * p], af, b0);
-            mma16816(acc[i][2 * p + 1], af, b1);
+            mma16816(acc[i][2 * p], af, bq[p][0], bq[p][1]);
+            mma16816(acc[i][2 * p + 1], af, bq[p][2], bq[p][3]);
           }
         }
       }
@@ -239,7 +211,7 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
         for (int q = 0; q < 4; ++q) sum[i][j][q] += acc[i][j][q];
   }
   const int g = lane >> 2, t = lane & 3;
-  float* out = a.part + ((long long)blockIdx.x * taps + tap) * a.cout_p * a.cin;
+  float* out = a.part + ((long long)blockIdx.x * 27 + tap) * a.cout_p * a.cin;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     if (i >= mt) continue;
@@ -250,7 +222,7 @@ __global__ void __launch_bounds__(128) k_wgrad(WgArgs a) {
         const int n0 = (warp + 4 * p) * 16 + h * 8;
         if (n0 >= a.cin) continue;
         const float* c = sum[i][2 * p + h];
-        const int co = mc * mcols + i * 16 + g, ci = n0 + 2 * t;
+        const int co = i * 16 + g, ci = n0 + 2 * t;
         out[(long long)co * a.cin + ci] = c[0];
         out[(long long)co * a.cin + ci + 1] = c[1];
         out[(long long)(co + 8) * a.cin + ci] = c[2];
@@ -742,7 +714,6 @@ cudaError_t pack_all(bfcs_net_s* N, const float* params) {
   return cudaGetLastError();
 }
 
-// forward GEMM of layer l: in -> out on the grid of level lv (coarse level for an up layer)
 int sm_count() {
   static int n = 0;
   if (n == 0) {
@@ -770,6 +741,7 @@ cudaError_t launch_conv(const ConvArgs& a, long long nvox, int* err, cudaStream_
   return cudaGetLastError();
 }
 
+// forward GEMM of layer l: in -> out on the grid of level lv (coarse level for an up layer)
 cudaError_t conv_fwd(bfcs_net_s* N, int l, const float* params, int B, View in, int lv, int out_mode, void* out,
                      int ldo, int offo) {
   const LayerDef& L = N->def[l];
@@ -780,7 +752,6 @@ cudaError_t conv_fwd(bfcs_net_s* N, int l, const float* params, int B, View in, 
   a.bias = params + L.boff;
   a.bias_mod = L.cout;
   a.cout_p = L.kind == 2 ? 8 * L.cout : L.cout_p;
-  a.cout = L.kind == 1 ? L.cout : a.cout_p;
   a.ksize = L.kind == 0 ? 3 : 1;
   a.v = N->vol[lv];
   a.batch = B;
@@ -864,8 +835,6 @@ cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View 
   const bool up = L.kind == 2;
   const int taps = L.kind == 0 ? 27 : 1;
   const long long rows = N->n[lv] * B;                  // GEMM K rows of the weight gradient
-  const long long orows = up ? rows * 8 : rows;         // rows of the output gradient
-  const int dch = up ? L.cout : L.cout_p;               // channels of the output gradient view
   // weight gradient
   WgArgs w{};
   w.dy = dout.p; w.ldd = dout.ld; w.offd = dout.off;
@@ -876,18 +845,22 @@ cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View 
   w.v = N->vol[lv];
   w.batch = B;
   w.up_c = up ? L.cout : 0;
-  const int mchunks = w.cout_p > 64 ? w.cout_p / 64 : 1;
-  const int want = 152 * 8;
-  int nchunks = std::max(1, std::min(ceil_div(want, taps * mchunks), ceil_div(rows, kWgRows)));
-  w.chunk = (long long)ceil_div(ceil_div(rows, nchunks), kWgRows) * kWgRows;
-  nchunks = ceil_div(rows, w.chunk);
   const long long per = (long long)taps * w.cout_p * w.cin;
-  const int bc = dch;
+  const int bc = up ? L.cout : L.cout_p;                // channels of the output gradient view
   const bool tc = wgrad3_ok(w) && tcgen05_enabled(), pw = wgrad1_ok(w);
-  if (tc) nchunks = wgrad3_chunks(w, sm_count());
-  else if (pw) nchunks = wgrad1_chunks(w, sm_count());
-  const int nblk = tc ? nchunks : pw ? (up ? nchunks / 2 : nchunks)
-                                     : std::max(1, std::min(kBiasBlocks, ceil_div(orows, 64)));
+  int nchunks, nblk;                                    // partials of the weights and of the bias
+  if (tc) {
+    nblk = nchunks = wgrad3_chunks(w, sm_count());
+  } else if (pw) {
+    nchunks = wgrad1_chunks(w, sm_count());
+    nblk = up ? nchunks / 2 : nchunks;
+  } else {
+    if (w.ksize != 3 || w.cout_p > 64) return cudaErrorInvalidValue;
+    nchunks = std::min(ceil_div(152 * 8, taps), ceil_div(rows, kWgRows));
+    w.chunk = (long long)ceil_div(ceil_div(rows, nchunks), kWgRows) * kWgRows;
+    nchunks = ceil_div(rows, w.chunk);
+    nblk = std::min(kBiasBlocks, ceil_div(rows, 64));
+  }
   if ((long long)nchunks * per + (long long)nblk * bc > N->part_cap) return cudaErrorInvalidValue;
   w.part = N->part;
   w.bpart = N->part + (long long)nchunks * per;
@@ -895,12 +868,10 @@ cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View 
     const cudaError_t e = tc ? launch_wgrad3(w, nchunks, N->err, N->st) : launch_wgrad1(w, sm_count(), N->st);
     if (e != cudaSuccess) return e;
   } else {
-    const int mcols = std::min(64, w.cout_p);
-    const size_t smem = (size_t)kWgRows * (mcols + 8 + w.cin + 8) * sizeof(bf16);
-    launch_chain(true, k_wgrad, dim3(nchunks, taps * mchunks), 128, smem, N->st, w);
-    const long long bper = (orows + nblk - 1) / nblk;
-    launch_chain(true, k_bias_grad, nblk, kBiasThreads, 0, N->st, dout.p, dout.ld, dout.off, bc, orows, bper,
-                 w.bpart);
+    const size_t smem = (size_t)kWgRows * (w.cout_p + 8 + w.cin + 8) * sizeof(bf16);
+    launch_chain(true, k_wgrad, dim3(nchunks, taps), 128, smem, N->st, w);
+    launch_chain(true, k_bias_grad, nblk, kBiasThreads, 0, N->st, dout.p, dout.ld, dout.off, bc, rows,
+                 (rows + nblk - 1) / nblk, w.bpart);
     count_launches(2);
   }
   launch_chain(true, k_reduce_grad, ceil_div(per, kRedOut) + ceil_div(bc, kRedOut), kRedOut * kRedLanes, 0, N->st,
@@ -913,7 +884,7 @@ cudaError_t layer_bwd(bfcs_net_s* N, float* grad, int l, int B, View dout, View 
     a.cin = up ? 8 * L.cout : L.cout_p;
     a.w = N->bw[l];
     a.bias = nullptr; a.bias_mod = 1;
-    a.cout_p = L.cin_p; a.cout = L.cin_p;
+    a.cout_p = L.cin_p;
     a.ksize = L.kind == 0 ? 3 : 1;
     a.v = N->vol[lv];
     a.batch = B;

@@ -21,14 +21,6 @@ namespace net {
 
 namespace {
 
-__device__ __forceinline__ void mma16816(float* c, const unsigned* a, uint2 b) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
-}
-
 constexpr int kRowWarps = 8;
 constexpr int kRowsPerWarp = 32;
 
@@ -123,8 +115,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows(ConvArgs a, unsigned ro
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const uint2 b = wfrag[((s * NG + grp) * 4 + j) * 32 + lane];
-            mma16816(acc[0][j], af[s][0], b);
-            mma16816(acc[1][j], af[s][1], b);
+            mma16816(acc[0][j], af[s][0], b.x, b.y);
+            mma16816(acc[1][j], af[s][1], b.x, b.y);
           }
         store(grp, acc);
         __syncwarp();
@@ -140,8 +132,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_rows(ConvArgs a, unsigned ro
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const uint2 b = wfrag[((s * NG + grp) * 4 + j) * 32 + lane];
-            mma16816(acc[grp][0][j], af[0], b);
-            mma16816(acc[grp][1][j], af[1], b);
+            mma16816(acc[grp][0][j], af[0], b.x, b.y);
+            mma16816(acc[grp][1][j], af[1], b.x, b.y);
           }
       }
 #pragma unroll
@@ -207,8 +199,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_head(HeadArgs<R> a) {
     float acc[2][4] = {};
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-      mma16816(acc[0], af[s][0], w[s]);
-      mma16816(acc[1], af[s][1], w[s]);
+      mma16816(acc[0], af[s][0], w[s].x, w[s].y);
+      mma16816(acc[1], af[s][1], w[s].x, w[s].y);
     }
     if (t < 3) {                                      // columns 6 and 7 are padding
 #pragma unroll

@@ -15,8 +15,23 @@ struct Vol { int nx, ny, nz; };
 
 __device__ __forceinline__ int wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
+// c += a b of one warp (m16n8k16, BF16 operands, FP32 accumulators)
+__device__ __forceinline__ void mma16816(float* c, const unsigned* a, unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// four transposed 8 x 8 matrices from the rows at the lanes' shared-memory addresses
+__device__ __forceinline__ void ldsm_x4_trans(unsigned* r, unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
 enum InMode : int { IN_CONV = 0, IN_GATHER_UP = 1 };
-enum OutMode : int { OUT_BF16 = 0, OUT_SHUFFLE_UP = 1, OUT_F32 = 2 };
+enum OutMode : int { OUT_BF16 = 0, OUT_SHUFFLE_UP = 1 };
 
 struct ConvArgs {
   const bf16* in;     // channels-last input: element (voxel, k) at in[voxel * ldi + offi + k]
@@ -26,7 +41,6 @@ struct ConvArgs {
   const float* bias;  // bias[col % bias_mod], or null
   int bias_mod;
   int cout_p;         // GEMM columns (multiple of 8)
-  int cout;           // columns stored (OUT_F32)
   int ksize;          // 1 or 3 (circular)
   Vol v;              // grid of the GEMM rows (coarse grid for the gather / shuffle modes)
   int batch;

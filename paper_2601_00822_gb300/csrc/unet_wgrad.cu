@@ -281,18 +281,6 @@ __global__ void __launch_bounds__(kTcWorkers + 32, 1) k_wgrad3(WgArgs a, int* er
 namespace {
 
 constexpr int kW1Rows = 32;
-__device__ __forceinline__ void ldsm_x4_trans(unsigned* r, unsigned addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
-}
-__device__ __forceinline__ void mma16816(float* c, const unsigned* a, const unsigned* b) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
 
 // row pitches: 16-byte multiples that put 8 consecutive rows on distinct banks
 template <int NP, bool UP> struct W1 {
@@ -348,7 +336,7 @@ __global__ void __launch_bounds__(256) k_wgrad1(WgArgs a, unsigned rows) {
   };
   // the bias gradient rides along as one more column tile, dY times a column of ones
   float sum[C::MT][2 * NP + 1][4] = {}, acc[C::MT][2 * NP + 1][4] = {};
-  const unsigned ones[2] = {0x3F803F80u, 0x3F803F80u};
+  const unsigned ones = 0x3F803F80u;
   auto flush = [&]() {
 #pragma unroll
     for (int i = 0; i < C::MT; ++i)
@@ -380,10 +368,10 @@ __global__ void __launch_bounds__(256) k_wgrad1(WgArgs a, unsigned rows) {
         ldsm_x4_trans(af, base + ((i >> 1) * kW1Rows + ks + (mi >> 1) * 8 + rr) * C::AP + ((i & 1) * 16 + (mi & 1) * 8) * 2u);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-          mma16816(acc[i][2 * p], af, bq[p]);
-          mma16816(acc[i][2 * p + 1], af, bq[p] + 2);
+          mma16816(acc[i][2 * p], af, bq[p][0], bq[p][1]);
+          mma16816(acc[i][2 * p + 1], af, bq[p][2], bq[p][3]);
         }
-        mma16816(acc[i][2 * NP], af, ones);
+        mma16816(acc[i][2 * NP], af, ones, ones);
       }
     }
     if (((u - u0) & 3) == 3) flush();
