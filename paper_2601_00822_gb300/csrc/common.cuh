@@ -131,9 +131,9 @@ template <typename R, int DIR> __device__ __forceinline__ C2<R> mul_di(C2<R> a) 
 
 // Complex sum and difference of the register butterflies.  FP32 with P (packed): both
 // parts in one instruction, with the same roundings; the passes along lines are short of
-// issue slots.  Cold, per launch: y pass of 256^3 117 -> 103 us, x pass 166 -> 160 us, of
-// 16 members of 64^3 52.9 -> 51.9 us, z pass 75.9 -> 74.8 us; the z pass of 256 lines took
-// 308 us instead of 298 and stays with single instructions (kPackZ).
+// issue slots.  Under the profiler (each launch alone): y pass of 256^3 117 -> 103 us, x
+// pass 166 -> 160 us, of 16 members of 64^3 52.9 -> 51.9 us, z pass 75.9 -> 74.8 us; the z pass of 256 lines took 308 us instead of 298 and stays with single instructions
+// (kPackZ).  In a solve, between other kernels, the 256^3 passes take 131 us (y) and 209 us (x).
 template <typename R, bool P> __device__ __forceinline__ C2<R> badd(C2<R> a, C2<R> b) {
   if constexpr (P && std::is_same<R, float>::value) {
     C2<R> r;

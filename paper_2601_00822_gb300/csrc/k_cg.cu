@@ -22,7 +22,8 @@ namespace bfcs {
 
 // Vector kernels.  In FP64 they are bound by the FP64 pipe (about 45 operations a mode
 // and two lanes an SM: 9.4 us at 64^3 when every SM has the same share), so the work has
-// to be even: blocks of 128 threads, one mode a thread, up to the eight blocks an SM holds.
+// to be even: blocks of 128 threads, one mode a thread, up to the eight blocks that each of
+// the 152 SMs holds (kCgParts; a chip with fewer would run a second round of blocks).
 // 512 blocks of 256 (20 us a launch) gave some SMs four blocks and others three, and 16
 // blocks a second round.  A 64^3 FP64 solve 37.8 -> 36.0 ms.  FP32 vectors, bound by
 // memory, keep 512 blocks of 256.

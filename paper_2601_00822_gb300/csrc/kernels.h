@@ -9,12 +9,12 @@ namespace bfcs {
 // Launch of a kernel that begins with chain_wait() (common.cuh), chained to its predecessor
 // when `chain` is set.  The Krylov loops chain their 8-10 launches per iteration (plain
 // stream launches with one-block kernels between the passes: a 128^3 solve by Algorithm 3
-// 38.9 -> 34.8 ms, a 64^3 FP64 solve by Algorithm 2 36.0 -> 33.6 ms with the vectors and
-// scalars chained instead of everything); the sweeps do not:
+// 38.9 -> 34.8 ms; a 64^3 FP64 solve by Algorithm 2 36.0 -> 33.6 ms beside each other with
+// the vectors and scalars chained instead of everything); the sweeps do not:
 // their launches sit in CUDA graphs, whose gaps are small already, and blocks that wait on
 // an SM disturb the placement of the running pass (32^3 FP64 8.7 -> 11.0 ms, 64^3 3.54 ->
 // 3.66 ms, 256^3 121 -> 124 ms when chained).  The network chains all of its launches (26 a
-// forward pass of some microseconds each at 32^3): one 32^3 sample 242 -> 195 us, and 160
+// forward pass of some microseconds each at 32^3): one 32^3 sample 242 -> 189 us, and 160
 // us with the layers' parameters loaded before the wait.
 //
 // Of an FP64 Krylov loop only the vector kernels and scalars are chained (chain_passes).
@@ -160,7 +160,7 @@ struct CgState {
   int best_it;           // iteration of `best`; no new best for kCgStagnation iterations ends the member
 };
 constexpr int kCgStagnation = 50;
-constexpr int kCgParts = 152 * 8;   // most partial sums per member: one block each, eight blocks an SM
+constexpr int kCgParts = 152 * 8;   // most partial sums per member: one block each, eight for each of a GB300's SMs
 template <typename R> struct CgArgs {
   C2<R>* c;              // iterate (state layout, members at ms)
   C2<R>* r;              // residual

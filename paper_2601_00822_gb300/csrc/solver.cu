@@ -811,7 +811,9 @@ int run_sets(std::vector<SweepSet<R>*>& sets, int maxit) {
   // The graph of G sweeps.  Its kernels take everything that belongs to a call from device
   // memory (Member, IterState), so a single set's graph depends on the plan, the batch size
   // and the material alone and is kept in the plan: capturing and instantiating it took
-  // 0.25 ms, three times in a 3.3 ms solve of 64^3 through the ladder.
+  // 0.25 ms, three times in a 3.3 ms solve of 64^3 through the ladder.  The plan keeps one: a
+  // call with another material or batch size than the last captures again, as every call did
+  // before.
   cudaGraphExec_t gexec = nullptr;
   long long gkernels = 0;
   struct GraphGuard {

@@ -385,8 +385,9 @@ struct SqSum {
 // relative squared L2 loss: per (block, sample) sums of (p - t)^2 and t^2; one voxel
 // per thread, planar fields (6 x n a sample).  The squares of a voxel are added in FP32
 // pieces without loss (SqSum), voxels in FP64: with every term on the FP64 pipe the pass
-// took 143 us for 8 samples of 64^3 instead of the 15 us its 100 MB take.  Voxels with
-// values outside the range of that form (tiny, huge, not finite) are formed in FP64.
+// took 143 us for 8 samples of 64^3, now 63 us alone under the profiler; its 100 MB take
+// 15.  Voxels with values outside the range of that form (tiny, huge, not finite) are
+// formed in FP64.
 constexpr int kLossBlocks = 64;
 __global__ void k_loss(const float* pred, const float* target, long long n, double* num, double* den) {
   chain_wait();

@@ -33,7 +33,9 @@
 // clock; 24 per tile, so 1344 clocks against 9 * 8 * 40 = 2880 with one MMA per (dy,
 // dx) on a plain dY plane, and staging three dY copies adds about 270 clocks of writes.
 // The 3^3 layers of a gradient over 8 samples of 64^3 take 0.79 ms together, 3.48 ms with
-// nine warps of mma.sync and sums over the blocks as a launch of their own.
+// nine warps of mma.sync and sums over the blocks as a launch of their own.  A thread keeps
+// 144 running sums; the ninth warp makes one quarter of an SM hold three, which leaves 168
+// registers a thread, and 420 bytes of the staging's state spill (-Xptxas -v).
 #include "unet_kernels.h"
 #include "unet_tc.cuh"
 #include "unet_wgrad_flow.h"
